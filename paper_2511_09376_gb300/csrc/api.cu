@@ -87,6 +87,7 @@ void free_ensemble(wdf_ensemble *e) {
     dfree(e->d_nodes); dfree(e->d_keys); dfree(e->d_group_leaf); dfree(e->d_leaf_row);
     dfree(e->d_w_rows); dfree(e->d_tiles); dfree(e->d_t32);
     dfree(e->d_rec); dfree(e->d_meta); dfree(e->d_flfeat); dfree(e->d_xmask); dfree(e->d_cols); dfree(e->d_col_thr);
+    dfree(e->d_unit); dfree(e->d_scol); dfree(e->d_spack); dfree(e->d_sgroup); dfree(e->d_sthr);
     dfree(e->d_apk); dfree(e->d_bpk); dfree(e->d_tiles128); dfree(e->d_err); dfree(e->d_A); dfree(e->d_ratio);
     dfree(e->d_hist); dfree(e->d_vc); dfree(e->d_scale); dfree(e->d_S); dfree(e->d_sfold); dfree(e->d_base);
     dfree(e->d_lines);
@@ -148,16 +149,15 @@ wdf_status ensure_staging(wdf_ensemble *e, int64_t rows, bool out) {
 // a multiple of the largest background tile), nbuf of them.
 constexpr int64_t kCodeRows = 1 << 20;
 wdf_status ensure_codes(wdf_ensemble *e, int64_t rows, int nbuf) {
-    const int64_t tile = wdf::kBgMaxTileRows;
+    const int64_t tile = wdf::kBgTileRows;
     rows = std::min((rows + tile - 1) / tile * tile, kCodeRows);
-    const size_t xb = e->pk.cols.size() * (size_t)e->pk.code_bytes;
     if (rows > e->code_rows) {
         WDF_CUDA(cudaDeviceSynchronize());
         for (int i = 0; i < 2; ++i) dfree(e->d_codes[i]);
         e->code_rows = rows;
     }
     for (int i = 0; i < nbuf; ++i)
-        if (!e->d_codes[i]) WDF_CUDA(dalloc(&e->d_codes[i], (size_t)e->code_rows * xb, &e->bytes));
+        if (!e->d_codes[i]) WDF_CUDA(dalloc(&e->d_codes[i], (size_t)e->code_rows / 32 * e->pk.quads * 16, &e->bytes));
     return WDF_OK;
 }
 
@@ -172,8 +172,8 @@ wdf_status count_device_rows(wdf_ensemble *ens, const float *B, int64_t m, int64
     if (s == WDF_OK && overlap) s = ensure_streams(ens);
     if (s != WDF_OK) return s;
     wdf::BgOverlap ov{ens->d_codes[1], ens->ist[0], {ens->ev_enc[0], ens->ev_enc[1]}, {ens->ev_cnt[0], ens->ev_cnt[1]}};
-    WDF_CUDA(wdf::launch_bg_hist(p.D, B, m, ldb, ens->arrays(), p.T, ens->d_codes[0], ens->code_rows, hist,
-                                 ens->ctx->dev, st, overlap ? &ov : nullptr));
+    WDF_CUDA(wdf::launch_bg_hist(p.D, B, m, ldb, ens->arrays(), ens->slices(), p.T, ens->d_codes[0],
+                                 ens->code_rows, hist, ens->ctx->dev, st, overlap ? &ov : nullptr));
     return WDF_OK;
 }
 
@@ -382,6 +382,11 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
     if (!p.xmask.empty()) chk(dalloc(&e->d_xmask, p.xmask.size(), &e->bytes));
     chk(dalloc(&e->d_cols, p.cols.size(), &e->bytes));
     chk(dalloc(&e->d_col_thr, std::max<size_t>(p.col_thr.size(), 1), &e->bytes));
+    chk(dalloc(&e->d_unit, p.unit.size(), &e->bytes));
+    chk(dalloc(&e->d_scol, p.scol.size(), &e->bytes));
+    chk(dalloc(&e->d_spack, p.spack.size(), &e->bytes));
+    chk(dalloc(&e->d_sgroup, p.sgroup.size(), &e->bytes));
+    chk(dalloc(&e->d_sthr, p.sthr.size(), &e->bytes));
     if (ce == cudaSuccess) {
         chk(cudaMemcpy(e->d_nodes, nodes.data(), nodes.size() * sizeof(int2), cudaMemcpyHostToDevice));
         if (e->G) chk(cudaMemcpy(e->d_keys, p.sig_key.data(), p.sig_key.size() * 4, cudaMemcpyHostToDevice));
@@ -398,6 +403,12 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
         chk(cudaMemcpy(e->d_cols, p.cols.data(), p.cols.size() * sizeof(wdf::CodeCol), cudaMemcpyHostToDevice));
         if (!p.col_thr.empty())
             chk(cudaMemcpy(e->d_col_thr, p.col_thr.data(), p.col_thr.size() * 4, cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(e->d_unit, p.unit.data(), p.unit.size() * sizeof(wdf::UnitNode), cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(e->d_scol, p.scol.data(), p.scol.size() * sizeof(wdf::SliceCol), cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(e->d_spack, p.spack.data(), p.spack.size() * sizeof(wdf::SlicePack), cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(e->d_sgroup, p.sgroup.data(), p.sgroup.size() * sizeof(wdf::SliceGroup),
+                       cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(e->d_sthr, p.sthr.data(), p.sthr.size() * 4, cudaMemcpyHostToDevice));
         if (e->n_tiles) chk(cudaMemcpy(e->d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice));
         // step 2 of Algorithm 3 depends only on the path signatures: build the tables now
         chk(wdf::launch_tables(p.D, e->metric, e->d_keys, e->G, e->d_t32, nullptr, 0));
@@ -490,8 +501,8 @@ wdf_status wdf_set_background(wdf_ensemble *ens, const float *B, int64_t m, int6
             const int b = (int)(chunk & 1);
             WDF_CUDA(copy_rows(ens->d_stage_in[b], p.F, B + r0 * ldb, ldb, rows, p.F, cudaMemcpyHostToDevice,
                                ens->ist[b]));
-            WDF_CUDA(wdf::launch_bg_hist(p.D, ens->d_stage_in[b], rows, p.F, ens->arrays(), p.T, ens->d_codes[b],
-                                         ens->code_rows, ens->d_hist, ens->ctx->dev, ens->ist[b]));
+            WDF_CUDA(wdf::launch_bg_hist(p.D, ens->d_stage_in[b], rows, p.F, ens->arrays(), ens->slices(), p.T,
+                                         ens->d_codes[b], ens->code_rows, ens->d_hist, ens->ctx->dev, ens->ist[b]));
         }
         for (int i = 0; i < 2; ++i) {
             WDF_CUDA(cudaEventRecord(ens->ev_join[i], ens->ist[i]));

@@ -2,18 +2,11 @@
 // (Algorithm 1, kept in registers) and their counts vc[l][p_b] (Eq.
 // "bg_shap_derivation" step (d)); plus the per-leaf marginals and E_b f(b).
 //
-// K1 counts, per tree and bottom subtree, the joint entry e = (pattern at the subtree
-// root, the three decisions inside the subtree) of every background row: one shared
-// memory increment per (row, tree, live bottom subtree) instead of one per leaf.  The
-// four leaf patterns of the subtree are functions of e, so per-leaf counts are exact
-// marginals of these joint counts (the sibling-leaf observation of section
-// "Algorithmic Improvements" item 3, applied two levels up).
-//
-// Work split: the rows are first encoded to decision codes (tree_layout.h, one pass
-// over B); the trees are cut into chunks whose counters fit in shared memory as 16-bit
-// halves of 32-bit words; blocks are numbered chunk-fastest, so the blocks that stage
-// the same code tile run at the same time and share it through L2.  A block flushes
-// its 16-bit counters into the global 32-bit counts before any can overflow.
+// The joint entry e = (pattern at a bottom subtree's root, the three decisions inside the
+// subtree) of every background row is counted per tree and live bottom subtree; the four leaf
+// patterns of the subtree are functions of e, so per-leaf counts are exact marginals of
+// these joint counts (the sibling-leaf observation of section "Algorithmic Improvements"
+// item 3, applied two levels up).
 #include <algorithm>
 #include <cstdlib>
 
@@ -22,268 +15,336 @@
 
 namespace wdf {
 
-// 16-bit counter slots in shared memory.  The rows of one warp increment the entries of
-// one (tree, subtree) together, and background entries are far from uniform (a warp's
-// most frequent entry is hit by about a quarter of its lanes), so lanes that land in
-// one bank serialise.  Two rules spread them: the two halves of a 32-bit word hold the
-// same entry of two sibling subtrees (so one instruction touches one entry per word),
-// and the word of entry e within its subtree pair is fold(e), which XORs the higher
-// entry bits into the five bank bits.  fold is its own inverse (bits 5 and up pass
-// through unchanged).
-__host__ __device__ __forceinline__ uint32_t bg_fold(uint32_t e) {
-    return e ^ ((e >> 5) & 31u) ^ ((e >> 10) & 31u);
+// Counting on the tensor cores.  A joint count is a sum over rows of products of indicators:
+// count(R, n) = sum_rows [ancestor decisions = R] [subtree decisions = n], so 16 ancestor
+// patterns x 8 subtree patterns of one bottom subtree are a small matrix product over rows
+// with operands built in registers from the rows' decision bits.  A warp owns one unit
+// (tree_layout.h) and keeps all its counters in registers; no counter is touched in memory
+// until the block's rows are done.
+//
+// Per tile of 128 rows a warp
+//   - evaluates its unit's 31 nodes, lane = node, for 32 rows at a time on the sliced codes
+//     (two or three 16-byte shared loads and 8 or 12 logic instructions per 32 x 32 decisions;
+//     the rank masks stay in registers for the whole launch) and exchanges the decision
+//     words through shared memory: lane (g, q) = (lane / 4, lane % 4) needs all nodes' words
+//     of row block q, the rows its MMA fragments cover;
+//   - forms the indicator words: ancestor pattern g (and g + 8, for the MMA's upper rows)
+//     per sibling pair of subtrees, which share their ancestors, and subtree pattern g;
+//   - expands each word into eight FP16-pair registers, two rows per FP16 value, so that four
+//     m16n8k16 MMAs cover the tile.  An FP16 value with only bits 0..10 set is that integer
+//     times 2^-24.  The ancestor side keeps bits j and j + 8 of each half (one AND, the shift
+//     shared by three registers); the subtree side, whose words are stored with the bits of
+//     each half reversed, puts the same two rows at bits 10 - j and 2 - j.  Every product is
+//     then 2^10 (a b + a' b') + 2^2 a b' + 2^18 a' b, in units of 2^-48: the wanted sum over
+//     the tile (at most 128) and the two cross sums (at most 64) are separate bytes of the
+//     FP32 accumulator, which starts from 2^-23 so that its mantissa is their integer;
+//   - adds the middle byte of every accumulator to an integer counter.
+// E4M3, 8-bit integer and 1-bit MMAs are emulated here (20, 17 and 142 issue slots per
+// instruction); one row per FP16 value takes twice the MMAs and nearly twice the logic.
+// Bound by the logic pipe (58 % busy, issue 55 %): 2.31 ms per 1M rows and 200 trees of depth 6,
+// where one shared-memory atomic per (row, bottom subtree), each row's decisions made node by
+// node, took 5.14 ms; depth 7, 100 trees: 3.95 ms per 1M rows against 6.5.  Depth 8 is
+// latency-bound at 8 warps per SM (128 counters per lane) and took as long either way.
+template <int D>
+struct Unit {
+    static constexpr int H = unit_height(D), TOP = unit_top(D), UPT = units_per_tree(D);
+    static constexpr int NLOC = (1 << H) - 1, NSU = 1 << (H - 2);  // nodes and bottom subtrees
+    static constexpr int TILES = TOP > 0 ? 1 << (TOP - 1) : 1;     // m16 tiles of ancestor patterns
+    static constexpr int WMAX = D <= 6 ? 16 : (D == 7 ? 12 : 8);   // warps per block (registers)
+};
+constexpr int kDecStride = 36;  // words of a row block's decision words: 9 * 16 bytes, so that the
+                                // four row blocks of a fragment lie in different banks
+
+constexpr float kCountBase = 0x1p-23f;  // an accumulator with all three sums zero
+
+__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                        uint32_t b1, const float *c) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
 }
 
-template <int D>
-__device__ __forceinline__ uint32_t bg_slot(int g, int s, uint32_t e) {
-    using S = Shape<D>;
-    if constexpr (S::NS == 1)
-        return (uint32_t)g * S::E + e;
-    else
-        return (((uint32_t)g * (S::NS / 2) + (uint32_t)(s >> 1)) * S::E + bg_fold(e)) * 2u + (uint32_t)(s & 1);
-}
-
-// Adds the shared counters of a block's trees into the global 32-bit counts ([tree]
-// [subtree][entry], gdst at the block's first tree) and zeroes them.
-template <int D>
-__device__ void bg_flush(uint32_t *sh, uint32_t *gdst, int bins, int tid, int nthreads) {
-    using S = Shape<D>;
-    for (int i = tid; i < bins / 2; i += nthreads) {
-        const uint32_t v = sh[i];
-        sh[i] = 0u;
-        if (!v) continue;
-        size_t i0, i1;
-        if constexpr (S::NS == 1) {
-            i0 = 2 * (size_t)i;
-            i1 = i0 + 1;
-        } else {
-            const uint32_t pair = (uint32_t)i / S::E, e = bg_fold((uint32_t)i % S::E);
-            i0 = (size_t)(2 * pair) * S::E + e;  // subtree 2k of the pair; 2k + 1 is E further
-            i1 = i0 + S::E;
-        }
-        if (v & 0xFFFFu) atomicAdd(gdst + i0, v & 0xFFFFu);
-        if (v >> 16) atomicAdd(gdst + i1, v >> 16);
+// A word and its shifts by 3 and 6, so that rows j and j + 8 of each half are bits i and i + 8
+// (i = j % 3) of shift j / 3.
+struct Shifts {
+    uint32_t w[3];
+    __device__ __forceinline__ void set(uint32_t x) {
+        w[0] = x; w[1] = (x >> 3); w[2] = (x >> 6);
     }
+};
+// Register j: rows j and j + 8 of each half of x & y, at bits i and i + 8.
+__device__ __forceinline__ void expand_a(const Shifts &x, const Shifts &y, uint32_t (&r)[8]) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) r[j] = x.w[j / 3] & y.w[j / 3] & (0x01010101u << (j % 3));
+}
+// The same rows, from a word with each half's bits reversed, at bits 10 - i and 2 - i.
+__device__ __forceinline__ void expand_b(uint32_t y, uint32_t (&r)[8]) {
+    const uint32_t y0 = (y >> 5), y3 = (y >> 2), y6 = y << 1;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) r[j] = (j < 3 ? y0 : j < 6 ? y3 : y6) & (0x01010101u << (2 - j % 3));
 }
 
-// Shared memory layout (bytes, 16-aligned pieces): code tile | tree metadata | node
-// records | 16-bit counters.
-template <int D>
-struct BgLayout {
-    size_t x, meta, rec, hist, total;
-    static __host__ __device__ size_t up(size_t v) { return (v + 15) & ~(size_t)15; }
-    __host__ __device__ BgLayout(int xb, int RT, int G, bool smem_hist) {
-        x = up((size_t)RT * xb);
-        meta = up((size_t)G * sizeof(TreeMeta));
-        rec = up((size_t)G * Shape<D>::NI * sizeof(NodeRec));
-        hist = smem_hist ? up((size_t)G * Shape<D>::NS * Shape<D>::E * 2) : 0;
-        total = x + meta + rec + hist;
+// The decision words of one node for the four row blocks of a tile.
+struct SliceNode {
+    uint32_t at, m[3][4];
+    __device__ __forceinline__ void load(const UnitNode *p) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        at = v.x;
+        set(m[0], v.y); set(m[1], v.z); set(m[2], v.w);
+    }
+    __device__ __forceinline__ static void set(uint32_t (&d)[4], uint32_t r) {
+        d[0] = rank_mask<0>(r); d[1] = rank_mask<1>(r); d[2] = rank_mask<2>(r); d[3] = rank_mask<3>(r);
+    }
+    __device__ __forceinline__ uint32_t decide1(const uint4 *block, const SliceArrays &sa) const {
+        const int col = (int)(at & 0xFFFFu), nq = (int)((at >> 16) & 15u);
+        uint32_t w = 0u - ((at >> 20) & 1u);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k < nq) w = slice_le(w, block[sa.qbase[k] + col], m[k]);
+        return w;
+    }
+    __device__ __forceinline__ void decide(const uint4 *tile, const SliceArrays &sa, uint32_t (&w)[4]) const {
+        const int col = (int)(at & 0xFFFFu), nq = (int)((at >> 16) & 15u);
+        const uint32_t le0 = 0u - ((at >> 20) & 1u);
+#pragma unroll
+        for (int b = 0; b < 4; ++b) w[b] = le0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            if (k < nq) {
+                uint4 q[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) q[b] = tile[b * sa.quads + sa.qbase[k] + col];
+#pragma unroll
+                for (int b = 0; b < 4; ++b) w[b] = slice_le(w[b], q[b], m[k]);
+            }
+        }
     }
 };
 
-// 16-byte code words per thread of the next tile held in registers (512-row tiles of up to
-// 128 one-byte codes per row fit entirely): 1.8 % off the large workload's background
-// step.  None at depth 5, where the registers made the compiler spill, nor for deep
-// trees, whose decision loop needs them.
-template <int D>
-__host__ __device__ constexpr int bg_prefetch() { return D <= 6 && D != 5 ? 8 : 0; }
-
-// codes: rows [0, m) of one encoded chunk, padded to a multiple of RT rows.
-template <int D, int RT, bool SMEM>
-__global__ void __launch_bounds__(RT) k_bg_hist(const unsigned char *__restrict__ codes, int64_t m, TreeArrays ta,
-                                                int T, int G, int chunks, uint32_t *__restrict__ hist) {
+// codes: rows [0, m) of one encoded chunk, padded to a multiple of 128 rows.  Block (chunk,
+// slice): units [chunk * W, ...), one per warp, over the tiles of 128 rows slice, slice +
+// nslices, ... in runs of SUB tiles.  STAGES runs in shared memory, filled by cp.async ahead
+// of their use (a barrier per run); STAGES = 0 reads the codes from global memory (rows too wide for two tiles).
+template <int D, int STAGES, int SUB>
+__global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsigned char *__restrict__ codes, int64_t m,
+                                                                   SliceArrays sa, const TreeMeta *__restrict__ meta,
+                                                                   int units, int chunks, uint32_t *__restrict__ hist) {
     using S = Shape<D>;
+    using N = Unit<D>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int cb = ta.code_bytes, xb = ta.n_cols * cb;
-    const BgLayout<D> L(xb, RT, G, SMEM);
-    unsigned char *sx = smem_raw;
-    TreeMeta *smeta = reinterpret_cast<TreeMeta *>(smem_raw + L.x);
-    int4 *srec = reinterpret_cast<int4 *>(smem_raw + L.x + L.meta);
-    uint32_t *sh = reinterpret_cast<uint32_t *>(smem_raw + L.x + L.meta + L.rec);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int chunk = blockIdx.x % chunks;
-    const int slice = blockIdx.x / chunks, nslices = gridDim.x / chunks;
-    const int t0 = chunk * G;
-    const int g_cnt = min(G, T - t0);
-    const int bins = g_cnt * S::NS * S::E;  // 16-bit counters, two per word
-    uint32_t *gdst = hist + (size_t)t0 * S::NS * S::E;
-    stage_trees<D>(t0, g_cnt, ta.rec, ta.meta, srec, smeta, tid, RT);
-    if (SMEM)
-        for (int i = tid; i < bins / 2; i += RT) sh[i] = 0u;
-    const CodeReader xr(sx + (size_t)warp * 32 * xb, lane, cb);
-    const int tile16 = RT * xb / 16;
-    // The first bg_prefetch 16-byte words per thread of the next tile are loaded into
-    // registers while the current tile is counted (the rest, for wide rows, at staging).
-    constexpr int PF = bg_prefetch<D>();
-    uint4 pf[PF > 0 ? PF : 1];
-    auto fetch = [&](int64_t r0) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(codes + r0 * xb);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
+    const int chunk = blockIdx.x % chunks, slice = blockIdx.x / chunks, nslices = gridDim.x / chunks;
+    const int unit = min(chunk * W + warp, units - 1);  // a spare warp repeats the last unit and adds nothing
+    const int t = unit / N::UPT, u = unit % N::UPT;
+    const int tile16 = 4 * sa.quads, run16 = SUB * tile16;  // 16-byte words of a tile, of a run
+    uint4 *ring = reinterpret_cast<uint4 *>(smem_raw);
+    uint32_t *dec = reinterpret_cast<uint32_t *>(smem_raw + (size_t)STAGES * run16 * 16) + warp * 4 * kDecStride;
+    const int64_t tiles = (m + kBgTileRows - 1) / kBgTileRows, runs = (tiles + SUB - 1) / SUB;
+
+    SliceNode node, top;  // this lane's node; top node 1 + lane / 4 of the unit's path, for row block lane % 4
+    {
+        const UnitNode *un = sa.unit + (size_t)unit * 32 + lane;
+        if (N::TOP > 0 && lane == 31) un = sa.unit + (size_t)t * N::UPT * 32 + 31;  // the root
+        node.load(un);
+        if constexpr (N::TOP > 1) {
+            const int k = min(1 + (lane >> 2), N::TOP - 1), v = (1 << k) - 1 + (u >> (N::TOP - k));
+            top.load(sa.unit + ((size_t)t * N::UPT + v) * 32 + 31);
+        }
+    }
+    const uint32_t live = (uint32_t)(__ldg(&meta[t].live) >> (u * N::NSU)) & ((1u << N::NSU) - 1u);
+    const bool flip = lane >= N::NSU - 1 && lane < N::NLOC;  // nodes of a bottom subtree
+    const int g = lane >> 2, q = lane & 3;
+    const uint32_t x0 = (g & 4) ? 0u : ~0u, x1 = (g & 2) ? 0u : ~0u, x2 = (g & 1) ? 0u : ~0u;
+    uint32_t count[N::NSU][N::TILES][4];
 #pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const int i = tid + k * RT;
-            if (i < tile16) pf[k] = __ldg(src + i);
+    for (int s = 0; s < N::NSU; ++s)
+#pragma unroll
+        for (int i = 0; i < N::TILES; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) count[s][i][k] = 0u;
+
+    const float base[4] = {kCountBase, kCountBase, kCountBase, kCountBase};
+    auto fetch = [&](int64_t run, int stage) {
+        if constexpr (STAGES > 0) {
+            if (run < runs) {
+                const int n = (int)min((int64_t)SUB, tiles - run * SUB) * tile16;
+                const uint4 *src = reinterpret_cast<const uint4 *>(codes) + run * run16 + tid;
+                uint32_t dst = (uint32_t)__cvta_generic_to_shared(ring + (size_t)stage * run16 + tid);
+                for (int i = tid; i < n; i += blockDim.x, src += blockDim.x, dst += 16u * blockDim.x)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src));
+            }
+            asm volatile("cp.async.commit_group;");
         }
     };
-    const int64_t step = (int64_t)nslices * RT;
-    if (PF > 0 && (int64_t)slice * RT < m) fetch((int64_t)slice * RT);
-    int64_t since_flush = 0;
-    for (int64_t row0 = (int64_t)slice * RT; row0 < m; row0 += step) {
-        __syncthreads();
-        if (SMEM && since_flush + RT > 65535) {  // a 16-bit counter could overflow: flush
-            bg_flush<D>(sh, gdst, bins, tid, RT);
-            since_flush = 0;
-        }
-        // the tile's RT rows are RT / 32 consecutive code blocks
 #pragma unroll
-        for (int k = 0; k < PF; ++k) {
-            const int i = tid + k * RT;
-            if (i < tile16) reinterpret_cast<uint4 *>(sx)[i] = pf[k];
+    for (int k = 0; k + 1 < STAGES; ++k) fetch(slice + (int64_t)k * nslices, k);
+    int stage = 0;
+    for (int64_t run = slice; run < runs; run += nslices) {
+        const uint4 *src;
+        if constexpr (STAGES > 0) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES > 1 ? STAGES - 2 : 0));
+            __syncthreads();
+            const int into = stage == 0 ? STAGES - 1 : stage - 1;
+            fetch(run + (int64_t)(STAGES - 1) * nslices, into);
+            src = ring + (size_t)stage * run16;
+            stage = stage + 1 == STAGES ? 0 : stage + 1;
+        } else {
+            src = reinterpret_cast<const uint4 *>(codes) + run * run16;
         }
-        const uint4 *src = reinterpret_cast<const uint4 *>(codes + row0 * xb);
-        for (int i = tid + PF * RT; i < tile16; i += RT) reinterpret_cast<uint4 *>(sx)[i] = __ldg(src + i);
-        __syncthreads();
-        if (PF > 0 && row0 + step < m) fetch(row0 + step);
-        since_flush += RT;
-        const bool valid = row0 + tid < m;
-        for (int g = 0; g < g_cnt; ++g) {
-            const TreeMeta &mt = smeta[g];
-            uint32_t dw[S::NW];
-            if (cb == 1)
-                tree_decisions<D, true>(srec + (size_t)g * S::NI, mt, xr, dw);
-            else
-                tree_decisions<D, false>(srec + (size_t)g * S::NI, mt, xr, dw);
-            uint32_t ent[S::NS];
-            subtree_entries<D>(dw, ent);
-            const uint64_t lv = mt.live;
+        const int here = (int)min((int64_t)SUB, tiles - run * SUB);
+        int left = (int)min(m - run * SUB * kBgTileRows, (int64_t)(1 << 30)) - 32 * q;  // rows from row block q on
+#pragma unroll 1
+        for (int sub = 0; sub < here; ++sub, src += tile16, left -= kBgTileRows) {
+            uint32_t w[4];
+            node.decide(src, sa, w);
 #pragma unroll
-            for (int s = 0; s < S::NS; ++s) {
-                if (((lv >> s) & 1ull) && valid) {
-                    if (SMEM) {
-                        const uint32_t sl = bg_slot<D>(g, s, ent[s]);
-                        atomicAdd(sh + (sl >> 1), 1u << ((sl & 1u) << 4));
-                    } else {
-                        atomicAdd(gdst + (uint32_t)(g * S::NS + s) * S::E + ent[s], 1u);
-                    }
+            for (int b = 0; b < 4; ++b) dec[b * kDecStride + lane] = flip ? __byte_perm(__brev(w[b]), 0u, 0x1032) : w[b];
+            if constexpr (N::TOP > 1) {
+                if (lane < 4 * (N::TOP - 1)) dec[q * kDecStride + 32 + (lane >> 2)] = top.decide1(src + q * sa.quads, sa);
+            }
+            __syncwarp();
+            constexpr int NV = (N::NLOC + 3) / 4;
+            uint32_t d[4 * NV > 32 ? 4 * NV : 32], pre[4];
+            const uint32_t *mine = dec + q * kDecStride;
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const uint4 v = reinterpret_cast<const uint4 *>(mine)[i];
+                d[4 * i] = v.x; d[4 * i + 1] = v.y; d[4 * i + 2] = v.z; d[4 * i + 3] = v.w;
+            }
+            pre[0] = N::TOP > 0 ? d[31] : 0u;
+            if constexpr (N::TOP > 1) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(mine + 32);
+                pre[1] = v.x; pre[2] = v.y;
+            }
+            __syncwarp();
+            const uint32_t valid = left >= 32 ? ~0u : (left > 0 ? (1u << left) - 1u : 0u);
+            // rows whose top decisions are c (root in the highest bit)
+            uint32_t path[1 << N::TOP];
+            path[0] = valid;
+#pragma unroll
+            for (int k = 0; k < N::TOP; ++k)
+#pragma unroll
+                for (int c = (1 << k) - 1; c >= 0; --c) {
+                    path[2 * c + 1] = path[c] & pre[k];
+                    path[2 * c] = path[c] & ~pre[k];
+                }
+            Shifts in[1 << N::TOP];
+#pragma unroll
+            for (int c = 0; c < 1 << N::TOP; ++c) in[c].set(path[c]);
+            constexpr int NP = N::NSU > 1 ? N::NSU / 2 : 1;  // sibling pairs
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                // the pair's ancestors inside the unit: the last three decisions of the pattern
+                uint32_t anc = ~0u;
+                if constexpr (N::H == 5) anc = (d[0] ^ x0) & (d[1 + (j >> 1)] ^ x1) & (d[3 + j] ^ x2);
+                if constexpr (N::H == 4) anc = (d[0] ^ x1) & (d[1 + j] ^ x2);
+                if constexpr (N::H == 3) anc = d[0] ^ x2;
+                Shifts own;
+                own.set(anc);
+                uint32_t rb[2][8];
+#pragma unroll
+                for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h) {
+                    const int r = N::NSU - 1 + 2 * j + h;  // subtree root; entry low bits: r, 2r + 2, 2r + 1
+                    expand_b((d[r] ^ x0) & (d[2 * r + 2] ^ x1) & (d[2 * r + 1] ^ x2), rb[h]);
+                }
+#pragma unroll
+                for (int i = 0; i < N::TILES; ++i) {
+                    uint32_t ra[2][8];
+                    expand_a(own, in[N::TOP > 0 ? 2 * i : 0], ra[0]);
+                    if constexpr (N::TOP > 0) expand_a(own, in[2 * i + 1], ra[1]);
+                    float acc[2][4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+#pragma unroll
+                        for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h)
+                            mma_f16(acc[h], ra[0][2 * k], N::TOP > 0 ? ra[1][2 * k] : 0u, ra[0][2 * k + 1],
+                                    N::TOP > 0 ? ra[1][2 * k + 1] : 0u, rb[h][2 * k], rb[h][2 * k + 1],
+                                    k == 0 ? base : acc[h]);
+#pragma unroll
+                    for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h)
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            count[2 * j + h][i][k] = __dp4a(__float_as_uint(acc[h][k]), 0x00000100u, count[2 * j + h][i][k]);
                 }
             }
         }
     }
-    if (SMEM) {
-        __syncthreads();
-        bg_flush<D>(sh, gdst, bins, tid, RT);
+    if (chunk * W + warp >= units) return;
+#pragma unroll
+    for (int s = 0; s < N::NSU; ++s) {
+        if (!((live >> s) & 1u)) continue;
+        uint32_t *h = hist + ((size_t)t * S::NS + u * N::NSU + s) * S::E;
+#pragma unroll
+        for (int i = 0; i < N::TILES; ++i)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                // accumulator k: pattern row g (+ 8 for k >= 2), subtree pattern 2q + (k & 1)
+                const uint32_t R = N::TOP > 0 ? (uint32_t)((2 * i + (k >> 1)) << 3) | (uint32_t)g
+                                              : (uint32_t)g + 8u * (k >> 1);
+                const uint32_t c = count[s][i][k];
+                if (R < (uint32_t)(S::E >> 3) && c) atomicAdd(h + ((R << 3) | (2 * q + (k & 1))), c);
+            }
     }
 }
 
-// Tree chunking of one launch: G trees per block with counters in shared memory whenever
-// one tree's counters fit beside the code tile; otherwise the counts go straight to
-// global memory and only the node records are chunked.  Deep trees (64 KB of counters
-// per depth-8 tree) then take one to a few trees per block and hundreds of chunks, each
-// block streaming every code tile through shared memory (from L2, where the blocks
-// walking the same tiles meet): 47.5 instead of 62.8 ms per 1M rows for 500 trees of
-// depth 7, 203 instead of 254 ms for 1000 of depth 8, against global-memory atomics.
-// With counters in shared memory G is chosen by a cost model rather than as
-// the most that fits: the blocks of a launch (chunks x row slices) are all resident, a
-// block's work is its tiles times (G trees + about one tree's worth for staging the
-// tile), and the busiest SM runs ceil(blocks / SMs) of them.  So 200 trees go in 8
-// chunks of 25 (152 blocks) rather than 7 of 32 (147 blocks, the last chunk nearly
-// empty): 6.1 ms against 6.9 ms per 1M rows.
-template <int D, int RT>
-static cudaError_t bg_hist_t(const unsigned char *codes, int64_t m, const TreeArrays &ta, int T, uint32_t *hist,
-                             const DevInfo &dev, cudaStream_t st) {
-    const int xb = ta.n_cols * ta.code_bytes;
-    const size_t budget = dev.smem_optin;
-    const int64_t tiles = (m + RT - 1) / RT;
-    int G = std::min(T, 256);
-    while (G > 1 && BgLayout<D>(xb, RT, G, true).total > budget) --G;
-    const bool smem_hist = BgLayout<D>(xb, RT, G, true).total <= budget;
-    cudaError_t err;
-    if (smem_hist) {
-        auto kern = k_bg_hist<D, RT, true>;
-        err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)BgLayout<D>(xb, RT, G, true).total);
-        if (err != cudaSuccess) return err;
-        int64_t best = -1;
-        int best_g = G;
-        for (int g = G; g >= 1; --g) {
-            const int chunks = (T + g - 1) / g;
-            int per_sm = 0;
-            err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RT, BgLayout<D>(xb, RT, g, true).total);
-            if (err != cudaSuccess) return err;
-            per_sm = std::max(per_sm, 1);
-            if (chunks > dev.sms * per_sm) break;
-            const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)dev.sms * per_sm / chunks));
-            const int64_t blocks = slices * chunks;
-            const int64_t cost = (int64_t)(g + 1) * ((tiles + slices - 1) / slices) * ((blocks + dev.sms - 1) / dev.sms);
-            if (best < 0 || cost < best) {
-                best = cost;
-                best_g = g;
-            }
+// Warps (units) per block and row slices of a launch: all blocks resident, one or more per
+// SM, and the busiest SM's warps x tiles as few as possible (a block also spends about
+// two tiles' worth on loading its nodes and adding its counters; fewer than 3/4 of the
+// warps an SM can hold take as long as that many).  On a tie the smaller blocks, which wait
+// less at their barriers.
+template <int D, int STAGES, int SUB>
+static cudaError_t bg_count_t(const unsigned char *codes, int64_t m, const SliceArrays &sa, const TreeMeta *meta, int T,
+                              uint32_t *hist, const DevInfo &dev, cudaStream_t st) {
+    using N = Unit<D>;
+    const int units = T * N::UPT;
+    const int64_t runs = ((m + kBgTileRows - 1) / kBgTileRows + SUB - 1) / SUB;
+    auto smem = [&](int W) { return (size_t)STAGES * SUB * sa.quads * 64 + (size_t)W * 4 * kDecStride * 4; };
+    int64_t best = -1, best_slices = 1;
+    int best_w = 1;
+    for (int W = std::min(units, N::WMAX); W >= 1; --W) {
+        const int64_t chunks = (units + W - 1) / W;
+        const int64_t per_sm = std::max<int64_t>(
+            1, std::min<int64_t>(N::WMAX / W, (int64_t)(dev.smem_optin / (smem(W) + 1024))));
+        const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(runs, dev.sms * per_sm / chunks));
+        const int64_t waves = (chunks * slices + dev.sms * per_sm - 1) / (dev.sms * per_sm);
+        const int64_t warps = W * std::min(per_sm, (chunks * slices + dev.sms - 1) / dev.sms);  // of one SM
+        const int64_t cost = waves * std::max<int64_t>(warps, 3 * N::WMAX / 4) * (((runs + slices - 1) / slices) * SUB + 2);
+        if (best < 0 || cost <= best) {
+            best = cost;
+            best_w = W;
+            best_slices = slices;
         }
-        G = best_g;
-    } else {
-        G = std::min(T, 256);
-        while (G > 1 && BgLayout<D>(xb, RT, G, false).total > budget) --G;
     }
-    const size_t smem = BgLayout<D>(xb, RT, G, smem_hist).total;
-    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
-    auto kern = smem_hist ? k_bg_hist<D, RT, true> : k_bg_hist<D, RT, false>;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int chunks = (units + best_w - 1) / best_w;
+    auto kern = k_bg_count<D, STAGES, SUB>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(best_w));
     if (err != cudaSuccess) return err;
-    int per_sm = 0;
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RT, smem);
-    if (err != cudaSuccess) return err;
-    per_sm = std::max(per_sm, 1);
-    const int chunks = (T + G - 1) / G;
-    const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(tiles, ((int64_t)dev.sms * per_sm) / chunks));
-    kern<<<(unsigned)(slices * chunks), RT, smem, st>>>(codes, m, ta, T, G, chunks, hist);
+    kern<<<(unsigned)(best_slices * chunks), 32 * best_w, smem(best_w), st>>>(codes, m, sa, meta, units, chunks, hist);
     count_launches(1);
     return cudaGetLastError();
 }
 
-// Rows per block: the largest tile whose codes take at most 30 % of shared memory.
-static int bg_tile_rows(int xb, const DevInfo &dev) {
-    for (int rt = kBgMaxTileRows; rt > 32; rt /= 2)
-        if ((size_t)rt * xb <= dev.smem_optin * 3 / 10) return rt;
-    return 32;
-}
-
-// Deep trees (depth 7, 8): the most rows per block (one warp per 32 rows) that fit beside
-// one tree's counters, since a block holds only one or two trees anyway: 32.5 instead of
-// 47.5 ms per 1M rows for 500 trees of depth 7 (512 instead of 256-row tiles), 150 instead
-// of 203 ms for 1000 of depth 8 (512 instead of 128).
+// Long chunks of rows run with four tiles per barrier, where three such runs fit: 2.31 ms per
+// 1M rows and 200 depth-6 trees against 2.53 with two tiles per run and two half-size blocks
+// per SM (the warps of a block drift apart and wait at every barrier).  Below 16,384 rows a
+// block would get too few runs to share evenly.
+constexpr int64_t kBgLongRows = 16384;
 template <int D>
-static int bg_tile_rows_d(int xb, const DevInfo &dev) {
-    if (D >= 7) {
-        for (int rt = kBgMaxTileRows; rt > 32; rt /= 2)
-            if (BgLayout<D>(xb, rt, 1, true).total <= dev.smem_optin) return rt;
-        return 32;
-    }
-    return bg_tile_rows(xb, dev);
+static cudaError_t bg_count(const unsigned char *codes, int64_t m, const SliceArrays &sa, const TreeMeta *meta, int T,
+                            uint32_t *hist, const DevInfo &dev, cudaStream_t st) {
+    const size_t dec = (size_t)Unit<D>::WMAX * 4 * kDecStride * 4;
+    if (3 * 4 * (size_t)sa.quads * 64 + dec <= dev.smem_optin && m >= kBgLongRows)
+        return bg_count_t<D, 3, 4>(codes, m, sa, meta, T, hist, dev, st);
+    if (3 * (size_t)sa.quads * 64 + dec <= dev.smem_optin)
+        return bg_count_t<D, 3, 1>(codes, m, sa, meta, T, hist, dev, st);
+    return bg_count_t<D, 0, 1>(codes, m, sa, meta, T, hist, dev, st);
 }
 
-template <int D>
-static cudaError_t bg_hist_d(const unsigned char *codes, int64_t m, const TreeArrays &ta, int T, uint32_t *hist,
-                             const DevInfo &dev, cudaStream_t st) {
-    switch (bg_tile_rows_d<D>(ta.n_cols * ta.code_bytes, dev)) {
-        case 512: return bg_hist_t<D, 512>(codes, m, ta, T, hist, dev, st);
-        case 256: return bg_hist_t<D, 256>(codes, m, ta, T, hist, dev, st);
-        case 128: return bg_hist_t<D, 128>(codes, m, ta, T, hist, dev, st);
-        case 64: return bg_hist_t<D, 64>(codes, m, ta, T, hist, dev, st);
-        default: return bg_hist_t<D, 32>(codes, m, ta, T, hist, dev, st);
-    }
-}
-
-template <int D>
-static cudaError_t bg_count_chunk(const unsigned char *codes, int64_t rows, const TreeArrays &ta, int T,
-                                  uint32_t *hist, const DevInfo &dev, cudaStream_t st) {
-    return bg_hist_d<D>(codes, rows, ta, T, hist, dev, st);
-}
-
-cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeArrays &ta, int T,
-                           unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
+cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeArrays &ta, const SliceArrays &sa,
+                           int T, unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
                            cudaStream_t st, const BgOverlap *ov) {
     if (m == 0) return cudaSuccess;
-    if (code_rows < kBgMaxTileRows || code_rows % kBgMaxTileRows) return cudaErrorInvalidValue;
+    if (code_rows < kBgTileRows || code_rows % kBgTileRows) return cudaErrorInvalidValue;
     cudaError_t err = cudaSuccess;
     if (ov) {
         // the side stream starts after everything already queued on st (B, the zeroed counts)
@@ -294,28 +355,28 @@ cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const 
     int64_t k = 0;
     for (int64_t r0 = 0; r0 < m; r0 += code_rows, ++k) {
         const int64_t rows = std::min(code_rows, m - r0);
-        const int64_t rows_pad = (rows + kBgMaxTileRows - 1) / kBgMaxTileRows * kBgMaxTileRows;
+        const int64_t rows_pad = (rows + kBgTileRows - 1) / kBgTileRows * kBgTileRows;
         const int b = ov ? (int)(k & 1) : 0;
         unsigned char *buf = b ? ov->codes1 : codes;
         if (ov) {
             // encode chunk k on the side stream once the count of chunk k - 2 (the last
             // reader of this buffer) is done; the count of chunk k waits for the encode
             if (k >= 2) err = cudaStreamWaitEvent(ov->side, ov->cnt[b], 0);
-            if (err == cudaSuccess) err = launch_encode_codes(B + r0 * ldb, rows, ldb, ta, rows_pad, buf, ov->side);
+            if (err == cudaSuccess) err = launch_encode_slices(B + r0 * ldb, rows, ldb, sa, rows_pad, buf, dev, ov->side);
             if (err == cudaSuccess) err = cudaEventRecord(ov->enc[b], ov->side);
             if (err == cudaSuccess) err = cudaStreamWaitEvent(st, ov->enc[b], 0);
         } else {
-            err = launch_encode_codes(B + r0 * ldb, rows, ldb, ta, rows_pad, buf, st);
+            err = launch_encode_slices(B + r0 * ldb, rows, ldb, sa, rows_pad, buf, dev, st);
         }
         if (err != cudaSuccess) return err;
         switch (D) {
-            case 2: err = bg_count_chunk<2>(buf, rows, ta, T, hist, dev, st); break;
-            case 3: err = bg_count_chunk<3>(buf, rows, ta, T, hist, dev, st); break;
-            case 4: err = bg_count_chunk<4>(buf, rows, ta, T, hist, dev, st); break;
-            case 5: err = bg_count_chunk<5>(buf, rows, ta, T, hist, dev, st); break;
-            case 6: err = bg_count_chunk<6>(buf, rows, ta, T, hist, dev, st); break;
-            case 7: err = bg_count_chunk<7>(buf, rows, ta, T, hist, dev, st); break;
-            case 8: err = bg_count_chunk<8>(buf, rows, ta, T, hist, dev, st); break;
+            case 2: err = bg_count<2>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 3: err = bg_count<3>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 4: err = bg_count<4>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 5: err = bg_count<5>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 6: err = bg_count<6>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 7: err = bg_count<7>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 8: err = bg_count<8>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
             default: return cudaErrorInvalidValue;
         }
         if (err == cudaSuccess && ov) err = cudaEventRecord(ov->cnt[b], st);

@@ -23,6 +23,17 @@ struct TreeArrays {
     const unsigned long long *xmask;  // [T][6] (depth <= 6) expand masks of the real nodes
 };
 
+// Device arrays of the sliced codes of an ensemble (tree_layout.h).
+struct SliceArrays {
+    const UnitNode *unit;     // [T][units_per_tree][32]
+    const SliceCol *col;
+    const SlicePack *pack;
+    const SliceGroup *group;
+    const float *thr;
+    int n_groups, max_group_thr;  // max_group_thr: floats of the largest group's thresholds
+    int qbase[3], quads;
+};
+
 // Everything the consumer kernel needs about one ensemble.
 struct ExplainJob {
     TreeArrays ta;
@@ -67,15 +78,18 @@ struct DevInfo {
 
 // Step 1 of Algorithm 3 (background): joint entry counts hist[T][NS][2^(D+1)] (u32,
 // must be zeroed by the caller) of the background rows at every bottom subtree.  The
-// rows are encoded to decision codes (tree_layout.h) in chunks of code_rows rows into
-// codes (code_rows * n_cols * code_bytes bytes; code_rows a positive multiple of
-// kBgMaxTileRows), each chunk then counted.
-constexpr int kBgMaxTileRows = 512;
+// rows are encoded to sliced codes (tree_layout.h) in chunks of code_rows rows into codes
+// (code_rows / 2 * quads bytes; code_rows a positive multiple of kBgTileRows), each chunk
+// then counted.
+constexpr int kBgTileRows = 128;
 
 // Decision codes of rows [0, rows) of X (row stride ldx) into codes, in 32-row code
 // blocks (wdf_device.cuh); rows up to rows_pad (a multiple of 32) get code 0.
 cudaError_t launch_encode_codes(const float *X, int64_t rows, int64_t ldx, const TreeArrays &ta, int64_t rows_pad,
                                 unsigned char *codes, cudaStream_t st);
+// The same codes sliced (tree_layout.h): quad q of block b at codes + (b * quads + q) * 16.
+cudaError_t launch_encode_slices(const float *X, int64_t rows, int64_t ldx, const SliceArrays &sa, int64_t rows_pad,
+                                 unsigned char *codes, const DevInfo &dev, cudaStream_t st);
 // With ov, chunks alternate between codes and ov->codes1 and are encoded on ov->side, so
 // the encode of chunk k + 1 overlaps the count of chunk k (events order each buffer's
 // encode after its previous count and each count after its encode); st still ends
@@ -85,8 +99,8 @@ struct BgOverlap {
     cudaStream_t side;
     cudaEvent_t enc[2], cnt[2];
 };
-cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeArrays &ta, int T,
-                           unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
+cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeArrays &ta, const SliceArrays &sa,
+                           int T, unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
                            cudaStream_t st, const BgOverlap *ov = nullptr);
 
 // Per-leaf pattern counts vc[row][p] (u32, 2^D per row) of the live leaves, marginals of

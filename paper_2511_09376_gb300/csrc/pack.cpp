@@ -164,6 +164,100 @@ void build_records(Packed *pp) {
     }
 }
 
+// Sliced codes of the counting kernel (tree_layout.h): columns sorted by width and grouped
+// into packs, their search trees, and the nodes of every unit.
+void build_slices(Packed *pp) {
+    Packed &p = *pp;
+    const int F = p.F, T = p.T, D = p.D, NI = p.NI;
+    constexpr int cap = (1 << kSliceBits) - 1;  // thresholds of one column
+    std::vector<std::vector<float>> thr((size_t)F);
+    for (size_t k = 0; k < p.node_feat.size(); ++k) {
+        const int f = p.node_feat[k];
+        if (f < F && p.node_thr[k] == p.node_thr[k]) thr[(size_t)f].push_back(p.node_thr[k]);
+    }
+    struct Col {
+        int f, lo, cnt, levels;
+    };
+    std::vector<Col> cols;
+    for (int f = 0; f < F; ++f) {
+        auto &v = thr[(size_t)f];
+        std::sort(v.begin(), v.end());
+        v.erase(std::unique(v.begin(), v.end(), [](float a, float b) { return a == b; }), v.end());
+        for (int lo = 0; lo < (int)v.size(); lo += cap) {
+            const int cnt = std::min((int)v.size() - lo, cap);
+            cols.push_back(Col{f, lo, cnt, ilog2(cnt) + 1});
+        }
+    }
+    if (cols.empty()) cols.push_back(Col{0, 0, 0, 1});  // no real threshold at all: one empty column
+    std::stable_sort(cols.begin(), cols.end(), [](const Col &a, const Col &b) { return a.levels > b.levels; });
+    while (cols.size() % 8) cols.push_back(Col{0, 0, 0, 1});
+    // column of the j-th threshold of feature f: at[f][j / cap]
+    std::vector<std::vector<int>> at((size_t)F);
+    p.scol.clear();
+    p.spack.clear();
+    p.sgroup.clear();
+    p.sthr.clear();
+    int wide[3] = {0, 0, 0};
+    for (size_t c0 = 0; c0 < cols.size(); c0 += 8) {
+        const int levels = cols[c0].levels;  // the widest of the pack
+        const int first = (int)p.sthr.size();
+        for (int k = 0; k < 3; ++k)
+            if (levels > 4 * k) wide[k] += 8;
+        p.sthr.resize(p.sthr.size() + ((size_t)8 << levels), std::numeric_limits<float>::quiet_NaN());
+        for (int j = 0; j < 8; ++j) {
+            const Col &c = cols[c0 + (size_t)j];
+            float *tree = p.sthr.data() + first + ((size_t)j << levels);
+            const float *src = c.cnt ? thr[(size_t)c.f].data() + c.lo : nullptr;
+            for (int i = 1; i < (1 << levels); ++i) {  // the threshold in the middle of node i's range
+                int d = ilog2(i);
+                const int rank = ((i - (1 << d)) << (levels - d)) + (1 << (levels - d - 1)) - 1;
+                if (rank < c.cnt) tree[i] = src[rank];
+            }
+            if (c.cnt) {
+                auto &a = at[(size_t)c.f];
+                if ((int)a.size() <= c.lo / cap) a.resize((size_t)(c.lo / cap + 1), 0);
+                a[(size_t)(c.lo / cap)] = (int)(c0 + (size_t)j);
+            }
+            p.scol.push_back(SliceCol{c.f, c.cnt});
+        }
+        p.spack.push_back(SlicePack{first, levels});
+        const int pack = (int)p.spack.size() - 1, size = 8 << levels;
+        if (p.sgroup.empty() || p.sgroup.back().thr_n + size > kSliceGroupFloats ||
+            pack - p.sgroup.back().pack0 >= kSliceGroupPacks)
+            p.sgroup.push_back(SliceGroup{pack, pack, first, 0});
+        p.sgroup.back().pack1 = pack + 1;
+        p.sgroup.back().thr_n += size;
+    }
+    p.qbase[0] = 0;
+    p.qbase[1] = wide[0];
+    p.qbase[2] = wide[0] + wide[1];
+    p.quads = wide[0] + wide[1] + wide[2];
+    const int U = units_per_tree(D), n_local = (1 << unit_height(D)) - 1;
+    p.unit.assign((size_t)T * U * 32, UnitNode{0u, {0u, 0u, 0u}});
+    for (int t = 0; t < T; ++t)
+        for (int u = 0; u < U; ++u)
+            for (int i = 0; i < 32; ++i) {
+                UnitNode &n = p.unit[((size_t)t * U + u) * 32 + i];
+                int v = -1;
+                if (i < n_local) v = unit_node(D, u, i);
+                else if (i == 31 && u < U - 1) v = u;  // a top node
+                if (v < 0) continue;
+                const int f = p.node_feat[(size_t)t * NI + v];
+                const float x = f < F ? p.node_thr[(size_t)t * NI + v] : 0.0f;
+                if (f == F) {
+                    n.at = 1u << 20;  // pass-through: always left
+                } else if (x == x) {
+                    const auto &s = thr[(size_t)f];
+                    const int j = (int)(std::lower_bound(s.begin(), s.end(), x) - s.begin());
+                    const int col = at[(size_t)f][(size_t)(j / cap)], rank = j % cap;
+                    const int levels = p.spack[(size_t)(col / 8)].levels;
+                    n.at = (uint32_t)col | ((uint32_t)((levels + 3) / 4) << 16) | (1u << 20);
+                    for (int b = 0; b < kSliceBits; ++b)
+                        if ((rank >> b) & 1) n.rank[b / 4] |= 0x80u << (8 * (b % 4));
+                }  // a NaN threshold: never left
+            }
+}
+
 }  // namespace
 
 int pack_ensemble(int F, int T, const int64_t *off, const int32_t *feat, const float *thr, const int32_t *left,
@@ -275,6 +369,7 @@ int pack_ensemble(int F, int T, const int64_t *off, const int32_t *feat, const f
         p.group_off.push_back((int32_t)p.group_leaf.size());
     }
     build_records(&p);
+    build_slices(&p);
     return 0;
 }
 

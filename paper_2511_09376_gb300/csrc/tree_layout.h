@@ -31,6 +31,53 @@
 
 namespace wdf {
 
+// Sliced codes (the counting kernel).  The same codes, stored bit by bit: the rows of a
+// 32-row block give one 32-bit word per code bit (bit r of the word = row r), four words
+// (a "quad", 16 bytes) per four code bits, and a node's decision for all 32 rows is
+//   le = all ones; for every code bit from the least significant: le = majority(~bit, rank bit, le)
+// (code <= rank), eight three-input logic instructions for 32 decisions.  Columns are sorted
+// by their number of code bits, largest first, and padded to packs of eight columns of equal
+// width; quad k of column c lies at quad index qbase[k] + c of the block, so columns with
+// more than k quads are exactly the first ones.  A column takes at most kSliceBits bits;
+// a feature with more thresholds is cut into several columns.
+//
+// The 31 inner nodes of a height-5 subtree, one per lane of a warp, are a "unit": a tree of
+// depth D >= 5 has 2^(D-5) of them, side by side below its 2^(D-5) - 1 top nodes; a smaller
+// tree is one unit of 2^D - 1 nodes.  Lane 31 of unit u carries top node u.
+constexpr int kSliceBits = 12;
+constexpr int kSliceGroupPacks = 16;      // most packs (of eight columns) encoded together
+constexpr int kSliceGroupFloats = 16384;  // most thresholds of an encoding group (one pack may exceed it)
+
+// A lane's node of a unit: its column and what its rank compares with.
+struct UnitNode {
+    uint32_t at;        // column index | quads << 16 (0: none to read) | always-left << 20 (the decision of a
+                        // node without quads; with quads it is 1: a code equal to the rank goes left)
+    uint32_t rank[3];   // byte b of rank[k]: bit 7 is bit 4k + b of the rank
+};
+// One column of a pack: its feature and its number of thresholds (the code of a NaN).
+struct SliceCol {
+    int32_t feature, count;
+};
+// Eight columns: their thresholds are search trees of 2^levels - 1 nodes (root at 1, children
+// of i at 2i and 2i + 1, NaN after the column's thresholds) at sthr[first + (j << levels)].
+struct SlicePack {
+    int32_t first, levels;
+};
+// Packs [pack0, pack1) whose thresholds [thr0, thr0 + thr_n) one encoding block keeps in
+// shared memory.
+struct SliceGroup {
+    int32_t pack0, pack1, thr0, thr_n;
+};
+WDF_HD constexpr int unit_height(int D) { return D < 5 ? D : 5; }
+WDF_HD constexpr int unit_top(int D) { return D > 5 ? D - 5 : 0; }      // levels above the units
+WDF_HD constexpr int units_per_tree(int D) { return 1 << unit_top(D); }
+// Heap index of local node i (heap order within the unit) of unit u.
+WDF_HD inline int unit_node(int D, int u, int i) {
+    int l = 0;
+    while ((2 << l) <= i + 1) ++l;
+    return (1 << (unit_top(D) + l)) - 1 + (u << l) + (i - ((1 << l) - 1));
+}
+
 // One real inner node of a tree, in the order the decision loop visits them (heap
 // order, so the nodes of each 32-node word of the heap index are contiguous).
 struct NodeRec {

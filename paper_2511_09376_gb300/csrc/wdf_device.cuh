@@ -200,6 +200,40 @@ __device__ __forceinline__ void subtree_entries(const uint32_t (&dw)[Shape<D>::N
     }
 }
 
+// Transpose of the 32 x 32 bit matrix whose row r is lane r's word: lane b gets bit b of
+// every lane's word, in lane order.
+__device__ __forceinline__ uint32_t transpose32(uint32_t w, int lane) {
+    uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, w, 16);
+    w = __byte_perm(w, y, (lane & 16) ? 0x3276 : 0x5410);
+    y = __shfl_xor_sync(0xFFFFFFFFu, w, 8);
+    w = __byte_perm(w, y, (lane & 8) ? 0x3715 : 0x6240);
+#pragma unroll
+    for (int s = 4; s > 0; s >>= 1) {
+        const uint32_t low = s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u : 0x55555555u;
+        const bool up = lane & s;
+        y = __shfl_xor_sync(0xFFFFFFFFu, w, s);
+        y = __funnelshift_l(y, y, up ? 32 - s : s);
+        const uint32_t keep = up ? ~low : low;
+        w = (w & keep) | (y & ~keep);
+    }
+    return w;
+}
+
+// Mask of one rank bit of a unit node (tree_layout.h): byte b of rank word k holds bit
+// 4k + b in its top bit, which the selector 8 + b spreads over the word.
+template <int b>
+__device__ __forceinline__ uint32_t rank_mask(uint32_t rank) {
+    uint32_t m;
+    asm("prmt.b32 %0, %1, 0, %2;" : "=r"(m) : "r"(rank), "n"(0x8888 + 0x1111 * b));
+    return m;
+}
+
+// Four more code bits of a sliced comparison (tree_layout.h): le for 32 rows.
+__device__ __forceinline__ uint32_t slice_le(uint32_t le, const uint4 &q, const uint32_t (&m)[4]) {
+    auto maj = [](uint32_t c, uint32_t mm, uint32_t l) { return (~c & mm) | (~c & l) | (mm & l); };
+    return maj(q.w, m[3], maj(q.z, m[2], maj(q.y, m[1], maj(q.x, m[0], le))));
+}
+
 // Decision code of value x in one code column (tree_layout.h): the number of the
 // column's sorted thresholds u with u <= x, by binary search; the count for NaN.
 __device__ __forceinline__ int decision_code(float x, const float *__restrict__ u, const CodeCol &c) {

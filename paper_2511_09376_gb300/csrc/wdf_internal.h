@@ -48,6 +48,15 @@ struct Packed {
     std::vector<CodeCol> cols;        // [n_cols]
     std::vector<float> col_thr;       // column segments of the sorted distinct thresholds
     int code_bytes = 1;               // 1 or 2
+    // sliced codes (tree_layout.h): per unit 32 nodes, the columns, their packs, the groups
+    // of packs encoded together, the packs' search trees and the quads' bases
+    std::vector<UnitNode> unit;       // [T][units_per_tree][32]
+    std::vector<SliceCol> scol;       // [packs * 8]
+    std::vector<SlicePack> spack;
+    std::vector<SliceGroup> sgroup;
+    std::vector<float> sthr;
+    int qbase[3] = {0, 0, 0};         // first quad index of code bits 4k .. 4k + 3
+    int quads = 0;                    // quads of a 32-row block
     // live leaves grouped by path signature (first-occurrence positions)
     std::vector<uint32_t> sig_key;    // [G] 3 bits per path position
     std::vector<int32_t> group_off;   // [G+1]

@@ -53,6 +53,18 @@ struct wdf_ensemble {
     int4 *d_tiles128 = nullptr;
     int n_tiles128 = 0;
     int *d_err = nullptr;
+    // sliced codes (tree_layout.h)
+    wdf::UnitNode *d_unit = nullptr;
+    wdf::SliceCol *d_scol = nullptr;
+    wdf::SlicePack *d_spack = nullptr;
+    wdf::SliceGroup *d_sgroup = nullptr;
+    float *d_sthr = nullptr;
+    wdf::SliceArrays slices() const {
+        int most = 0;
+        for (const wdf::SliceGroup &g : pk.sgroup) most = g.thr_n > most ? g.thr_n : most;
+        return wdf::SliceArrays{d_unit, d_scol, d_spack, d_sgroup, d_sthr, (int)pk.sgroup.size(), most,
+                                {pk.qbase[0], pk.qbase[1], pk.qbase[2]}, pk.quads};
+    }
     wdf::TreeArrays arrays() const {
         return wdf::TreeArrays{d_nodes, d_rec, d_meta, d_cols, d_col_thr, (int)pk.cols.size(), pk.code_bytes,
                               d_xmask};
