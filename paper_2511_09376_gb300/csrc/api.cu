@@ -86,7 +86,7 @@ namespace {
 void free_ensemble(wdf_ensemble *e) {
     dfree(e->d_nodes); dfree(e->d_keys); dfree(e->d_group_leaf); dfree(e->d_leaf_row);
     dfree(e->d_w_rows); dfree(e->d_tiles); dfree(e->d_t32);
-    dfree(e->d_rec); dfree(e->d_meta); dfree(e->d_flfeat); dfree(e->d_xmask); dfree(e->d_cols); dfree(e->d_col_thr);
+    dfree(e->d_rec); dfree(e->d_meta); dfree(e->d_image);
     dfree(e->d_unit); dfree(e->d_scol); dfree(e->d_spack); dfree(e->d_sgroup); dfree(e->d_sthr);
     dfree(e->d_apk); dfree(e->d_bpk); dfree(e->d_tiles128); dfree(e->d_err); dfree(e->d_A); dfree(e->d_ratio);
     dfree(e->d_hist); dfree(e->d_vc); dfree(e->d_scale); dfree(e->d_S); dfree(e->d_sfold); dfree(e->d_base);
@@ -172,7 +172,7 @@ wdf_status count_device_rows(wdf_ensemble *ens, const float *B, int64_t m, int64
     if (s == WDF_OK && overlap) s = ensure_streams(ens);
     if (s != WDF_OK) return s;
     wdf::BgOverlap ov{ens->d_codes[1], ens->ist[0], {ens->ev_enc[0], ens->ev_enc[1]}, {ens->ev_cnt[0], ens->ev_cnt[1]}};
-    WDF_CUDA(wdf::launch_bg_hist(p.D, B, m, ldb, ens->arrays(), ens->slices(), p.T, ens->d_codes[0],
+    WDF_CUDA(wdf::launch_bg_hist(p.D, B, m, ldb, ens->d_meta, ens->slices(), p.T, ens->d_codes[0],
                                  ens->code_rows, hist, ens->ctx->dev, st, overlap ? &ov : nullptr));
     return WDF_OK;
 }
@@ -236,7 +236,7 @@ wdf_status ensure_frequency_state(wdf_ensemble *ens, wdf_precision precision) {
         WDF_CUDA(dalloc(&ens->d_A, (size_t)ens->n_live * K, &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_scale, (size_t)ens->n_live, &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_S, (size_t)ens->n_live * N, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_sfold, hist_n * wdf::slots_per_entry(p.D), &ens->bytes));
+        WDF_CUDA(dalloc(&ens->d_sfold, hist_n * (wdf::slots_per_entry(p.D) + wdf::extra_slots(p.D)), &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_lines, (size_t)p.T * wdf::lines_words(p.D), &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_base, 1, &ens->bytes));
     }
@@ -275,7 +275,7 @@ wdf_status finish_background(wdf_ensemble *ens, int64_t m, wdf_precision precisi
     WDF_CUDA(wdf::launch_leaf_counts(p.D, ens->d_hist, ens->d_group_leaf, ens->n_live, ens->d_vc, ens->d_A, st));
     WDF_CUDA(wdf::launch_scale(ens->d_w_rows, ens->n_live, m, ens->d_scale, st));
     WDF_CUDA(wdf::launch_base_value(p.D, ens->d_vc, nullptr, ens->d_w_rows, ens->n_live, m, ens->d_base, st));
-    WDF_CUDA(wdf::launch_line_maps(p.D, ens->d_hist, p.T, ens->d_lines, st));
+    WDF_CUDA(wdf::launch_line_maps(p.D, ens->d_hist, ens->d_meta, p.T, ens->d_lines, st));
     wdf_status s1 = contract_and_fold(ens, precision, st);
     if (s1 != WDF_OK) return s1;
     ens->m = m;
@@ -378,10 +378,12 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
     chk(dalloc(&e->d_t32, (size_t)e->G * K * N, &e->bytes));
     chk(dalloc(&e->d_rec, p.rec.size(), &e->bytes));
     chk(dalloc(&e->d_meta, p.meta.size(), &e->bytes));
-    chk(dalloc(&e->d_flfeat, p.flush_feat.size(), &e->bytes));
-    if (!p.xmask.empty()) chk(dalloc(&e->d_xmask, p.xmask.size(), &e->bytes));
-    chk(dalloc(&e->d_cols, p.cols.size(), &e->bytes));
-    chk(dalloc(&e->d_col_thr, std::max<size_t>(p.col_thr.size(), 1), &e->bytes));
+    chk(dalloc(&e->d_image, (size_t)wdf::kImages * p.T * wdf::image_bytes(p.D), &e->bytes));
+    int32_t *flfeat = nullptr;  // inputs of the images
+    uint8_t *flrep = nullptr;
+    int64_t scratch = 0;
+    chk(dalloc(&flfeat, p.flush_feat.size(), &scratch));
+    chk(dalloc(&flrep, p.flush_rep.size(), &scratch));
     chk(dalloc(&e->d_unit, p.unit.size(), &e->bytes));
     chk(dalloc(&e->d_scol, p.scol.size(), &e->bytes));
     chk(dalloc(&e->d_spack, p.spack.size(), &e->bytes));
@@ -397,12 +399,8 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
         chk(cudaMemcpy(e->d_leaf_row, p.leaf_row.data(), p.leaf_row.size() * 4, cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_rec, p.rec.data(), p.rec.size() * sizeof(wdf::NodeRec), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_meta, p.meta.data(), p.meta.size() * sizeof(wdf::TreeMeta), cudaMemcpyHostToDevice));
-        chk(cudaMemcpy(e->d_flfeat, p.flush_feat.data(), p.flush_feat.size() * 4, cudaMemcpyHostToDevice));
-        if (!p.xmask.empty())
-            chk(cudaMemcpy(e->d_xmask, p.xmask.data(), p.xmask.size() * 8, cudaMemcpyHostToDevice));
-        chk(cudaMemcpy(e->d_cols, p.cols.data(), p.cols.size() * sizeof(wdf::CodeCol), cudaMemcpyHostToDevice));
-        if (!p.col_thr.empty())
-            chk(cudaMemcpy(e->d_col_thr, p.col_thr.data(), p.col_thr.size() * 4, cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(flfeat, p.flush_feat.data(), p.flush_feat.size() * 4, cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(flrep, p.flush_rep.data(), p.flush_rep.size(), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_unit, p.unit.data(), p.unit.size() * sizeof(wdf::UnitNode), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_scol, p.scol.data(), p.scol.size() * sizeof(wdf::SliceCol), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_spack, p.spack.data(), p.spack.size() * sizeof(wdf::SlicePack), cudaMemcpyHostToDevice));
@@ -410,10 +408,13 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
                        cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_sthr, p.sthr.data(), p.sthr.size() * 4, cudaMemcpyHostToDevice));
         if (e->n_tiles) chk(cudaMemcpy(e->d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice));
+        chk(wdf::launch_images(p.D, p.T, e->d_unit, e->d_meta, flfeat, flrep, e->d_image, 0));
         // step 2 of Algorithm 3 depends only on the path signatures: build the tables now
         chk(wdf::launch_tables(p.D, e->metric, e->d_keys, e->G, e->d_t32, nullptr, 0));
         chk(cudaStreamSynchronize(0));
     }
+    dfree(flfeat);
+    dfree(flrep);
     if (ce != cudaSuccess) {
         free_ensemble(e);
         delete e;
@@ -501,7 +502,7 @@ wdf_status wdf_set_background(wdf_ensemble *ens, const float *B, int64_t m, int6
             const int b = (int)(chunk & 1);
             WDF_CUDA(copy_rows(ens->d_stage_in[b], p.F, B + r0 * ldb, ldb, rows, p.F, cudaMemcpyHostToDevice,
                                ens->ist[b]));
-            WDF_CUDA(wdf::launch_bg_hist(p.D, ens->d_stage_in[b], rows, p.F, ens->arrays(), ens->slices(), p.T,
+            WDF_CUDA(wdf::launch_bg_hist(p.D, ens->d_stage_in[b], rows, p.F, ens->d_meta, ens->slices(), p.T,
                                          ens->d_codes[b], ens->code_rows, ens->d_hist, ens->ctx->dev, ens->ist[b]));
         }
         for (int i = 0; i < 2; ++i) {
@@ -583,7 +584,7 @@ wdf_status wdf_set_path_dependent(wdf_ensemble *ens, wdf_precision precision, vo
     WDF_CUDA(wdf::launch_pd_freq(p.D, ens->d_ratio, ens->n_live, ens->d_A, st));
     WDF_CUDA(wdf::launch_scale(ens->d_w_rows, ens->n_live, 1, ens->d_scale, st));
     WDF_CUDA(wdf::launch_base_value(p.D, nullptr, ens->d_ratio, ens->d_w_rows, ens->n_live, 1, ens->d_base, st));
-    WDF_CUDA(wdf::launch_line_maps(p.D, nullptr, p.T, ens->d_lines, st));
+    WDF_CUDA(wdf::launch_line_maps(p.D, nullptr, ens->d_meta, p.T, ens->d_lines, st));
     wdf_status s1 = contract_and_fold(ens, precision, st);
     if (s1 != WDF_OK) return s1;
     ens->m = 0;
@@ -661,7 +662,7 @@ wdf_status wdf_explain_interactions(wdf_ensemble *ens, const float *C, int64_t n
         e = folded ? wdf::launch_iv_fold(D, s2, ens->d_leaf_row, p.T, s2t, st)
                    : wdf::launch_iv_pack(D, PP, s2, ens->n_live, s2t, st);
     if (e == cudaSuccess)
-        e = wdf::launch_explain_iv(D, C, n, ldc, p.F, ens->arrays(), p.T, ens->d_group_leaf, ens->n_live,
+        e = wdf::launch_explain_iv(D, C, n, ldc, p.F, ens->arrays(), ens->slices(), p.T, ens->d_group_leaf, ens->n_live,
                                    folded ? nullptr : s2t, folded ? s2t : nullptr, out, ldo, ens->ctx->dev, st);
     const cudaError_t fe = cudaFreeAsync(buf, st);
     WDF_CUDA(e);

@@ -3,7 +3,7 @@
 //
 // Ensembles are grouped into depth classes (one kernel instantiation per depth).  A
 // call writes every class's work description -- the ensembles' device arrays (jobs),
-// the requests, the encode items (request, 32-row block) and the work items (job,
+// the requests, the encode items (request, group of columns, 32-row blocks) and the work items (job,
 // request, first row) of tile_rows consumer rows each -- into one pinned host blob; the
 // captured graph copies that blob to the device with a single memcpy and then runs, per
 // class on parallel branches, k_encode_batch (the rows' decision codes into the batch's
@@ -41,7 +41,7 @@ wdf_status fail(wdf_status s, const std::string &msg) {
     } while (0)
 
 struct Cls {
-    int D = 0, F_max = 0, xb_max = 0, tile_rows = 0;
+    int D = 0, F_max = 0, q_max = 0, thr_max = 0, tile_rows = 0;
     std::vector<int> members;  // batch ensemble indices, in job-slot order
     int cap_reqs = 0, cap_items = 0, cap_eitems = 0;
     size_t off_jobs = 0, off_reqs = 0, off_items = 0, off_count = 0, off_eitems = 0, off_ecount = 0;
@@ -102,7 +102,7 @@ wdf_status place_codes(wdf_batch *b, std::vector<Req> *reqs) {
     for (Req &r : *reqs) {
         const wdf::Packed &p = b->ens[(size_t)r.e]->pk;
         r.codes_off = total;
-        total += (size_t)padded_rows(r.n) * p.cols.size() * (size_t)p.code_bytes;
+        total += (size_t)padded_rows(r.n) / 32 * (size_t)p.quads * 16;
     }
     if (total > b->codes_cap) {
         wdf_status s = wait_copied(b);
@@ -146,7 +146,7 @@ wdf_status ensure_blob(wdf_batch *b, const std::vector<int> &need_reqs, const st
         k.off_count = off;
         off = up16(off + 2 * sizeof(int));
         k.off_eitems = off;
-        off = up16(off + (size_t)k.cap_eitems * sizeof(int2));
+        off = up16(off + (size_t)k.cap_eitems * sizeof(int4));
         k.off_ecount = off;
         off = up16(off + sizeof(int));
     }
@@ -168,14 +168,17 @@ int fill_class(wdf_batch *b, int c, const std::vector<Req> &reqs, int tile_rows)
     for (size_t j = 0; j < k.members.size(); ++j) jobs[j] = b->ens[(size_t)k.members[j]]->job();
     auto *rq = reinterpret_cast<wdf::BatchRequest *>(b->h_blob + k.off_reqs);
     auto *items = reinterpret_cast<int4 *>(b->h_blob + k.off_items);
-    auto *eitems = reinterpret_cast<int2 *>(b->h_blob + k.off_eitems);
+    auto *eitems = reinterpret_cast<int4 *>(b->h_blob + k.off_eitems);
     int nr = 0, ni = 0, ne = 0;
     for (const Req &r : reqs) {
         if (b->cls_of[(size_t)r.e] != c) continue;
         rq[nr] = wdf::BatchRequest{r.C, r.phi, b->d_codes + r.codes_off, r.n, r.ldc, r.ldp, b->slot_of[(size_t)r.e]};
         for (int64_t c0 = 0; c0 < r.n; c0 += tile_rows)
             items[ni++] = make_int4(b->slot_of[(size_t)r.e], nr, (int)(c0 >> 31), (int)(c0 & 0x7FFFFFFF));
-        for (int64_t blk = 0; blk < padded_rows(r.n) / 32; ++blk) eitems[ne++] = make_int2(nr, (int)blk);
+        const int64_t blocks = padded_rows(r.n) / 32;
+        for (int64_t blk = 0; blk < blocks; blk += wdf::kEncodeItemBlocks)
+            for (int g = 0; g < (int)b->ens[(size_t)r.e]->pk.sgroup.size(); ++g)
+                eitems[ne++] = make_int4(nr, g, (int)blk, (int)std::min<int64_t>(wdf::kEncodeItemBlocks, blocks - blk));
         ++nr;
     }
     // longest first: tiles of ensembles with more trees cost more; blocks claim items in
@@ -190,9 +193,6 @@ int fill_class(wdf_batch *b, int c, const std::vector<Req> &reqs, int tile_rows)
     return ni;
 }
 
-// Blocks of the batched encode: eight per SM walk the (request, 32-row block) items.
-int kEncodeGrid(const wdf_batch *b) { return 8 * std::max(1, b->ctx->dev.sms); }
-
 wdf_status capture(wdf_batch *b) {
     drop_graph(b);
     WDF_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeRelaxed));
@@ -206,15 +206,15 @@ wdf_status capture(wdf_batch *b) {
         if (e == cudaSuccess)
             e = wdf::launch_encode_batch(reinterpret_cast<const wdf::ExplainJob *>(b->d_blob + k.off_jobs),
                                          reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),
-                                         reinterpret_cast<const int2 *>(b->d_blob + k.off_eitems),
-                                         reinterpret_cast<const int *>(b->d_blob + k.off_ecount), kEncodeGrid(b),
+                                         reinterpret_cast<const int4 *>(b->d_blob + k.off_eitems),
+                                         reinterpret_cast<const int *>(b->d_blob + k.off_ecount), k.thr_max, b->ctx->dev,
                                          b->branch[c]);
         if (e == cudaSuccess)
             e = wdf::launch_explain_batch(
                 k.D, reinterpret_cast<const wdf::ExplainJob *>(b->d_blob + k.off_jobs),
                 reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),
                 reinterpret_cast<const int4 *>(b->d_blob + k.off_items),
-                reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.xb_max, k.tile_rows, 0, b->ctx->dev,
+                reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.q_max, k.tile_rows, 0, b->ctx->dev,
                 b->branch[c]);
         if (e == cudaSuccess) e = cudaEventRecord(b->ev_join[c], b->branch[c]);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->ev_join[c], 0);
@@ -257,7 +257,9 @@ void count_needs(const wdf_batch *b, const std::vector<Req> &reqs, const std::ve
         const int c = b->cls_of[(size_t)r.e];
         (*need_reqs)[(size_t)c] += 1;
         (*need_items)[(size_t)c] += (int)((r.n + tile_rows[(size_t)c] - 1) / tile_rows[(size_t)c]);
-        (*need_eitems)[(size_t)c] += (int)(padded_rows(r.n) / 32);
+        (*need_eitems)[(size_t)c] +=
+            (int)((padded_rows(r.n) / 32 + wdf::kEncodeItemBlocks - 1) / wdf::kEncodeItemBlocks) *
+            (int)b->ens[(size_t)r.e]->pk.sgroup.size();
     }
 }
 
@@ -290,7 +292,8 @@ wdf_status wdf_batch_create(wdf_ctx *ctx, int32_t n_ensembles, wdf_ensemble *con
         }
         Cls &k = b->cls[(size_t)c];
         k.F_max = std::max(k.F_max, b->ens[(size_t)i]->pk.F);
-        k.xb_max = std::max(k.xb_max, (int)b->ens[(size_t)i]->pk.cols.size() * b->ens[(size_t)i]->pk.code_bytes);
+        k.q_max = std::max(k.q_max, b->ens[(size_t)i]->pk.quads);
+        k.thr_max = std::max(k.thr_max, b->ens[(size_t)i]->slices().max_group_thr);
         b->cls_of[(size_t)i] = c;
         b->slot_of[(size_t)i] = (int)k.members.size();
         k.members.push_back(i);
@@ -302,8 +305,8 @@ wdf_status wdf_batch_create(wdf_ctx *ctx, int32_t n_ensembles, wdf_ensemble *con
     b->ev_join.assign(b->cls.size(), nullptr);
     for (size_t c = 0; c < b->cls.size() && e == cudaSuccess; ++c) {
         Cls &k = b->cls[c];
-        k.tile_rows = wdf::default_tile_rows(k.D, k.F_max, k.xb_max, ctx->dev);
-        if (wdf::explain_smem_bytes(k.D, k.F_max, k.xb_max, k.tile_rows) > ctx->dev.smem_optin) {
+        k.tile_rows = wdf::default_tile_rows(k.D, k.F_max, k.q_max, ctx->dev);
+        if (wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, k.tile_rows) > ctx->dev.smem_optin) {
             e = cudaErrorInvalidConfiguration;
             break;
         }
@@ -412,10 +415,12 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
     for (size_t c = 0; c < b->cls.size() && s == WDF_OK; ++c) {
         Cls &k = b->cls[c];
         if (need_reqs[c] == 0) continue;
-        const int fkey = (k.F_max + 31) / 32 * 32, xkey = (k.xb_max + 31) / 32 * 32;
+        const int fkey = (k.F_max + 31) / 32 * 32, xkey = (k.q_max / 2 + 31) / 32 * 32;  // half a byte per quad and row
         int hit = 0;
         for (const auto &row : cached)
-            if (row[0] == k.D && row[1] == fkey && row[2] == xkey) hit = row[3];
+            if (row[0] == k.D && row[1] == fkey && row[2] == xkey && (row[3] == 32 || row[3] == 64 || row[3] == 128) &&
+                wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, row[3]) <= b->ctx->dev.smem_optin)
+                hit = row[3];
         if (hit) {
             k.tile_rows = hit;
             continue;
@@ -429,16 +434,16 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
             if (e == cudaSuccess)
                 e = wdf::launch_encode_batch(reinterpret_cast<const wdf::ExplainJob *>(b->d_blob + k.off_jobs),
                                              reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),
-                                             reinterpret_cast<const int2 *>(b->d_blob + k.off_eitems),
-                                             reinterpret_cast<const int *>(b->d_blob + k.off_ecount), kEncodeGrid(b),
-                                             st);
+                                             reinterpret_cast<const int4 *>(b->d_blob + k.off_eitems),
+                                             reinterpret_cast<const int *>(b->d_blob + k.off_ecount), k.thr_max,
+                                             b->ctx->dev, st);
             if (e != cudaSuccess) {
                 s = fail(WDF_ECUDA, std::string("autotune: ") + cudaGetErrorString(e));
                 break;
             }
         }
         for (int tc : cand) {
-            if (wdf::explain_smem_bytes(k.D, k.F_max, k.xb_max, tc) > b->ctx->dev.smem_optin) continue;
+            if (wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, tc) > b->ctx->dev.smem_optin) continue;
             fill_class(b, (int)c, reqs, tc);
             cudaError_t e = cudaMemcpyAsync(b->d_blob, b->h_blob, b->blob_bytes, cudaMemcpyHostToDevice, st);
             float ms = 0.0f;
@@ -450,7 +455,7 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
                     e = wdf::launch_explain_batch(k.D, reinterpret_cast<const wdf::ExplainJob *>(b->d_blob + k.off_jobs),
                                                   reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),
                                                   reinterpret_cast<const int4 *>(b->d_blob + k.off_items),
-                                                  reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.xb_max, tc,
+                                                  reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.q_max, tc,
                                                   0, b->ctx->dev, st);
             }
             if (e == cudaSuccess) e = cudaEventRecord(e1, st);

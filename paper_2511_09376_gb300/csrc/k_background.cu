@@ -88,12 +88,10 @@ __device__ __forceinline__ void expand_b(uint32_t y, uint32_t (&r)[8]) {
 struct SliceNode {
     uint32_t at, m[3][4];
     __device__ __forceinline__ void load(const UnitNode *p) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+        const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
         at = v.x;
-        set(m[0], v.y); set(m[1], v.z); set(m[2], v.w);
-    }
-    __device__ __forceinline__ static void set(uint32_t (&d)[4], uint32_t r) {
-        d[0] = rank_mask<0>(r); d[1] = rank_mask<1>(r); d[2] = rank_mask<2>(r); d[3] = rank_mask<3>(r);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) rank_masks(v.y, k, m[k]);
     }
     __device__ __forceinline__ uint32_t decide1(const uint4 *block, const SliceArrays &sa) const {
         const int col = (int)(at & 0xFFFFu), nq = (int)((at >> 16) & 15u);
@@ -244,8 +242,8 @@ __global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsign
                 uint32_t rb[2][8];
 #pragma unroll
                 for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h) {
-                    const int r = N::NSU - 1 + 2 * j + h;  // subtree root; entry low bits: r, 2r + 2, 2r + 1
-                    expand_b((d[r] ^ x0) & (d[2 * r + 2] ^ x1) & (d[2 * r + 1] ^ x2), rb[h]);
+                    const int c = N::NSU - 1 + 3 * (2 * j + h);  // the root's left child, right child and the root
+                    expand_b((d[c + 2] ^ x0) & (d[c + 1] ^ x1) & (d[c] ^ x2), rb[h]);
                 }
 #pragma unroll
                 for (int i = 0; i < N::TILES; ++i) {
@@ -340,7 +338,7 @@ static cudaError_t bg_count(const unsigned char *codes, int64_t m, const SliceAr
     return bg_count_t<D, 0, 1>(codes, m, sa, meta, T, hist, dev, st);
 }
 
-cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeArrays &ta, const SliceArrays &sa,
+cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeMeta *meta, const SliceArrays &sa,
                            int T, unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
                            cudaStream_t st, const BgOverlap *ov) {
     if (m == 0) return cudaSuccess;
@@ -370,13 +368,13 @@ cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const 
         }
         if (err != cudaSuccess) return err;
         switch (D) {
-            case 2: err = bg_count<2>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
-            case 3: err = bg_count<3>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
-            case 4: err = bg_count<4>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
-            case 5: err = bg_count<5>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
-            case 6: err = bg_count<6>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
-            case 7: err = bg_count<7>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
-            case 8: err = bg_count<8>(buf, rows, sa, ta.meta, T, hist, dev, st); break;
+            case 2: err = bg_count<2>(buf, rows, sa, meta, T, hist, dev, st); break;
+            case 3: err = bg_count<3>(buf, rows, sa, meta, T, hist, dev, st); break;
+            case 4: err = bg_count<4>(buf, rows, sa, meta, T, hist, dev, st); break;
+            case 5: err = bg_count<5>(buf, rows, sa, meta, T, hist, dev, st); break;
+            case 6: err = bg_count<6>(buf, rows, sa, meta, T, hist, dev, st); break;
+            case 7: err = bg_count<7>(buf, rows, sa, meta, T, hist, dev, st); break;
+            case 8: err = bg_count<8>(buf, rows, sa, meta, T, hist, dev, st); break;
             default: return cudaErrorInvalidValue;
         }
         if (err == cudaSuccess && ov) err = cudaEventRecord(ov->cnt[b], st);

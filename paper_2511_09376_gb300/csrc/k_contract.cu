@@ -143,11 +143,12 @@ cudaError_t launch_contract_fp32(int D, const float *A, const float *scale, cons
 // collects sum over leaves of S[leaf][k][p] per path position k: positions above r
 // (slots 0..D-3) and r itself (slot D-2) from all four leaves, the left child of r
 // (slot D-1) from leaves 0-1 and the right child (slot D) from leaves 2-3.  The vector
-// of entry e is stored at line_pos(e) of the subtree's line map.
+// of entry e is stored at line_pos(e) of the subtree's line map (depth 8: slots 1..8, slot 0
+// in an array of its own after all vectors).
 __global__ void k_fold(int D, const float *__restrict__ S, const int32_t *__restrict__ leaf_row, int T,
                        const uint32_t *__restrict__ lines, float *__restrict__ sfold) {
     const int NS = 1 << (D - 2), E = 1 << (D + 1), NL = 1 << D, N = D << D;
-    const int SP = (D + 1) <= 4 ? 4 : ((D + 1) <= 8 ? 8 : 12);
+    const int SP = slots_per_entry(D), X1 = extra_slots(D);
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)T * NS * E) return;
     const int e = (int)(idx % E);
@@ -171,8 +172,11 @@ __global__ void k_fold(int D, const float *__restrict__ S, const int32_t *__rest
     }
     const uint32_t rot = (__ldg(lines + (size_t)t * lines_words(D) + (s >> 2)) >> (8 * (s & 3))) & 0xFFu;
     const int64_t at = ((int64_t)t * NS + s) * E + line_pos((uint32_t)e, rot, D);
+    if (rot == kLineDead && e) return;  // every row reads entry 0 (zeros)
     float4 *dst = reinterpret_cast<float4 *>(sfold + at * SP);
-    for (int k = 0; k < SP; k += 4) dst[k / 4] = make_float4(out[k], out[k + 1], out[k + 2], out[k + 3]);
+    for (int k = 0; k < SP; k += 4)
+        dst[k / 4] = make_float4(out[k + X1], out[k + 1 + X1], out[k + 2 + X1], out[k + 3 + X1]);
+    if (X1) sfold[(int64_t)T * NS * E * SP + at] = out[0];
 }
 
 cudaError_t launch_fold(int D, const float *S, const int32_t *leaf_row, int T, const uint32_t *lines, float *sfold,
@@ -188,7 +192,8 @@ cudaError_t launch_fold(int D, const float *S, const int32_t *leaf_row, int T, c
 // pair (bits r and r + 1 mod D + 1) is the least certain: the largest sum of
 // min(p, 1 - p).  Ties keep the smaller r; a subtree no row reaches, and the padding
 // bytes past the last subtree, keep the identity 0.
-__global__ void k_line_maps(int D, const uint32_t *__restrict__ hist, int T, uint8_t *__restrict__ lines) {
+__global__ void k_line_maps(int D, const uint32_t *__restrict__ hist, const TreeMeta *__restrict__ meta, int T,
+                            uint8_t *__restrict__ lines) {
     const int NS = 1 << (D - 2), E = 1 << (D + 1), B = 4 * lines_words(D), NB = D + 1;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)T * B) return;
@@ -217,13 +222,16 @@ __global__ void k_line_maps(int D, const uint32_t *__restrict__ hist, int T, uin
             }
         }
     }
+    if (s < NS && !((__ldg(&meta[t].live) >> s) & 1ull)) rot = kLineDead;
     lines[idx] = (uint8_t)rot;
 }
 
-cudaError_t launch_line_maps(int D, const uint32_t *hist, int T, uint32_t *lines, cudaStream_t st) {
+cudaError_t launch_line_maps(int D, const uint32_t *hist, const TreeMeta *meta, int T, uint32_t *lines,
+                             cudaStream_t st) {
     const int64_t total = (int64_t)T * 4 * lines_words(D);
     if (total == 0) return cudaSuccess;
-    k_line_maps<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(D, hist, T, reinterpret_cast<uint8_t *>(lines));
+    k_line_maps<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(D, hist, meta, T,
+                                                                  reinterpret_cast<uint8_t *>(lines));
     count_launches(1);
     return cudaGetLastError();
 }

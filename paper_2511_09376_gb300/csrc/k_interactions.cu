@@ -163,14 +163,14 @@ __global__ void k_iv_fold(int D, const float *__restrict__ S2, const int32_t *__
 // Words of the depth <= 6 interaction scratch: the folded vectors, then a byte per
 // complete-layout node of every tree (its feature; 16 words per tree), then every tree's
 // decision records packed into words (kIvPackWords per tree); the last two are used when
-// F <= 255 and the codes take one byte.
+// F <= 255 and no code takes more than eight bits.
 constexpr int kIvPackWords = 68;
 static size_t iv_fold_only(int D, int T) { return ((size_t)T << (D - 2 + D + 1)) * iv_fpp(D); }
 size_t iv_fold_floats(int D, int T) { return D <= 6 ? iv_fold_only(D, T) + (size_t)T * (16 + kIvPackWords) : 0; }
 
 // prec[t]: words 0-2 = the tree's pass-through decision words and its real inner-node
 // count, then one word per real node: column << 16 | (rank + 1) << 7 | decision bit (the
-// row goes left at the node when its code < rank + 1).  One-byte codes only.
+// row goes left at the node when its code < rank + 1).  Codes of at most eight bits.
 __global__ void k_iv_pack_records(int NW, int NI, const int4 *__restrict__ rec, const TreeMeta *__restrict__ meta,
                                   int T, uint32_t *__restrict__ prec) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -187,7 +187,7 @@ __global__ void k_iv_pack_records(int NW, int NI, const int4 *__restrict__ rec, 
     } else if (k >= 4 && k - 4 < cnt) {
         const int4 r = rec[(size_t)t * NI + (k - 4)];
         const int bit = r.z ? __ffs(r.z) - 1 : 32 + __ffs(r.w) - 1;
-        w = ((uint32_t)(r.x >> 5) << 16) | ((uint32_t)(r.y + 1) << 7) | (uint32_t)bit;
+        w = ((uint32_t)r.x << 16) | ((uint32_t)(r.y + 1) << 7) | (uint32_t)bit;
     }
     prec[i] = w;
 }
@@ -246,7 +246,7 @@ __host__ __device__ __forceinline__ size_t iv_up16(size_t v) { return (v + 15) &
 // row's matrix.  Without SMEM the triangle accumulates in place in out (global atomics).
 template <int D, bool SMEM>
 __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restrict__ C, int64_t n, int64_t ldc,
-                                                         int F, TreeArrays ta, int T,
+                                                         int F, TreeArrays ta, SliceArrays sa, int T,
                                                          const int32_t *__restrict__ group_leaf, int n_live,
                                                          const float *__restrict__ S2T, float *__restrict__ out,
                                                          int64_t ldo) {
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
     constexpr int NW = S::NW, NI = S::NI, NL = S::NL, K = 1 << D;
     constexpr int P = D * (D - 1) / 2, PP = (P + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int ncol = ta.n_cols, cshift = ta.code_bytes == 1 ? 5 : 6;  // column = col_off >> cshift
+    const int ncol = sa.n_cols;
     int *scode = reinterpret_cast<int *>(smem_raw);
     uint32_t *sdw = reinterpret_cast<uint32_t *>(smem_raw + iv_up16((size_t)ncol * 4));
     float *acc = reinterpret_cast<float *>(smem_raw + iv_up16((size_t)ncol * 4) + iv_up16((size_t)T * NW * 4));
@@ -269,11 +269,8 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
             for (int64_t k = tid; k < (int64_t)F * F; k += kIvThreads) orow[k] = 0.0f;
         }
         const float *x = C + row * ldc;
-        for (int c = tid; c < ncol; c += kIvThreads) {
-            const int4 cv = __ldg(reinterpret_cast<const int4 *>(ta.cols) + c);
-            const CodeCol col{cv.x, cv.y, cv.z, cv.w};
-            scode[c] = decision_code(__ldg(x + col.feature), ta.col_thr + col.first, col);
-        }
+        for (int c = tid; c < ncol; c += kIvThreads)
+            scode[c] = decision_code(__ldg(x + __ldg(&sa.col[c].feature)), sa, c);
         __syncthreads();
         // decision words of every tree (bit v of word v / 32: left at inner node v)
         for (int t = tid; t < T; t += kIvThreads) {
@@ -283,7 +280,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
                 uint32_t lo = 0u, hi = 0u;
                 for (int i = 0; i < m.wend[NW - 1]; ++i) {
                     const int4 r = __ldg(rec + i);
-                    const uint32_t s = 0u - (uint32_t)(scode[r.x >> cshift] <= r.y);
+                    const uint32_t s = 0u - (uint32_t)(scode[r.x] <= r.y);
                     lo |= (uint32_t)r.z & s;
                     hi |= (uint32_t)r.w & s;
                 }
@@ -295,7 +292,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
                     uint32_t bits = 0u;
                     for (; i < m.wend[w]; ++i) {
                         const int4 r = __ldg(rec + i);
-                        bits |= (uint32_t)r.z & (0u - (uint32_t)(scode[r.x >> cshift] <= r.y));
+                        bits |= (uint32_t)r.z & (0u - (uint32_t)(scode[r.x] <= r.y));
                     }
                     sdw[t * NW + w] = m.pt[w] | bits;
                 }
@@ -346,12 +343,12 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
 // pairs with r or its children go straight into the triangle, while the pairs of two
 // nodes above the bottom subtrees accumulate in registers (one per (node, ancestor))
 // and are added once per tree.
-// FB (F <= 255, one-byte codes): the node features come from a byte table, loaded as
+// FB (F <= 255, codes of at most eight bits): the node features come from a byte table, loaded as
 // 64 bytes per tree into registers, instead of one scattered load per feature, and the
 // decision records from the packed table (four nodes per 16-byte load).
 template <int D, bool SMEM, bool FB>
 __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__restrict__ C, int64_t n, int64_t ldc,
-                                                              int F, TreeArrays ta, int T,
+                                                              int F, TreeArrays ta, SliceArrays sa, int T,
                                                               const float *__restrict__ fold,
                                                               const uint4 *__restrict__ ftab,
                                                               const uint4 *__restrict__ prec, float *__restrict__ out,
@@ -362,7 +359,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__r
     // (node, ancestor) pairs above the bottom subtrees: node v of depth d has d of them
     constexpr int UP = (D - 4) * (1 << (D - 2)) + 2 > 1 ? (D - 4) * (1 << (D - 2)) + 2 : 1;  // sum of depths, nodes 0..NS-2
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int ncol = ta.n_cols, cshift = ta.code_bytes == 1 ? 5 : 6;
+    const int ncol = sa.n_cols;
     int *scode = reinterpret_cast<int *>(smem_raw);
     uint32_t *sdw = reinterpret_cast<uint32_t *>(smem_raw + iv_up16((size_t)ncol * 4));
     float *acc = reinterpret_cast<float *>(smem_raw + iv_up16((size_t)ncol * 4) + iv_up16((size_t)T * NW * 4));
@@ -376,11 +373,8 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__r
             for (int64_t k = tid; k < (int64_t)F * F; k += kIvThreads) orow[k] = 0.0f;
         }
         const float *x = C + row * ldc;
-        for (int c = tid; c < ncol; c += kIvThreads) {
-            const int4 cv = __ldg(reinterpret_cast<const int4 *>(ta.cols) + c);
-            const CodeCol col{cv.x, cv.y, cv.z, cv.w};
-            scode[c] = decision_code(__ldg(x + col.feature), ta.col_thr + col.first, col);
-        }
+        for (int c = tid; c < ncol; c += kIvThreads)
+            scode[c] = decision_code(__ldg(x + __ldg(&sa.col[c].feature)), sa, c);
         __syncthreads();
         for (int t = tid; t < T; t += kIvThreads) {
             if constexpr (FB) {
@@ -404,7 +398,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__r
                 uint32_t lo = 0u, hi = 0u;
                 for (int i = 0; i < m.wend[NW - 1]; ++i) {
                     const int4 r = __ldg(rec + i);
-                    const uint32_t s = 0u - (uint32_t)(scode[r.x >> cshift] <= r.y);
+                    const uint32_t s = 0u - (uint32_t)(scode[r.x] <= r.y);
                     lo |= (uint32_t)r.z & s;
                     hi |= (uint32_t)r.w & s;
                 }
@@ -509,10 +503,11 @@ size_t iv_smem_bytes(int D, int F, int T, int n_cols, bool smem_acc) {
 }
 
 template <int D, bool SMEM>
-static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta, int T,
+static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta,
+                        const SliceArrays &sa, int T,
                         const int32_t *group_leaf, int n_live, const float *S2T, float *fold, float *out,
                         int64_t ldo, const DevInfo &dev, cudaStream_t st) {
-    const size_t smem = iv_smem_bytes(D, F, T, ta.n_cols, SMEM);
+    const size_t smem = iv_smem_bytes(D, F, T, sa.n_cols, SMEM);
     if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
     int per_sm = 0;
     cudaError_t err;
@@ -522,7 +517,7 @@ static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const Tre
         if (fold != nullptr) {
             // node features as bytes and packed decision records when they fit (the tables
             // follow the folded vectors)
-            const bool fb = F <= 255 && ta.code_bytes == 1;
+            const bool fb = F <= 255 && sa.max_levels <= 8;
             uint4 *ftab = reinterpret_cast<uint4 *>(fold + iv_fold_only(D, T));
             uint4 *prec = ftab + (size_t)T * 4;
             if (fb) {
@@ -539,7 +534,7 @@ static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const Tre
                 err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIvThreads, smem);
             if (err != cudaSuccess) return err;
             const int64_t grid = std::min<int64_t>(cap, (int64_t)dev.sms * std::max(per_sm, 1));
-            kern<<<(unsigned)grid, kIvThreads, smem, st>>>(C, n, ldc, F, ta, T, fold, ftab, prec, out, ldo);
+            kern<<<(unsigned)grid, kIvThreads, smem, st>>>(C, n, ldc, F, ta, sa, T, fold, ftab, prec, out, ldo);
             done = true;
         }
     }
@@ -549,34 +544,36 @@ static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const Tre
         if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIvThreads, smem);
         if (err != cudaSuccess) return err;
         const int64_t grid = std::min<int64_t>(cap, (int64_t)dev.sms * std::max(per_sm, 1));
-        kern<<<(unsigned)grid, kIvThreads, smem, st>>>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, out, ldo);
+        kern<<<(unsigned)grid, kIvThreads, smem, st>>>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, out, ldo);
     }
     count_launches(1);
     return cudaGetLastError();
 }
 
 template <int D>
-static cudaError_t iv_d(const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta, int T,
+static cudaError_t iv_d(const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta,
+                        const SliceArrays &sa, int T,
                         const int32_t *group_leaf, int n_live, const float *S2T, float *fold, float *out,
                         int64_t ldo, const DevInfo &dev, cudaStream_t st) {
     // the triangle in shared memory while two blocks still fit per SM, else in place
-    if (iv_smem_bytes(D, F, T, ta.n_cols, true) <= dev.smem_optin / 2)
-        return iv_t<D, true>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-    return iv_t<D, false>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+    if (iv_smem_bytes(D, F, T, sa.n_cols, true) <= dev.smem_optin / 2)
+        return iv_t<D, true>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+    return iv_t<D, false>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
 }
 
-cudaError_t launch_explain_iv(int D, const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta, int T,
+cudaError_t launch_explain_iv(int D, const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta,
+                        const SliceArrays &sa, int T,
                               const int32_t *group_leaf, int n_live, const float *S2T, float *fold, float *out,
                               int64_t ldo, const DevInfo &dev, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     switch (D) {
-        case 2: return iv_d<2>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-        case 3: return iv_d<3>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-        case 4: return iv_d<4>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-        case 5: return iv_d<5>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-        case 6: return iv_d<6>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-        case 7: return iv_d<7>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
-        case 8: return iv_d<8>(C, n, ldc, F, ta, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 2: return iv_d<2>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 3: return iv_d<3>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 4: return iv_d<4>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 5: return iv_d<5>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 6: return iv_d<6>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 7: return iv_d<7>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
+        case 8: return iv_d<8>(C, n, ldc, F, ta, sa, T, group_leaf, n_live, S2T, fold, out, ldo, dev, st);
         default: return cudaErrorInvalidValue;
     }
 }

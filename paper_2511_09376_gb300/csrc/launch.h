@@ -17,13 +17,9 @@ struct TreeArrays {
     const int2 *nodes;        // [T][NI] (feature, threshold bits); feature F = pass-through
     const NodeRec *rec;       // [T][NI] real inner nodes of every tree
     const TreeMeta *meta;     // [T]
-    const CodeCol *cols;      // [n_cols] decision-code columns
-    const float *col_thr;     // their sorted thresholds
-    int n_cols, code_bytes;   // code_bytes: 1 or 2
-    const unsigned long long *xmask;  // [T][6] (depth <= 6) expand masks of the real nodes
 };
 
-// Device arrays of the sliced codes of an ensemble (tree_layout.h).
+// Device arrays of the decision codes of an ensemble (tree_layout.h).
 struct SliceArrays {
     const UnitNode *unit;     // [T][units_per_tree][32]
     const SliceCol *col;
@@ -31,17 +27,27 @@ struct SliceArrays {
     const SliceGroup *group;
     const float *thr;
     int n_groups, max_group_thr;  // max_group_thr: floats of the largest group's thresholds
+    int n_cols, max_levels;       // columns (packs x 8); code bits of the widest
     int qbase[3], quads;
 };
 
 // Everything the consumer kernel needs about one ensemble.
 struct ExplainJob {
-    TreeArrays ta;
-    const float *sfold;     // folded slot vectors [T][NS][2^(D+1)][SP], entry e at line_pos(e)
+    SliceArrays sa;
+    const unsigned char *image;  // [kImages][T][image_bytes(D)] (tree_layout.h)
+    const float *sfold;     // folded slot vectors [T][NS][2^(D+1)][slots_per_entry], entry e at line_pos(e), then
+                            // (depth 8) the root slots [T][NS][2^(D+1)]
     const uint32_t *lines;  // per tree lines_words(D) words: byte s = line map of subtree s
-    const int32_t *flfeat;  // [T][flush_len(D)] feature of the node at each flush position (F: none)
     int T, F;
 };
+// A row's phi is the sum of the sums of its ensemble's parts, in part order: part p of P holds
+// trees [T p / P, T (p + 1) / P), each part's trees added in order from zero.  The split
+// depends on the ensemble alone, so a row's result does not depend on how many blocks
+// share its parts.
+inline __host__ __device__ int explain_parts(int T, int D) {
+    const long long p = (((long long)T << D) + 1600) / 3200;  // about 50 trees of depth 6 to a part
+    return p < 1 ? 1 : p > 8 ? 8 : (int)p;
+}
 
 // Where the consumer gathers land.  A warp's 32-byte gathers of one bottom subtree are
 // served a quarter warp at a time, one L1 wavefront per distinct 128-byte line, and a
@@ -50,11 +56,13 @@ struct ExplainJob {
 // bits that land in the two lowest positions (within a line) are the adjacent pair
 // (cyclically) whose background frequencies are closest to one half: the rows of a
 // quarter warp mostly agree on the more certain decisions, so they land in fewer lines.
-// The map of subtree s is the byte r_s (0 is the identity).  A rotation keeps nearly all
+// The map of subtree s is the byte r_s (0 is the identity); a dead subtree, whose slots are
+// all zero, has kLineDead, which sends every row to entry 0.  A rotation keeps nearly all
 // of the gain of moving the best two bits anywhere, for a third of the instructions.
+constexpr uint32_t kLineDead = 31;
 __host__ __device__ __forceinline__ uint32_t line_pos(uint32_t e, uint32_t r, int D) {
     const uint32_t nb = (uint32_t)D + 1u;
-    return ((e >> r) | (e << (nb - r))) & ((1u << nb) - 1u);
+    return ((e | (e << nb)) >> r) & ((1u << nb) - 1u);  // at most 18 bits, so r = kLineDead gives 0
 }
 // 32-bit words of line maps per tree: one byte per bottom subtree, at least four words
 // so that a tree's maps are whole 16-byte loads.
@@ -83,11 +91,9 @@ struct DevInfo {
 // then counted.
 constexpr int kBgTileRows = 128;
 
-// Decision codes of rows [0, rows) of X (row stride ldx) into codes, in 32-row code
-// blocks (wdf_device.cuh); rows up to rows_pad (a multiple of 32) get code 0.
-cudaError_t launch_encode_codes(const float *X, int64_t rows, int64_t ldx, const TreeArrays &ta, int64_t rows_pad,
-                                unsigned char *codes, cudaStream_t st);
-// The same codes sliced (tree_layout.h): quad q of block b at codes + (b * quads + q) * 16.
+// Decision codes of rows [0, rows) of X (row stride ldx), sliced (tree_layout.h): quad q of
+// 32-row block b at codes + (b * quads + q) * 16; rows up to rows_pad (a multiple of 32) get
+// code 0.
 cudaError_t launch_encode_slices(const float *X, int64_t rows, int64_t ldx, const SliceArrays &sa, int64_t rows_pad,
                                  unsigned char *codes, const DevInfo &dev, cudaStream_t st);
 // With ov, chunks alternate between codes and ov->codes1 and are encoded on ov->side, so
@@ -99,7 +105,7 @@ struct BgOverlap {
     cudaStream_t side;
     cudaEvent_t enc[2], cnt[2];
 };
-cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeArrays &ta, const SliceArrays &sa,
+cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeMeta *meta, const SliceArrays &sa,
                            int T, unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
                            cudaStream_t st, const BgOverlap *ov = nullptr);
 
@@ -152,7 +158,8 @@ cudaError_t launch_fold(int D, const float *S, const int32_t *leaf_row, int T, c
                         cudaStream_t st);
 // Line maps of every bottom subtree from the joint background counts hist (hist null:
 // the identity map, used for the path-dependent frequencies).
-cudaError_t launch_line_maps(int D, const uint32_t *hist, int T, uint32_t *lines, cudaStream_t st);
+cudaError_t launch_line_maps(int D, const uint32_t *hist, const TreeMeta *meta, int T, uint32_t *lines,
+                             cudaStream_t st);
 
 // scale[row] = w[row] / m.
 cudaError_t launch_scale(const double *w, int n_live, int64_t m, float *scale, cudaStream_t st);
@@ -161,6 +168,11 @@ cudaError_t launch_scale(const double *w, int n_live, int64_t m, float *scale, c
 // ratio is non-null (path-dependent game), of w * (product of the leaf's cover ratios).
 cudaError_t launch_base_value(int D, const uint32_t *vc, const double *ratio, const double *leaf_w_rows, int n_live,
                               int64_t m, double *out, cudaStream_t st);
+
+// The tree images (tree_layout.h) from the unit nodes, the metadata, the features flfeat
+// [T][flush_len(D)] and repeats flrep [T][flush_batches(D)] of the flush positions.
+cudaError_t launch_images(int D, int T, const UnitNode *unit, const TreeMeta *meta, const int32_t *flfeat,
+                          const uint8_t *flrep, unsigned char *image, cudaStream_t st);
 
 // Step 4: phi of n consumer rows, tile_rows consumer rows per block (32, 64 or 128;
 // 0 picks the default for the shared-memory budget).
@@ -172,21 +184,24 @@ cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const 
 // forgets them.  Turning it on or off also forgets them.
 void explain_timing(bool on);
 cudaError_t explain_timing_read(double *ms, int64_t *launches);
-// xb: decision-code bytes per row (code columns x code bytes).
-int default_tile_rows(int D, int F, int xb, const DevInfo &dev);
-size_t explain_smem_bytes(int D, int F, int xb, int tile_rows);
+// quads: 16-byte quads of a 32-row code block.
+int default_tile_rows(int D, int F, int quads, const DevInfo &dev);
+size_t explain_smem_bytes(int D, int F, int quads, int tile_rows);
 
-// Decision codes of a ragged batch's rows: items (request, 32-row block), *n_items read on
-// the device; a grid of `grid` blocks walks them.
-cudaError_t launch_encode_batch(const ExplainJob *jobs, const BatchRequest *reqs, const int2 *items,
-                                const int *n_items, int grid, cudaStream_t st);
+// Decision codes of a ragged batch's rows: items (request, group of packs, first 32-row block,
+// blocks), *n_items read on the device; a grid of `grid` blocks walks them.  max_group_thr:
+// the largest of the jobs' groups.
+constexpr int kEncodeItemBlocks = 16;
+int encode_batch_grid(int max_group_thr, const DevInfo &dev);
+cudaError_t launch_encode_batch(const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items,
+                                const int *n_items, int max_group_thr, const DevInfo &dev, cudaStream_t st);
 
 // Step 4 for a ragged batch of one depth: a persistent grid (grid <= 0: one wave at full
 // occupancy) walks the work items (job, request, first row split as hi/lo words);
-// *n_items is read on the device; the rows' codes come from launch_encode_batch.  F_max and xb_max bound the feature count and the
-// decision-code bytes per row of every job.
+// *n_items is read on the device; the rows' codes come from launch_encode_batch.  F_max and q_max bound the
+// feature count and the quads of a code block of every job.
 cudaError_t launch_explain_batch(int D, const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items,
-                                 int *n_items, int F_max, int xb_max, int tile_rows, int grid, const DevInfo &dev,
+                                 int *n_items, int F_max, int q_max, int tile_rows, int grid, const DevInfo &dev,
                                  cudaStream_t st);
 
 // Interaction values (k_interactions.cu).  Pair tables t2 [G][2^D][P * 2^D] (P =
@@ -200,7 +215,8 @@ cudaError_t launch_iv_pack(int D, int PP, const float *S2, int n_live, float *S2
 // table); the consumer kernel then takes whole trees (fold non-null) instead of leaves
 size_t iv_fold_floats(int D, int T);
 cudaError_t launch_iv_fold(int D, const float *S2, const int32_t *leaf_row, int T, float *fold, cudaStream_t st);
-cudaError_t launch_explain_iv(int D, const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta, int T,
+cudaError_t launch_explain_iv(int D, const float *C, int64_t n, int64_t ldc, int F, const TreeArrays &ta,
+                              const SliceArrays &sa, int T,
                               const int32_t *group_leaf, int n_live, const float *S2T, float *fold, float *out,
                               int64_t ldo, const DevInfo &dev, cudaStream_t st);
 

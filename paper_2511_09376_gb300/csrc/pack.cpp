@@ -63,110 +63,10 @@ void place(const Src &s, int t, int32_t node, int h, int depth, float w, bool ke
     place(s, t, -1, 2 * h + 2, depth + 1, 0.0f, false, p, -1);
 }
 
-// Code columns, node records and tree metadata of the decision kernels (tree_layout.h).
+// Decision codes, node records and tree metadata (tree_layout.h): columns sorted by width
+// and grouped into packs, their search trees, the nodes of every unit, the real inner nodes
+// and the flush order's features and batch flags.
 void build_records(Packed *pp) {
-    Packed &p = *pp;
-    const int F = p.F, T = p.T, D = p.D, NI = p.NI;
-    // distinct thresholds of every feature, sorted (NaN thresholds send every row right
-    // and take no part in the codes)
-    std::vector<std::vector<float>> thr(F);
-    for (size_t k = 0; k < p.node_feat.size(); ++k) {
-        const int f = p.node_feat[k];
-        if (f < F && p.node_thr[k] == p.node_thr[k]) thr[(size_t)f].push_back(p.node_thr[k]);
-    }
-    int64_t cols8 = 0, cols16 = 0;
-    for (auto &v : thr) {
-        std::sort(v.begin(), v.end());
-        v.erase(std::unique(v.begin(), v.end(), [](float a, float b) { return a == b; }), v.end());
-        cols8 += ((int64_t)v.size() + 254) / 255;
-        cols16 += ((int64_t)v.size() + 65534) / 65535;
-    }
-    // one-byte codes unless they would take more shared memory than two-byte codes
-    p.code_bytes = cols8 <= 2 * cols16 ? 1 : 2;
-    const int cap = p.code_bytes == 1 ? 255 : 65535;
-    std::vector<int32_t> first_col((size_t)F, -1);
-    p.cols.clear();
-    p.col_thr.clear();
-    for (int f = 0; f < F; ++f) {
-        const auto &v = thr[(size_t)f];
-        if (v.empty()) continue;
-        first_col[(size_t)f] = (int32_t)p.cols.size();
-        for (size_t lo = 0; lo < v.size(); lo += (size_t)cap) {
-            const int cnt = (int)std::min(v.size() - lo, (size_t)cap);
-            int top = 1;
-            while (2 * top <= cnt) top *= 2;
-            p.cols.push_back(CodeCol{f, (int32_t)p.col_thr.size(), cnt, top});
-            p.col_thr.insert(p.col_thr.end(), v.begin() + (int64_t)lo, v.begin() + (int64_t)lo + cnt);
-            // one-byte columns are padded to 255 entries with NaN (u <= x is false for a NaN
-            // u), so the encoder can search them in 8 fixed steps without bound checks
-            if (p.code_bytes == 1)
-                p.col_thr.insert(p.col_thr.end(), (size_t)(255 - cnt), std::numeric_limits<float>::quiet_NaN());
-        }
-    }
-    if (p.cols.empty()) {  // no real threshold at all: one empty column
-        p.cols.push_back(CodeCol{0, 0, 0, 0});
-        if (p.code_bytes == 1) p.col_thr.assign(255, std::numeric_limits<float>::quiet_NaN());
-    }
-    const int64_t blk = 32 * (int64_t)p.code_bytes;             // bytes of one column in a code block
-    p.rec.assign((size_t)T * NI, NodeRec{0, -1, 0u, 0u});
-    p.meta.assign((size_t)T, TreeMeta{});
-    const int FL = flush_len(D);
-    p.flush_feat.assign((size_t)T * FL, F);
-    if (D <= 6) p.xmask.assign((size_t)T * 6, 0ull);
-    for (int t = 0; t < T; ++t) {
-        TreeMeta &m = p.meta[(size_t)t];
-        int c = 0;
-        for (int v = 0; v < NI; ++v) {  // heap order, so the nodes of word v/32 are contiguous
-            const size_t k = (size_t)t * NI + v;
-            const int f = p.node_feat[k];
-            if (f == F) {
-                m.pt[v >> 5] |= 1u << (v & 31);
-            } else {
-                NodeRec r{0, -1, (D >= 7 || v < 32) ? 1u << (v & 31) : 0u, (D <= 6 && v >= 32) ? 1u << (v - 32) : 0u};
-                const float x = p.node_thr[k];
-                if (x == x) {
-                    const auto &u = thr[(size_t)f];
-                    const int64_t j = std::lower_bound(u.begin(), u.end(), x) - u.begin();
-                    r.col_off = (int32_t)((first_col[(size_t)f] + j / cap) * blk);
-                    r.rank = (int32_t)(j % cap);
-                }
-                p.rec[(size_t)t * NI + c++] = r;
-            }
-            if ((v & 31) == 31 || v == NI - 1) m.wend[v >> 5] = (uint8_t)c;
-        }
-        for (int w = (NI - 1) / 32 + 1; w < 8; ++w) m.wend[w] = (uint8_t)c;
-        m.live = p.live[(size_t)t];
-        if (D <= 6) {  // the real (not pass-through) nodes, one bit per heap position
-            const uint64_t all = NI == 64 ? ~0ull : ((1ull << NI) - 1ull);
-            const uint64_t real = ~((uint64_t)m.pt[0] | ((uint64_t)m.pt[1] << 32)) & all;
-            expand_masks(real, &p.xmask[(size_t)t * 6]);
-        }
-        for (int i = 0; i < FL; ++i) {
-            const int v = flush_node(D, i);
-            if (v >= 0) p.flush_feat[(size_t)t * FL + i] = p.node_feat[(size_t)t * NI + v];
-        }
-        // flush batches of the consumer kernel whose real features are all distinct
-        for (int b = 0; b < flush_batches(D); ++b) {
-            bool ok = true;
-            for (int i = 8 * b; i < 8 * b + 8 && ok; ++i)
-                for (int j = 8 * b; j < i && ok; ++j) {
-                    const int vi = flush_node(D, i), vj = flush_node(D, j);
-                    if (vi < 0 || vj < 0) continue;
-                    const int32_t fi = p.node_feat[(size_t)t * NI + vi], fj = p.node_feat[(size_t)t * NI + vj];
-                    ok = fi == F || fi != fj;  // pass-through nodes all write the scratch row
-                }
-            if (ok) m.flush |= 1ull << b;
-            for (int i = 8 * b; i < 8 * b + 8; ++i) {
-                const int v = flush_node(D, i);
-                if (v >= 0 && p.node_feat[(size_t)t * NI + v] != F) m.real |= 1ull << b;
-            }
-        }
-    }
-}
-
-// Sliced codes of the counting kernel (tree_layout.h): columns sorted by width and grouped
-// into packs, their search trees, and the nodes of every unit.
-void build_slices(Packed *pp) {
     Packed &p = *pp;
     const int F = p.F, T = p.T, D = p.D, NI = p.NI;
     constexpr int cap = (1 << kSliceBits) - 1;  // thresholds of one column
@@ -232,30 +132,75 @@ void build_slices(Packed *pp) {
     p.qbase[1] = wide[0];
     p.qbase[2] = wide[0] + wide[1];
     p.quads = wide[0] + wide[1] + wide[2];
-    const int U = units_per_tree(D), n_local = (1 << unit_height(D)) - 1;
-    p.unit.assign((size_t)T * U * 32, UnitNode{0u, {0u, 0u, 0u}});
-    for (int t = 0; t < T; ++t)
-        for (int u = 0; u < U; ++u)
-            for (int i = 0; i < 32; ++i) {
-                UnitNode &n = p.unit[((size_t)t * U + u) * 32 + i];
-                int v = -1;
-                if (i < n_local) v = unit_node(D, u, i);
-                else if (i == 31 && u < U - 1) v = u;  // a top node
-                if (v < 0) continue;
-                const int f = p.node_feat[(size_t)t * NI + v];
-                const float x = f < F ? p.node_thr[(size_t)t * NI + v] : 0.0f;
-                if (f == F) {
-                    n.at = 1u << 20;  // pass-through: always left
-                } else if (x == x) {
-                    const auto &s = thr[(size_t)f];
-                    const int j = (int)(std::lower_bound(s.begin(), s.end(), x) - s.begin());
-                    const int col = at[(size_t)f][(size_t)(j / cap)], rank = j % cap;
-                    const int levels = p.spack[(size_t)(col / 8)].levels;
-                    n.at = (uint32_t)col | ((uint32_t)((levels + 3) / 4) << 16) | (1u << 20);
-                    for (int b = 0; b < kSliceBits; ++b)
-                        if ((rank >> b) & 1) n.rank[b / 4] |= 0x80u << (8 * (b % 4));
-                }  // a NaN threshold: never left
+    // per complete-layout node: its column and rank (-1: pass-through, or a NaN threshold)
+    std::vector<int32_t> col((size_t)T * NI, -1), rank((size_t)T * NI, -1);
+    for (size_t k = 0; k < col.size(); ++k) {
+        const int f = p.node_feat[k];
+        const float x = p.node_thr[k];
+        if (f == F || x != x) continue;
+        const auto &s = thr[(size_t)f];
+        const int j = (int)(std::lower_bound(s.begin(), s.end(), x) - s.begin());
+        col[k] = at[(size_t)f][(size_t)(j / cap)];
+        rank[k] = j % cap;
+    }
+    const int U = units_per_tree(D), n_local = (1 << unit_height(D)) - 1, FL = flush_len(D);
+    std::vector<int> lane_node((size_t)U * 32, -1), pos_node((size_t)FL);
+    for (int u = 0; u < U; ++u)
+        for (int i = 0; i < 32; ++i)
+            lane_node[(size_t)u * 32 + i] = i < n_local ? unit_node(D, u, i) : (i == 31 && u < U - 1 ? u : -1);
+    for (int i = 0; i < FL; ++i) pos_node[(size_t)i] = flush_node(D, i);
+    p.unit.assign((size_t)T * U * 32, UnitNode{0u, 0u});
+    p.rec.assign((size_t)T * NI, NodeRec{0, -1, 0u, 0u});
+    p.meta.assign((size_t)T, TreeMeta{});
+    p.flush_feat.assign((size_t)T * FL, F);
+    p.flush_rep.assign((size_t)T * (FL / 8), 0);
+    for (int t = 0; t < T; ++t) {
+        const int32_t *feat = &p.node_feat[(size_t)t * NI], *tc = &col[(size_t)t * NI], *tr = &rank[(size_t)t * NI];
+        for (int i = 0; i < U * 32; ++i) {
+            const int v = lane_node[(size_t)i];
+            if (v < 0) continue;
+            UnitNode &n = p.unit[(size_t)t * U * 32 + i];
+            if (feat[v] == F) {
+                n.at = 1u << 20;  // pass-through: always left
+            } else if (tc[v] >= 0) {
+                const int levels = p.spack[(size_t)(tc[v] / 8)].levels;
+                n.at = (uint32_t)tc[v] | ((uint32_t)((levels + 3) / 4) << 16) | (1u << 20);
+                for (int b = 0; b < kSliceBits; ++b)
+                    if ((tr[v] >> b) & 1) n.rank |= (0x80u >> (b / 4)) << (8 * (b % 4));
+            }  // a NaN threshold: never left
+        }
+        TreeMeta &m = p.meta[(size_t)t];
+        int c = 0;
+        for (int v = 0; v < NI; ++v) {  // heap order, so the nodes of word v/32 are contiguous
+            if (feat[v] == F)
+                m.pt[v >> 5] |= 1u << (v & 31);
+            else
+                p.rec[(size_t)t * NI + c++] =
+                    NodeRec{tc[v] >= 0 ? tc[v] : 0, tr[v], (D >= 7 || v < 32) ? 1u << (v & 31) : 0u,
+                            (D <= 6 && v >= 32) ? 1u << (v - 32) : 0u};
+            if ((v & 31) == 31 || v == NI - 1) m.wend[v >> 5] = (uint8_t)c;
+        }
+        for (int w = (NI - 1) / 32 + 1; w < 8; ++w) m.wend[w] = (uint8_t)c;
+        m.live = p.live[(size_t)t];
+        for (int b = 0; b < flush_batches(D); ++b) {
+            uint32_t rep = 0;
+            bool real = false, again = false;
+            for (int i = 8 * b; i < 8 * b + 8; ++i) {
+                const int v = pos_node[(size_t)i];
+                if (v < 0 || feat[v] == F) continue;  // pass-through nodes all write the scratch row
+                p.flush_feat[(size_t)t * FL + i] = feat[v];
+                real = true;
+                for (int j = 8 * b; j < i; ++j)
+                    if (pos_node[(size_t)j] >= 0 && feat[pos_node[(size_t)j]] == feat[v]) {
+                        again = again || ((rep >> (j - 8 * b)) & 1u);
+                        rep |= 1u << (i - 8 * b);
+                    }
             }
+            if (!rep) m.flush |= 1ull << b;
+            p.flush_rep[(size_t)t * (FL / 8) + b] = (uint8_t)(again ? 0xFFu : rep);
+            if (real) m.real |= 1ull << b;
+        }
+    }
 }
 
 }  // namespace
@@ -369,7 +314,6 @@ int pack_ensemble(int F, int T, const int64_t *off, const int32_t *feat, const f
         p.group_off.push_back((int32_t)p.group_leaf.size());
     }
     build_records(&p);
-    build_slices(&p);
     return 0;
 }
 

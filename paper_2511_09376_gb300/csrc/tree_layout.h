@@ -3,23 +3,23 @@
 //
 // Decision codes.  Every real inner node tests x[f] < thr (Def. "decision_tree").  The
 // packer sorts the distinct thresholds of each feature and cuts the sorted list into
-// "code columns" of at most 255 (one-byte codes) or 65535 (two-byte codes) thresholds.
-// A row's code in column c is the number of the column's thresholds u with u <= x (the
-// column's threshold count when x is NaN).  A node whose threshold is the k-th of its
-// column (rank k, 0-based) sends the row left exactly when code <= k, because the
-// thresholds are sorted: x < u_k  <=>  fewer than k + 1 of them are <= x.  A NaN
-// threshold never sends a row left (rank -1).  The kernels stage codes instead of
-// floats: one or two bytes per column and row instead of four per feature.
+// "code columns" of at most 2^kSliceBits - 1 thresholds.  A row's code in column c is the
+// number of the column's thresholds u with u <= x (the column's threshold count when x is
+// NaN).  A node whose threshold is the k-th of its column (rank k, 0-based) sends the row
+// left exactly when code <= k, because the thresholds are sorted: x < u_k  <=>  fewer than
+// k + 1 of them are <= x.  A NaN threshold never sends a row left (rank -1).  The kernels
+// stage codes instead of floats: half a byte to one and a half bytes per column and row
+// instead of four bytes per feature.
 //
-// Flush sequence of a tree of depth D (NS = 2^(D-2) bottom subtrees, cut into NG groups
-// of GS = gather_group(D) consecutive subtrees, the gather groups of the consumer
-// kernel).  Per group g: the three inner nodes r, 2r+1, 2r+2 of each of its subtrees (r =
-// NS - 1 + s), padded to a multiple of 8; then the GS - 1 inner nodes of the height-
-// log2(GS) subtree whose leaves are the group's subtree roots (heap order within it),
-// padded to a multiple of 8.  After the groups: the NG - 1 nodes above them (heap 0 ..
-// NG - 2), padded to a multiple of 8.  With one group (D <= 6) this is all bottom nodes,
-// then all nodes above them.  Batch b is positions [8b, 8b + 8).  A batch whose real
-// features are all distinct can read all its phi values before writing any.
+// Flush sequence of a tree of depth D, the order in which the consumer kernel adds node
+// values into phi.  The bottom subtrees come in groups of GS = gather_group(D) consecutive
+// ones, those of one unit (below); NG groups.  Per group: the three inner nodes r, 2r+1, 2r+2
+// of its subtrees, two subtrees to a batch of eight positions (a pair whose nodes are all
+// pass-through nodes, as below an early leaf, is skipped as a whole), then the GS - 1 inner
+// nodes above them inside the group (heap order within it), padded to a batch.  After the
+// groups: the NG - 1 nodes above them, padded to a batch.  Batch b is positions [8b, 8b + 8).
+// A batch whose real features are all distinct can read all its phi values before writing
+// any.
 #pragma once
 #include <cstdint>
 
@@ -31,8 +31,7 @@
 
 namespace wdf {
 
-// Sliced codes (the counting kernel).  The same codes, stored bit by bit: the rows of a
-// 32-row block give one 32-bit word per code bit (bit r of the word = row r), four words
+// Sliced codes.  The codes are stored bit by bit: the rows of a 32-row block give one 32-bit word per code bit (bit r of the word = row r), four words
 // (a "quad", 16 bytes) per four code bits, and a node's decision for all 32 rows is
 //   le = all ones; for every code bit from the least significant: le = majority(~bit, rank bit, le)
 // (code <= rank), eight three-input logic instructions for 32 decisions.  Columns are sorted
@@ -43,16 +42,19 @@ namespace wdf {
 //
 // The 31 inner nodes of a height-5 subtree, one per lane of a warp, are a "unit": a tree of
 // depth D >= 5 has 2^(D-5) of them, side by side below its 2^(D-5) - 1 top nodes; a smaller
-// tree is one unit of 2^D - 1 nodes.  Lane 31 of unit u carries top node u.
+// tree is one unit of 2^D - 1 nodes.  Lanes of a unit with S bottom subtrees: the S - 1 nodes
+// above them in heap order, then per subtree its root's left child, right child and the root,
+// so that the three low bits of a row's entry lie side by side in its decision word.  Lane 31
+// of unit u carries top node u.
 constexpr int kSliceBits = 12;
 constexpr int kSliceGroupPacks = 16;      // most packs (of eight columns) encoded together
 constexpr int kSliceGroupFloats = 16384;  // most thresholds of an encoding group (one pack may exceed it)
 
-// A lane's node of a unit: its column and what its rank compares with.
+// A lane's node of a unit: its column and the rank it compares with.
 struct UnitNode {
-    uint32_t at;        // column index | quads << 16 (0: none to read) | always-left << 20 (the decision of a
-                        // node without quads; with quads it is 1: a code equal to the rank goes left)
-    uint32_t rank[3];   // byte b of rank[k]: bit 7 is bit 4k + b of the rank
+    uint32_t at;    // column index | quads << 16 (0: none to read) | start << 20 (the comparison's start: 1 when
+                    // a code equal to the rank goes left; without quads it is the decision itself)
+    uint32_t rank;  // bit 7 - k of byte b is bit 4k + b of the rank
 };
 // One column of a pack: its feature and its number of thresholds (the code of a NaN).
 struct SliceCol {
@@ -71,17 +73,22 @@ struct SliceGroup {
 WDF_HD constexpr int unit_height(int D) { return D < 5 ? D : 5; }
 WDF_HD constexpr int unit_top(int D) { return D > 5 ? D - 5 : 0; }      // levels above the units
 WDF_HD constexpr int units_per_tree(int D) { return 1 << unit_top(D); }
-// Heap index of local node i (heap order within the unit) of unit u.
+WDF_HD constexpr int unit_subtrees(int D) { return 1 << (unit_height(D) - 2); }
+// Heap index of the node of lane i of unit u (i < 2^unit_height - 1).
 WDF_HD inline int unit_node(int D, int u, int i) {
-    int l = 0;
-    while ((2 << l) <= i + 1) ++l;
-    return (1 << (unit_top(D) + l)) - 1 + (u << l) + (i - ((1 << l) - 1));
+    const int S = unit_subtrees(D), top = unit_top(D);
+    if (i < S - 1) {
+        int l = 0;
+        while ((2 << l) <= i + 1) ++l;
+        return (1 << (top + l)) - 1 + (u << l) + (i - ((1 << l) - 1));
+    }
+    const int r = (1 << (D - 2)) - 1 + u * S + (i - (S - 1)) / 3, c = (i - (S - 1)) % 3;
+    return c == 2 ? r : 2 * r + 1 + c;
 }
 
-// One real inner node of a tree, in the order the decision loop visits them (heap
-// order, so the nodes of each 32-node word of the heap index are contiguous).
+// One real inner node of a tree, in heap order (the interaction kernels).
 struct NodeRec {
-    int32_t col_off;  // byte offset of the node's code column in a 32-row code block
+    int32_t col;      // the node's code column
     int32_t rank;     // left when code <= rank; -1 for a NaN threshold
     // the node's decision bit: trees of at most 64 inner nodes (depth <= 6) carry it in
     // two words (bit_lo: heap index < 32, bit_hi: the rest), deeper trees as the bit
@@ -99,27 +106,18 @@ struct TreeMeta {
 static_assert(sizeof(NodeRec) == 16, "NodeRec is one 16-byte load");
 static_assert(sizeof(TreeMeta) == 64, "TreeMeta layout");
 
-// One code column: source feature, first threshold in the sorted threshold array,
-// threshold count, and the largest power of two <= count (0 when count is 0).  With
-// one-byte codes every column occupies 255 entries of the array (NaN after its count).
-struct CodeCol {
-    int32_t feature, first, count, top;
-};
-
-// Floats per entry of the folded slot vectors: D - 2 ancestors and the three nodes of the
-// bottom subtree, padded to 4, 8 or 12.
-WDF_HD constexpr int slots_per_entry(int D) { return (D + 1) <= 4 ? 4 : ((D + 1) <= 8 ? 8 : 12); }
-// Bottom subtrees per gather group: the largest power of two <= NS whose slot vectors fit
-// in 128 registers.
-WDF_HD constexpr int gather_group(int D) {
-    int g = 1 << (D - 2);
-    while (g > 1 && g * slots_per_entry(D) > 128) g /= 2;
-    return g;
-}
+// Slots per entry of the folded slot vectors: D - 2 ancestors and the three nodes of the
+// bottom subtree.  An entry is one 16- or 32-byte vector of slots; at depth 8, whose nine
+// slots do not fit, the root's slot is kept apart (one float per entry after all vectors).
+WDF_HD constexpr int slots_per_entry(int D) { return (D + 1) <= 4 ? 4 : 8; }
+WDF_HD constexpr int extra_slots(int D) { return D == 8 ? 1 : 0; }
+// Bottom subtrees per gather group: those of a unit, whose slot vectors are in flight together
+// in at most 64 registers.
+WDF_HD constexpr int gather_group(int D) { return 1 << (unit_height(D) - 2); }
 WDF_HD constexpr int pad8(int n) { return (n + 7) & ~7; }
 WDF_HD constexpr int ilog2(int n) { return n <= 1 ? 0 : 1 + ilog2(n / 2); }
 WDF_HD constexpr int flush_groups(int D) { return (1 << (D - 2)) / gather_group(D); }
-WDF_HD constexpr int flush_group_bottom(int D) { return pad8(3 * gather_group(D)); }
+WDF_HD constexpr int flush_group_bottom(int D) { return 8 * ((gather_group(D) + 1) / 2); }
 WDF_HD constexpr int flush_group_len(int D) { return flush_group_bottom(D) + pad8(gather_group(D) - 1); }
 WDF_HD constexpr int flush_len(int D) { return flush_groups(D) * flush_group_len(D) + pad8(flush_groups(D) - 1); }
 WDF_HD constexpr int flush_batches(int D) { return flush_len(D) / 8; }
@@ -132,8 +130,10 @@ WDF_HD inline int flush_node(int D, int i) {
         return u < NG - 1 ? u : -1;
     }
     const int g = i / GL, k = i - g * GL;
-    if (k < 3 * GS) {
-        const int r = NS - 1 + g * GS + k / 3, c = k % 3;
+    if (k < flush_group_bottom(D)) {
+        const int s = 2 * (k / 8) + k % 8 / 3, c = k % 8 % 3;  // two subtrees to a batch
+        if (k % 8 >= 6 || s >= GS) return -1;
+        const int r = NS - 1 + g * GS + s;
         return c == 0 ? r : 2 * r + c;
     }
     const int u = k - flush_group_bottom(D);  // node of the group's upper subtree, heap order
@@ -144,5 +144,18 @@ WDF_HD inline int flush_node(int D, int i) {
 }
 
 static_assert(flush_batches(8) <= 64, "batch flags are one 64-bit word per tree");
+
+// Everything of a tree that the consumer kernel stages, but its line maps, as one block of
+// 16-byte words (copied asynchronously, no registers): the unit nodes; live, flush and real
+// flags; the phi offset (feature x row stride of the phi tile) of every flush position, 16
+// bits; per batch the positions whose feature an earlier position of the batch has (0xFF when
+// they repeat among themselves).  The offsets depend on the tile's rows, so an ensemble has
+// an image of its trees for every tile size.
+WDF_HD constexpr int image_flags(int D) { return units_per_tree(D) * 32 * (int)sizeof(UnitNode); }
+WDF_HD constexpr int image_offsets(int D) { return image_flags(D) + 32; }
+WDF_HD constexpr int image_repeats(int D) { return image_offsets(D) + flush_len(D) * 2; }
+WDF_HD constexpr int image_bytes(int D) { return (image_repeats(D) + flush_batches(D) + 15) & ~15; }
+constexpr int kImages = 3;
+WDF_HD constexpr int image_rows(int i) { return 32 << i; }  // tile rows of image i
 
 }  // namespace wdf

@@ -37,18 +37,13 @@ struct Packed {
     std::vector<float> node_thr;      // [T][NI]
     std::vector<float> leaf_w;        // [T][NL]
     std::vector<uint64_t> live;       // [T] bit s: bottom subtree s has a non-zero leaf
-    // decision records of the kernels (tree_layout.h): per tree the real inner nodes
-    // (rec[t * NI ...], meta[t].wend[7] of them) and the tree's metadata; the code
-    // columns and their sorted thresholds
+    // per tree its real inner nodes (rec[t * NI ...], meta[t].wend[7] of them) and its metadata
     std::vector<NodeRec> rec;         // [T][NI]
     std::vector<TreeMeta> meta;       // [T]
     std::vector<int32_t> flush_feat;  // [T][flush_len(D)] feature at each consumer flush position (F: padding
                                       // and pass-through nodes)
-    std::vector<uint64_t> xmask;      // [T][6] (depth <= 6) expand_masks of the tree's real nodes
-    std::vector<CodeCol> cols;        // [n_cols]
-    std::vector<float> col_thr;       // column segments of the sorted distinct thresholds
-    int code_bytes = 1;               // 1 or 2
-    // sliced codes (tree_layout.h): per unit 32 nodes, the columns, their packs, the groups
+    std::vector<uint8_t> flush_rep;   // [T][flush_batches(D)] repeats of every batch (tree_layout.h)
+    // decision codes (tree_layout.h): per unit 32 nodes, the columns, their packs, the groups
     // of packs encoded together, the packs' search trees and the quads' bases
     std::vector<UnitNode> unit;       // [T][units_per_tree][32]
     std::vector<SliceCol> scol;       // [packs * 8]
@@ -91,9 +86,8 @@ struct TraceRange {
 
 // Move masks of the expand of Hacker's Delight section 7-5 for mask m: expanding x with
 // them puts bit k of x at the position of the k-th set bit of m (bits of x at or above
-// popcount(m) must be zero) and leaves copies of bits only at positions outside m, which
-// the consumer kernel ORs with the pass-through bits (all ones there) instead of
-// masking.  Six steps, for shifts of 32, 16, ..., 1.
+// popcount(m) must be zero) and leaves copies of bits only at positions outside m.  Six
+// steps, for shifts of 32, 16, ..., 1.
 inline void expand_masks(uint64_t m, uint64_t mv[6]) {
     uint64_t mk = ~m << 1;  // bit p: the number of zeros of m below p is odd, after the prefix steps
     for (int i = 0; i < 6; ++i) {

@@ -41,10 +41,7 @@ struct wdf_ensemble {
     float *d_t32 = nullptr;
     wdf::NodeRec *d_rec = nullptr;
     wdf::TreeMeta *d_meta = nullptr;
-    int32_t *d_flfeat = nullptr;  // features in consumer flush order (Packed::flush_feat)
-    unsigned long long *d_xmask = nullptr;  // per tree expand masks of the real nodes (depth <= 6)
-    wdf::CodeCol *d_cols = nullptr;
-    float *d_col_thr = nullptr;
+    unsigned char *d_image = nullptr;  // the trees as the consumer kernel stages them (tree_layout.h)
     // tensor-core contraction: split operand stages (A for any mode, B for bpk_mode),
     // 128-row tiles, wait-expiry flag
     unsigned char *d_apk = nullptr;
@@ -53,7 +50,7 @@ struct wdf_ensemble {
     int4 *d_tiles128 = nullptr;
     int n_tiles128 = 0;
     int *d_err = nullptr;
-    // sliced codes (tree_layout.h)
+    // decision codes (tree_layout.h)
     wdf::UnitNode *d_unit = nullptr;
     wdf::SliceCol *d_scol = nullptr;
     wdf::SlicePack *d_spack = nullptr;
@@ -63,13 +60,10 @@ struct wdf_ensemble {
         int most = 0;
         for (const wdf::SliceGroup &g : pk.sgroup) most = g.thr_n > most ? g.thr_n : most;
         return wdf::SliceArrays{d_unit, d_scol, d_spack, d_sgroup, d_sthr, (int)pk.sgroup.size(), most,
-                                {pk.qbase[0], pk.qbase[1], pk.qbase[2]}, pk.quads};
+                                (int)pk.scol.size(), pk.spack[0].levels, {pk.qbase[0], pk.qbase[1], pk.qbase[2]}, pk.quads};
     }
-    wdf::TreeArrays arrays() const {
-        return wdf::TreeArrays{d_nodes, d_rec, d_meta, d_cols, d_col_thr, (int)pk.cols.size(), pk.code_bytes,
-                              d_xmask};
-    }
-    wdf::ExplainJob job() const { return wdf::ExplainJob{arrays(), d_sfold, d_lines, d_flfeat, pk.T, pk.F}; }
+    wdf::TreeArrays arrays() const { return wdf::TreeArrays{d_nodes, d_rec, d_meta}; }
+    wdf::ExplainJob job() const { return wdf::ExplainJob{slices(), d_image, d_sfold, d_lines, pk.T, pk.F}; }
     // background state (set_background)
     int has_bg = 0;
     int64_t m = 0;
