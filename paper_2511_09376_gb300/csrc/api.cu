@@ -86,7 +86,7 @@ namespace {
 void free_ensemble(wdf_ensemble *e) {
     dfree(e->d_nodes); dfree(e->d_keys); dfree(e->d_group_leaf); dfree(e->d_leaf_row);
     dfree(e->d_w_rows); dfree(e->d_tiles); dfree(e->d_t32);
-    dfree(e->d_rec); dfree(e->d_meta); dfree(e->d_image);
+    dfree(e->d_rec); dfree(e->d_meta); dfree(e->d_image); dfree(e->d_vlist); dfree(e->d_voff);
     dfree(e->d_unit); dfree(e->d_scol); dfree(e->d_spack); dfree(e->d_sgroup); dfree(e->d_sthr);
     dfree(e->d_apk); dfree(e->d_bpk); dfree(e->d_tiles128); dfree(e->d_err); dfree(e->d_A); dfree(e->d_ratio);
     dfree(e->d_hist); dfree(e->d_vc); dfree(e->d_scale); dfree(e->d_S); dfree(e->d_sfold); dfree(e->d_base);
@@ -327,6 +327,17 @@ wdf_status wdf_ctx_create(int32_t device, wdf_ctx **out) {
     }
     c->dev.sms = sms;
     c->dev.smem_optin = (size_t)smem;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keeps = wdf_ctx::kPoolKeeps;
+    cudaError_t e3 = cudaMemPoolCreate(&c->dev.pool, &props);
+    if (e3 == cudaSuccess) e3 = cudaMemPoolSetAttribute(c->dev.pool, cudaMemPoolAttrReleaseThreshold, &keeps);
+    if (e3 != cudaSuccess) {
+        delete c;
+        return cuda_fail(e3, "wdf_ctx_create: memory pool");
+    }
     *out = c;
     return WDF_OK;
 }
@@ -379,6 +390,8 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
     chk(dalloc(&e->d_rec, p.rec.size(), &e->bytes));
     chk(dalloc(&e->d_meta, p.meta.size(), &e->bytes));
     chk(dalloc(&e->d_image, (size_t)wdf::kImages * p.T * wdf::image_bytes(p.D), &e->bytes));
+    chk(dalloc(&e->d_vlist, std::max<size_t>(p.vlist.size(), 1), &e->bytes));
+    chk(dalloc(&e->d_voff, p.voff.size(), &e->bytes));
     int32_t *flfeat = nullptr;  // inputs of the images
     uint8_t *flrep = nullptr;
     int64_t scratch = 0;
@@ -399,6 +412,9 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
         chk(cudaMemcpy(e->d_leaf_row, p.leaf_row.data(), p.leaf_row.size() * 4, cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_rec, p.rec.data(), p.rec.size() * sizeof(wdf::NodeRec), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_meta, p.meta.data(), p.meta.size() * sizeof(wdf::TreeMeta), cudaMemcpyHostToDevice));
+        if (!p.vlist.empty())
+            chk(cudaMemcpy(e->d_vlist, p.vlist.data(), p.vlist.size() * 4, cudaMemcpyHostToDevice));
+        chk(cudaMemcpy(e->d_voff, p.voff.data(), p.voff.size() * 4, cudaMemcpyHostToDevice));
         chk(cudaMemcpy(flfeat, p.flush_feat.data(), p.flush_feat.size() * 4, cudaMemcpyHostToDevice));
         chk(cudaMemcpy(flrep, p.flush_rep.data(), p.flush_rep.size(), cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_unit, p.unit.data(), p.unit.size() * sizeof(wdf::UnitNode), cudaMemcpyHostToDevice));
@@ -653,7 +669,8 @@ wdf_status wdf_explain_interactions(wdf_ensemble *ens, const float *C, int64_t n
     const size_t n_t2 = (size_t)ens->G * K * P * K, n_s2 = (size_t)ens->n_live * P * K;
     const size_t n_s2t = folded ? wdf::iv_fold_floats(D, p.T) : (size_t)ens->n_live * K * PP;
     float *buf = nullptr;
-    WDF_CUDA(cudaMallocAsync(reinterpret_cast<void **>(&buf), std::max<size_t>(n_t2 + n_s2 + n_s2t, 4) * 4, st));
+    WDF_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void **>(&buf), std::max<size_t>(n_t2 + n_s2 + n_s2t, 4) * 4,
+                                     ens->ctx->dev.pool, st));
     float *t2 = buf, *s2 = buf + n_t2, *s2t = buf + n_t2 + n_s2;
     cudaError_t e = wdf::launch_tables_iv(D, ens->metric, ens->d_keys, ens->G, t2, st);
     if (e == cudaSuccess)
@@ -690,7 +707,7 @@ wdf_status wdf_global_attribution(wdf_ctx *ctx, const float *phi, int64_t n, int
     cudaStream_t st = (cudaStream_t)stream;
     const size_t pn = (size_t)wdf::global_attr_partial_doubles(n, n_features);
     double *partial = nullptr;
-    WDF_CUDA(cudaMallocAsync((void **)&partial, pn * sizeof(double), st));
+    WDF_CUDA(cudaMallocFromPoolAsync((void **)&partial, pn * sizeof(double), ctx->dev.pool, st));
     cudaError_t e = wdf::launch_global_attr(phi, n, ldphi, n_features, partial, mean_abs, mean, st);
     cudaFreeAsync(partial, st);
     if (e != cudaSuccess) return cuda_fail(e, "wdf_global_attribution");

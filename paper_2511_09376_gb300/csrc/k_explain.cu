@@ -55,11 +55,12 @@ WDF_EXPLAIN_DEPTH(8, extern)
 
 template <int D>
 static cudaError_t explain_depth(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi,
-                                 int64_t ldp, int tile_rows, const DevInfo &dev, cudaStream_t st) {
+                                 int64_t ldp, int tile_rows, int splits, float *scratch, const DevInfo &dev,
+                                 cudaStream_t st) {
     switch (tile_rows) {
-        case 32: return explain_t<D, 32>(codes, n, job, phi, ldp, dev, st);
-        case 128: return explain_t<D, 128>(codes, n, job, phi, ldp, dev, st);
-        default: return explain_t<D, 64>(codes, n, job, phi, ldp, dev, st);
+        case 32: return explain_t<D, 32>(codes, n, job, phi, ldp, splits, scratch, dev, st);
+        case 128: return explain_t<D, 128>(codes, n, job, phi, ldp, splits, scratch, dev, st);
+        default: return explain_t<D, 64>(codes, n, job, phi, ldp, splits, scratch, dev, st);
     }
 }
 
@@ -91,20 +92,131 @@ int default_tile_rows(int D, int F, int quads, const DevInfo &dev) {
     return best;
 }
 
+// phi = the parts' sums, added in part order; one thread per element of a row.
+__global__ void k_add_parts(const float *__restrict__ scratch, int P, int64_t n, int F, float *__restrict__ phi,
+                            int64_t ldp) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n * F) return;
+    float x = __ldg(scratch + i);
+    for (int p = 1; p < P; ++p) x += __ldg(scratch + (size_t)p * n * F + i);
+    phi[i / F * ldp + i % F] = x;
+}
+
+// phi from the node values of k_values: a warp adds one feature's nodes of 32 rows in their
+// order, a block takes eight features.  The node list is read 32 entries at a time and the
+// values 16 at a time, so their latency overlaps; only the additions are a chain.
+constexpr int kSumWarps = 8;
+__global__ void __launch_bounds__(32 * kSumWarps) k_sum_values(const float *__restrict__ values, int FL,
+                                                              const int32_t *__restrict__ vlist,
+                                                              const int32_t *__restrict__ voff, int T, int F, int P,
+                                                              int64_t n, float *__restrict__ phi, int64_t ldp) {
+    __shared__ float out[32][kSumWarps + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, f = blockIdx.x * kSumWarps + warp;
+    const float *v = values + (size_t)blockIdx.y * T * FL * 32 + lane;
+    float total = 0.0f;
+    if (f < F) {
+        for (int p = 0; p < P; ++p) {
+            const int beg = __ldg(voff + (size_t)f * P + p), end = __ldg(voff + (size_t)f * P + p + 1);
+            float acc = 0.0f;
+            for (int k0 = beg; k0 < end; k0 += 32) {
+                const int mine = k0 + lane < end ? __ldg(vlist + k0 + lane) : 0, cnt = min(32, end - k0);
+#pragma unroll
+                for (int h = 0; h < 32; h += 16) {
+                    float x[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const int i = __shfl_sync(0xFFFFFFFFu, mine, h + k);
+                        x[k] = h + k < cnt ? __ldg(v + (size_t)i * 32) : 0.0f;
+                    }
+#pragma unroll
+                    for (int k = 0; k < 16; ++k)
+                        if (h + k < cnt) acc += x[k];
+                }
+            }
+            total = p == 0 ? acc : total + acc;
+        }
+    }
+    out[lane][warp] = total;
+    __syncthreads();
+    const int r = threadIdx.x / kSumWarps, c = threadIdx.x % kSumWarps, fc = blockIdx.x * kSumWarps + c;
+    const int64_t row = (int64_t)blockIdx.y * 32 + r;
+    if (row < n && fc < F) phi[row * ldp + fc] = out[r][c];
+}
+
+template <int D>
+static cudaError_t explain_values(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi, int64_t ldp,
+                                  float *values, const DevInfo &dev, cudaStream_t st) {
+    cudaError_t err = values_t<D>(codes, n, job, values, dev, st);
+    if (err != cudaSuccess) return err;
+    const dim3 grid((unsigned)((job.F + kSumWarps - 1) / kSumWarps), (unsigned)((n + 31) / 32));
+    k_sum_values<<<grid, 32 * kSumWarps, 0, st>>>(values, flush_len(D), job.vlist, job.voff, job.T, job.F,
+                                                  explain_parts(job.T, D), n, phi, ldp);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 // Rows per encoded chunk: the decision codes of a chunk live in a stream-ordered
 // scratch allocation (so concurrent calls on other streams never share it).
 constexpr int64_t kExplainChunkRows = 1 << 20;
+// Most scratch of the node values; the context's pool keeps as much between calls.
+constexpr int64_t kValuesBytes = 320ll << 20;
+
+// How a call is spread over the GPU: splits = 0: node values (k_values, k_sum_values), else the
+// tile kernel with its tiles' parts on that many blocks.  The least of estimated microseconds:
+//  - tile kernel: its waves of resident blocks times a tile's walk of its trees, 0.034 us per
+//    tree and leaf position at full occupancy, down to half of it with a block to itself;
+//    split, the parts' sums are written and read once more;
+//  - node values: 1.4 ps (depth 8: 2.2) per row and flush position, 8 ps per row and feature.
+// Measured at 200 trees of depth 6, 127 features (node values / parts on blocks / one block a
+// tile): 1,000 rows 36 / 70 / 205 us, 2,000 rows 56 / 71, 4,000 rows 100 / 86, 8,000 rows 177 /
+// 121; 1000 trees of depth 8, 100 rows 236 / 728; 500 trees of depth 7, 777 rows 130 / 156 /
+// 1380; 50 trees of depth 4, 255 features, 20,000 rows 87 / 49.
+static int explain_splits(int D, int64_t n, const ExplainJob &job, int tile_rows, const DevInfo &dev) {
+    const int P = explain_parts(job.T, D);
+    const size_t smem = explain_smem_bytes(D, job.F, job.sa.quads, tile_rows);
+    const int64_t per_sm = std::max<int64_t>(
+        1, std::min<int64_t>((int64_t)((dev.smem_optin + 1024) / (smem + 1024)), explain_warps(D) * 16 / tile_rows));
+    const int64_t tiles = (n + tile_rows - 1) / tile_rows, room = (int64_t)dev.sms * per_sm;
+    const double walk = 0.034 * job.T * (1 << D);
+    int best = 1;
+    double least = 0.0;
+    for (int s = 1; s <= P; ++s) {
+        const double full = (double)(tiles * s) / (double)room;
+        const double waves = (double)((tiles * s + room - 1) / room) * ((P + s - 1) / s) / P;
+        const double cost = 15.0 + waves * walk * (full < 1.0 ? 0.5 + 0.5 * full : 1.0) +
+                            (s > 1 ? 4.0 + 2e-6 * (double)P * (double)n * job.F : 0.0);
+        if (s == 1 || cost < least) {
+            best = s;
+            least = cost;
+        }
+    }
+    const int64_t rows = (n + 31) / 32 * 32, positions = (int64_t)job.T * flush_len(D);
+    if (rows * positions <= kValuesBytes / (int64_t)sizeof(float)) {
+        const double cost = 20.0 + (double)rows * ((D == 8 ? 2.2e-6 : 1.4e-6) * (double)positions + 8e-6 * job.F);
+        if (cost < least) best = 0;
+    }
+    return best;
+}
 
 cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const ExplainJob &job, float *phi,
                            int64_t ldp, int tile_rows, const DevInfo &dev, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (D < 2 || D > 8) return cudaErrorInvalidValue;
     if (tile_rows <= 0) tile_rows = default_tile_rows(D, job.F, job.sa.quads, dev);
+    if (explain_smem_bytes(D, job.F, job.sa.quads, tile_rows) > dev.smem_optin) return cudaErrorInvalidConfiguration;
     const int64_t chunk = std::min(n, kExplainChunkRows);
     const int64_t pad = 128;  // every tile size divides it
+    const size_t code_bytes = (size_t)((chunk + pad - 1) / pad * pad) / 32 * job.sa.quads * 16;
+    const int splits = explain_splits(D, chunk, job, tile_rows, dev);
+    const bool values = splits == 0;  // then one chunk
+    const size_t scratch_floats = values ? (size_t)((n + 31) / 32 * 32) * job.T * flush_len(D)
+                                         : (splits > 1 ? (size_t)explain_parts(job.T, D) * chunk * job.F : 0);
+    const size_t at = (code_bytes + 255) & ~(size_t)255;
     unsigned char *codes = nullptr;
-    cudaError_t err = cudaMallocAsync(reinterpret_cast<void **>(&codes), (size_t)((chunk + pad - 1) / pad * pad) / 32 * job.sa.quads * 16, st);
+    cudaError_t err =
+        cudaMallocFromPoolAsync(reinterpret_cast<void **>(&codes), at + scratch_floats * sizeof(float), dev.pool, st);
     if (err != cudaSuccess) return err;
+    float *scratch = scratch_floats ? reinterpret_cast<float *>(codes + at) : nullptr;
     for (int64_t r0 = 0; r0 < n && err == cudaSuccess; r0 += chunk) {
         const int64_t rows = std::min(chunk, n - r0);
         err = launch_encode_slices(C + r0 * ldc, rows, ldc, job.sa, (rows + pad - 1) / pad * pad, codes, dev, st);
@@ -123,13 +235,20 @@ cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const 
             }
         }
         switch (D) {
-            case 2: err = explain_depth<2>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
-            case 3: err = explain_depth<3>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
-            case 4: err = explain_depth<4>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
-            case 5: err = explain_depth<5>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
-            case 6: err = explain_depth<6>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
-            case 7: err = explain_depth<7>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
-            default: err = explain_depth<8>(codes, rows, job, out, ldp, tile_rows, dev, st); break;
+#define WDF_EXPLAIN_CASE(d)                                                                                       \
+    case d:                                                                                                       \
+        err = values ? explain_values<d>(codes, rows, job, out, ldp, scratch, dev, st)                            \
+                     : explain_depth<d>(codes, rows, job, out, ldp, tile_rows, splits, scratch, dev, st);         \
+        break;
+            WDF_EXPLAIN_CASE(2) WDF_EXPLAIN_CASE(3) WDF_EXPLAIN_CASE(4) WDF_EXPLAIN_CASE(5)
+            WDF_EXPLAIN_CASE(6) WDF_EXPLAIN_CASE(7) WDF_EXPLAIN_CASE(8)
+#undef WDF_EXPLAIN_CASE
+        }
+        if (err == cudaSuccess && splits > 1) {
+            k_add_parts<<<(unsigned)((rows * job.F + 255) / 256), 256, 0, st>>>(scratch, explain_parts(job.T, D), rows,
+                                                                               job.F, out, ldp);
+            count_launches(1);
+            err = cudaGetLastError();
         }
         if (ev1) {  // the pair is kept only once both ends are recorded
             std::lock_guard<std::mutex> lk(g_tmu);

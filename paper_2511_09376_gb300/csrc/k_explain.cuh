@@ -49,8 +49,6 @@ template <int D>
 struct ExplainCfg {
     static constexpr int TOP = unit_top(D), UPT = units_per_tree(D);  // levels above the units, units
     static constexpr int GS = gather_group(D);                        // bottom subtrees of a unit
-    static constexpr int LG = ilog2(GS);                              // levels above them inside it
-    static constexpr int Q = slots_per_entry(D) / 4;
     static constexpr int LW = lines_words(D);
     // deep trees loop over their units (unrolled, the code of a tree does not stay in the
     // instruction cache)
@@ -147,19 +145,91 @@ __device__ __forceinline__ void load_offsets8(const uint16_t *p, int (&o)[8]) {
     o[4] = (int)(a.z & 0xFFFFu); o[5] = (int)(a.z >> 16); o[6] = (int)(a.w & 0xFFFFu); o[7] = (int)(a.w >> 16);
 }
 
-// Slot k of a gathered entry held as Q float4 registers and, at depth 8, the root's slot x0
-// apart (k a compile-time constant after unrolling).
-template <int D, int Q>
-__device__ __forceinline__ float slot_of(const float4 (&vj)[Q], float x0, int k) {
-    if (extra_slots(D) && k == 0) return x0;
-    const int at = k - extra_slots(D);
-    const float4 &x = vj[at >> 2];
-    return (at & 3) == 0 ? x.x : (at & 3) == 1 ? x.y : (at & 3) == 2 ? x.z : x.w;
+// The gathered entries of a unit's bottom subtrees: Q float4 each and, at depth 8, the root's
+// slot apart.
+template <int D>
+struct UnitSlots {
+    static constexpr int GS = gather_group(D), Q = slots_per_entry(D) / 4;
+    float4 v[GS][Q];
+    float x0[GS];
+    // slot k of subtree j (both compile-time constants after unrolling)
+    __device__ __forceinline__ float slot(int j, int k) const {
+        if (extra_slots(D) && k == 0) return x0[j];
+        const int at = k - extra_slots(D);
+        const float4 &x = v[j][at >> 2];
+        return (at & 3) == 0 ? x.x : (at & 3) == 1 ? x.y : (at & 3) == 2 ? x.z : x.w;
+    }
+};
+
+// Entries and gathers of unit u of tree t: live and lm are the live flags and line maps of its
+// subtrees, w and topw the row's decisions in the unit and at the nodes above the units.
+template <int D>
+__device__ __forceinline__ void gather_unit(const float *sfold, int T, int t, int u, uint32_t live,
+                                            const uint32_t (&lm)[(gather_group(D) + 3) / 4], uint32_t w, uint32_t topw,
+                                            UnitSlots<D> &v) {
+    using S = Shape<D>;
+    constexpr int GS = UnitSlots<D>::GS, Q = UnitSlots<D>::Q, TOP = unit_top(D);
+    constexpr uint32_t EB = 4 * S::SP;  // bytes of an entry
+    // decisions on the path to the unit's root, then R of the children of every node above its
+    // bottom subtrees (wdf_internal.h), in units of 8 entries repeated twice (line_pos), in bytes
+    constexpr uint32_t ONE = EB * ((1u << (D + 1)) + 1u);
+    uint32_t path = 0u, R[GS > 1 ? GS - 1 : 1];
+#pragma unroll
+    for (int k = 0; k < TOP; ++k) path = (path << 1) | ((topw >> ((1 << k) - 1 + (u >> (TOP - k)))) & 1u);
+    R[0] = 0u;
+#pragma unroll
+    for (int k = 0; k < GS - 1; ++k)
+        R[k] = 2u * (k == 0 ? path * (8u * ONE) : R[(k - 1) >> 1]) + ((w >> k) & 1u) * (8u * ONE);
+    const char *tf = reinterpret_cast<const char *>(sfold) + ((size_t)t * S::NS + u * GS) * S::E * EB;
+    const char *tx =
+        reinterpret_cast<const char *>(sfold + (size_t)T * S::NS * S::E * S::SP + ((size_t)t * S::NS + u * GS) * S::E);
+#pragma unroll
+    for (int j = 0; j < GS; ++j) {
+        const uint32_t on = (live >> j) & 1u;
+        const uint32_t e = (GS > 1 ? R[(GS - 2 + j) >> 1] : 0u) + ((w >> (GS - 1 + 3 * j)) & 7u) * ONE;
+        // the shift amount is the low five bits of the map's byte
+        const uint32_t at = __funnelshift_r(e, 0u, lm[j >> 2] >> (8 * (j & 3))) & ((S::E - 1) * EB);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) v.v[j][k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if constexpr (Q == 2) ldg_f8_if(tf + j * (int)(S::E * EB) + at, v.v[j][0], v.v[j][Q - 1], on);
+        else ldg_f4_if(tf + j * (int)(S::E * EB) + at, v.v[j][0], on);
+        if (extra_slots(D))
+            asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v.x0[j]) : "l"(tx + j * (int)(S::E * 4) + at / 8));
+        else
+            v.x0[j] = 0.0f;
+    }
+}
+
+// Values of the nodes above a unit's bottom subtrees: up, inside the unit (heap order); top, the
+// nodes above the units, on the unit's path (the first unit below one starts its sum).
+template <int D>
+__device__ __forceinline__ void unit_sums(const UnitSlots<D> &v, int u, float (&up)[gather_group(D) > 1 ? gather_group(D) - 1 : 1],
+                                          float (&top)[units_per_tree(D) > 1 ? units_per_tree(D) - 1 : 1]) {
+    constexpr int GS = gather_group(D), TOP = unit_top(D), LG = ilog2(GS);
+#pragma unroll
+    for (int k = 0; k < GS - 1; ++k) up[k] = 0.0f;
+#pragma unroll
+    for (int j = 0; j < GS; ++j)
+#pragma unroll
+        for (int l = 0; l < LG; ++l) up[(1 << l) - 1 + (j >> (LG - l))] += v.slot(j, TOP + l);
+#pragma unroll
+    for (int k = 0; k < TOP; ++k) {
+        float x = v.slot(0, k);
+#pragma unroll
+        for (int j = 1; j < GS; ++j) x += v.slot(j, k);
+        const int node = u >> (TOP - k);
+#pragma unroll
+        for (int p = 0; p < 1 << k; ++p) {
+            float &tp = top[(1 << k) - 1 + p];
+            if (p == node) tp = u & ((1 << (TOP - k)) - 1) ? tp + x : x;
+        }
+    }
 }
 
 // One tile of TC consumer rows starting at row c0 (of n rows), for one ensemble: parts
-// [part0, part1) of its trees, the first stored into phi, the others added.  The rows' decision
-// codes are copied from codes, the code blocks of all n rows written by k_encode_slices or
+// [part0, part1) of its trees.  With scratch null the parts are all of them, the first stored
+// into phi, the others added; else part p is stored at scratch + p * n * F, row stride F, and
+// k_add_parts adds them.  The rows' decision codes are copied from codes, the code blocks of all n rows written by k_encode_slices or
 // k_encode_batch (padded to a multiple of TC rows).
 //
 // Two warps share 32 rows, their codes and their phi columns: the first takes the even trees of
@@ -170,10 +240,9 @@ __device__ __forceinline__ float slot_of(const float4 (&vj)[Q], float x0, int k)
 template <int D, int TC>
 __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsigned char *__restrict__ codes,
                                              int64_t n, float *__restrict__ phi, int64_t ldp, int64_t c0, int part0,
-                                             int part1, unsigned char *smem_raw) {
-    using S = Shape<D>;
+                                             int part1, float *__restrict__ scratch, unsigned char *smem_raw) {
     using X = ExplainCfg<D>;
-    constexpr int XS = TC + 1, GS = X::GS, Q = X::Q, TOP = X::TOP, UPT = X::UPT, LG = X::LG;
+    constexpr int XS = TC + 1, GS = X::GS, TOP = X::TOP, UPT = X::UPT;
     constexpr int NT = explain_threads(TC), SLOTS = ExLayout<D>::SLOTS;
     constexpr int FB = flush_group_bottom(D), GL = flush_group_len(D), LW = X::LW;
     constexpr int IMG = image_bytes(D), LINE = ExLayout<D>::LINE, TREE = ExLayout<D>::TREE;
@@ -239,44 +308,14 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         }
         return q;
     };
-    float4 v[GS][Q];
-    float x0[GS];  // depth 8: the root's slots
-    // Entries and gathers of unit u of tree t.
+    UnitSlots<D> v;
     auto gather = [&](int t, const unsigned char *slot, int u, const Words &p, bool mine) {
-        constexpr uint32_t EB = 4 * S::SP;  // bytes of an entry
-        const uint32_t live = (uint32_t)(*reinterpret_cast<const uint64_t *>(slot + image_flags(D)) >> (u * GS)) & (mine ? ~0u : 0u);
-        uint32_t lm[GS / 4 > 0 ? GS / 4 : 1];
+        const uint32_t live = (uint32_t)(*reinterpret_cast<const uint64_t *>(slot + image_flags(D)) >> (u * GS));
+        uint32_t lm[(GS + 3) / 4];
 #pragma unroll
         for (int k = 0; k < (GS + 3) / 4; ++k)
             lm[k] = reinterpret_cast<const uint32_t *>(slot + LINE)[u * (GS / 4) + k];
-        // decisions on the path to the unit's root, then R of the children of every node above its
-        // bottom subtrees (wdf_internal.h), in units of 8 entries repeated twice (line_pos), in bytes
-        constexpr uint32_t ONE = EB * ((1u << (D + 1)) + 1u);
-        uint32_t path = 0u, R[GS > 1 ? GS - 1 : 1];
-#pragma unroll
-        for (int k = 0; k < TOP; ++k) path = (path << 1) | ((p.top >> ((1 << k) - 1 + (u >> (TOP - k)))) & 1u);
-        R[0] = 0u;
-#pragma unroll
-        for (int k = 0; k < GS - 1; ++k)
-            R[k] = 2u * (k == 0 ? path * (8u * ONE) : R[(k - 1) >> 1]) + ((p.w >> k) & 1u) * (8u * ONE);
-        const char *tf = reinterpret_cast<const char *>(job.sfold) + ((size_t)t * S::NS + u * GS) * S::E * EB;
-        const char *tx = reinterpret_cast<const char *>(job.sfold + (size_t)T * S::NS * S::E * S::SP +
-                                                        ((size_t)t * S::NS + u * GS) * S::E);
-#pragma unroll
-        for (int j = 0; j < GS; ++j) {
-            const uint32_t on = (live >> j) & 1u;
-            const uint32_t e = (GS > 1 ? R[(GS - 2 + j) >> 1] : 0u) + ((p.w >> (GS - 1 + 3 * j)) & 7u) * ONE;
-            // the shift amount is the low five bits of the map's byte
-            const uint32_t at = __funnelshift_r(e, 0u, lm[j >> 2] >> (8 * (j & 3))) & ((S::E - 1) * EB);
-#pragma unroll
-            for (int k = 0; k < Q; ++k) v[j][k] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if constexpr (Q == 2) ldg_f8_if(tf + j * (int)(S::E * EB) + at, v[j][0], v[j][Q - 1], on);
-            else ldg_f4_if(tf + j * (int)(S::E * EB) + at, v[j][0], on);
-            if (extra_slots(D))
-                asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(x0[j]) : "l"(tx + j * (int)(S::E * 4) + at / 8));
-            else
-                x0[j] = 0.0f;
-        }
+        gather_unit<D>(job.sfold, T, t, u, mine ? live : 0u, lm, p.w, p.top, v);
     };
     float top[UPT > 1 ? UPT - 1 : 1];
     // Adds unit u's node values into phi; the top nodes' sums are kept until the tree's last unit.
@@ -286,28 +325,10 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         const uint32_t real = (uint32_t)(reinterpret_cast<const uint64_t *>(slot + image_flags(D))[2] >> (u * (GL / 8))) &
                               (mine ? ~0u : 0u);
         const unsigned char *rep = slot + image_repeats(D) + u * (GL / 8);
-        auto val = [&](int j, int k) { return slot_of<D>(v[j], x0[j], k); };
         int o[8];
         load_offsets8(off, o);
         float up[GS > 1 ? GS - 1 : 1];
-#pragma unroll
-        for (int k = 0; k < GS - 1; ++k) up[k] = 0.0f;
-#pragma unroll
-        for (int j = 0; j < GS; ++j)
-#pragma unroll
-            for (int l = 0; l < LG; ++l) up[(1 << l) - 1 + (j >> (LG - l))] += val(j, TOP + l);
-#pragma unroll
-        for (int k = 0; k < TOP; ++k) {
-            float x = val(0, k);
-#pragma unroll
-            for (int j = 1; j < GS; ++j) x += val(j, k);
-            const int node = u >> (TOP - k);
-#pragma unroll
-            for (int p = 0; p < 1 << k; ++p) {
-                float &tp = top[(1 << k) - 1 + p];
-                if (p == node) tp = u & ((1 << (TOP - k)) - 1) ? tp + x : x;
-            }
-        }
+        unit_sums<D>(v, u, up, top);
 #pragma unroll
         for (int b = 0; b < GL / 8; ++b) {
             int on[8];
@@ -316,7 +337,7 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 if (b < FB / 8)  // two subtrees to a batch
-                    x[q] = q < 6 ? val(2 * b + q / 3 < GS ? 2 * b + q / 3 : 0, D - 2 + q % 3) : 0.0f;
+                    x[q] = q < 6 ? v.slot(2 * b + q / 3 < GS ? 2 * b + q / 3 : 0, D - 2 + q % 3) : 0.0f;
                 else
                     x[q] = q < GS - 1 ? up[q < GS - 1 ? q : 0] : 0.0f;
             }
@@ -376,10 +397,10 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         for (int r = half; r < 32; r += 2) {
             const int64_t row = c0 + 32 * pair + r;
             if (row >= n) break;
-            float *dst = phi + row * ldp;
+            float *dst = scratch ? scratch + ((size_t)part * n + row) * F : phi + row * ldp;
             for (int f = lane; f < F; f += 32) {
                 const float x = sp[f * XS + 32 * pair + r];
-                dst[f] = part > part0 ? dst[f] + x : x;
+                dst[f] = part > part0 && !scratch ? dst[f] + x : x;
                 sp[f * XS + 32 * pair + r] = 0.0f;
             }
         }
@@ -387,11 +408,73 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
     }
 }
 
+// Block (tile, y): parts [P y / gridDim.y, P (y + 1) / gridDim.y) of the tile's rows (scratch
+// non-null when there is more than one y).
 template <int D, int TC>
-__global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16 / TC) k_explain(const unsigned char *__restrict__ codes, int64_t n,
-                                                   ExplainJob job, float *__restrict__ phi, int64_t ldp) {
+__global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16 / TC) k_explain(const unsigned char *__restrict__ codes, int64_t n, ExplainJob job, float *__restrict__ phi, int64_t ldp,
+              float *__restrict__ scratch) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    explain_tile<D, TC>(job, codes, n, phi, ldp, (int64_t)blockIdx.x * TC, 0, explain_parts(job.T, D), smem_raw);
+    const int P = explain_parts(job.T, D), y = blockIdx.y, Y = gridDim.y;
+    explain_tile<D, TC>(job, codes, n, phi, ldp, (int64_t)blockIdx.x * TC, P * y / Y, P * (y + 1) / Y, scratch, smem_raw);
+}
+
+// Few rows: the node values of 32 rows and one tree per warp, every tree at once, position i of
+// the flush order at values + (((row block) * T + t) * flush_len + i) * 32 + row;
+// k_sum_values then adds each feature's in the order of the tile kernel.  Latency-bound.
+constexpr int kValueWarps = 4;
+template <int D>
+__global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char *__restrict__ codes, ExplainJob job,
+                                                            float *__restrict__ values) {
+    using X = ExplainCfg<D>;
+    constexpr int GS = X::GS, TOP = X::TOP, UPT = X::UPT, LW = X::LW;
+    constexpr int FB = flush_group_bottom(D), GL = flush_group_len(D), FL = flush_len(D);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, quads = job.sa.quads;
+    uint4 *block = reinterpret_cast<uint4 *>(smem_raw);
+    const int t = blockIdx.x * kValueWarps + (tid >> 5), tt = min(t, job.T - 1);
+    const uint2 *rec = reinterpret_cast<const uint2 *>(job.sa.unit) + (size_t)tt * UPT * 32;
+    const uint64_t *flags = reinterpret_cast<const uint64_t *>(job.image + (size_t)tt * image_bytes(D) + image_flags(D));
+    const uint64_t live = __ldg(flags), real = __ldg(flags + 2);
+    const uint4 *src = reinterpret_cast<const uint4 *>(codes) + (size_t)blockIdx.y * quads;
+    for (int i = tid; i < quads; i += 32 * kValueWarps) block[i] = __ldg(src + i);
+    __syncthreads();
+    if (t >= job.T) return;
+    uint32_t topw = 0u;
+    if (TOP > 1)
+        topw = transpose32(lane < UPT - 1 ? unit_decide(__ldg(rec + lane * 32 + 31), block, job.sa) : 0u, lane);
+    float *out = values + ((size_t)blockIdx.y * job.T + t) * FL * 32 + lane;
+    float top[UPT > 1 ? UPT - 1 : 1];
+    uint2 node = __ldg(rec + lane);
+#pragma unroll X::UNROLL
+    for (int u = 0; u < UPT; ++u) {
+        const uint32_t w = transpose32(unit_decide(node, block, job.sa), lane);
+        if (TOP == 1 && u == 0) topw = w >> 31;
+        uint32_t lm[(GS + 3) / 4];
+#pragma unroll
+        for (int k = 0; k < (GS + 3) / 4; ++k) lm[k] = __ldg(job.lines + (size_t)t * LW + u * (GS / 4) + k);
+        UnitSlots<D> v;
+        gather_unit<D>(job.sfold, job.T, t, u, (uint32_t)(live >> (u * GS)), lm, w, topw, v);
+        if (u + 1 < UPT) node = __ldg(rec + (u + 1) * 32 + lane);
+        float up[GS > 1 ? GS - 1 : 1];
+        unit_sums<D>(v, u, up, top);
+        const uint32_t some = (uint32_t)(real >> (u * (GL / 8)));
+        float *dst = out + (size_t)u * GL * 32;
+#pragma unroll
+        for (int b = 0; b < GL / 8; ++b) {
+            if (!((some >> b) & 1u)) continue;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                if (b < FB / 8) {
+                    if (q < 6 && 2 * b + q / 3 < GS)
+                        dst[(8 * b + q) * 32] = v.slot(2 * b + q / 3 < GS ? 2 * b + q / 3 : 0, D - 2 + q % 3);
+                } else if (q < GS - 1) {
+                    dst[(8 * b + q) * 32] = up[q < GS - 1 ? q : 0];
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < UPT - 1; ++k) out[(size_t)(UPT * GL + k) * 32] = top[k];
 }
 
 // Persistent form over a ragged batch: work item i is (job, request, first row).  Blocks
@@ -416,21 +499,35 @@ __global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16
         const ExplainJob job = jobs[it.x];
         const BatchRequest rq = reqs[it.y];
         const int64_t c0 = ((int64_t)it.z << 31) | (uint32_t)it.w;
-        explain_tile<D, TC>(job, rq.codes, rq.n, rq.phi, rq.ldp, c0, 0, explain_parts(job.T, D), smem_raw);
+        explain_tile<D, TC>(job, rq.codes, rq.n, rq.phi, rq.ldp, c0, 0, explain_parts(job.T, D), nullptr, smem_raw);
         __syncthreads();
     }
 }
 
 template <int D, int TC>
 cudaError_t explain_t(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi, int64_t ldp,
-                      const DevInfo &dev, cudaStream_t st) {
+                      int splits, float *scratch, const DevInfo &dev, cudaStream_t st) {
     const size_t smem = ExLayout<D>(job.F, job.sa.quads, TC).total;
     if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
     auto kern = k_explain<D, TC>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const int64_t blocks = (n + TC - 1) / TC;
-    kern<<<(unsigned)blocks, explain_threads(TC), smem, st>>>(codes, n, job, phi, ldp);
+    kern<<<dim3((unsigned)blocks, (unsigned)splits), explain_threads(TC), smem, st>>>(codes, n, job, phi, ldp, scratch);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
+template <int D>
+cudaError_t values_t(const unsigned char *codes, int64_t n, const ExplainJob &job, float *values, const DevInfo &dev,
+                     cudaStream_t st) {
+    const size_t smem = (size_t)job.sa.quads * 16;
+    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
+    auto kern = k_values<D>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    const dim3 grid((unsigned)((job.T + kValueWarps - 1) / kValueWarps), (unsigned)((n + 31) / 32));
+    kern<<<grid, 32 * kValueWarps, smem, st>>>(codes, job, values);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -458,10 +555,13 @@ cudaError_t batch_t(const ExplainJob *jobs, const BatchRequest *reqs, const int4
 // compiled in one of the k_explain_d*.cu translation units.
 #define WDF_EXPLAIN_TILE(d, tc, spec)                                                                            \
     spec template cudaError_t explain_t<d, tc>(const unsigned char *, int64_t, const ExplainJob &, float *,       \
-                                               int64_t, const DevInfo &, cudaStream_t);                          \
+                                               int64_t, int, float *, const DevInfo &, cudaStream_t);            \
     spec template cudaError_t batch_t<d, tc>(const ExplainJob *, const BatchRequest *, const int4 *, int *, int,  \
                                              int, int, const DevInfo &, cudaStream_t);
+#define WDF_EXPLAIN_VALUES(d, spec)                                                                              \
+    spec template cudaError_t values_t<d>(const unsigned char *, int64_t, const ExplainJob &, float *,           \
+                                          const DevInfo &, cudaStream_t);
 #define WDF_EXPLAIN_DEPTH(d, spec) WDF_EXPLAIN_TILE(d, 32, spec) WDF_EXPLAIN_TILE(d, 64, spec) \
-    WDF_EXPLAIN_TILE(d, 128, spec)
+    WDF_EXPLAIN_TILE(d, 128, spec) WDF_EXPLAIN_VALUES(d, spec)
 
 }  // namespace wdf

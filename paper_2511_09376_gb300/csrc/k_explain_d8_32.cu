@@ -3,4 +3,5 @@
 
 namespace wdf {
 WDF_EXPLAIN_TILE(8, 32, )
+WDF_EXPLAIN_VALUES(8, )
 }  // namespace wdf

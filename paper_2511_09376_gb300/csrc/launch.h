@@ -37,18 +37,10 @@ struct ExplainJob {
     const unsigned char *image;  // [kImages][T][image_bytes(D)] (tree_layout.h)
     const float *sfold;     // folded slot vectors [T][NS][2^(D+1)][slots_per_entry], entry e at line_pos(e), then
                             // (depth 8) the root slots [T][NS][2^(D+1)]
+    const int32_t *vlist, *voff;  // nodes of every feature and part in the order of addition (Packed)
     const uint32_t *lines;  // per tree lines_words(D) words: byte s = line map of subtree s
     int T, F;
 };
-// A row's phi is the sum of the sums of its ensemble's parts, in part order: part p of P holds
-// trees [T p / P, T (p + 1) / P), each part's trees added in order from zero.  The split
-// depends on the ensemble alone, so a row's result does not depend on how many blocks
-// share its parts.
-inline __host__ __device__ int explain_parts(int T, int D) {
-    const long long p = (((long long)T << D) + 1600) / 3200;  // about 50 trees of depth 6 to a part
-    return p < 1 ? 1 : p > 8 ? 8 : (int)p;
-}
-
 // Where the consumer gathers land.  A warp's 32-byte gathers of one bottom subtree are
 // served a quarter warp at a time, one L1 wavefront per distinct 128-byte line, and a
 // line holds four consecutive entries.  Entries are formed from D + 1 decision bits;
@@ -82,6 +74,7 @@ struct BatchRequest {
 struct DevInfo {
     int sms = 0;
     size_t smem_optin = 0;  // max dynamic shared memory per block
+    cudaMemPool_t pool = nullptr;  // the context's stream-ordered scratch
 };
 
 // Step 1 of Algorithm 3 (background): joint entry counts hist[T][NS][2^(D+1)] (u32,
@@ -175,7 +168,8 @@ cudaError_t launch_images(int D, int T, const UnitNode *unit, const TreeMeta *me
                           const uint8_t *flrep, unsigned char *image, cudaStream_t st);
 
 // Step 4: phi of n consumer rows, tile_rows consumer rows per block (32, 64 or 128;
-// 0 picks the default for the shared-memory budget).
+// 0 picks the default for the shared-memory budget).  Scratch (codes, partial sums) comes
+// from dev.pool in stream order.
 cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const ExplainJob &job, float *phi,
                            int64_t ldp, int tile_rows, const DevInfo &dev, cudaStream_t st);
 // Consumer-kernel timing (process-wide): while on, launch_explain brackets every

@@ -203,6 +203,38 @@ void build_records(Packed *pp) {
     }
 }
 
+// The nodes of every feature in the order of the consumer kernel (k_explain.cuh): within a part
+// its trees two by two, in turns unit by unit; within a unit its flush positions; the nodes
+// above the units with the tree's last unit.
+void build_value_lists(Packed *pp) {
+    Packed &p = *pp;
+    const int F = p.F, T = p.T, D = p.D, FL = flush_len(D), GL = flush_group_len(D), U = units_per_tree(D);
+    const int P = explain_parts(T, D);
+    p.voff.assign((size_t)F * P + 1, 0);
+    std::vector<int32_t> count((size_t)F * P + 1, 0);
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int part = 0; part < P; ++part) {
+            const int tb = (int)((long long)T * part / P), te = (int)((long long)T * (part + 1) / P);
+            for (int t0 = tb; t0 < te; t0 += 2)
+                for (int u = 0; u < U; ++u)
+                    for (int t = t0; t < te && t < t0 + 2; ++t) {
+                        const int end = u == U - 1 ? FL : (u + 1) * GL;
+                        for (int i = u * GL; i < end; ++i) {
+                            const int f = p.flush_feat[(size_t)t * FL + i];
+                            if (f == F) continue;
+                            const size_t k = (size_t)f * P + part;
+                            if (pass == 0) ++p.voff[k + 1];
+                            else p.vlist[(size_t)p.voff[k] + count[k]++] = t * FL + i;
+                        }
+                    }
+        }
+        if (pass == 0) {
+            for (size_t k = 0; k < (size_t)F * P; ++k) p.voff[k + 1] += p.voff[k];
+            p.vlist.assign((size_t)p.voff[(size_t)F * P], 0);
+        }
+    }
+}
+
 }  // namespace
 
 int pack_ensemble(int F, int T, const int64_t *off, const int32_t *feat, const float *thr, const int32_t *left,
@@ -314,6 +346,7 @@ int pack_ensemble(int F, int T, const int64_t *off, const int32_t *feat, const f
         p.group_off.push_back((int32_t)p.group_leaf.size());
     }
     build_records(&p);
+    build_value_lists(&p);
     return 0;
 }
 

@@ -125,12 +125,12 @@ cudaError_t launch_wave(wdf_server *s, Wave &w, bool *recorded) {
     cudaError_t err = cudaSuccess;
     for (Part &r : w.parts) {
         const size_t row_bytes = (size_t)r.F * sizeof(float);
-        err = cudaMallocAsync((void **)&r.d_C, r.n * row_bytes, st);
+        err = cudaMallocFromPoolAsync((void **)&r.d_C, r.n * row_bytes, s->ctx->dev.pool, st);
         if (err != cudaSuccess) {
             r.d_C = nullptr;
             break;
         }
-        err = cudaMallocAsync((void **)&r.d_phi, r.n * row_bytes, st);
+        err = cudaMallocFromPoolAsync((void **)&r.d_phi, r.n * row_bytes, s->ctx->dev.pool, st);
         if (err != cudaSuccess) {
             r.d_phi = nullptr;
             break;

@@ -155,6 +155,16 @@ WDF_HD constexpr int image_flags(int D) { return units_per_tree(D) * 32 * (int)s
 WDF_HD constexpr int image_offsets(int D) { return image_flags(D) + 32; }
 WDF_HD constexpr int image_repeats(int D) { return image_offsets(D) + flush_len(D) * 2; }
 WDF_HD constexpr int image_bytes(int D) { return (image_repeats(D) + flush_batches(D) + 15) & ~15; }
+// A row's phi is the sum of the sums of its ensemble's parts, in part order: part p of P holds
+// trees [T p / P, T (p + 1) / P), each part's nodes added in the consumer kernel's order from
+// zero.  The split depends on the ensemble alone, so a row's result does not depend on how
+// many blocks share its parts.  About 50 trees of depth 6 to a part: a part's end costs what
+// 1.3 such trees cost.
+WDF_HD inline int explain_parts(int T, int D) {
+    const long long p = (((long long)T << D) + 1600) / 3200;
+    return p < 1 ? 1 : p > 8 ? 8 : (int)p;
+}
+
 constexpr int kImages = 3;
 WDF_HD constexpr int image_rows(int i) { return 32 << i; }  // tile rows of image i
 

@@ -43,6 +43,10 @@ struct Packed {
     std::vector<int32_t> flush_feat;  // [T][flush_len(D)] feature at each consumer flush position (F: padding
                                       // and pass-through nodes)
     std::vector<uint8_t> flush_rep;   // [T][flush_batches(D)] repeats of every batch (tree_layout.h)
+    // per feature and part (explain_parts) the real nodes, as tree * flush_len + flush position, in
+    // the order the consumer kernel adds them: vlist[voff[f * parts + p] ...]
+    std::vector<int32_t> vlist;
+    std::vector<int32_t> voff;        // [F * parts + 1]
     // decision codes (tree_layout.h): per unit 32 nodes, the columns, their packs, the groups
     // of packs encoded together, the packs' search trees and the quads' bases
     std::vector<UnitNode> unit;       // [T][units_per_tree][32]

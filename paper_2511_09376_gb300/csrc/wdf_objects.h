@@ -9,6 +9,13 @@
 struct wdf_ctx {
     int device = 0;
     wdf::DevInfo dev;
+    // Scratch of the calls on this context's objects is allocated in stream order from a pool of
+    // its own, which keeps up to this much between calls (the default pool gives everything
+    // back at each synchronisation, and mapping it again cost 0.2 ms a call).
+    static constexpr uint64_t kPoolKeeps = 384ull << 20;
+    ~wdf_ctx() {
+        if (dev.pool) cudaMemPoolDestroy(dev.pool);
+    }
     // the caller's handle plus one reference per ensemble, batch and server made from the
     // context, so wdf_ctx_destroy may come before theirs: the last reference frees it
     std::atomic<int> refs{1};
@@ -50,6 +57,7 @@ struct wdf_ensemble {
     int4 *d_tiles128 = nullptr;
     int n_tiles128 = 0;
     int *d_err = nullptr;
+    int32_t *d_vlist = nullptr, *d_voff = nullptr;  // Packed::vlist, voff
     // decision codes (tree_layout.h)
     wdf::UnitNode *d_unit = nullptr;
     wdf::SliceCol *d_scol = nullptr;
@@ -63,7 +71,7 @@ struct wdf_ensemble {
                                 (int)pk.scol.size(), pk.spack[0].levels, {pk.qbase[0], pk.qbase[1], pk.qbase[2]}, pk.quads};
     }
     wdf::TreeArrays arrays() const { return wdf::TreeArrays{d_nodes, d_rec, d_meta}; }
-    wdf::ExplainJob job() const { return wdf::ExplainJob{slices(), d_image, d_sfold, d_lines, pk.T, pk.F}; }
+    wdf::ExplainJob job() const { return wdf::ExplainJob{slices(), d_image, d_sfold, d_vlist, d_voff, d_lines, pk.T, pk.F}; }
     // background state (set_background)
     int has_bg = 0;
     int64_t m = 0;

@@ -29,6 +29,10 @@ def _check(ctx, D, T, F, n, seed, early=0.12):
     got = wdf.explain(e, torch.from_numpy(C).cuda()).cpu().numpy()
     want = oracle.values_hist(ens, oracle.bg_hist(ens, B), B.shape[0], C)
     assert_phi_close(got, want, f"D={D} T={T} F={F} n={n}")
+    batch = wdf.batch_create(ctx, [e])
+    tile = wdf.batch_explain(batch, [(0, torch.from_numpy(C).cuda())])[0]
+    np.testing.assert_array_equal(got, tile.cpu().numpy())
+    batch.close()
     e.close()
 
 
@@ -49,3 +53,9 @@ def test_repeated_features(ctx, depth, features):
                                          (7, 39), (3, 601)])
 def test_parts(ctx, depth, trees):
     _check(ctx, depth, trees, 30, 65, 1200 + depth)
+
+
+# more rows, with fewer tiles than the GPU holds blocks: the tile kernel, parts on several blocks
+@pytest.mark.parametrize("depth,trees,rows", [(8, 101, 5000), (7, 260, 4033), (6, 230, 6001), (5, 640, 5000)])
+def test_parts_on_several_blocks(ctx, depth, trees, rows):
+    _check(ctx, depth, trees, 40, rows, 1300 + depth)
