@@ -89,7 +89,7 @@ void free_ensemble(wdf_ensemble *e) {
     dfree(e->d_rec); dfree(e->d_meta); dfree(e->d_image); dfree(e->d_vlist); dfree(e->d_voff);
     dfree(e->d_unit); dfree(e->d_scol); dfree(e->d_spack); dfree(e->d_sgroup); dfree(e->d_sthr);
     dfree(e->d_apk); dfree(e->d_bpk); dfree(e->d_tiles128); dfree(e->d_err); dfree(e->d_A); dfree(e->d_ratio);
-    dfree(e->d_hist); dfree(e->d_vc); dfree(e->d_scale); dfree(e->d_S); dfree(e->d_sfold); dfree(e->d_base);
+    dfree(e->d_hist); dfree(e->d_scale); dfree(e->d_S); dfree(e->d_sfold); dfree(e->d_base);
     dfree(e->d_lines);
     for (int i = 0; i < 2; ++i) {
         dfree(e->d_codes[i]);
@@ -224,21 +224,23 @@ bool valid_precision(wdf_precision p) {
 // The tensor-core kernel's operand split: 0 = TF32 two parts, 1 = BF16 two, 2 = BF16 three.
 int tc_mode(wdf_precision p) { return p == WDF_TF32X3 ? 0 : (p == WDF_BF16X3 ? 1 : 2); }
 
-// Buffers of the consumer-independent half (counts, frequencies, S, folded vectors) and,
-// for the tensor-core precisions, the K-major tables.
-wdf_status ensure_frequency_state(wdf_ensemble *ens, wdf_precision precision) {
+// Buffers of the consumer-independent half (counts, folded vectors), for a dense contraction
+// (path-dependent frequencies, tensor-core precisions) its operands and per-leaf values, and
+// for the tensor-core precisions the K-major tables.
+wdf_status ensure_frequency_state(wdf_ensemble *ens, wdf_precision precision, bool path_dependent) {
     const wdf::Packed &p = ens->pk;
     const int K = 1 << p.D, N = p.D << p.D;
     const size_t hist_n = (size_t)p.T * p.NS * (2 * K);
     if (!ens->d_hist) {
         WDF_CUDA(dalloc(&ens->d_hist, hist_n, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_vc, (size_t)ens->n_live * K, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_A, (size_t)ens->n_live * K, &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_scale, (size_t)ens->n_live, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_S, (size_t)ens->n_live * N, &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_sfold, hist_n * (wdf::slots_per_entry(p.D) + wdf::extra_slots(p.D)), &ens->bytes));
         WDF_CUDA(dalloc(&ens->d_lines, (size_t)p.T * wdf::lines_words(p.D), &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_base, 1, &ens->bytes));
+        WDF_CUDA(dalloc(&ens->d_base, wdf::kBaseBlocks + 1, &ens->bytes));
+    }
+    if ((path_dependent || precision != WDF_FP32) && !ens->d_S) {
+        if (!ens->d_A) WDF_CUDA(dalloc(&ens->d_A, (size_t)ens->n_live * K, &ens->bytes));
+        WDF_CUDA(dalloc(&ens->d_S, (size_t)ens->n_live * N, &ens->bytes));
     }
     ens->has_bg = 0;
     if (precision != WDF_FP32) return ensure_tensor_core_state(ens, tc_mode(precision));
@@ -268,16 +270,23 @@ wdf_status contract_and_fold(wdf_ensemble *ens, wdf_precision precision, cudaStr
     return WDF_OK;
 }
 
-// Steps 2-3 of Algorithm 3 after the joint counts are in d_hist: per-leaf counts (and
-// the FP32 frequency operand), scales w_l / m, E_b f(b), contraction and fold.
+// Steps 2-3 of Algorithm 3 after the joint counts are in d_hist: scales w_l / m, E_b f(b),
+// line maps, and the folded vectors: in FP32 straight from the counts, else through the
+// per-leaf counts and the tensor-core contraction.
 wdf_status finish_background(wdf_ensemble *ens, int64_t m, wdf_precision precision, cudaStream_t st) {
     const wdf::Packed &p = ens->pk;
-    WDF_CUDA(wdf::launch_leaf_counts(p.D, ens->d_hist, ens->d_group_leaf, ens->n_live, ens->d_vc, ens->d_A, st));
     WDF_CUDA(wdf::launch_scale(ens->d_w_rows, ens->n_live, m, ens->d_scale, st));
-    WDF_CUDA(wdf::launch_base_value(p.D, ens->d_vc, nullptr, ens->d_w_rows, ens->n_live, m, ens->d_base, st));
+    WDF_CUDA(wdf::launch_base_value(p.D, ens->d_hist, ens->d_group_leaf, nullptr, ens->d_w_rows, ens->n_live, m,
+                                    ens->d_base, st));
     WDF_CUDA(wdf::launch_line_maps(p.D, ens->d_hist, ens->d_meta, p.T, ens->d_lines, st));
-    wdf_status s1 = contract_and_fold(ens, precision, st);
-    if (s1 != WDF_OK) return s1;
+    if (precision == WDF_FP32) {
+        WDF_CUDA(wdf::launch_subtree_fold(p.D, ens->metric, ens->d_hist, ens->d_nodes, p.F, ens->d_leaf_row,
+                                          ens->d_scale, p.T, ens->d_lines, ens->d_sfold, ens->ctx->dev, st));
+    } else {
+        WDF_CUDA(wdf::launch_leaf_counts(p.D, ens->d_hist, ens->d_group_leaf, ens->n_live, nullptr, ens->d_A, st));
+        wdf_status s1 = contract_and_fold(ens, precision, st);
+        if (s1 != WDF_OK) return s1;
+    }
     ens->m = m;
     ens->pd = 0;
     ens->has_bg = 1;
@@ -500,7 +509,7 @@ wdf_status wdf_set_background(wdf_ensemble *ens, const float *B, int64_t m, int6
     const wdf::Packed &p = ens->pk;
     const int K = 1 << p.D;
     const size_t hist_n = (size_t)p.T * p.NS * (2 * K);
-    wdf_status s0 = ensure_frequency_state(ens, precision);
+    wdf_status s0 = ensure_frequency_state(ens, precision, false);
     if (s0 != WDF_OK) return s0;
     WDF_CUDA(cudaMemsetAsync(ens->d_hist, 0, hist_n * 4, st));
     if (kind == WDF_MEM_DEVICE) {
@@ -565,7 +574,7 @@ wdf_status wdf_set_background_counts(wdf_ensemble *ens, const uint32_t *counts, 
         return fail(WDF_EINVAL, "unknown precision");
     DeviceGuard g(ens->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
-    wdf_status s0 = ensure_frequency_state(ens, precision);
+    wdf_status s0 = ensure_frequency_state(ens, precision, false);
     if (s0 != WDF_OK) return s0;
     WDF_CUDA(cudaMemcpyAsync(ens->d_hist, counts, (size_t)wdf_background_counts_size(ens) * 4,
                              cudaMemcpyDeviceToDevice, st));
@@ -595,11 +604,11 @@ wdf_status wdf_set_path_dependent(wdf_ensemble *ens, wdf_precision precision, vo
     DeviceGuard g(ens->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const wdf::Packed &p = ens->pk;
-    wdf_status s0 = ensure_frequency_state(ens, precision);
+    wdf_status s0 = ensure_frequency_state(ens, precision, true);
     if (s0 != WDF_OK) return s0;
     WDF_CUDA(wdf::launch_pd_freq(p.D, ens->d_ratio, ens->n_live, ens->d_A, st));
     WDF_CUDA(wdf::launch_scale(ens->d_w_rows, ens->n_live, 1, ens->d_scale, st));
-    WDF_CUDA(wdf::launch_base_value(p.D, nullptr, ens->d_ratio, ens->d_w_rows, ens->n_live, 1, ens->d_base, st));
+    WDF_CUDA(wdf::launch_base_value(p.D, nullptr, nullptr, ens->d_ratio, ens->d_w_rows, ens->n_live, 1, ens->d_base, st));
     WDF_CUDA(wdf::launch_line_maps(p.D, nullptr, ens->d_meta, p.T, ens->d_lines, st));
     wdf_status s1 = contract_and_fold(ens, precision, st);
     if (s1 != WDF_OK) return s1;
@@ -663,21 +672,27 @@ wdf_status wdf_explain_interactions(wdf_ensemble *ens, const float *C, int64_t n
     DeviceGuard g(ens->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const int D = p.D, K = 1 << D, P = D * (D - 1) / 2, PP = (P + 3) & ~3;
-    // pair tables, the contraction and its repacking live in one stream-ordered block
-    // depth <= 6: pair values folded per bottom-subtree entry; deeper: per leaf
+    // pair values in one stream-ordered block, before it (path-dependent game) the pair tables
+    // and their contraction; depth <= 6: folded per bottom-subtree entry; deeper: per leaf
     const bool folded = D <= 6;
-    const size_t n_t2 = (size_t)ens->G * K * P * K, n_s2 = (size_t)ens->n_live * P * K;
+    const size_t n_t2 = ens->pd ? (size_t)ens->G * K * P * K : 0, n_s2 = ens->pd ? (size_t)ens->n_live * P * K : 0;
     const size_t n_s2t = folded ? wdf::iv_fold_floats(D, p.T) : (size_t)ens->n_live * K * PP;
     float *buf = nullptr;
     WDF_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void **>(&buf), std::max<size_t>(n_t2 + n_s2 + n_s2t, 4) * 4,
                                      ens->ctx->dev.pool, st));
     float *t2 = buf, *s2 = buf + n_t2, *s2t = buf + n_t2 + n_s2;
-    cudaError_t e = wdf::launch_tables_iv(D, ens->metric, ens->d_keys, ens->G, t2, st);
-    if (e == cudaSuccess)
-        e = wdf::launch_contract_fp32(D, ens->d_A, ens->d_scale, ens->d_tiles, ens->n_tiles, t2, s2, st, P);
-    if (e == cudaSuccess)
-        e = folded ? wdf::launch_iv_fold(D, s2, ens->d_leaf_row, p.T, s2t, st)
-                   : wdf::launch_iv_pack(D, PP, s2, ens->n_live, s2t, st);
+    cudaError_t e;
+    if (ens->pd) {
+        e = wdf::launch_tables_iv(D, ens->metric, ens->d_keys, ens->G, t2, st);
+        if (e == cudaSuccess)
+            e = wdf::launch_contract_fp32(D, ens->d_A, ens->d_scale, ens->d_tiles, ens->n_tiles, t2, s2, st, P);
+        if (e == cudaSuccess)
+            e = folded ? wdf::launch_iv_fold(D, s2, ens->d_leaf_row, p.T, s2t, st)
+                       : wdf::launch_iv_pack(D, PP, s2, ens->n_live, s2t, st);
+    } else {
+        e = wdf::launch_subtree_pairs(D, ens->metric, ens->d_hist, ens->d_nodes, p.F, ens->d_leaf_row, ens->d_scale,
+                                      p.T, ens->d_meta, s2t, ens->ctx->dev, st);
+    }
     if (e == cudaSuccess)
         e = wdf::launch_explain_iv(D, C, n, ldc, p.F, ens->arrays(), ens->slices(), p.T, ens->d_group_leaf, ens->n_live,
                                    folded ? nullptr : s2t, folded ? s2t : nullptr, out, ldo, ens->ctx->dev, st);

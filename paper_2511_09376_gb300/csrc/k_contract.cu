@@ -3,7 +3,8 @@
 // baseline pattern frequencies, s_{l,i} = w_l * M_{l,i} * f_l (Eq.
 // "bg_shap_derivation" step (f); f from background counts or, for the path-dependent
 // game, Eq. "path_dependent_estimation"), then the fold of the four leaves of every
-// bottom subtree into the per-entry vectors the consumer kernel gathers.
+// bottom subtree into the per-entry vectors the consumer kernel gathers.  Background counts
+// in FP32 take k_subtree.cu instead.
 #include "launch.h"
 
 namespace wdf {
@@ -187,51 +188,58 @@ cudaError_t launch_fold(int D, const float *S, const int32_t *leaf_row, int T, c
     return cudaGetLastError();
 }
 
-// One thread per (tree, map byte): for its bottom subtree s, the background frequency of
+// One warp per (tree, map byte): for its bottom subtree s, the background frequency of
 // every entry bit b (the share of rows with bit b set), and the rotation r whose low
 // pair (bits r and r + 1 mod D + 1) is the least certain: the largest sum of
 // min(p, 1 - p).  Ties keep the smaller r; a subtree no row reaches, and the padding
-// bytes past the last subtree, keep the identity 0.
-__global__ void k_line_maps(int D, const uint32_t *__restrict__ hist, const TreeMeta *__restrict__ meta, int T,
-                            uint8_t *__restrict__ lines) {
+// bytes past the last subtree, keep the identity 0.  (A thread per subtree, one entry after
+// another, took 155 us for 19,200 subtrees of depth 8, this 21.)
+__global__ void __launch_bounds__(256) k_line_maps(int D, const uint32_t *__restrict__ hist,
+                                                   const TreeMeta *__restrict__ meta, int T,
+                                                   uint8_t *__restrict__ lines) {
     const int NS = 1 << (D - 2), E = 1 << (D + 1), B = 4 * lines_words(D), NB = D + 1;
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t idx = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
     if (idx >= (int64_t)T * B) return;
     const int t = (int)(idx / B), s = (int)(idx % B);
     uint32_t rot = 0;
     if (s < NS && hist) {
         const uint32_t *h = hist + ((size_t)t * NS + s) * E;
-        uint64_t total = 0, ones[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int e = 0; e < E; ++e) {
-            const uint64_t c = __ldg(h + e);
+        uint32_t total = 0, ones[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};  // at most the background rows, below 2^32
+        for (int e = lane; e < E; e += 32) {
+            const uint32_t c = __ldg(h + e);
             total += c;
-            for (int b = 0; b < NB; ++b) ones[b] += ((e >> b) & 1) ? c : 0;
+#pragma unroll
+            for (int b = 0; b < 9; ++b) ones[b] += ((e >> b) & 1) ? c : 0u;
         }
+        total = __reduce_add_sync(0xFFFFFFFFu, total);
+#pragma unroll
+        for (int b = 0; b < 9; ++b) ones[b] = __reduce_add_sync(0xFFFFFFFFu, ones[b]);
         if (total > 0) {
-            double best = -1.0;
-            for (int r = 0; r < NB; ++r) {
-                double u = 0.0;
-                for (int k = 0; k < 2; ++k) {
-                    const double p = (double)ones[(r + k) % NB] / (double)total;
-                    u += p < 1.0 - p ? p : 1.0 - p;
-                }
-                if (u > best) {
-                    best = u;
+            // uncertainties as integers: min(ones, total - ones)
+            uint64_t u[9], best = 0;
+#pragma unroll
+            for (int b = 0; b < 9; ++b) u[b] = ones[b] < total - ones[b] ? ones[b] : total - ones[b];
+#pragma unroll
+            for (int r = 0; r < 9; ++r) {
+                if (r >= NB) break;
+                const uint64_t x = u[r] + (r + 1 < NB ? u[r + 1 < 9 ? r + 1 : 0] : u[0]);
+                if (r == 0 || x > best) {
+                    best = x;
                     rot = (uint32_t)r;
                 }
             }
         }
     }
     if (s < NS && !((__ldg(&meta[t].live) >> s) & 1ull)) rot = kLineDead;
-    lines[idx] = (uint8_t)rot;
+    if (lane == 0) lines[idx] = (uint8_t)rot;
 }
 
 cudaError_t launch_line_maps(int D, const uint32_t *hist, const TreeMeta *meta, int T, uint32_t *lines,
                              cudaStream_t st) {
     const int64_t total = (int64_t)T * 4 * lines_words(D);
     if (total == 0) return cudaSuccess;
-    k_line_maps<<<(unsigned)((total + 127) / 128), 128, 0, st>>>(D, hist, meta, T,
-                                                                  reinterpret_cast<uint8_t *>(lines));
+    k_line_maps<<<(unsigned)((total + 7) / 8), 256, 0, st>>>(D, hist, meta, T, reinterpret_cast<uint8_t *>(lines));
     count_launches(1);
     return cudaGetLastError();
 }

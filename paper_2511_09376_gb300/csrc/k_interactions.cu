@@ -2,9 +2,10 @@
 // "table_shap_iv", Def. "banzhaf_iv_def" with Formula
 // "banzhaf_simplified_formula_interactions") of the game the ensemble holds.  By
 // linearity (the derivation of Eq. "bg_shap_derivation" uses only linearity) the
-// pipeline is the one of the values with a pair table in place of the value table:
-//   k_tables_iv   per path signature, for every (p_b, p_c) cube and every pair of path
-//                 positions, the pair's cell (FP64 built, stored FP32);
+// pipeline is the one of the values with pairs of variables in place of variables:
+//   k_subtree_pairs  (k_subtree.cu) background counts: the pair values by subset sums;
+//   k_tables_iv   path-dependent game: per path signature, for every (p_b, p_c) cube and
+//                 every pair of path positions, the pair's cell (FP64 built, stored FP32);
 //   contraction   s2_{l,q}[p_c] = w_l sum_{p_b} M2[p_c][p_b][q] f_l[p_b] (the FP32 GEMM of
 //                 the values with P = D(D-1)/2 pair slots per pattern);
 //   k_iv_fold     (depth <= 6) the four leaves of every bottom subtree folded per entry
@@ -115,15 +116,7 @@ cudaError_t launch_iv_pack(int D, int PP, const float *S2, int n_live, float *S2
 // The four leaves of a bottom subtree share their path above the subtree root r.  Slots
 // of a subtree: 0..D-3 the ancestors of r (root first), D-2 = r, D-1 = its left child,
 // D = its right child.  A folded vector holds, per entry, the pair values of every slot
-// pair (u, v), u < v, except (left child, right child) (never on one path), summed
-// over the four leaves: IV_FP(D) = C(D+1, 2) - 1 values, padded to a multiple of 4.
-__host__ __device__ constexpr int iv_fp(int D) { return (D + 1) * D / 2 - 1; }
-__host__ __device__ constexpr int iv_fpp(int D) { return (iv_fp(D) + 3) & ~3; }
-// index of slot pair (u, v), u < v, in a folded vector (pairs ordered by u, then v)
-__host__ __device__ constexpr int iv_pidx(int D, int u, int v) {
-    return u * D - u * (u - 1) / 2 + (v - u - 1);
-}
-
+// pair (iv_fp, iv_pidx of wdf_device.cuh) summed over the four leaves.
 // One thread per (tree, bottom subtree, entry): fold the per-leaf pair values S2 [leaf
 // row][q * 2^D + p] of the subtree's four leaves (q over the leaf's position pairs).
 __global__ void k_iv_fold(int D, const float *__restrict__ S2, const int32_t *__restrict__ leaf_row, int T,

@@ -102,8 +102,8 @@ cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const 
                            int T, unsigned char *codes, int64_t code_rows, uint32_t *hist, const DevInfo &dev,
                            cudaStream_t st, const BgOverlap *ov = nullptr);
 
-// Per-leaf pattern counts vc[row][p] (u32, 2^D per row) of the live leaves, marginals of
-// the joint entry counts; A (nullable) receives them as FP32.
+// Per-leaf pattern counts vc[row][p] (u32, 2^D per row; nullable) of the live leaves,
+// marginals of the joint entry counts; A (nullable) receives them as FP32.
 cudaError_t launch_leaf_counts(int D, const uint32_t *hist, const int32_t *group_leaf, int n_live, uint32_t *vc,
                                float *A, cudaStream_t st);
 
@@ -145,6 +145,19 @@ cudaError_t launch_contract_tc(int D, int mode, const float *A, const float *sca
 // restores the normal limit).
 void set_contract_first_wait_limit(uint32_t polls);
 
+// Steps 2 and 3 at once for background counts in FP32: the folded slot vectors sfold of every
+// bottom subtree (as launch_fold's) straight from the joint entry counts hist, with the
+// cube values of the metric (k_subtree.cu).
+cudaError_t launch_subtree_fold(int D, int metric, const uint32_t *hist, const int2 *nodes, int F,
+                                const int32_t *leaf_row, const float *scale, int T, const uint32_t *lines,
+                                float *sfold, const DevInfo &dev, cudaStream_t st);
+
+// The same for the pairs of slots: for D <= 6 the folded vectors of launch_iv_fold, else the
+// per-leaf vectors of launch_iv_pack (of the live leaves, by leaf_row).
+cudaError_t launch_subtree_pairs(int D, int metric, const uint32_t *hist, const int2 *nodes, int F,
+                                 const int32_t *leaf_row, const float *scale, int T, const TreeMeta *meta,
+                                 float *out, const DevInfo &dev, cudaStream_t st);
+
 // Folds the per-leaf S rows of every bottom subtree into per-entry slot vectors
 // sfold[T][NS][2^(D+1)][SP] (see wdf_internal.h).
 cudaError_t launch_fold(int D, const float *S, const int32_t *leaf_row, int T, const uint32_t *lines, float *sfold,
@@ -157,10 +170,12 @@ cudaError_t launch_line_maps(int D, const uint32_t *hist, const TreeMeta *meta, 
 // scale[row] = w[row] / m.
 cudaError_t launch_scale(const double *w, int n_live, int64_t m, float *scale, cudaStream_t st);
 
-// v({}) in FP64 (one block): sum over live leaves of w * vc[all ones] / m, or, when
-// ratio is non-null (path-dependent game), of w * (product of the leaf's cover ratios).
-cudaError_t launch_base_value(int D, const uint32_t *vc, const double *ratio, const double *leaf_w_rows, int n_live,
-                              int64_t m, double *out, cudaStream_t st);
+// v({}) in FP64: sum over live leaves of w * (rows that reach the leaf, from the joint counts
+// hist) / m, or, when ratio is non-null (path-dependent game), of w * (product of the leaf's
+// cover ratios).  out: kBaseBlocks + 1 doubles, the value first.
+constexpr int kBaseBlocks = 64;
+cudaError_t launch_base_value(int D, const uint32_t *hist, const int32_t *group_leaf, const double *ratio,
+                              const double *leaf_w_rows, int n_live, int64_t m, double *out, cudaStream_t st);
 
 // The tree images (tree_layout.h) from the unit nodes, the metadata, the features flfeat
 // [T][flush_len(D)] and repeats flrep [T][flush_batches(D)] of the flush positions.

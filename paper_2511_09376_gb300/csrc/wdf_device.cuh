@@ -116,6 +116,39 @@ __device__ __forceinline__ uint32_t unit_decide(const uint2 &node, const uint4 *
     return le;
 }
 
+// Rows with pattern p at leaf q = 4s + j of tree t: the leaf pattern p has the subtree-root
+// pattern in its high D-2 bits, then the bit for node r and the bit for the child of r on the
+// path; the decision at the other child of r is summed out.
+__device__ __forceinline__ uint32_t leaf_count(int D, const uint32_t *__restrict__ hist, int leaf, uint32_t p) {
+    const int t = leaf >> D, q = leaf & ((1 << D) - 1);
+    const int s = q >> 2, j = q & 3;
+    const int NS = 1 << (D - 2), E = 1 << (D + 1);
+    const uint32_t pp = p >> 2, fn = (p >> 1) & 1u, fc = p & 1u;
+    const uint32_t dn = (j < 2) ? fn : (fn ^ 1u);         // path goes left at r for j < 2
+    const uint32_t dch = ((j & 1) == 0) ? fc : (fc ^ 1u);  // and left at the child for even j
+    const uint32_t *h = hist + ((size_t)t * NS + s) * E;
+    const uint32_t R = pp ^ (uint32_t)s;  // ancestors' raw decisions (wdf_internal.h)
+    uint32_t e0, e1;
+    if (j < 2) {  // the path takes 2r+1 (entry bit 0); sum over the decision at 2r+2
+        e0 = (R << 3) | (dn << 2) | dch;
+        e1 = e0 | 2u;
+    } else {  // the path takes 2r+2 (entry bit 1); sum over the decision at 2r+1
+        e0 = (R << 3) | (dn << 2) | (dch << 1);
+        e1 = e0 | 1u;
+    }
+    return __ldg(h + e0) + __ldg(h + e1);
+}
+
+// Folded pair values (depth <= 6) of a bottom subtree with slots 0..D-3 = the ancestors of its
+// root r (root first), D-2 = r, D-1 and D = r's children: every slot pair (u, v), u < v, except
+// the two children (never on one path): iv_fp(D) values, padded to a multiple of 4.
+__host__ __device__ constexpr int iv_fp(int D) { return (D + 1) * D / 2 - 1; }
+__host__ __device__ constexpr int iv_fpp(int D) { return (iv_fp(D) + 3) & ~3; }
+// index of slot pair (u, v), u < v, in a folded vector (pairs ordered by u, then v)
+__host__ __device__ constexpr int iv_pidx(int D, int u, int v) {
+    return u * D - u * (u - 1) / 2 + (v - u - 1);
+}
+
 // Decision code of value x in code column c (tree_layout.h).
 __device__ __forceinline__ int decision_code(float x, const SliceArrays &sa, int c) {
     if (x != x) return __ldg(&sa.col[c].count);

@@ -76,7 +76,6 @@ struct wdf_ensemble {
     int has_bg = 0;
     int64_t m = 0;
     uint32_t *d_hist = nullptr;
-    uint32_t *d_vc = nullptr;
     float *d_scale = nullptr;
     float *d_S = nullptr;
     float *d_sfold = nullptr;
