@@ -4,7 +4,7 @@
 // Ensembles are grouped into depth classes (one kernel instantiation per depth).  A
 // call writes every class's work description -- the ensembles' device arrays (jobs),
 // the requests, the encode items (request, group of columns, 32-row blocks) and the work items (job,
-// request, first row) of tile_rows consumer rows each -- into one pinned host blob; the
+// request, first row, group of parts) of tile_rows consumer rows each -- into one pinned host blob; the
 // captured graph copies that blob to the device with a single memcpy and then runs, per
 // class on parallel branches, k_encode_batch (the rows' decision codes into the batch's
 // code arena) and one persistent k_explain_batch.  The item count is read on the device, so the same graph serves
@@ -15,6 +15,7 @@
 // caller's own requests and keeps the fastest per class; results can be cached in a text
 // file keyed by (depth, feature count rounded up to 32).
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <fstream>
@@ -43,13 +44,16 @@ wdf_status fail(wdf_status s, const std::string &msg) {
 struct Cls {
     int D = 0, F_max = 0, q_max = 0, thr_max = 0, tile_rows = 0;
     std::vector<int> members;  // batch ensemble indices, in job-slot order
-    int cap_reqs = 0, cap_items = 0, cap_eitems = 0;
+    int cap_reqs = 0, cap_items = 0, cap_eitems = 0, cap_tiles = 0;
     size_t off_jobs = 0, off_reqs = 0, off_items = 0, off_count = 0, off_eitems = 0, off_ecount = 0;
 };
 
 // Rows of a request's code region: a multiple of every tile size (and of 32).
 constexpr int64_t kCodePad = 128;
 int64_t padded_rows(int64_t n) { return (n + kCodePad - 1) / kCodePad * kCodePad; }
+
+// Most scratch of the parts of one call's split requests; kept until the batch is destroyed.
+constexpr size_t kPartsBytes = (size_t)128 << 20;
 
 }  // namespace
 
@@ -69,6 +73,8 @@ struct wdf_batch {
     bool copied_pending = false;
     unsigned char *d_codes = nullptr;  // decision codes of the requests' rows
     size_t codes_cap = 0;
+    unsigned char *d_parts = nullptr;  // parts of the split requests' rows
+    size_t parts_cap = 0;
 };
 
 namespace {
@@ -79,6 +85,8 @@ struct Req {
     float *phi;
     int64_t n, ldc, ldp;
     size_t codes_off = 0;  // the request's region of the code arena
+    int groups = 1;        // work items per tile (launch.h)
+    size_t parts_off = 0;  // split: the request's region of the parts' scratch
 };
 
 void drop_graph(wdf_batch *b) {
@@ -118,13 +126,67 @@ wdf_status place_codes(wdf_batch *b, std::vector<Req> *reqs) {
     return WDF_OK;
 }
 
+// Splits the requests whose tiles would be the call's tail.  A tile walks all trees of its
+// ensemble one after another (0.034 us per tree and leaf position, 2.2 ms for 257 trees of depth
+// 8), and parts of the walk are independent; storing and adding parts costs a few percent, so a
+// tile is cut into pieces of at most a quarter of the time that the whole call takes with
+// every SM busy, as far as the scratch goes.  A call with many tiles is not split at all.
+// Twelve ensembles, 87,079 rows in all: 2.45 -> 1.26 ms; a burst of 24 server requests 11.2 ->
+// 10.5 ms; 163 tiles against 257 trees of depth 8 alone 2.3 -> 0.75 ms.
+// tile_rows: of every class.
+void plan_groups(const wdf_batch *b, const std::vector<int> &tile_rows, std::vector<Req> *reqs) {
+    double call = 0.0;  // in tree leaves walked by one block at full occupancy
+    for (const Req &r : *reqs) {
+        const wdf::Packed &p = b->ens[(size_t)r.e]->pk;
+        const Cls &k = b->cls[(size_t)b->cls_of[(size_t)r.e]];
+        const int tc = tile_rows[(size_t)b->cls_of[(size_t)r.e]];
+        call += (double)((r.n + tc - 1) / tc) * ((double)p.T * p.NL) /
+                ((double)b->ctx->dev.sms * wdf::explain_blocks_per_sm(k.D, k.F_max, k.q_max, tc, b->ctx->dev));
+    }
+    size_t used = 0;
+    for (Req &r : *reqs) {
+        const wdf::Packed &p = b->ens[(size_t)r.e]->pk;
+        const int P = wdf::explain_parts(p.T, p.D);
+        const double want = std::ceil((double)p.T * p.NL / (0.25 * call));
+        const size_t bytes = ((size_t)P * (size_t)r.n * (size_t)p.F * sizeof(float) + 255) & ~(size_t)255;
+        r.groups = want >= P ? P : std::max(1, (int)want);
+        if (r.n > (int64_t)(kPartsBytes / sizeof(float)) || used + bytes > kPartsBytes) r.groups = 1;
+        if (r.groups > 1) {
+            r.parts_off = used;
+            used += bytes;
+        }
+    }
+}
+
+// Scratch for the planned parts, grown like the code arena.
+wdf_status place_parts(wdf_batch *b, const std::vector<Req> &reqs) {
+    size_t total = 0;
+    for (const Req &r : reqs) {
+        const wdf::Packed &p = b->ens[(size_t)r.e]->pk;
+        if (r.groups > 1)
+            total = r.parts_off + (size_t)wdf::explain_parts(p.T, p.D) * (size_t)r.n * (size_t)p.F * sizeof(float);
+    }
+    if (total > b->parts_cap) {
+        wdf_status s = wait_copied(b);
+        if (s != WDF_OK) return s;
+        WDF_CUDA(cudaDeviceSynchronize());  // earlier launches may still use the old scratch
+        if (b->d_parts) cudaFree(b->d_parts);
+        b->d_parts = nullptr;
+        b->parts_cap = 0;
+        const size_t cap = std::min(std::max<size_t>(total + total / 2, 1 << 20), kPartsBytes);
+        WDF_CUDA(cudaMalloc((void **)&b->d_parts, cap));
+        b->parts_cap = cap;
+    }
+    return WDF_OK;
+}
+
 // Blob layout for the current capacities; reallocates (and drops the graph) if it grew.
 wdf_status ensure_blob(wdf_batch *b, const std::vector<int> &need_reqs, const std::vector<int> &need_items,
-                       const std::vector<int> &need_eitems) {
+                       const std::vector<int> &need_eitems, const std::vector<int> &need_tiles) {
     bool grow = b->h_blob == nullptr;
     for (size_t c = 0; c < b->cls.size(); ++c)
         if (need_reqs[c] > b->cls[c].cap_reqs || need_items[c] > b->cls[c].cap_items ||
-            need_eitems[c] > b->cls[c].cap_eitems)
+            need_eitems[c] > b->cls[c].cap_eitems || need_tiles[c] > b->cls[c].cap_tiles)
             grow = true;
     if (!grow) return WDF_OK;
     wdf_status s = wait_copied(b);
@@ -137,6 +199,7 @@ wdf_status ensure_blob(wdf_batch *b, const std::vector<int> &need_reqs, const st
         k.cap_reqs = std::max(k.cap_reqs, std::max(need_reqs[c], 4) * 3 / 2);
         k.cap_items = std::max(k.cap_items, std::max(need_items[c], 64) * 3 / 2);
         k.cap_eitems = std::max(k.cap_eitems, std::max(need_eitems[c], 64) * 3 / 2);
+        k.cap_tiles = std::max(k.cap_tiles, std::max(need_tiles[c], 64) * 3 / 2);
         k.off_jobs = off;
         off = up16(off + k.members.size() * sizeof(wdf::ExplainJob));
         k.off_reqs = off;
@@ -144,7 +207,7 @@ wdf_status ensure_blob(wdf_batch *b, const std::vector<int> &need_reqs, const st
         k.off_items = off;
         off = up16(off + (size_t)k.cap_items * sizeof(int4));
         k.off_count = off;
-        off = up16(off + 2 * sizeof(int));
+        off = up16(off + (2 + (size_t)k.cap_tiles) * sizeof(int));
         k.off_eitems = off;
         off = up16(off + (size_t)k.cap_eitems * sizeof(int4));
         k.off_ecount = off;
@@ -169,26 +232,40 @@ int fill_class(wdf_batch *b, int c, const std::vector<Req> &reqs, int tile_rows)
     auto *rq = reinterpret_cast<wdf::BatchRequest *>(b->h_blob + k.off_reqs);
     auto *items = reinterpret_cast<int4 *>(b->h_blob + k.off_items);
     auto *eitems = reinterpret_cast<int4 *>(b->h_blob + k.off_eitems);
-    int nr = 0, ni = 0, ne = 0;
+    int nr = 0, ni = 0, ne = 0, nt = 0;
     for (const Req &r : reqs) {
         if (b->cls_of[(size_t)r.e] != c) continue;
-        rq[nr] = wdf::BatchRequest{r.C, r.phi, b->d_codes + r.codes_off, r.n, r.ldc, r.ldp, b->slot_of[(size_t)r.e]};
+        rq[nr] = wdf::BatchRequest{r.C,   r.phi, b->d_codes + r.codes_off, nullptr, r.n, r.ldc,
+                                   r.ldp, b->slot_of[(size_t)r.e],  r.groups, nt};
+        if (r.groups > 1) {
+            rq[nr].parts = reinterpret_cast<float *>(b->d_parts + r.parts_off);
+            nt += (int)((r.n + tile_rows - 1) / tile_rows);
+        }
         for (int64_t c0 = 0; c0 < r.n; c0 += tile_rows)
-            items[ni++] = make_int4(b->slot_of[(size_t)r.e], nr, (int)(c0 >> 31), (int)(c0 & 0x7FFFFFFF));
+            for (int g = 0; g < r.groups; ++g)
+                items[ni++] = make_int4(b->slot_of[(size_t)r.e], nr, (int)(c0 >> 31) | g << wdf::kBatchGroupShift,
+                                        (int)(c0 & 0x7FFFFFFF));
         const int64_t blocks = padded_rows(r.n) / 32;
         for (int64_t blk = 0; blk < blocks; blk += wdf::kEncodeItemBlocks)
             for (int g = 0; g < (int)b->ens[(size_t)r.e]->pk.sgroup.size(); ++g)
                 eitems[ne++] = make_int4(nr, g, (int)blk, (int)std::min<int64_t>(wdf::kEncodeItemBlocks, blocks - blk));
         ++nr;
     }
-    // longest first: tiles of ensembles with more trees cost more; blocks claim items in
-    // this order, so the cheap ones fill the tail of the launch
+    // longest first: blocks claim items in this order, so the cheap ones fill the tail of the
+    // launch; then by ensemble and group, so that blocks at work together walk the same trees
+    // (the folded vectors of 350 trees of depth 8 are three times the L2 cache: 56,000 rows 6.7
+    // ms, with a tile's groups next to one another 8.1)
+    auto cost = [&](const int4 &i) {
+        return (double)b->ens[(size_t)k.members[(size_t)i.x]]->pk.T / rq[i.y].groups;
+    };
     std::stable_sort(items, items + ni, [&](const int4 &a, const int4 &c) {
-        return b->ens[(size_t)k.members[(size_t)a.x]]->pk.T > b->ens[(size_t)k.members[(size_t)c.x]]->pk.T;
+        const double ca = cost(a), cc = cost(c);
+        if (ca != cc) return ca > cc;
+        return a.x != c.x ? a.x < c.x : a.z >> wdf::kBatchGroupShift < c.z >> wdf::kBatchGroupShift;
     });
     int *hdr = reinterpret_cast<int *>(b->h_blob + k.off_count);
     hdr[0] = ni;  // item count
-    hdr[1] = 0;   // claim counter, zero at every launch
+    std::memset(hdr + 1, 0, (1 + (size_t)nt) * sizeof(int));  // claim counter and tile counters, zero at every launch
     *reinterpret_cast<int *>(b->h_blob + k.off_ecount) = ne;
     return ni;
 }
@@ -241,7 +318,7 @@ wdf_status gather_requests(wdf_batch *b, int32_t nreq, const int32_t *idx, const
         if (idx[i] < 0 || idx[i] >= (int)b->ens.size()) return fail(WDF_EINVAL, "ensemble index out of range");
         const wdf_ensemble *e = b->ens[(size_t)idx[i]];
         if (!e->has_bg) return fail(WDF_EINVAL, "an ensemble of the batch has no background");
-        if (n[i] < 0 || (n[i] > 0 && (!C[i] || !phi[i])) || ldc[i] < e->pk.F || ldphi[i] < e->pk.F)
+        if (n[i] < 0 || n[i] > wdf::kBatchMaxRows || (n[i] > 0 && (!C[i] || !phi[i])) || ldc[i] < e->pk.F || ldphi[i] < e->pk.F)
             return fail(WDF_EINVAL, "bad request " + std::to_string(i));
         if (n[i] > 0) out->push_back(Req{idx[i], C[i], phi[i], n[i], ldc[i], ldphi[i]});
     }
@@ -249,14 +326,18 @@ wdf_status gather_requests(wdf_batch *b, int32_t nreq, const int32_t *idx, const
 }
 
 void count_needs(const wdf_batch *b, const std::vector<Req> &reqs, const std::vector<int> &tile_rows,
-                 std::vector<int> *need_reqs, std::vector<int> *need_items, std::vector<int> *need_eitems) {
+                 std::vector<int> *need_reqs, std::vector<int> *need_items, std::vector<int> *need_eitems,
+                 std::vector<int> *need_tiles) {
     need_reqs->assign(b->cls.size(), 0);
     need_items->assign(b->cls.size(), 0);
     need_eitems->assign(b->cls.size(), 0);
+    need_tiles->assign(b->cls.size(), 0);
     for (const Req &r : reqs) {
         const int c = b->cls_of[(size_t)r.e];
         (*need_reqs)[(size_t)c] += 1;
-        (*need_items)[(size_t)c] += (int)((r.n + tile_rows[(size_t)c] - 1) / tile_rows[(size_t)c]);
+        const int tiles = (int)((r.n + tile_rows[(size_t)c] - 1) / tile_rows[(size_t)c]);
+        (*need_items)[(size_t)c] += tiles * r.groups;
+        (*need_tiles)[(size_t)c] += r.groups > 1 ? tiles : 0;
         (*need_eitems)[(size_t)c] +=
             (int)((padded_rows(r.n) / 32 + wdf::kEncodeItemBlocks - 1) / wdf::kEncodeItemBlocks) *
             (int)b->ens[(size_t)r.e]->pk.sgroup.size();
@@ -332,6 +413,7 @@ void wdf_batch_destroy(wdf_batch *b) {
     if (b->h_blob) cudaFreeHost(b->h_blob);
     if (b->d_blob) cudaFree(b->d_blob);
     if (b->d_codes) cudaFree(b->d_codes);
+    if (b->d_parts) cudaFree(b->d_parts);
     for (cudaStream_t s : b->branch)
         if (s) cudaStreamDestroy(s);
     for (cudaEvent_t ev : b->ev_join)
@@ -355,11 +437,13 @@ wdf_status wdf_batch_explain(wdf_batch *b, int32_t n_requests, const int32_t *en
     int prev = -1;
     cudaGetDevice(&prev);
     if (prev != b->ctx->device) cudaSetDevice(b->ctx->device);
-    std::vector<int> tiles, need_reqs, need_items, need_eitems;
+    std::vector<int> tiles, need_reqs, need_items, need_eitems, need_tiles;
     for (const Cls &k : b->cls) tiles.push_back(k.tile_rows);
-    count_needs(b, reqs, tiles, &need_reqs, &need_items, &need_eitems);
-    s = ensure_blob(b, need_reqs, need_items, need_eitems);
+    plan_groups(b, tiles, &reqs);
+    count_needs(b, reqs, tiles, &need_reqs, &need_items, &need_eitems, &need_tiles);
+    s = ensure_blob(b, need_reqs, need_items, need_eitems, need_tiles);
     if (s == WDF_OK) s = place_codes(b, &reqs);
+    if (s == WDF_OK) s = place_parts(b, reqs);
     if (s == WDF_OK) s = wait_copied(b);
     if (s == WDF_OK) {
         for (size_t c = 0; c < b->cls.size(); ++c) fill_class(b, (int)c, reqs, b->cls[c].tile_rows);
@@ -402,9 +486,11 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
     if (prev != b->ctx->device) cudaSetDevice(b->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const int cand[3] = {32, 64, 128};
-    std::vector<int> t32(b->cls.size(), 32), need_reqs, need_items, need_eitems;
-    count_needs(b, reqs, t32, &need_reqs, &need_items, &need_eitems);  // tile_rows 32 needs the most items
-    s = ensure_blob(b, need_reqs, need_items, need_eitems);
+    // tile_rows 32 and every part an item needs the most
+    std::vector<int> t32(b->cls.size(), 32), need_reqs, need_items, need_eitems, need_tiles;
+    for (Req &r : reqs) r.groups = wdf::explain_parts(b->ens[(size_t)r.e]->pk.T, b->ens[(size_t)r.e]->pk.D);
+    count_needs(b, reqs, t32, &need_reqs, &need_items, &need_eitems, &need_tiles);
+    s = ensure_blob(b, need_reqs, need_items, need_eitems, need_tiles);
     if (s == WDF_OK) s = place_codes(b, &reqs);
     if (s == WDF_OK) s = wait_copied(b);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -428,6 +514,7 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
         float best_ms = 1e30f;
         int best = k.tile_rows;
         // the rows' codes do not depend on the tile size: encode them once
+        for (Req &r : reqs) r.groups = 1;
         fill_class(b, (int)c, reqs, k.tile_rows);
         {
             cudaError_t e = cudaMemcpyAsync(b->d_blob, b->h_blob, b->blob_bytes, cudaMemcpyHostToDevice, st);
@@ -444,13 +531,19 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
         }
         for (int tc : cand) {
             if (wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, tc) > b->ctx->dev.smem_optin) continue;
+            std::vector<int> tiles;
+            for (const Cls &o : b->cls) tiles.push_back(&o == &k ? tc : o.tile_rows);
+            plan_groups(b, tiles, &reqs);
+            s = place_parts(b, reqs);
+            if (s != WDF_OK) break;
             fill_class(b, (int)c, reqs, tc);
             cudaError_t e = cudaMemcpyAsync(b->d_blob, b->h_blob, b->blob_bytes, cudaMemcpyHostToDevice, st);
             float ms = 0.0f;
             for (int r = -1; r < reps && e == cudaSuccess; ++r) {  // r = -1 warms up
                 if (r == 0) e = cudaEventRecord(e0, st);
-                if (e == cudaSuccess)  // reset the claim counter of this class
-                    e = cudaMemsetAsync(b->d_blob + k.off_count + sizeof(int), 0, sizeof(int), st);
+                if (e == cudaSuccess)  // reset the claim and tile counters of this class
+                    e = cudaMemsetAsync(b->d_blob + k.off_count + sizeof(int), 0, (1 + (size_t)k.cap_tiles) * sizeof(int),
+                                        st);
                 if (e == cudaSuccess)
                     e = wdf::launch_explain_batch(k.D, reinterpret_cast<const wdf::ExplainJob *>(b->d_blob + k.off_jobs),
                                                   reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),

@@ -92,6 +92,11 @@ int default_tile_rows(int D, int F, int quads, const DevInfo &dev) {
     return best;
 }
 
+int explain_blocks_per_sm(int D, int F, int quads, int tile_rows, const DevInfo &dev) {
+    const size_t smem = explain_smem_bytes(D, F, quads, tile_rows);
+    return std::max(1, std::min((int)((dev.smem_optin + 1024) / (smem + 1024)), explain_warps(D) * 16 / tile_rows));
+}
+
 // phi = the parts' sums, added in part order; one thread per element of a row.
 __global__ void k_add_parts(const float *__restrict__ scratch, int P, int64_t n, int F, float *__restrict__ phi,
                             int64_t ldp) {
@@ -173,9 +178,7 @@ constexpr int64_t kValuesBytes = 320ll << 20;
 // 1380; 50 trees of depth 4, 255 features, 20,000 rows 87 / 49.
 static int explain_splits(int D, int64_t n, const ExplainJob &job, int tile_rows, const DevInfo &dev) {
     const int P = explain_parts(job.T, D);
-    const size_t smem = explain_smem_bytes(D, job.F, job.sa.quads, tile_rows);
-    const int64_t per_sm = std::max<int64_t>(
-        1, std::min<int64_t>((int64_t)((dev.smem_optin + 1024) / (smem + 1024)), explain_warps(D) * 16 / tile_rows));
+    const int64_t per_sm = explain_blocks_per_sm(D, job.F, job.sa.quads, tile_rows, dev);
     const int64_t tiles = (n + tile_rows - 1) / tile_rows, room = (int64_t)dev.sms * per_sm;
     const double walk = 0.034 * job.T * (1 << D);
     int best = 1;

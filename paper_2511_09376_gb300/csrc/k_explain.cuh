@@ -477,18 +477,18 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
     for (int k = 0; k < UPT - 1; ++k) out[(size_t)(UPT * GL + k) * 32] = top[k];
 }
 
-// Persistent form over a ragged batch: work item i is (job, request, first row).  Blocks
-// claim items in order from a counter (n_items[1], zero at launch), so expensive items,
-// which the host puts first, spread over the whole grid and cheap ones fill the tail.
-// The item count n_items[0] is read from device memory, so one captured graph serves
-// batches of any size up to its capacity.  Which block computes a tile does not change
-// any row's arithmetic.
+// Persistent form over a ragged batch: work item i is a tile of a request, or one of its groups
+// of parts (launch.h).  Blocks claim items in order from a counter (n_items[1], zero at launch),
+// so expensive items, which the host puts first, spread over the whole grid and cheap ones fill
+// the tail.  The item count n_items[0] is read from device memory, so one captured graph serves
+// batches of any size up to its capacity.  Which block computes a tile does not change any
+// row's arithmetic, nor do the groups: parts are always added in their order.
 template <int D, int TC>
 __global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16 / TC) k_explain_batch(const ExplainJob *__restrict__ jobs,
                                                          const BatchRequest *__restrict__ reqs,
-                                                         const int4 *__restrict__ items, int *__restrict__ n_items) {
+                                                         const int4 *__restrict__ items, int *n_items) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int claimed;
+    __shared__ int claimed, arrived;
     const int count = n_items[0];
     for (;;) {
         if (threadIdx.x == 0) claimed = atomicAdd(n_items + 1, 1);
@@ -498,9 +498,29 @@ __global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16
         const int4 it = items[i];
         const ExplainJob job = jobs[it.x];
         const BatchRequest rq = reqs[it.y];
-        const int64_t c0 = ((int64_t)it.z << 31) | (uint32_t)it.w;
-        explain_tile<D, TC>(job, rq.codes, rq.n, rq.phi, rq.ldp, c0, 0, explain_parts(job.T, D), nullptr, smem_raw);
+        const int group = it.z >> kBatchGroupShift, P = explain_parts(job.T, D), groups = rq.groups;
+        const int64_t c0 = ((int64_t)(it.z & ((1 << kBatchGroupShift) - 1)) << 31) | (uint32_t)it.w;
+        explain_tile<D, TC>(job, rq.codes, rq.n, rq.phi, rq.ldp, c0, P * group / groups, P * (group + 1) / groups,
+                            groups > 1 ? rq.parts : nullptr, smem_raw);
         __syncthreads();
+        if (groups > 1) {  // the last of the tile's items adds its parts
+            if (threadIdx.x == 0) {
+                __threadfence();
+                arrived = atomicAdd(n_items + 2 + rq.tile0 + (int)(c0 / TC), 1);
+                __threadfence();
+            }
+            __syncthreads();
+            if (arrived == groups - 1) {
+                const int64_t rows = min((int64_t)TC, rq.n - c0), cells = rows * job.F, step = rq.n * job.F;
+                const float *src = rq.parts + c0 * job.F;
+                for (int64_t k = threadIdx.x; k < cells; k += explain_threads(TC)) {
+                    float x = __ldcg(src + k);
+                    for (int p = 1; p < P; ++p) x += __ldcg(src + p * step + k);
+                    rq.phi[(c0 + k / job.F) * rq.ldp + k % job.F] = x;
+                }
+            }
+            __syncthreads();
+        }
     }
 }
 

@@ -62,14 +62,20 @@ __host__ __device__ constexpr int lines_words(int D) { return (1 << (D - 2)) / 4
 
 // One request of a ragged batch: n consumer rows at C (row stride ldc), phi out; codes
 // receives the rows' decision code blocks (rows padded to a multiple of 128), job is
-// the slot of the request's ensemble among its class's jobs.
+// the slot of the request's ensemble among its class's jobs.  groups > 1: every tile's parts
+// go over that many work items, which store them at parts + p * n * F; the one that counts
+// to groups in done[tile0 + tile] (n_items + 2 of the class) adds them into phi.
 struct BatchRequest {
     const float *C;
     float *phi;
     unsigned char *codes;
+    float *parts;
     int64_t n, ldc, ldp;
-    int job;
+    int job, groups, tile0;
 };
+// A work item is (job, request, first row >> 31 | group << 24, first row & 0x7FFFFFFF).
+constexpr int kBatchGroupShift = 24;
+constexpr int64_t kBatchMaxRows = 1ll << 55;
 
 struct DevInfo {
     int sms = 0;
@@ -196,6 +202,7 @@ cudaError_t explain_timing_read(double *ms, int64_t *launches);
 // quads: 16-byte quads of a 32-row code block.
 int default_tile_rows(int D, int F, int quads, const DevInfo &dev);
 size_t explain_smem_bytes(int D, int F, int quads, int tile_rows);
+int explain_blocks_per_sm(int D, int F, int quads, int tile_rows, const DevInfo &dev);
 
 // Decision codes of a ragged batch's rows: items (request, group of packs, first 32-row block,
 // blocks), *n_items read on the device; a grid of `grid` blocks walks them.  max_group_thr:
