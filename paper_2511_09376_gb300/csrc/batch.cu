@@ -54,6 +54,7 @@ int64_t padded_rows(int64_t n) { return (n + kCodePad - 1) / kCodePad * kCodePad
 
 // Most scratch of the parts of one call's split requests; kept until the batch is destroyed.
 constexpr size_t kPartsBytes = (size_t)128 << 20;
+constexpr int kMostItemBlocks = 16;  // 32-row blocks of an encode item
 
 }  // namespace
 
@@ -224,6 +225,16 @@ wdf_status ensure_blob(wdf_batch *b, const std::vector<int> &need_reqs, const st
     return WDF_OK;
 }
 
+// 32-row blocks of an encode item: as few as give every resident block of an encode grid an
+// item (an item reads its thresholds once, some 2 us, and takes 5 us a block), 16 at most.
+int encode_item_blocks(const wdf_batch *b, const std::vector<Req> &reqs) {
+    int64_t total = 0;
+    for (const Req &r : reqs)
+        total += padded_rows(r.n) / 32 * (int64_t)b->ens[(size_t)r.e]->pk.sgroup.size();
+    const int64_t grid = 3 * (int64_t)b->ctx->dev.sms;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kMostItemBlocks, (total + grid - 1) / grid));
+}
+
 // Writes one class's jobs, requests and items into the host blob.
 int fill_class(wdf_batch *b, int c, const std::vector<Req> &reqs, int tile_rows) {
     Cls &k = b->cls[(size_t)c];
@@ -233,6 +244,7 @@ int fill_class(wdf_batch *b, int c, const std::vector<Req> &reqs, int tile_rows)
     auto *items = reinterpret_cast<int4 *>(b->h_blob + k.off_items);
     auto *eitems = reinterpret_cast<int4 *>(b->h_blob + k.off_eitems);
     int nr = 0, ni = 0, ne = 0, nt = 0;
+    const int eb = encode_item_blocks(b, reqs);
     for (const Req &r : reqs) {
         if (b->cls_of[(size_t)r.e] != c) continue;
         rq[nr] = wdf::BatchRequest{r.C,   r.phi, b->d_codes + r.codes_off, nullptr, r.n, r.ldc,
@@ -246,9 +258,9 @@ int fill_class(wdf_batch *b, int c, const std::vector<Req> &reqs, int tile_rows)
                 items[ni++] = make_int4(b->slot_of[(size_t)r.e], nr, (int)(c0 >> 31) | g << wdf::kBatchGroupShift,
                                         (int)(c0 & 0x7FFFFFFF));
         const int64_t blocks = padded_rows(r.n) / 32;
-        for (int64_t blk = 0; blk < blocks; blk += wdf::kEncodeItemBlocks)
+        for (int64_t blk = 0; blk < blocks; blk += eb)
             for (int g = 0; g < (int)b->ens[(size_t)r.e]->pk.sgroup.size(); ++g)
-                eitems[ne++] = make_int4(nr, g, (int)blk, (int)std::min<int64_t>(wdf::kEncodeItemBlocks, blocks - blk));
+                eitems[ne++] = make_int4(nr, g, (int)blk, (int)std::min<int64_t>(eb, blocks - blk));
         ++nr;
     }
     // longest first: blocks claim items in this order, so the cheap ones fill the tail of the
@@ -332,6 +344,7 @@ void count_needs(const wdf_batch *b, const std::vector<Req> &reqs, const std::ve
     need_items->assign(b->cls.size(), 0);
     need_eitems->assign(b->cls.size(), 0);
     need_tiles->assign(b->cls.size(), 0);
+    const int eb = encode_item_blocks(b, reqs);
     for (const Req &r : reqs) {
         const int c = b->cls_of[(size_t)r.e];
         (*need_reqs)[(size_t)c] += 1;
@@ -339,7 +352,7 @@ void count_needs(const wdf_batch *b, const std::vector<Req> &reqs, const std::ve
         (*need_items)[(size_t)c] += tiles * r.groups;
         (*need_tiles)[(size_t)c] += r.groups > 1 ? tiles : 0;
         (*need_eitems)[(size_t)c] +=
-            (int)((padded_rows(r.n) / 32 + wdf::kEncodeItemBlocks - 1) / wdf::kEncodeItemBlocks) *
+            (int)((padded_rows(r.n) / 32 + eb - 1) / eb) *
             (int)b->ens[(size_t)r.e]->pk.sgroup.size();
     }
 }

@@ -392,6 +392,7 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
             }
             at = (at + 1) % SLOTS;
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");  // copies past the end: their slots are staged anew
         if (!half) turn();
         // the part's sums, stored or added, and the tile zeroed for the next part
         for (int r = half; r < 32; r += 2) {

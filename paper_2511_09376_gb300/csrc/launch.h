@@ -207,7 +207,6 @@ int explain_blocks_per_sm(int D, int F, int quads, int tile_rows, const DevInfo 
 // Decision codes of a ragged batch's rows: items (request, group of packs, first 32-row block,
 // blocks), *n_items read on the device; a grid of `grid` blocks walks them.  max_group_thr:
 // the largest of the jobs' groups.
-constexpr int kEncodeItemBlocks = 16;
 int encode_batch_grid(int max_group_thr, const DevInfo &dev);
 cudaError_t launch_encode_batch(const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items,
                                 const int *n_items, int max_group_thr, const DevInfo &dev, cudaStream_t st);
