@@ -8,6 +8,7 @@
 // these joint counts (the sibling-leaf observation of section "Algorithmic Improvements"
 // item 3, applied two levels up).
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 
 #include "launch.h"
@@ -15,7 +16,7 @@
 
 namespace wdf {
 
-// Counting on the tensor cores.  A joint count is a sum over rows of products of indicators:
+// Depth <= 6: counting on the tensor cores.  A joint count is a sum over rows of products of indicators:
 // count(R, n) = sum_rows [ancestor decisions = R] [subtree decisions = n], so 16 ancestor
 // patterns x 8 subtree patterns of one bottom subtree are a small matrix product over rows
 // with operands built in registers from the rows' decision bits.  A warp owns one unit
@@ -31,7 +32,7 @@ namespace wdf {
 //   - forms the indicator words: ancestor pattern g (and g + 8, for the MMA's upper rows)
 //     per sibling pair of subtrees, which share their ancestors, and subtree pattern g;
 //   - expands each word into eight FP16-pair registers, two rows per FP16 value, so that four
-//     m16n8k16 MMAs cover the tile.  An FP16 value with only bits 0..10 set is that integer
+//     m16n8k16 MMAs cover the tile (depth 6's sixteen ancestor patterns are one m16).  An FP16 value with only bits 0..10 set is that integer
 //     times 2^-24.  The ancestor side keeps bits j and j + 8 of each half (one AND, the shift
 //     shared by three registers); the subtree side, whose words are stored with the bits of
 //     each half reversed, puts the same two rows at bits 10 - j and 2 - j.  Every product is
@@ -43,15 +44,13 @@ namespace wdf {
 // instruction); one row per FP16 value takes twice the MMAs and nearly twice the logic.
 // Bound by the logic pipe (58 % busy, issue 55 %): 2.31 ms per 1M rows and 200 trees of depth 6,
 // where one shared-memory atomic per (row, bottom subtree), each row's decisions made node by
-// node, took 5.14 ms; depth 7, 100 trees: 3.95 ms per 1M rows against 6.5.  Depth 8 is
-// latency-bound at 8 warps per SM (128 counters per lane) and took as long either way.
+// node, took 5.14 ms, and k_bg_add below takes 20 % more (depth 5: 12 %).
 template <int D>
 struct Unit {
     static constexpr int H = unit_height(D), TOP = unit_top(D), UPT = units_per_tree(D);
     static constexpr int NLOC = (1 << H) - 1, NSU = 1 << (H - 2);  // nodes and bottom subtrees
-    static constexpr int TILES = TOP > 0 ? 1 << (TOP - 1) : 1;     // m16 tiles of ancestor patterns
-    static constexpr int WMAX = D <= 6 ? 16 : (D == 7 ? 12 : 8);   // warps per block (registers)
 };
+constexpr int kCountWarps = 16;  // of an SM (k_bg_count's registers)
 constexpr int kDecStride = 36;  // words of a row block's decision words: 9 * 16 bytes, so that the
                                 // four row blocks of a fragment lie in different banks
 
@@ -84,7 +83,7 @@ __device__ __forceinline__ void expand_b(uint32_t y, uint32_t (&r)[8]) {
     for (int j = 0; j < 8; ++j) r[j] = (j < 3 ? y0 : j < 6 ? y3 : y6) & (0x01010101u << (2 - j % 3));
 }
 
-// The decision words of one node for the four row blocks of a tile.
+// The decision words of one node for the row blocks of a tile.
 struct SliceNode {
     uint32_t at, m[3][4];
     __device__ __forceinline__ void load(const UnitNode *p) {
@@ -101,19 +100,20 @@ struct SliceNode {
             if (k < nq) w = slice_le(w, block[sa.qbase[k] + col], m[k]);
         return w;
     }
-    __device__ __forceinline__ void decide(const uint4 *tile, const SliceArrays &sa, uint32_t (&w)[4]) const {
+    template <int N>
+    __device__ __forceinline__ void decide(const uint4 *tile, const SliceArrays &sa, uint32_t (&w)[N]) const {
         const int col = (int)(at & 0xFFFFu), nq = (int)((at >> 16) & 15u);
         const uint32_t le0 = 0u - ((at >> 20) & 1u);
 #pragma unroll
-        for (int b = 0; b < 4; ++b) w[b] = le0;
+        for (int b = 0; b < N; ++b) w[b] = le0;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             if (k < nq) {
-                uint4 q[4];
+                uint4 q[N];
 #pragma unroll
-                for (int b = 0; b < 4; ++b) q[b] = tile[b * sa.quads + sa.qbase[k] + col];
+                for (int b = 0; b < N; ++b) q[b] = tile[b * sa.quads + sa.qbase[k] + col];
 #pragma unroll
-                for (int b = 0; b < 4; ++b) w[b] = slice_le(w[b], q[b], m[k]);
+                for (int b = 0; b < N; ++b) w[b] = slice_le(w[b], q[b], m[k]);
             }
         }
     }
@@ -124,11 +124,12 @@ struct SliceNode {
 // nslices, ... in runs of SUB tiles.  STAGES runs in shared memory, filled by cp.async ahead
 // of their use (a barrier per run); STAGES = 0 reads the codes from global memory (rows too wide for two tiles).
 template <int D, int STAGES, int SUB>
-__global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsigned char *__restrict__ codes, int64_t m,
+__global__ void __launch_bounds__(32 * kCountWarps, 1) k_bg_count(const unsigned char *__restrict__ codes, int64_t m,
                                                                    SliceArrays sa, const TreeMeta *__restrict__ meta,
                                                                    int units, int chunks, uint32_t *__restrict__ hist) {
     using S = Shape<D>;
     using N = Unit<D>;
+    static_assert(N::TOP <= 1, "one m16 of ancestor patterns");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
     const int chunk = blockIdx.x % chunks, slice = blockIdx.x / chunks, nslices = gridDim.x / chunks;
@@ -139,27 +140,21 @@ __global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsign
     uint32_t *dec = reinterpret_cast<uint32_t *>(smem_raw + (size_t)STAGES * run16 * 16) + warp * 4 * kDecStride;
     const int64_t tiles = (m + kBgTileRows - 1) / kBgTileRows, runs = (tiles + SUB - 1) / SUB;
 
-    SliceNode node, top;  // this lane's node; top node 1 + lane / 4 of the unit's path, for row block lane % 4
+    SliceNode node;
     {
         const UnitNode *un = sa.unit + (size_t)unit * 32 + lane;
         if (N::TOP > 0 && lane == 31) un = sa.unit + (size_t)t * N::UPT * 32 + 31;  // the root
         node.load(un);
-        if constexpr (N::TOP > 1) {
-            const int k = min(1 + (lane >> 2), N::TOP - 1), v = (1 << k) - 1 + (u >> (N::TOP - k));
-            top.load(sa.unit + ((size_t)t * N::UPT + v) * 32 + 31);
-        }
     }
     const uint32_t live = (uint32_t)(__ldg(&meta[t].live) >> (u * N::NSU)) & ((1u << N::NSU) - 1u);
     const bool flip = lane >= N::NSU - 1 && lane < N::NLOC;  // nodes of a bottom subtree
     const int g = lane >> 2, q = lane & 3;
     const uint32_t x0 = (g & 4) ? 0u : ~0u, x1 = (g & 2) ? 0u : ~0u, x2 = (g & 1) ? 0u : ~0u;
-    uint32_t count[N::NSU][N::TILES][4];
+    uint32_t count[N::NSU][4];
 #pragma unroll
     for (int s = 0; s < N::NSU; ++s)
 #pragma unroll
-        for (int i = 0; i < N::TILES; ++i)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) count[s][i][k] = 0u;
+        for (int k = 0; k < 4; ++k) count[s][k] = 0u;
 
     const float base[4] = {kCountBase, kCountBase, kCountBase, kCountBase};
     auto fetch = [&](int64_t run, int stage) {
@@ -197,38 +192,21 @@ __global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsign
             node.decide(src, sa, w);
 #pragma unroll
             for (int b = 0; b < 4; ++b) dec[b * kDecStride + lane] = flip ? __byte_perm(__brev(w[b]), 0u, 0x1032) : w[b];
-            if constexpr (N::TOP > 1) {
-                if (lane < 4 * (N::TOP - 1)) dec[q * kDecStride + 32 + (lane >> 2)] = top.decide1(src + q * sa.quads, sa);
-            }
             __syncwarp();
             constexpr int NV = (N::NLOC + 3) / 4;
-            uint32_t d[4 * NV > 32 ? 4 * NV : 32], pre[4];
+            uint32_t d[4 * NV > 32 ? 4 * NV : 32];
             const uint32_t *mine = dec + q * kDecStride;
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
                 const uint4 v = reinterpret_cast<const uint4 *>(mine)[i];
                 d[4 * i] = v.x; d[4 * i + 1] = v.y; d[4 * i + 2] = v.z; d[4 * i + 3] = v.w;
             }
-            pre[0] = N::TOP > 0 ? d[31] : 0u;
-            if constexpr (N::TOP > 1) {
-                const uint2 v = *reinterpret_cast<const uint2 *>(mine + 32);
-                pre[1] = v.x; pre[2] = v.y;
-            }
             __syncwarp();
             const uint32_t valid = left >= 32 ? ~0u : (left > 0 ? (1u << left) - 1u : 0u);
-            // rows whose top decisions are c (root in the highest bit)
-            uint32_t path[1 << N::TOP];
-            path[0] = valid;
-#pragma unroll
-            for (int k = 0; k < N::TOP; ++k)
-#pragma unroll
-                for (int c = (1 << k) - 1; c >= 0; --c) {
-                    path[2 * c + 1] = path[c] & pre[k];
-                    path[2 * c] = path[c] & ~pre[k];
-                }
+            // depth 6: rows that the root sends right and left
             Shifts in[1 << N::TOP];
-#pragma unroll
-            for (int c = 0; c < 1 << N::TOP; ++c) in[c].set(path[c]);
+            in[0].set(N::TOP > 0 ? valid & ~d[31] : valid);
+            if constexpr (N::TOP > 0) in[1].set(valid & d[31]);
             constexpr int NP = N::NSU > 1 ? N::NSU / 2 : 1;  // sibling pairs
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
@@ -245,25 +223,22 @@ __global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsign
                     const int c = N::NSU - 1 + 3 * (2 * j + h);  // the root's left child, right child and the root
                     expand_b((d[c + 2] ^ x0) & (d[c + 1] ^ x1) & (d[c] ^ x2), rb[h]);
                 }
+                uint32_t ra[2][8];
+                expand_a(own, in[0], ra[0]);
+                if constexpr (N::TOP > 0) expand_a(own, in[1], ra[1]);
+                float acc[2][4];
 #pragma unroll
-                for (int i = 0; i < N::TILES; ++i) {
-                    uint32_t ra[2][8];
-                    expand_a(own, in[N::TOP > 0 ? 2 * i : 0], ra[0]);
-                    if constexpr (N::TOP > 0) expand_a(own, in[2 * i + 1], ra[1]);
-                    float acc[2][4];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-#pragma unroll
-                        for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h)
-                            mma_f16(acc[h], ra[0][2 * k], N::TOP > 0 ? ra[1][2 * k] : 0u, ra[0][2 * k + 1],
-                                    N::TOP > 0 ? ra[1][2 * k + 1] : 0u, rb[h][2 * k], rb[h][2 * k + 1],
-                                    k == 0 ? base : acc[h]);
+                for (int k = 0; k < 4; ++k)
 #pragma unroll
                     for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h)
+                        mma_f16(acc[h], ra[0][2 * k], N::TOP > 0 ? ra[1][2 * k] : 0u, ra[0][2 * k + 1],
+                                N::TOP > 0 ? ra[1][2 * k + 1] : 0u, rb[h][2 * k], rb[h][2 * k + 1],
+                                k == 0 ? base : acc[h]);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            count[2 * j + h][i][k] = __dp4a(__float_as_uint(acc[h][k]), 0x00000100u, count[2 * j + h][i][k]);
-                }
+                for (int h = 0; h < (N::NSU > 1 ? 2 : 1); ++h)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        count[2 * j + h][k] = __dp4a(__float_as_uint(acc[h][k]), 0x00000100u, count[2 * j + h][k]);
             }
         }
     }
@@ -273,15 +248,12 @@ __global__ void __launch_bounds__(32 * Unit<D>::WMAX, 1) k_bg_count(const unsign
         if (!((live >> s) & 1u)) continue;
         uint32_t *h = hist + ((size_t)t * S::NS + u * N::NSU + s) * S::E;
 #pragma unroll
-        for (int i = 0; i < N::TILES; ++i)
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                // accumulator k: pattern row g (+ 8 for k >= 2), subtree pattern 2q + (k & 1)
-                const uint32_t R = N::TOP > 0 ? (uint32_t)((2 * i + (k >> 1)) << 3) | (uint32_t)g
-                                              : (uint32_t)g + 8u * (k >> 1);
-                const uint32_t c = count[s][i][k];
-                if (R < (uint32_t)(S::E >> 3) && c) atomicAdd(h + ((R << 3) | (2 * q + (k & 1))), c);
-            }
+        for (int k = 0; k < 4; ++k) {
+            // accumulator k: pattern row g (+ 8 for k >= 2), subtree pattern 2q + (k & 1)
+            const uint32_t R = (uint32_t)g + 8u * (k >> 1);
+            const uint32_t c = count[s][k];
+            if (R < (uint32_t)(S::E >> 3) && c) atomicAdd(h + ((R << 3) | (2 * q + (k & 1))), c);
+        }
     }
 }
 
@@ -299,14 +271,14 @@ static cudaError_t bg_count_t(const unsigned char *codes, int64_t m, const Slice
     auto smem = [&](int W) { return (size_t)STAGES * SUB * sa.quads * 64 + (size_t)W * 4 * kDecStride * 4; };
     int64_t best = -1, best_slices = 1;
     int best_w = 1;
-    for (int W = std::min(units, N::WMAX); W >= 1; --W) {
+    for (int W = std::min(units, kCountWarps); W >= 1; --W) {
         const int64_t chunks = (units + W - 1) / W;
         const int64_t per_sm = std::max<int64_t>(
-            1, std::min<int64_t>(N::WMAX / W, (int64_t)(dev.smem_optin / (smem(W) + 1024))));
+            1, std::min<int64_t>(kCountWarps / W, (int64_t)(dev.smem_optin / (smem(W) + 1024))));
         const int64_t slices = std::max<int64_t>(1, std::min<int64_t>(runs, dev.sms * per_sm / chunks));
         const int64_t waves = (chunks * slices + dev.sms * per_sm - 1) / (dev.sms * per_sm);
         const int64_t warps = W * std::min(per_sm, (chunks * slices + dev.sms - 1) / dev.sms);  // of one SM
-        const int64_t cost = waves * std::max<int64_t>(warps, 3 * N::WMAX / 4) * (((runs + slices - 1) / slices) * SUB + 2);
+        const int64_t cost = waves * std::max<int64_t>(warps, 3 * kCountWarps / 4) * (((runs + slices - 1) / slices) * SUB + 2);
         if (best < 0 || cost <= best) {
             best = cost;
             best_w = W;
@@ -322,6 +294,146 @@ static cudaError_t bg_count_t(const unsigned char *codes, int64_t m, const Slice
     return cudaGetLastError();
 }
 
+// Depth 7 and 8: counting by shared-memory atomics (a unit's 8 x 2^(D+1) counters grow with the
+// depth, and with them the MMAs, but not a row's 8 entries per unit).  Two warps own one unit and
+// its counters in shared memory, each takes two of a tile's four row blocks.  A warp evaluates
+// the unit's nodes on the sliced codes as above, turns the words of 32 rows so that each lane
+// has its row's 31 decisions (wdf_device.cuh), and adds one to the row's entry of every live
+// subtree.  Latency-bound (issue 53 %, shared-memory wavefronts 60 %, 5.6 of them per atomic);
+// four warps per unit with one row block each take 15 % longer, one warp with four 7 %.
+// 60,013 rows and 300 trees of depth 8 2.48 -> 1.44 ms, 60,000 rows and 300 trees of depth 7 0.77
+// -> 0.66 (from MMAs with four and two m16 tiles of ancestor patterns), encoding included.
+template <int D, int STAGES>
+__global__ void __launch_bounds__(512, 1) k_bg_add(const unsigned char *__restrict__ codes, int64_t m, SliceArrays sa,
+                                                  const TreeMeta *__restrict__ meta, int units, int chunks,
+                                                  uint32_t *__restrict__ hist) {
+    using S = Shape<D>;
+    using N = Unit<D>;
+    constexpr int GS = N::NSU, TOP = N::TOP, CELLS = GS * S::E;
+    static_assert(N::H == 5, "units of 31 nodes");
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 6, half = (tid >> 5) & 1, W = blockDim.x >> 6;
+    const int chunk = blockIdx.x % chunks, slice = blockIdx.x / chunks, nslices = gridDim.x / chunks;
+    const bool spare = chunk * W + warp >= units;
+    const int unit = min(chunk * W + warp, units - 1), t = unit / N::UPT, u = unit % N::UPT;
+    const int tile16 = 4 * sa.quads;  // 16-byte words of a tile
+    uint4 *ring = reinterpret_cast<uint4 *>(smem_raw);
+    uint32_t *cells = reinterpret_cast<uint32_t *>(smem_raw + (size_t)STAGES * tile16 * 16) + warp * CELLS;
+    const uint32_t at = (uint32_t)__cvta_generic_to_shared(cells);
+    const int64_t tiles = (m + kBgTileRows - 1) / kBgTileRows;
+
+    SliceNode node, top;  // as in k_bg_count
+    {
+        const UnitNode *un = sa.unit + (size_t)unit * 32 + lane;
+        if (TOP > 0 && lane == 31) un = sa.unit + (size_t)t * N::UPT * 32 + 31;  // the root
+        node.load(un);
+        if constexpr (TOP > 1) {
+            const int k = min(1 + (lane >> 1), TOP - 1), v = (1 << k) - 1 + (u >> (TOP - k));
+            top.load(sa.unit + ((size_t)t * N::UPT + v) * 32 + 31);
+        }
+    }
+    const uint32_t live = spare ? 0u : (uint32_t)(__ldg(&meta[t].live) >> (u * GS)) & ((1u << GS) - 1u);
+    for (int i = tid; i < W * CELLS; i += blockDim.x)
+        reinterpret_cast<uint32_t *>(smem_raw + (size_t)STAGES * tile16 * 16)[i] = 0u;
+    __syncthreads();
+
+    auto fetch = [&](int64_t tile, int stage) {
+        if constexpr (STAGES > 0) {
+            if (tile < tiles) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(codes) + tile * tile16 + tid;
+                uint32_t dst = (uint32_t)__cvta_generic_to_shared(ring + (size_t)stage * tile16 + tid);
+                for (int i = tid; i < tile16; i += blockDim.x, src += blockDim.x, dst += 16u * blockDim.x)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src));
+            }
+            asm volatile("cp.async.commit_group;");
+        }
+    };
+#pragma unroll
+    for (int k = 0; k + 1 < STAGES; ++k) fetch(slice + (int64_t)k * nslices, k);
+    int stage = 0;
+    for (int64_t tile = slice; tile < tiles; tile += nslices) {
+        const uint4 *src;
+        if constexpr (STAGES > 0) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(STAGES > 1 ? STAGES - 2 : 0));
+            __syncthreads();
+            fetch(tile + (int64_t)(STAGES - 1) * nslices, stage == 0 ? STAGES - 1 : stage - 1);
+            src = ring + (size_t)stage * tile16;
+            stage = stage + 1 == STAGES ? 0 : stage + 1;
+        } else {
+            src = reinterpret_cast<const uint4 *>(codes) + tile * tile16;
+        }
+        src += 2 * half * sa.quads;
+        const int left = (int)min(m - tile * kBgTileRows, (int64_t)kBgTileRows) - 64 * half;  // rows of this warp
+        uint32_t w[2], tw = 0u;
+        node.decide(src, sa, w);
+        if constexpr (TOP > 1) {
+            if (lane < 2 * (TOP - 1)) tw = top.decide1(src + (lane & 1) * sa.quads, sa);
+        }
+        transpose32(w, lane);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            uint32_t path = TOP > 0 ? w[b] >> 31 : 0u;
+#pragma unroll
+            for (int k = 1; k < TOP; ++k) path = 2u * path + ((__shfl_sync(0xFFFFFFFFu, tw, 2 * (k - 1) + b) >> lane) & 1u);
+            // byte offsets, entry e of subtree j at 4 (j E + e): R of the children of the unit's
+            // nodes above its subtrees, 32 bytes (eight entries) apart
+            uint32_t R[GS - 1];
+            R[0] = 64u * path | ((w[b] << 5) & 32u);
+#pragma unroll
+            for (int k = 1; k < GS - 1; ++k) {
+                R[k] = 2u * R[(k - 1) >> 1] | ((k < 5 ? w[b] << (5 - k) : w[b] >> (k - 5)) & 32u);
+            }
+#pragma unroll
+            for (int k = GS / 2 - 1; k < GS - 1; ++k) R[k] += at;
+            if (32 * b + lane < left) {
+#pragma unroll
+                for (int j = 0; j < GS; ++j)
+                    if ((live >> j) & 1u)  // the same for all lanes
+                        asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(
+                                         (((w[b] >> (GS - 3 + 3 * j)) & 28u) | R[(GS - 2 + j) >> 1]) + 4u * j * S::E)
+                                     : "memory");
+            }
+        }
+    }
+    __syncthreads();
+    if (spare) return;
+    uint32_t *h = hist + ((size_t)t * S::NS + u * GS) * S::E;
+    for (int i = (tid & 63); i < CELLS; i += 64) {
+        const uint32_t c = cells[i];
+        if (c) atomicAdd(h + i, c);
+    }
+}
+
+// Eight units per block (as many as fit) and the number of row slices with the least time by
+// this measure: a block takes its tiles' time and four tiles' more for its counters; blocks go
+// round the SMs; they differ in live subtrees, so a round ends 14 % of a block's time late.
+// 300 trees, 60,000 rows: depth 8, 1, 2 and 3 slices 1.54, 1.46 and 1.43 ms; depth 7, 1, 2, 4
+// and 6 slices 709, 684, 655 and 648 us.
+constexpr int kAddUnits = 8;
+template <int D, int STAGES>
+static cudaError_t bg_add_t(const unsigned char *codes, int64_t m, const SliceArrays &sa, const TreeMeta *meta, int T,
+                            int W, uint32_t *hist, const DevInfo &dev, cudaStream_t st) {
+    const int units = T * Unit<D>::UPT, chunks = (units + W - 1) / W;
+    const int64_t tiles = (m + kBgTileRows - 1) / kBgTileRows;
+    int64_t slices = 1;
+    double least = 0.0;
+    for (int64_t s = 1; s <= std::min<int64_t>(tiles, 64); ++s) {
+        const double one = (double)((tiles + s - 1) / s + 4), rounds = (double)(chunks * s) / dev.sms;
+        const double cost = one * (0.14 + (rounds <= 1.0 ? 1.0 : 0.5 * (rounds + std::ceil(rounds))));
+        if (s == 1 || cost < least) {
+            slices = s;
+            least = cost;
+        }
+    }
+    const size_t smem = (size_t)STAGES * sa.quads * 64 + (size_t)W * Unit<D>::NSU * Shape<D>::E * 4;
+    auto kern = k_bg_add<D, STAGES>;
+    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err != cudaSuccess) return err;
+    kern<<<(unsigned)(slices * chunks), 64 * W, smem, st>>>(codes, m, sa, meta, units, chunks, hist);
+    count_launches(1);
+    return cudaGetLastError();
+}
+
 // Long chunks of rows run with four tiles per barrier, where three such runs fit: 2.31 ms per
 // 1M rows and 200 depth-6 trees against 2.53 with two tiles per run and two half-size blocks
 // per SM (the warps of a block drift apart and wait at every barrier).  Below 16,384 rows a
@@ -330,12 +442,21 @@ constexpr int64_t kBgLongRows = 16384;
 template <int D>
 static cudaError_t bg_count(const unsigned char *codes, int64_t m, const SliceArrays &sa, const TreeMeta *meta, int T,
                             uint32_t *hist, const DevInfo &dev, cudaStream_t st) {
-    const size_t dec = (size_t)Unit<D>::WMAX * 4 * kDecStride * 4;
-    if (3 * 4 * (size_t)sa.quads * 64 + dec <= dev.smem_optin && m >= kBgLongRows)
-        return bg_count_t<D, 3, 4>(codes, m, sa, meta, T, hist, dev, st);
-    if (3 * (size_t)sa.quads * 64 + dec <= dev.smem_optin)
-        return bg_count_t<D, 3, 1>(codes, m, sa, meta, T, hist, dev, st);
-    return bg_count_t<D, 0, 1>(codes, m, sa, meta, T, hist, dev, st);
+    if constexpr (D >= 7) {
+        // rows too wide for two tiles beside four units' counters are read from global memory
+        const size_t unit = (size_t)Unit<D>::NSU * Shape<D>::E * 4, ring = (size_t)2 * sa.quads * 64;
+        const int most = std::min(kAddUnits, T * Unit<D>::UPT);
+        const int fit = ring < dev.smem_optin ? (int)std::min<size_t>(most, (dev.smem_optin - ring) / unit) : 0;
+        if (fit >= std::min(most, 4)) return bg_add_t<D, 2>(codes, m, sa, meta, T, fit, hist, dev, st);
+        return bg_add_t<D, 0>(codes, m, sa, meta, T, most, hist, dev, st);
+    } else {
+        const size_t dec = (size_t)kCountWarps * 4 * kDecStride * 4;
+        if (3 * 4 * (size_t)sa.quads * 64 + dec <= dev.smem_optin && m >= kBgLongRows)
+            return bg_count_t<D, 3, 4>(codes, m, sa, meta, T, hist, dev, st);
+        if (3 * (size_t)sa.quads * 64 + dec <= dev.smem_optin)
+            return bg_count_t<D, 3, 1>(codes, m, sa, meta, T, hist, dev, st);
+        return bg_count_t<D, 0, 1>(codes, m, sa, meta, T, hist, dev, st);
+    }
 }
 
 cudaError_t launch_bg_hist(int D, const float *B, int64_t m, int64_t ldb, const TreeMeta *meta, const SliceArrays &sa,

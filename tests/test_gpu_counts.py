@@ -82,3 +82,10 @@ def test_wide_rows(ctx):
     ens, _, B = synth.make(synth.Workload("c", 980, 1, 260, 3000, 2500, 60, 6, 0.5, 0.0, True))
     assert np.unique(ens.feature).size > 1400
     _counts_equal(ctx, ens, B)
+
+
+@pytest.mark.parametrize("depth", [7, 8])
+@pytest.mark.parametrize("features", [1000, 3000])  # fewer units per block; codes read from global memory
+def test_wide_rows_of_deep_trees(ctx, depth, features):
+    ens, _, B = synth.make(synth.Workload("c", 990 + depth, 1, 200, features, features, 40, depth, 0.5, 0.1, False))
+    _counts_equal(ctx, ens, B)
