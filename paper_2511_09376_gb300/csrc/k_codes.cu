@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(kSliceThreads, 3) k_encode_slices(const float 
                                                                    int64_t ldx, SliceArrays sa, int64_t blocks,
                                                                    unsigned char *__restrict__ codes) {
     extern __shared__ __align__(16) float slice_smem_raw[];
+    early_launch();
     encode_group(X, rows, ldx, sa, blockIdx.y, blockIdx.x, blocks, gridDim.x, codes, slice_smem_raw);
 }
 

@@ -119,9 +119,11 @@ __global__ void __launch_bounds__(32 * kSumWarps) k_sum_values(const float *__re
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, f = blockIdx.x * kSumWarps + warp;
     const float *v = values + (size_t)blockIdx.y * T * FL * 32 + lane;
     float total = 0.0f;
+    int off = f < F && lane <= P ? __ldg(voff + (size_t)f * P + lane) : 0;  // at most nine
+    previous_done();  // the node values
     if (f < F) {
         for (int p = 0; p < P; ++p) {
-            const int beg = __ldg(voff + (size_t)f * P + p), end = __ldg(voff + (size_t)f * P + p + 1);
+            const int beg = __shfl_sync(0xFFFFFFFFu, off, p), end = __shfl_sync(0xFFFFFFFFu, off, p + 1);
             float acc = 0.0f;
             for (int k0 = beg; k0 < end; k0 += 32) {
                 const int mine = k0 + lane < end ? __ldg(vlist + k0 + lane) : 0, cnt = min(32, end - k0);
@@ -131,7 +133,7 @@ __global__ void __launch_bounds__(32 * kSumWarps) k_sum_values(const float *__re
 #pragma unroll
                     for (int k = 0; k < 16; ++k) {
                         const int i = __shfl_sync(0xFFFFFFFFu, mine, h + k);
-                        x[k] = h + k < cnt ? __ldg(v + (size_t)i * 32) : 0.0f;
+                        x[k] = h + k < cnt ? v[(size_t)i * 32] : 0.0f;
                     }
 #pragma unroll
                     for (int k = 0; k < 16; ++k)
@@ -154,10 +156,10 @@ static cudaError_t explain_values(const unsigned char *codes, int64_t n, const E
     cudaError_t err = values_t<D>(codes, n, job, values, dev, st);
     if (err != cudaSuccess) return err;
     const dim3 grid((unsigned)((job.F + kSumWarps - 1) / kSumWarps), (unsigned)((n + 31) / 32));
-    k_sum_values<<<grid, 32 * kSumWarps, 0, st>>>(values, flush_len(D), job.vlist, job.voff, job.T, job.F,
-                                                  explain_parts(job.T, D), n, phi, ldp);
+    err = launch_dependent(k_sum_values, grid, 32 * kSumWarps, 0, st, (const float *)values, flush_len(D), job.vlist,
+                           job.voff, job.T, job.F, explain_parts(job.T, D), n, phi, ldp);
     count_launches(1);
-    return cudaGetLastError();
+    return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 // Rows per encoded chunk: the decision codes of a chunk live in a stream-ordered

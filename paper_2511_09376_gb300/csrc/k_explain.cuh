@@ -437,7 +437,10 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
     const uint64_t *flags = reinterpret_cast<const uint64_t *>(job.image + (size_t)tt * image_bytes(D) + image_flags(D));
     const uint64_t live = __ldg(flags), real = __ldg(flags + 2);
     const uint4 *src = reinterpret_cast<const uint4 *>(codes) + (size_t)blockIdx.y * quads;
-    for (int i = tid; i < quads; i += 32 * kValueWarps) block[i] = __ldg(src + i);
+    uint2 node = __ldg(rec + lane);
+    early_launch();
+    previous_done();  // the rows' codes
+    for (int i = tid; i < quads; i += 32 * kValueWarps) block[i] = src[i];
     __syncthreads();
     if (t >= job.T) return;
     uint32_t topw = 0u;
@@ -445,7 +448,6 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
         topw = transpose32(lane < UPT - 1 ? unit_decide(__ldg(rec + lane * 32 + 31), block, job.sa) : 0u, lane);
     float *out = values + ((size_t)blockIdx.y * job.T + t) * FL * 32 + lane;
     float top[UPT > 1 ? UPT - 1 : 1];
-    uint2 node = __ldg(rec + lane);
 #pragma unroll X::UNROLL
     for (int u = 0; u < UPT; ++u) {
         const uint32_t w = transpose32(unit_decide(node, block, job.sa), lane);
@@ -548,9 +550,9 @@ cudaError_t values_t(const unsigned char *codes, int64_t n, const ExplainJob &jo
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
     const dim3 grid((unsigned)((job.T + kValueWarps - 1) / kValueWarps), (unsigned)((n + 31) / 32));
-    kern<<<grid, 32 * kValueWarps, smem, st>>>(codes, job, values);
+    err = launch_dependent(kern, grid, 32 * kValueWarps, smem, st, codes, job, values);
     count_launches(1);
-    return cudaGetLastError();
+    return err != cudaSuccess ? err : cudaGetLastError();
 }
 
 template <int D, int TC>
