@@ -74,6 +74,12 @@ static cudaError_t batch_depth(const ExplainJob *jobs, const BatchRequest *reqs,
     }
 }
 
+int explain_blocks_per_sm(int D, int F, int quads, int tile_rows, const DevInfo &dev) {
+    const size_t smem = explain_smem_bytes(D, F, quads, tile_rows);
+    const size_t room = explain_carveout(D, tile_rows, smem) ? kExplainCarveout : dev.smem_optin + 1024;
+    return std::max(1, std::min((int)(room / (smem + 1024)), kExplainWarps * 16 / tile_rows));
+}
+
 // The tile that keeps most warps on an SM; 32 rows where 64 keep no more (the same speed at
 // depth 6 and 127 features, 545-560 SM clocks per warp and tree; 3-7 % faster for deeper trees
 // and 20 % at 255 features, whose smaller blocks fill the shared memory better).
@@ -83,18 +89,13 @@ int default_tile_rows(int D, int F, int quads, const DevInfo &dev) {
     for (int tc : {32, 64}) {
         const size_t smem = explain_smem_bytes(D, F, quads, tc);
         if (smem > dev.smem_optin) continue;
-        const size_t warps = std::min<size_t>(explain_warps(D), (dev.smem_optin + 1024) / (smem + 1024) * (tc / 16));
+        const size_t warps = std::min<size_t>(kExplainWarps, (dev.smem_optin + 1024) / (smem + 1024) * (tc / 16));
         if (warps > most) {
             most = warps;
             best = tc;
         }
     }
     return best;
-}
-
-int explain_blocks_per_sm(int D, int F, int quads, int tile_rows, const DevInfo &dev) {
-    const size_t smem = explain_smem_bytes(D, F, quads, tile_rows);
-    return std::max(1, std::min((int)((dev.smem_optin + 1024) / (smem + 1024)), explain_warps(D) * 16 / tile_rows));
 }
 
 // phi = the parts' sums, added in part order; one thread per element of a row.
@@ -284,18 +285,36 @@ cudaError_t launch_explain_batch(int D, const ExplainJob *jobs, const BatchReque
 __global__ void k_images(int D, int T, const UnitNode *__restrict__ unit, const TreeMeta *__restrict__ meta,
                          const int32_t *__restrict__ flfeat, const uint8_t *__restrict__ flrep,
                          unsigned char *__restrict__ image) {
-    const int t = blockIdx.x, i = blockIdx.y, tid = threadIdx.x;
+    const int t = blockIdx.x, i = blockIdx.y, tid = threadIdx.x, nt = blockDim.x, xs = image_rows(i) + 1;
+    const int UPT = units_per_tree(D), CU = chunk_units(D), GS = gather_group(D), GB = flush_group_len(D) / 8;
+    const int CP = chunk_positions(D);
     unsigned char *dst = image + ((size_t)i * T + t) * image_bytes(D);
-    const int nu = units_per_tree(D) * 32, fl = flush_len(D), xs = image_rows(i) + 1;
-    for (int k = tid; k < nu; k += blockDim.x) reinterpret_cast<UnitNode *>(dst)[k] = unit[(size_t)t * nu + k];
-    if (tid < 4) {
-        const TreeMeta &m = meta[t];
-        reinterpret_cast<uint64_t *>(dst + image_flags(D))[tid] =
-            tid == 0 ? m.live : tid == 1 ? m.flush : tid == 2 ? m.real : 0ull;
+    const UnitNode *src = unit + (size_t)t * UPT * 32;
+    const int32_t *feat = flfeat + (size_t)t * flush_len(D);
+    const uint8_t *rep = flrep + (size_t)t * flush_batches(D);
+    const TreeMeta &m = meta[t];
+    for (int c = 0; c < tree_chunks(D); ++c, dst += chunk_bytes(D)) {
+        // batch b of the chunk is batch at(b) of the tree
+        auto at = [&](int b) { return b < CU * GB ? c * CU * GB + b : UPT * GB; };
+        for (int k = tid; k < 32 * CU; k += nt) reinterpret_cast<UnitNode *>(dst)[k] = src[c * CU * 32 + k];
+        for (int k = tid; k < CP; k += nt)
+            reinterpret_cast<uint16_t *>(dst + chunk_offsets(D))[k] = (uint16_t)(feat[8 * at(k / 8) + k % 8] * xs);
+        for (int k = chunk_repeats(D) + tid; k < chunk_bytes(D); k += nt) {
+            const int b = k - chunk_repeats(D);
+            dst[k] = b < CP / 8 ? rep[at(b)] : 0;
+        }
+        if (tid < CU) {
+            const int u = c * CU + tid, nb = GB + (UPT > 1 ? 1 : 0);
+            uint32_t f = (uint32_t)(m.live >> (u * GS)) & ((1u << GS) - 1u);
+            for (int b = 0; b < nb; ++b) {
+                const int tb = b < GB ? u * GB + b : UPT * GB;
+                f |= (uint32_t)((m.flush >> tb) & 1u) << (8 + b) | (uint32_t)((m.real >> tb) & 1u) << (16 + b);
+            }
+            reinterpret_cast<uint32_t *>(dst + chunk_flags(D))[tid] = f;
+        }
     }
-    for (int k = tid; k < fl; k += blockDim.x)
-        reinterpret_cast<uint16_t *>(dst + image_offsets(D))[k] = (uint16_t)(flfeat[(size_t)t * fl + k] * xs);
-    for (int k = tid; k < fl / 8; k += blockDim.x) dst[image_repeats(D) + k] = flrep[(size_t)t * (fl / 8) + k];
+    if (unit_top(D) > 1 && tid < 8)  // lane 31 of unit u is node u
+        reinterpret_cast<UnitNode *>(dst)[tid] = src[(tid < UPT ? tid : 0) * 32 + 31];
 }
 
 cudaError_t launch_images(int D, int T, const UnitNode *unit, const TreeMeta *meta, const int32_t *flfeat,

@@ -27,7 +27,7 @@
 // 32 rows (L1 pipe 78 %); with one warp per 32 rows 677 (two units' gathers in flight, ten
 // warps per SM), with two rows per thread 860 (five warps), and 624 for the kernel that
 // evaluated nodes one by one, lane = row.  Depth 5: 290, depth 7: 1220 (1940 with node-by-
-// node decisions), depth 8: 3100 (6350; slots in twelve floats, three loads per gather).
+// node decisions), depth 8: 2620 (6350; slots in twelve floats, three loads per gather).
 //
 // The kernels are templates of the depth; every depth is instantiated in its own
 // translation unit so that they compile in parallel.
@@ -42,8 +42,19 @@
 namespace wdf {
 
 // Warps per SM that the registers allow: at depth 6, 20 (96 registers) measured no faster than
-// 16 and 12 (168) 5 % slower; depth 8 keeps the root's slots apart in 8 more.
-constexpr int explain_warps(int D) { return D == 8 ? 12 : 16; }
+// 16 and 12 (168) 5 % slower.
+constexpr int kExplainWarps = 16;
+
+// Depth 8 leaves the L1 cache a good part of the SM's memory: a gather in flight holds its lines
+// there, some 300 KB for twelve warps if they could, and waits for them otherwise.  233,472 rows and
+// 40 trees of 134 features with blocks in up to 132 / 164 / 196 / 228 KB: 2773 / 2655 / 2869 / 2865 us;
+// 191 features (four blocks in 164 KB) are as fast in all of it, 60 features (ten) 2 % faster by
+// the driver's choice; depth 5 to 7 do not gain.
+constexpr size_t kExplainCarveout = (size_t)164 << 10;
+constexpr bool explain_carveout(int D, int tile_rows, size_t smem) {
+    const size_t blocks = kExplainCarveout / (smem + 1024);
+    return D == 8 && tile_rows == 32 && blocks >= 5 && blocks <= 8;
+}
 
 template <int D>
 struct ExplainCfg {
@@ -53,23 +64,25 @@ struct ExplainCfg {
     // deep trees loop over their units (unrolled, the code of a tree does not stay in the
     // instruction cache)
     static constexpr int UNROLL = D >= 7 ? 1 : UPT;
-    static constexpr int WARPS = explain_warps(D);
 };
 WDF_HD constexpr int explain_threads(int tc) { return 2 * tc; }
 
 // Shared memory of one block: code tile (TC / 32 blocks of quads) | phi tile ((F + 1) x (TC + 1)
-// floats, feature-major, row F a scratch row) | per warp, SLOTS trees' images and line maps.
+// floats, feature-major, row F a scratch row) | per warp, a ring of SLOTS chunks and their line
+// maps, then the nodes above a tree's units.  (Depth 8 a tree at a time, 33.5 KB a block instead
+// of 24.7: 3063 us where the above took 2655, 3371 where 191 features take 3090; depth 7 a unit
+// at a time 3 % slower.)
 template <int D>
 struct ExLayout {
     size_t x, p, total;
-    static constexpr int LINE = image_bytes(D), TREE = LINE + 4 * lines_words(D);
-    // a tree is copied while the tree before it (with several units) or the two trees before it
-    // are processed
-    static constexpr int SLOTS = units_per_tree(D) > 1 ? 2 : 3;
+    // a chunk is copied while the one (of two units) or the two before it are processed
+    static constexpr int SLOTS = chunk_units(D) > 1 ? 2 : 3;
+    static constexpr int LINE = chunk_bytes(D), SLOT = LINE + (chunk_units(D) > 2 ? 8 * chunk_units(D) : 16);
+    static constexpr int WARP = SLOTS * SLOT + (unit_top(D) > 1 ? 8 * (int)sizeof(UnitNode) : 0);
     __host__ __device__ ExLayout(int F, int quads, int TC) {
         x = (size_t)(TC / 32) * quads * 16;
         p = ((size_t)(F + 1) * (TC + 1) * 4 + 15) & ~(size_t)15;
-        total = x + p + (size_t)(TC / 16) * SLOTS * TREE;
+        total = x + p + (size_t)(TC / 16) * WARP;
     }
 };
 
@@ -243,15 +256,17 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
                                              int part1, float *__restrict__ scratch, unsigned char *smem_raw) {
     using X = ExplainCfg<D>;
     constexpr int XS = TC + 1, GS = X::GS, TOP = X::TOP, UPT = X::UPT;
-    constexpr int NT = explain_threads(TC), SLOTS = ExLayout<D>::SLOTS;
+    constexpr int NT = explain_threads(TC), SLOTS = ExLayout<D>::SLOTS, SLOT = ExLayout<D>::SLOT;
     constexpr int FB = flush_group_bottom(D), GL = flush_group_len(D), LW = X::LW;
-    constexpr int IMG = image_bytes(D), LINE = ExLayout<D>::LINE, TREE = ExLayout<D>::TREE;
+    constexpr int IMG = image_bytes(D), CHUNK = chunk_bytes(D), LINE = ExLayout<D>::LINE;
+    constexpr int CU = chunk_units(D), CPT = tree_chunks(D);
     const int F = job.F, T = job.T, quads = job.sa.quads;
     const ExLayout<D> L(F, quads, TC);
     uint4 *sx = reinterpret_cast<uint4 *>(smem_raw);
     float *sp = reinterpret_cast<float *>(smem_raw + L.x);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, pair = warp >> 1, half = warp & 1;
-    unsigned char *slots = smem_raw + L.x + L.p + (size_t)warp * SLOTS * TREE;  // this warp's
+    unsigned char *ring = smem_raw + L.x + L.p + (size_t)warp * ExLayout<D>::WARP;  // this warp's
+    const uint2 *above = reinterpret_cast<const uint2 *>(ring + SLOTS * SLOT);
     {
         const uint4 *src = reinterpret_cast<const uint4 *>(codes) + (c0 / 32) * quads;
         for (int i = tid; i < TC / 32 * quads; i += NT) sx[i] = __ldg(src + i);
@@ -268,21 +283,33 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         else asm volatile("bar.sync 4, 64;" ::: "memory");
     };
 
-    // Copies tree t's image and line maps into a slot (all lanes of the warp).
+    // Copies chunk c of tree t into a slot of the ring, with a tree's first chunk the nodes above
+    // its units too (read with the decisions of its first unit, CPT chunks before the next copy).
     const unsigned char *image = job.image + (size_t)(ilog2(TC) - 5) * T * IMG;
-    auto stage = [&](int t, unsigned char *slot) {
-        const unsigned char *src = image + (size_t)t * IMG;
-        const unsigned char *lsrc = reinterpret_cast<const unsigned char *>(job.lines + (size_t)t * LW) - LINE;
-        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(slot);
+    auto stage = [&](int t, int c, const unsigned char *slot) {
+        const unsigned char *tree = image + (size_t)t * IMG;
 #pragma unroll
-        for (int i = 0; i < TREE / 16; i += 32) {
-            const int k = 16 * (i + lane);
-            if (k < TREE)
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst + k), "l"((k < LINE ? src : lsrc) + k)
-                             : "memory");
+        for (int i = 0; i < CHUNK / 16 + (TOP > 1 ? 4 : 0); i += 32) {
+            const unsigned char *src = tree + c * CHUNK + 16 * (i + lane);
+            uint32_t dst = (uint32_t)__cvta_generic_to_shared(slot) + 16 * (i + lane);
+            bool on = i + lane < CHUNK / 16;
+            if (TOP > 1 && c == 0 && i + 32 >= CHUNK / 16 + 4 && lane >= 28) {
+                src = tree + image_top(D) + 16 * (lane - 28);
+                dst = (uint32_t)__cvta_generic_to_shared(above) + 16 * (lane - 28);
+                on = true;
+            }
+            if (on) asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
         }
+        // the line maps: two words a unit (a tree has at least four)
+        const uint32_t ldst = (uint32_t)__cvta_generic_to_shared(slot) + LINE;
+        const uint32_t *lsrc = job.lines + (size_t)t * LW + c * CU * (GS / 4);
+        if (CU == 1) {
+            if (lane == 24) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ldst), "l"(lsrc) : "memory");
+        } else if (lane < CU / 2) {
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(ldst + 16 * lane), "l"(lsrc + 4 * lane) : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    auto commit = [&]() { asm volatile("cp.async.commit_group;" ::: "memory"); };
     auto arrived = [&]() {  // all copies but the newest SLOTS - 2 groups are in shared memory
         asm volatile("cp.async.wait_group %0;" ::"n"(SLOTS - 2) : "memory");
         __syncwarp();
@@ -293,38 +320,37 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
     struct Words {
         uint32_t w, top;
     };
-    auto decide = [&](const unsigned char *slot, int u, const Words &p) -> Words {
+    auto decide = [&](const unsigned char *slot, int u, int i, const Words &p) -> Words {
         Words q = p;
-        const uint2 *rec = reinterpret_cast<const uint2 *>(slot);
-        if (TOP > 1 && u == 0) {  // lane 31 of unit k holds node k
+        const uint2 *rec = reinterpret_cast<const uint2 *>(slot) + i * 32;
+        if (TOP > 1 && u == 0) {
             uint32_t w[2] = {unit_decide(rec[lane], block, job.sa),
-                             lane < UPT - 1 ? unit_decide(rec[lane * 32 + 31], block, job.sa) : 0u};
+                             lane < UPT - 1 ? unit_decide(above[lane], block, job.sa) : 0u};
             transpose32(w, lane);
             q.w = w[0];
             q.top = w[1];
         } else {
-            q.w = transpose32(unit_decide(rec[u * 32 + lane], block, job.sa), lane);
+            q.w = transpose32(unit_decide(rec[lane], block, job.sa), lane);
             if (TOP == 1 && u == 0) q.top = q.w >> 31;
         }
         return q;
     };
     UnitSlots<D> v;
-    auto gather = [&](int t, const unsigned char *slot, int u, const Words &p, bool mine) {
-        const uint32_t live = (uint32_t)(*reinterpret_cast<const uint64_t *>(slot + image_flags(D)) >> (u * GS));
+    auto gather = [&](int t, const unsigned char *slot, int u, int i, const Words &p, bool mine) {
+        const uint32_t live = reinterpret_cast<const uint32_t *>(slot + chunk_flags(D))[i];
         uint32_t lm[(GS + 3) / 4];
 #pragma unroll
         for (int k = 0; k < (GS + 3) / 4; ++k)
-            lm[k] = reinterpret_cast<const uint32_t *>(slot + LINE)[u * (GS / 4) + k];
+            lm[k] = reinterpret_cast<const uint32_t *>(slot + LINE)[i * (GS / 4) + k];
         gather_unit<D>(job.sfold, T, t, u, mine ? live : 0u, lm, p.w, p.top, v);
     };
     float top[UPT > 1 ? UPT - 1 : 1];
     // Adds unit u's node values into phi; the top nodes' sums are kept until the tree's last unit.
-    auto flush = [&](const unsigned char *slot, int u, bool mine) {
-        const uint16_t *off = reinterpret_cast<const uint16_t *>(slot + image_offsets(D)) + u * GL;
-        const uint32_t fok = (uint32_t)(reinterpret_cast<const uint64_t *>(slot + image_flags(D))[1] >> (u * (GL / 8)));
-        const uint32_t real = (uint32_t)(reinterpret_cast<const uint64_t *>(slot + image_flags(D))[2] >> (u * (GL / 8))) &
-                              (mine ? ~0u : 0u);
-        const unsigned char *rep = slot + image_repeats(D) + u * (GL / 8);
+    auto flush = [&](const unsigned char *slot, int u, int i, bool mine) {
+        const uint16_t *off = reinterpret_cast<const uint16_t *>(slot + chunk_offsets(D)) + i * GL;
+        const uint32_t flags = reinterpret_cast<const uint32_t *>(slot + chunk_flags(D))[i];
+        const uint32_t fok = flags >> 8, real = (flags >> 16) & (mine ? ~0u : 0u);
+        const unsigned char *rep = slot + chunk_repeats(D) + i * (GL / 8);
         int o[8];
         load_offsets8(off, o);
         float up[GS > 1 ? GS - 1 : 1];
@@ -348,11 +374,11 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
                 if (b + 1 < GL / 8) o[q] = on[q];
         }
         if (UPT > 1 && u == UPT - 1 && mine) {
-            load_offsets8(off + GL, o);
+            load_offsets8(off + (CU - i) * GL, o);
             float x[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) x[q] = q < UPT - 1 ? top[q < UPT - 1 ? q : 0] : 0.0f;
-            flush_batch(myphi, o, x, UPT - 1, (fok >> (GL / 8)) & 1u, rep + GL / 8);
+            flush_batch(myphi, o, x, UPT - 1, (fok >> (GL / 8)) & 1u, rep + (CU - i) * (GL / 8));
         }
     };
 
@@ -363,34 +389,38 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         // both warps take the same number of turns; past the part's end the second repeats a tree
         // without gathers and additions (a branch around the gathers would wait for them)
         auto tree = [&](int t) { return min(t, te - 1); };
-        int at = 0;  // slot of the current tree
-        auto slot = [&](int k) { return slots + ((at + k) % SLOTS) * TREE; };
-#pragma unroll
-        for (int k = 0; k < SLOTS - 1; ++k) {
-            stage(tree(tb + half + 2 * k), slot(k));
-            commit();
-        }
+        // chunk c + k of tree t, past the tree's end of the warp's next trees
+        auto stage_ahead = [&](int t, int c, int k, const unsigned char *slot) {
+            stage(tree(t + 2 * ((c + k) / CPT)), (c + k) % CPT, slot);
+        };
+        // the chunk at work, the next one and (of three) the one to copy into
+        const unsigned char *now = ring, *next = ring + SLOT, *free = ring + (SLOTS - 1) * SLOT;
+        stage_ahead(tb + half, 0, 0, now);
+        if (SLOTS == 3) stage_ahead(tb + half, 0, 1, next);
         arrived();
-        Words p = decide(slot(0), 0, Words{});
+        Words p = decide(now, 0, 0, Words{});
         if (half) turn();
         for (int t = tb + half; t < te + half; t += 2) {
             const bool mine = t < te;
-            stage(tree(t + 2 * (SLOTS - 1)), slot(SLOTS - 1));
-            commit();
+#pragma unroll 1
+            for (int c = 0; c < CPT; ++c) {
+                stage_ahead(t, c, SLOTS - 1, free);
 #pragma unroll X::UNROLL
-            for (int u = 0; u < UPT; ++u) {
-                gather(tree(t), slot(0), u, p, mine);
-                if (u + 1 < UPT) {
-                    p = decide(slot(0), u + 1, p);
-                } else {
-                    arrived();
-                    p = decide(slot(1), 0, p);
+                for (int i = 0; i < CU; ++i) {
+                    const int u = c * CU + i;
+                    const bool last = i + 1 == CU;
+                    gather(tree(t), now, u, i, p, mine);
+                    if (last) arrived();
+                    p = decide(last ? next : now, u + 1 < UPT ? u + 1 : 0, last ? 0 : i + 1, p);
+                    turn();
+                    flush(now, u, i, mine);
+                    turn();
                 }
-                turn();
-                flush(slot(0), u, mine);
-                turn();
+                const unsigned char *done = now;
+                now = next;
+                next = SLOTS == 3 ? free : done;
+                free = done;
             }
-            at = (at + 1) % SLOTS;
         }
         asm volatile("cp.async.wait_group 0;" ::: "memory");  // copies past the end: their slots are staged anew
         if (!half) turn();
@@ -412,7 +442,7 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
 // Block (tile, y): parts [P y / gridDim.y, P (y + 1) / gridDim.y) of the tile's rows (scratch
 // non-null when there is more than one y).
 template <int D, int TC>
-__global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16 / TC) k_explain(const unsigned char *__restrict__ codes, int64_t n, ExplainJob job, float *__restrict__ phi, int64_t ldp,
+__global__ void __launch_bounds__(explain_threads(TC), kExplainWarps * 16 / TC) k_explain(const unsigned char *__restrict__ codes, int64_t n, ExplainJob job, float *__restrict__ phi, int64_t ldp,
               float *__restrict__ scratch) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P = explain_parts(job.T, D), y = blockIdx.y, Y = gridDim.y;
@@ -434,8 +464,9 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
     uint4 *block = reinterpret_cast<uint4 *>(smem_raw);
     const int t = blockIdx.x * kValueWarps + (tid >> 5), tt = min(t, job.T - 1);
     const uint2 *rec = reinterpret_cast<const uint2 *>(job.sa.unit) + (size_t)tt * UPT * 32;
-    const uint64_t *flags = reinterpret_cast<const uint64_t *>(job.image + (size_t)tt * image_bytes(D) + image_flags(D));
-    const uint64_t live = __ldg(flags), real = __ldg(flags + 2);
+    const unsigned char *chunk = job.image + (size_t)tt * image_bytes(D) + lane / chunk_units(D) * chunk_bytes(D);
+    const uint32_t flags =
+        lane < UPT ? __ldg(reinterpret_cast<const uint32_t *>(chunk + chunk_flags(D)) + lane % chunk_units(D)) : 0u;
     const uint4 *src = reinterpret_cast<const uint4 *>(codes) + (size_t)blockIdx.y * quads;
     uint2 node = __ldg(rec + lane);
     early_launch();
@@ -456,11 +487,12 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
 #pragma unroll
         for (int k = 0; k < (GS + 3) / 4; ++k) lm[k] = __ldg(job.lines + (size_t)t * LW + u * (GS / 4) + k);
         UnitSlots<D> v;
-        gather_unit<D>(job.sfold, job.T, t, u, (uint32_t)(live >> (u * GS)), lm, w, topw, v);
+        const uint32_t unit_flags = __shfl_sync(0xFFFFFFFFu, flags, u);
+        gather_unit<D>(job.sfold, job.T, t, u, unit_flags, lm, w, topw, v);
         if (u + 1 < UPT) node = __ldg(rec + (u + 1) * 32 + lane);
         float up[GS > 1 ? GS - 1 : 1];
         unit_sums<D>(v, u, up, top);
-        const uint32_t some = (uint32_t)(real >> (u * (GL / 8)));
+        const uint32_t some = unit_flags >> 16;
         float *dst = out + (size_t)u * GL * 32;
 #pragma unroll
         for (int b = 0; b < GL / 8; ++b) {
@@ -487,7 +519,7 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
 // batches of any size up to its capacity.  Which block computes a tile does not change any
 // row's arithmetic, nor do the groups: parts are always added in their order.
 template <int D, int TC>
-__global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16 / TC) k_explain_batch(const ExplainJob *__restrict__ jobs,
+__global__ void __launch_bounds__(explain_threads(TC), kExplainWarps * 16 / TC) k_explain_batch(const ExplainJob *__restrict__ jobs,
                                                          const BatchRequest *__restrict__ reqs,
                                                          const int4 *__restrict__ items, int *n_items) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -527,6 +559,14 @@ __global__ void __launch_bounds__(explain_threads(TC), ExplainCfg<D>::WARPS * 16
     }
 }
 
+// The part of an SM's memory that a kernel's blocks want (228 KB in all).
+template <class K>
+cudaError_t set_carveout(K kern, int D, int tile_rows, size_t smem) {
+    const int percent = explain_carveout(D, tile_rows, smem) ? (int)(100 * (kExplainCarveout >> 10) / 228 + 1)
+                                                             : cudaSharedmemCarveoutDefault;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
+}
+
 template <int D, int TC>
 cudaError_t explain_t(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi, int64_t ldp,
                       int splits, float *scratch, const DevInfo &dev, cudaStream_t st) {
@@ -534,6 +574,7 @@ cudaError_t explain_t(const unsigned char *codes, int64_t n, const ExplainJob &j
     if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
     auto kern = k_explain<D, TC>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (err == cudaSuccess) err = set_carveout(kern, D, TC, smem);
     if (err != cudaSuccess) return err;
     const int64_t blocks = (n + TC - 1) / TC;
     kern<<<dim3((unsigned)blocks, (unsigned)splits), explain_threads(TC), smem, st>>>(codes, n, job, phi, ldp, scratch);
@@ -563,12 +604,9 @@ cudaError_t batch_t(const ExplainJob *jobs, const BatchRequest *reqs, const int4
     auto kern = k_explain_batch<D, TC>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    if (grid <= 0) {
-        int per_sm = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, explain_threads(TC), smem);
-        if (err != cudaSuccess) return err;
-        grid = dev.sms * (per_sm > 0 ? per_sm : 1);
-    }
+    if (err == cudaSuccess) err = set_carveout(kern, D, TC, smem);
+    if (err != cudaSuccess) return err;
+    if (grid <= 0) grid = dev.sms * explain_blocks_per_sm(D, F_max, q_max, TC, dev);
     kern<<<grid, explain_threads(TC), smem, st>>>(jobs, reqs, items, n_items);
     count_launches(1);
     return cudaGetLastError();

@@ -145,16 +145,27 @@ WDF_HD inline int flush_node(int D, int i) {
 
 static_assert(flush_batches(8) <= 64, "batch flags are one 64-bit word per tree");
 
-// Everything of a tree that the consumer kernel stages, but its line maps, as one block of
-// 16-byte words (copied asynchronously, no registers): the unit nodes; live, flush and real
-// flags; the phi offset (feature x row stride of the phi tile) of every flush position, 16
-// bits; per batch the positions whose feature an earlier position of the batch has (0xFF when
-// they repeat among themselves).  The offsets depend on the tile's rows, so an ensemble has
-// an image of its trees for every tile size.
-WDF_HD constexpr int image_flags(int D) { return units_per_tree(D) * 32 * (int)sizeof(UnitNode); }
-WDF_HD constexpr int image_offsets(int D) { return image_flags(D) + 32; }
-WDF_HD constexpr int image_repeats(int D) { return image_offsets(D) + flush_len(D) * 2; }
-WDF_HD constexpr int image_bytes(int D) { return (image_repeats(D) + flush_batches(D) + 15) & ~15; }
+// Everything of a tree that the consumer kernel stages, but its line maps, as 16-byte words
+// (copied asynchronously, no registers), in chunks of a whole tree, at depth 8 of a unit: the units'
+// nodes; the phi offset (feature x row stride of the phi tile) of every flush position,
+// 16 bits; with several units those of the tree's last batch, the nodes above the units; per
+// unit a word of flags, live subtrees in bits 0-7, flush (no repeated feature) and real of its
+// batches and the last batch in bits 8-15 and 16-23; per batch the positions whose feature an
+// earlier position of the batch has (0xFF when they repeat among themselves).  After the
+// chunks, with several levels above the units, the nodes of those.  The offsets depend on the
+// tile's rows, so an ensemble has an image of its trees for every tile size.
+WDF_HD constexpr int chunk_units(int D) { return D == 8 ? 1 : units_per_tree(D); }
+WDF_HD constexpr int tree_chunks(int D) { return units_per_tree(D) / chunk_units(D); }
+WDF_HD constexpr int chunk_positions(int D) {
+    return chunk_units(D) * flush_group_len(D) + (units_per_tree(D) > 1 ? 8 : 0);
+}
+WDF_HD constexpr int chunk_offsets(int D) { return chunk_units(D) * 32 * (int)sizeof(UnitNode); }
+WDF_HD constexpr int chunk_flags(int D) { return chunk_offsets(D) + 2 * chunk_positions(D); }
+WDF_HD constexpr int chunk_repeats(int D) { return chunk_flags(D) + 4 * chunk_units(D); }
+WDF_HD constexpr int chunk_bytes(int D) { return (chunk_repeats(D) + chunk_positions(D) / 8 + 15) & ~15; }
+WDF_HD constexpr int image_top(int D) { return tree_chunks(D) * chunk_bytes(D); }
+WDF_HD constexpr int image_bytes(int D) { return image_top(D) + (unit_top(D) > 1 ? 8 * (int)sizeof(UnitNode) : 0); }
+static_assert(flush_group_len(8) / 8 < 8 && image_bytes(8) % 16 == 0, "chunk layout");
 // A row's phi is the sum of the sums of its ensemble's parts, in part order: part p of P holds
 // trees [T p / P, T (p + 1) / P), each part's nodes added in the consumer kernel's order from
 // zero.  The split depends on the ensemble alone, so a row's result does not depend on how
