@@ -145,15 +145,16 @@ wdf_status ensure_staging(wdf_ensemble *e, int64_t rows, bool out) {
     return WDF_OK;
 }
 
-// Rows per chunk of an explain call on host rows: an even number of equal chunks of about
-// 10 MB, so that the two streams' copies and kernels overlap from the first chunk to the last
-// and each chunk still fills the GPU; one chunk below 4 MB.  Rows of 127 floats, 1 / 2 / 4 / 8 /
-// 16 chunks: 150,001 rows and 150 trees of depth 5 1637 / 1299 / 1143 / 1126 / 1554 us, 60,000
-// rows and 400 trees 1203 / 1155 / 1061 / 1045 / 1323, 20,000 rows 334 / 271 / 299 / 348 / 366.
+// Rows per chunk of an explain call on host rows: two to eight equal chunks, an even number of
+// about 10 MB or more each, so that the two streams' copies and kernels overlap from the first
+// chunk to the last and each chunk still fills the GPU; one chunk below 4 MB.  Rows of 127
+// floats, 1 / 2 / 4 / 8 / 16 chunks: 150,001 rows and 150 trees of depth 5 1637 / 1299 / 1143 / 1126 /
+// 1554 us, 60,000 rows and 400 trees 1203 / 1155 / 1061 / 1045 / 1323, 20,000 rows 334 / 271 / 299 /
+// 348 / 366.
 int64_t explain_stage_rows(int64_t n, int F) {
     const double mb = 4e-6 * (double)n * F;
     if (mb < 4.0) return std::min(n, kStageRows);
-    const int64_t chunks = 2 * std::max<int64_t>(1, (int64_t)(mb / 20.0 + 0.5));
+    const int64_t chunks = 2 * std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(mb / 20.0 + 0.5)));
     const int64_t rows = (n + chunks - 1) / chunks;
     return std::min(kStageRows, (rows + 127) / 128 * 128);
 }
