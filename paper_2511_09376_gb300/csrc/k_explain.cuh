@@ -87,12 +87,15 @@ struct ExLayout {
 };
 
 // 16-byte and 32-byte read-only loads predicated on `on` (the outputs keep their values
-// when off): a dead bottom subtree issues no load.  (A branch around the loads makes the
+// when off): a dead bottom subtree issues no load.  Without a line of their own in the L1 cache
+// (one gather in four hits it at depth 6, one in twenty-five at depth 8) the gathers in flight
+// wait less for one: 233,472 rows, depth 5 to 8 1391 -> 1349, 1409 -> 1358, 2321 -> 2202, 2637 -> 2580 us
+// (200, 100, 80, 40 trees).  (A branch around the loads makes the
 // compiler wait for them at its end, and sending a dead subtree's rows to one entry costs the
 // eight wavefronts that return 32 bytes to 32 lanes.)
 __device__ __forceinline__ void ldg_f4_if(const void *p, float4 &r, uint32_t on) {
     asm volatile(
-        "{\n.reg .pred q;\nsetp.ne.u32 q, %5, 0;\n@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n}\n"
+        "{\n.reg .pred q;\nsetp.ne.u32 q, %5, 0;\n@q ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];\n}\n"
         : "+f"(r.x), "+f"(r.y), "+f"(r.z), "+f"(r.w)
         : "l"(p), "r"(on));
 }
@@ -100,7 +103,7 @@ __device__ __forceinline__ void ldg_f4_if(const void *p, float4 &r, uint32_t on)
 // One 32-byte vector in a single 256-bit load (the address is 32-byte aligned).
 __device__ __forceinline__ void ldg_f8_if(const void *p, float4 &a, float4 &b, uint32_t on) {
     asm volatile(
-        "{\n.reg .pred q;\nsetp.ne.u32 q, %9, 0;\n@q ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n}\n"
+        "{\n.reg .pred q;\nsetp.ne.u32 q, %9, 0;\n@q ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n}\n"
         : "+f"(a.x), "+f"(a.y), "+f"(a.z), "+f"(a.w), "+f"(b.x), "+f"(b.y), "+f"(b.z), "+f"(b.w)
         : "l"(p), "r"(on));
 }
@@ -207,7 +210,7 @@ __device__ __forceinline__ void gather_unit(const float *sfold, int T, int t, in
         if constexpr (Q == 2) ldg_f8_if(tf + j * (int)(S::E * EB) + at, v.v[j][0], v.v[j][Q - 1], on);
         else ldg_f4_if(tf + j * (int)(S::E * EB) + at, v.v[j][0], on);
         if (extra_slots(D))
-            asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v.x0[j]) : "l"(tx + j * (int)(S::E * 4) + at / 8));
+            asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v.x0[j]) : "l"(tx + j * (int)(S::E * 4) + at / 8));
         else
             v.x0[j] = 0.0f;
     }
@@ -298,7 +301,7 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
                 dst = (uint32_t)__cvta_generic_to_shared(above) + 16 * (lane - 28);
                 on = true;
             }
-            if (on) asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+            if (on) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
         }
         // the line maps: two words a unit (a tree has at least four)
         const uint32_t ldst = (uint32_t)__cvta_generic_to_shared(slot) + LINE;
@@ -306,7 +309,7 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         if (CU == 1) {
             if (lane == 24) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(ldst), "l"(lsrc) : "memory");
         } else if (lane < CU / 2) {
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(ldst + 16 * lane), "l"(lsrc + 4 * lane) : "memory");
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ldst + 16 * lane), "l"(lsrc + 4 * lane) : "memory");
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
