@@ -163,11 +163,12 @@ wdf_status wdf_set_metric(wdf_ensemble *ens, wdf_metric metric);
  * phi[c, i] for the n consumer rows C (leading dimension ldc) into phi (leading
  * dimension ldphi >= F): Algorithm 3 step 4 / Eq. "bg_shap_derivation" step (g).
  * C and phi live in the same memory kind.  WDF_EINVAL if no background was set.
- * Device kind: asynchronous; the rows' decision codes (one or two bytes per code column
- * and row, at most 2^20 rows at a time) live in a temporary stream-ordered allocation,
- * so calls on different streams never share scratch memory.  Host kind: copies
- * through the ensemble's device staging buffers and returns once phi is written on the
- * host.  phi of a row does not depend on the other rows of the call (the same
+ * Device kind: asynchronous; the rows' decision codes (four to twelve bits per code column
+ * and row, at most 2^20 rows at a time) and, for calls of few rows, node values (at most
+ * 320 MB) or partial sums live in a temporary stream-ordered allocation from the context's
+ * pool (which keeps up to 384 MB between calls), so calls on different streams never share
+ * scratch memory.  Host kind: copies through the ensemble's device staging buffers, in up
+ * to eight chunks, and returns once phi is written on the host.  phi of a row does not depend on the other rows of the call (the same
  * floating-point additions in the same order).
  */
 wdf_status wdf_explain(wdf_ensemble *ens, const float *C, int64_t n, int64_t ldc, wdf_memkind kind,
@@ -210,10 +211,11 @@ wdf_status wdf_global_attribution(wdf_ctx *ctx, const float *phi, int64_t n, int
  * Ragged batches (project addition; the paper runs one tree ensemble at a time).
  * A batch groups ensembles of one context -- any depths 2..8 and feature counts -- so a
  * single call explains many requests against them with ONE CUDA-graph launch: the graph
- * copies a packed work description (one memcpy) and runs, per depth class on parallel
- * branches, an encode kernel (the requests' decision codes into a device arena the
+ * copies a packed work description (one memcpy) and runs, per class (of one depth and about
+ * the same shared memory per block) on parallel branches, an encode kernel (the requests' decision codes into a device arena the
  * batch keeps and grows as needed) and a persistent consumer kernel over (ensemble,
- * request, tile of consumer rows) work items.  Per-row results equal those of
+ * request, tile of consumer rows, group of trees) work items (partial sums of up to
+ * 128 MB in scratch the batch keeps).  Per-row results equal those of
  * wdf_explain bit for bit.
  *
  * wdf_batch_create: the ensembles must outlive the batch; their backgrounds may be set
