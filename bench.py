@@ -352,7 +352,7 @@ def run_ours(args, rank, world, local_rank):
         "reduce_ms": ms - explain_ms - background_ms,
         "explain_only_rows_per_s": world * n / (explain_ms * 1e-3),
         "roofline": {
-            "kernel": f"k_explain<{info['depth']},64> alone (decisions, entries, gathers, phi accumulation): "
+            "kernel": f"k_explain<{info['depth']}> alone (decisions, entries, gathers, phi accumulation): "
                       f"{launches_per_call} launches per explain call of {n} rows, {kernel_launches} timed "
                       "with CUDA events on the call's stream (wdf_explain_timing)",
             "bound": "alu",
@@ -385,15 +385,15 @@ def run_ours(args, rank, world, local_rank):
             },
         },
         "roofline_background": {
-            "kernel": "set_background: k_encode_codes (on a side stream, overlapping) + k_bg_hist (patterns, "
-                      "joint counts) + the small per-leaf, line-map, contraction and fold kernels",
+            "kernel": "set_background: k_encode_slices (on a side stream, overlapping) + k_bg_count (decisions, "
+                      "joint counts on the tensor cores) + the small line-map, base-value and subset-sum kernels",
             "bound": "alu",
             "achieved": bg_ops * m / (background_ms * 1e-3) / 1e12,
             "peak": alu_peak_max,
             "unit": "Top/s",
             "frac": bg_ops * m / (background_ms * 1e-3) / 1e12 / alu_peak_max,
-            "traffic": profiled_traffic("k_bg_hist_large.md", BACKGROUND_SOURCES, m),
-            "limiter_ncu": profiled_limiter("k_bg_hist_large.md", BACKGROUND_SOURCES),
+            "traffic": profiled_traffic("k_bg_count_large.md", BACKGROUND_SOURCES, m),
+            "limiter_ncu": profiled_limiter("k_bg_count_large.md", BACKGROUND_SOURCES),
             "ops_per_row": {"compares": ops["compares"], "leaf_counts": info["n_live_leaves"], "ops": bg_ops},
             "hbm_gbs": B.nbytes / (background_ms * 1e-3) / 1e9,
         },

@@ -22,12 +22,13 @@
 // depends only on the ensemble, never on which rows share a block.
 //
 // Per row and depth-6 tree: about 13 32-byte gathers (four 128-byte lines per quarter warp) and
-// 50 phi read-modify-writes, some 430 L1 data-pipe wavefronts per warp and tree.  5.45 ms
-// per 486,400 rows and 200 trees of depth 6 (127 features), 546 SM clocks per warp and tree of
-// 32 rows (L1 pipe 78 %); with one warp per 32 rows 677 (two units' gathers in flight, ten
-// warps per SM), with two rows per thread 860 (five warps), and 624 for the kernel that
-// evaluated nodes one by one, lane = row.  Depth 5: 290, depth 7: 1220 (1940 with node-by-
-// node decisions), depth 8: 2620 (6350; slots in twelve floats, three loads per gather).
+// 50 phi read-modify-writes, some 430 L1 data-pipe wavefronts per warp and tree.  10.2 ms per 1M
+// rows and 200 trees of depth 6 (127 features), 515 SM clocks per warp and tree of 32 rows (L1
+// pipe 81 %), 546 while its gathers allocated in the L1 cache; of that form, one warp per 32
+// rows took 677 (two units' gathers in flight, ten warps per SM), two rows per thread 860 (five
+// warps), and 624 the kernel that evaluated nodes one by one, lane = row.  Depth 5: 280, depth 7:
+// 1170 (1940 with node-by-node decisions), depth 8: 2560 (6350; slots in twelve floats, three
+// loads per gather).
 //
 // The kernels are templates of the depth; every depth is instantiated in its own
 // translation unit so that they compile in parallel.
