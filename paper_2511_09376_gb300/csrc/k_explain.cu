@@ -108,47 +108,54 @@ __global__ void k_add_parts(const float *__restrict__ scratch, int P, int64_t n,
     phi[i / F * ldp + i % F] = x;
 }
 
-// phi from the node values of k_values: a warp adds one feature's nodes of 32 rows in their
-// order, a block takes eight features.  The node list is read 32 entries at a time and the
-// values 16 at a time, so their latency overlaps; only the additions are a chain.
+// phi from the node values of k_values: a warp adds one feature's nodes of one part and 32 rows in
+// their order, then a thread adds the parts in theirs.  part_warps (a power of two, at most
+// kSumWarps) warps per feature, so that a large ensemble's parts are summed side by side; the
+// node list is read 32 entries at a time and the values 16 at a time, so their latency
+// overlaps; only the additions are a chain.  777 rows, 500 trees of depth 7 and 112 features, the
+// whole call: 122 us with a warp per feature for all parts, 88 so.
 constexpr int kSumWarps = 8;
 __global__ void __launch_bounds__(32 * kSumWarps) k_sum_values(const float *__restrict__ values, int FL,
                                                               const int32_t *__restrict__ vlist,
                                                               const int32_t *__restrict__ voff, int T, int F, int P,
-                                                              int64_t n, float *__restrict__ phi, int64_t ldp) {
+                                                              int part_warps, int64_t n, float *__restrict__ phi,
+                                                              int64_t ldp) {
     __shared__ float out[32][kSumWarps + 1];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, f = blockIdx.x * kSumWarps + warp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, here = kSumWarps / part_warps;  // features of a block
+    const int f = blockIdx.x * here + warp / part_warps, p = warp % part_warps;
     const float *v = values + (size_t)blockIdx.y * T * FL * 32 + lane;
-    float total = 0.0f;
-    int off = f < F && lane <= P ? __ldg(voff + (size_t)f * P + lane) : 0;  // at most nine
+    const bool on = f < F && p < P;
+    const int off = on && lane < 2 ? __ldg(voff + (size_t)f * P + p + lane) : 0;
+    const int beg = __shfl_sync(0xFFFFFFFFu, off, 0), end = __shfl_sync(0xFFFFFFFFu, off, 1);
+    int mine = beg + lane < end ? __ldg(vlist + beg + lane) : 0;
     previous_done();  // the node values
-    if (f < F) {
-        for (int p = 0; p < P; ++p) {
-            const int beg = __shfl_sync(0xFFFFFFFFu, off, p), end = __shfl_sync(0xFFFFFFFFu, off, p + 1);
-            float acc = 0.0f;
-            for (int k0 = beg; k0 < end; k0 += 32) {
-                const int mine = k0 + lane < end ? __ldg(vlist + k0 + lane) : 0, cnt = min(32, end - k0);
+    float acc = 0.0f;
+    for (int k0 = beg; k0 < end; k0 += 32) {
+        const int cnt = min(32, end - k0), ahead = k0 + 32 + lane;
+        const int next = ahead < end ? __ldg(vlist + ahead) : 0;
 #pragma unroll
-                for (int h = 0; h < 32; h += 16) {
-                    float x[16];
+        for (int h = 0; h < 32; h += 16) {
+            float x[16];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const int i = __shfl_sync(0xFFFFFFFFu, mine, h + k);
-                        x[k] = h + k < cnt ? v[(size_t)i * 32] : 0.0f;
-                    }
-#pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        if (h + k < cnt) acc += x[k];
-                }
+            for (int k = 0; k < 16; ++k) {
+                const int i = __shfl_sync(0xFFFFFFFFu, mine, h + k);
+                x[k] = h + k < cnt ? v[(size_t)i * 32] : 0.0f;
             }
-            total = p == 0 ? acc : total + acc;
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (h + k < cnt) acc += x[k];
         }
+        mine = next;
     }
-    out[lane][warp] = total;
+    out[lane][warp] = acc;
     __syncthreads();
-    const int r = threadIdx.x / kSumWarps, c = threadIdx.x % kSumWarps, fc = blockIdx.x * kSumWarps + c;
+    const int r = threadIdx.x / kSumWarps, c = threadIdx.x % kSumWarps, fc = blockIdx.x * here + c;
     const int64_t row = (int64_t)blockIdx.y * 32 + r;
-    if (row < n && fc < F) phi[row * ldp + fc] = out[r][c];
+    if (c < here && row < n && fc < F) {
+        float total = out[r][c * part_warps];
+        for (int k = 1; k < P; ++k) total += out[r][c * part_warps + k];
+        phi[row * ldp + fc] = total;
+    }
 }
 
 template <int D>
@@ -156,9 +163,14 @@ static cudaError_t explain_values(const unsigned char *codes, int64_t n, const E
                                   float *values, const DevInfo &dev, cudaStream_t st) {
     cudaError_t err = values_t<D>(codes, n, job, values, dev, st);
     if (err != cudaSuccess) return err;
-    const dim3 grid((unsigned)((job.F + kSumWarps - 1) / kSumWarps), (unsigned)((n + 31) / 32));
+    const int P = explain_parts(job.T, D);
+    int part_warps = 1;
+    while (part_warps < P) part_warps *= 2;
+    static_assert(kSumWarps >= 8, "a warp per part");
+    const int here = kSumWarps / part_warps;
+    const dim3 grid((unsigned)((job.F + here - 1) / here), (unsigned)((n + 31) / 32));
     err = launch_dependent(k_sum_values, grid, 32 * kSumWarps, 0, st, (const float *)values, flush_len(D), job.vlist,
-                           job.voff, job.T, job.F, explain_parts(job.T, D), n, phi, ldp);
+                           job.voff, job.T, job.F, P, part_warps, n, phi, ldp);
     count_launches(1);
     return err != cudaSuccess ? err : cudaGetLastError();
 }
@@ -178,7 +190,8 @@ constexpr int64_t kValuesBytes = 320ll << 20;
 // Measured at 200 trees of depth 6, 127 features (node values / parts on blocks / one block a
 // tile): 1,000 rows 36 / 70 / 205 us, 2,000 rows 56 / 71, 4,000 rows 100 / 86, 8,000 rows 177 /
 // 121; 1000 trees of depth 8, 100 rows 236 / 728; 500 trees of depth 7, 777 rows 130 / 156 /
-// 1380; 50 trees of depth 4, 255 features, 20,000 rows 87 / 49.
+// 1380; 50 trees of depth 4, 255 features, 20,000 rows 87 / 49 (all before k_sum_values took its
+// parts side by side, which only moves the line further to where node values already win).
 static int explain_splits(int D, int64_t n, const ExplainJob &job, int tile_rows, const DevInfo &dev) {
     const int P = explain_parts(job.T, D);
     const int64_t per_sm = explain_blocks_per_sm(D, job.F, job.sa.quads, tile_rows, dev);
