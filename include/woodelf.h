@@ -108,7 +108,8 @@ wdf_status wdf_ensemble_info(const wdf_ensemble *ens, wdf_info *out);
  * 2) and their contraction (step 3), in the given precision.  B is not retained; its
  * decision codes pass through a buffer the ensemble keeps (up to 2^20 rows of codes).
  * Calls on one ensemble must not overlap on the GPU.
- * WDF_EUNSUPPORTED: m == 0 (an empty background is the path-dependent variant).
+ * WDF_EUNSUPPORTED: m == 0 (an empty background is the path-dependent variant), or more
+ * than 2^24 code columns (split features; one of more than 4095 thresholds takes several).
  * precision WDF_TF32X3 / WDF_BF16X3 / WDF_BF16X6 runs the contraction on the tensor cores (tcgen05,
  * TMEM accumulators) and then waits for the stream to check the kernel's bounded waits:
  * WDF_ETIMEOUT if one expired.  WDF_FP32 is stream-ordered without waiting; a later

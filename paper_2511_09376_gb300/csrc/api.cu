@@ -175,6 +175,14 @@ wdf_status ensure_codes(wdf_ensemble *e, int64_t rows, int nbuf) {
     return WDF_OK;
 }
 
+// A unit node names its code column in 24 bits (tree_layout.h), and the kernels index a row
+// block's quads, three per column at most, in 32.
+wdf_status check_columns(const wdf_ensemble *e) {
+    if ((int64_t)e->pk.scol.size() <= wdf::kMostColumns) return WDF_OK;
+    return fail(WDF_EUNSUPPORTED, "more than 2^24 code columns (split features, or features of more than 4095 "
+                                  "thresholds cut into several)");
+}
+
 // Counts of device rows B (m rows) added into hist: with more than one chunk of codes,
 // the encode of the next chunk overlaps the count of this one (two code buffers, the
 // side stream ist[0]).
@@ -518,6 +526,8 @@ wdf_status wdf_set_background(wdf_ensemble *ens, const float *B, int64_t m, int6
     if (kind != WDF_MEM_HOST && kind != WDF_MEM_DEVICE) return fail(WDF_EINVAL, "bad memory kind");
     if (!valid_precision(precision))
         return fail(WDF_EINVAL, "unknown precision");
+    const wdf_status cols = check_columns(ens);
+    if (cols != WDF_OK) return cols;
     DeviceGuard g(ens->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
     const wdf::Packed &p = ens->pk;
@@ -570,10 +580,10 @@ wdf_status wdf_background_counts(wdf_ensemble *ens, const float *B, int64_t m, i
     if (!B || !counts) return fail(WDF_EINVAL, "B and counts must be non-null");
     if (ldb < ens->pk.F) return fail(WDF_EINVAL, "ldb < n_features");
     if (m > (int64_t)0xFFFFFFFF) return fail(WDF_EUNSUPPORTED, "more than 2^32-1 background rows");
+    const wdf_status cols = check_columns(ens);
+    if (cols != WDF_OK) return cols;
     DeviceGuard g(ens->ctx->device);
     cudaStream_t st = (cudaStream_t)stream;
-    const wdf::Packed &p = ens->pk;
-    (void)p;
     return count_device_rows(ens, B, m, ldb, counts, st);
 }
 

@@ -93,8 +93,8 @@ struct SliceNode {
         for (int k = 0; k < 3; ++k) rank_masks(v.y, k, m[k]);
     }
     __device__ __forceinline__ uint32_t decide1(const uint4 *block, const SliceArrays &sa) const {
-        const int col = (int)(at & 0xFFFFu), nq = (int)((at >> 16) & 15u);
-        uint32_t w = 0u - ((at >> 20) & 1u);
+        const int col = unit_column(at), nq = unit_quads(at);
+        uint32_t w = 0u - unit_start(at);
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             if (k < nq) w = slice_le(w, block[sa.qbase[k] + col], m[k]);
@@ -102,8 +102,8 @@ struct SliceNode {
     }
     template <int N>
     __device__ __forceinline__ void decide(const uint4 *tile, const SliceArrays &sa, uint32_t (&w)[N]) const {
-        const int col = (int)(at & 0xFFFFu), nq = (int)((at >> 16) & 15u);
-        const uint32_t le0 = 0u - ((at >> 20) & 1u);
+        const int col = unit_column(at), nq = unit_quads(at);
+        const uint32_t le0 = 0u - unit_start(at);
 #pragma unroll
         for (int b = 0; b < N; ++b) w[b] = le0;
 #pragma unroll

@@ -161,10 +161,10 @@ void build_records(Packed *pp) {
             if (v < 0) continue;
             UnitNode &n = p.unit[(size_t)t * U * 32 + i];
             if (feat[v] == F) {
-                n.at = 1u << 20;  // pass-through: always left
+                n.at = unit_at(0u, 0u, 1u);  // pass-through: always left
             } else if (tc[v] >= 0) {
                 const int levels = p.spack[(size_t)(tc[v] / 8)].levels;
-                n.at = (uint32_t)tc[v] | ((uint32_t)((levels + 3) / 4) << 16) | (1u << 20);
+                n.at = unit_at((uint32_t)tc[v], (uint32_t)((levels + 3) / 4), 1u);  // at most kMostColumns: api.cu
                 for (int b = 0; b < kSliceBits; ++b)
                     if ((tr[v] >> b) & 1) n.rank |= (0x80u >> (b / 4)) << (8 * (b % 4));
             }  // a NaN threshold: never left

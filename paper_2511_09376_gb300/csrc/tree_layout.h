@@ -52,10 +52,18 @@ constexpr int kSliceGroupFloats = 16384;  // most thresholds of an encoding grou
 
 // A lane's node of a unit: its column and the rank it compares with.
 struct UnitNode {
-    uint32_t at;    // column index | quads << 16 (0: none to read) | start << 20 (the comparison's start: 1 when
-                    // a code equal to the rank goes left; without quads it is the decision itself)
+    uint32_t at;    // unit_at: column index | quads << 24 (0: none to read) | start << 28 (the comparison's start:
+                    // 1 when a code equal to the rank goes left; without quads it is the decision itself)
     uint32_t rank;  // bit 7 - k of byte b is bit 4k + b of the rank
 };
+// Columns that a node can name; an ensemble with more of them cannot be counted or explained.
+constexpr int64_t kMostColumns = (int64_t)1 << 24;
+WDF_HD constexpr uint32_t unit_at(uint32_t column, uint32_t quads, uint32_t start) {
+    return column | quads << 24 | start << 28;
+}
+WDF_HD constexpr int unit_column(uint32_t at) { return (int)(at & (uint32_t)(kMostColumns - 1)); }
+WDF_HD constexpr int unit_quads(uint32_t at) { return (int)((at >> 24) & 15u); }
+WDF_HD constexpr uint32_t unit_start(uint32_t at) { return (at >> 28) & 1u; }
 // One column of a pack: its feature and its number of thresholds (the code of a NaN).
 struct SliceCol {
     int32_t feature, count;

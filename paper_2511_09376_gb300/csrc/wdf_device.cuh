@@ -130,8 +130,8 @@ __device__ __forceinline__ uint32_t slice_le(uint32_t le, const uint4 &q, const 
 
 // Decisions of a unit node for the 32 rows of a code block (quads at `block`).
 __device__ __forceinline__ uint32_t unit_decide(const uint2 &node, const uint4 *block, const SliceArrays &sa) {
-    const int col = (int)(node.x & 0xFFFFu), nq = (int)((node.x >> 16) & 15u);
-    uint32_t le = 0u - ((node.x >> 20) & 1u), m[4];
+    const int col = unit_column(node.x), nq = unit_quads(node.x);
+    uint32_t le = 0u - unit_start(node.x), m[4];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         if (k < nq) {
