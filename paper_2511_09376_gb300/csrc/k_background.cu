@@ -287,7 +287,7 @@ static cudaError_t bg_count_t(const unsigned char *codes, int64_t m, const Slice
     }
     const int chunks = (units + best_w - 1) / best_w;
     auto kern = k_bg_count<D, STAGES, SUB>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(best_w));
+    cudaError_t err = allow_shared(kern, smem(best_w), dev);
     if (err != cudaSuccess) return err;
     kern<<<(unsigned)(best_slices * chunks), 32 * best_w, smem(best_w), st>>>(codes, m, sa, meta, units, chunks, hist);
     count_launches(1);
@@ -427,7 +427,7 @@ static cudaError_t bg_add_t(const unsigned char *codes, int64_t m, const SliceAr
     }
     const size_t smem = (size_t)STAGES * sa.quads * 64 + (size_t)W * Unit<D>::NSU * Shape<D>::E * 4;
     auto kern = k_bg_add<D, STAGES>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_shared(kern, smem, dev);
     if (err != cudaSuccess) return err;
     kern<<<(unsigned)(slices * chunks), 64 * W, smem, st>>>(codes, m, sa, meta, units, chunks, hist);
     count_launches(1);

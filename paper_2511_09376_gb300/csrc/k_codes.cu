@@ -125,8 +125,7 @@ int encode_batch_grid(int max_group_thr, const DevInfo &dev) {
 cudaError_t launch_encode_batch(const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items,
                                 const int *n_items, int max_group_thr, const DevInfo &dev, cudaStream_t st) {
     const size_t smem = slice_smem(max_group_thr);
-    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
-    cudaError_t err = cudaFuncSetAttribute(k_encode_batch, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_shared(k_encode_batch, smem, dev);
     if (err != cudaSuccess) return err;
     k_encode_batch<<<encode_batch_grid(max_group_thr, dev), kSliceThreads, smem, st>>>(jobs, reqs, items, n_items);
     count_launches(1);
@@ -138,8 +137,7 @@ cudaError_t launch_encode_slices(const float *X, int64_t rows, int64_t ldx, cons
     const int64_t blocks = rows_pad / 32;
     if (blocks == 0) return cudaSuccess;
     const size_t smem = slice_smem(sa.max_group_thr);
-    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
-    cudaError_t err = cudaFuncSetAttribute(k_encode_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_shared(k_encode_slices, smem, dev);
     if (err != cudaSuccess) return err;
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(3, dev.smem_optin / (smem + 1024)));
     const int64_t fill = std::max<int64_t>(1, (int64_t)dev.sms * per_sm / sa.n_groups);

@@ -395,7 +395,10 @@ cudaError_t launch_contract_tc(int D, int mode, const float *A, const float *sca
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     auto kern = mode == 0 ? k_contract_tc<false, 2> : (mode == 1 ? k_contract_tc<true, 2> : k_contract_tc<true, 3>);
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem);
+    // the kernel serves all depths: one limit for them all, whichever host thread sets it
+    size_t most = 0;
+    for (int d = 2; d <= 8; ++d) most = std::max(most, tc_geom(d, mode).smem);
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
     const uint32_t first = g_first_wait_limit.load();
     kern<<<(unsigned)((int64_t)n_tiles * g.NB), 128, g.smem, st>>>(D, apk, bpk, scale, tiles, S, g.NT, g.NB, g.nk, g.ring, err,

@@ -522,6 +522,7 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
 // the tail.  The item count n_items[0] is read from device memory, so one captured graph serves
 // batches of any size up to its capacity.  Which block computes a tile does not change any
 // row's arithmetic, nor do the groups: parts are always added in their order.
+constexpr size_t kBatchShared = 16;  // room for the two words below
 template <int D, int TC>
 __global__ void __launch_bounds__(explain_threads(TC), kExplainWarps * 16 / TC) k_explain_batch(const ExplainJob *__restrict__ jobs,
                                                          const BatchRequest *__restrict__ reqs,
@@ -575,9 +576,8 @@ template <int D, int TC>
 cudaError_t explain_t(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi, int64_t ldp,
                       int splits, float *scratch, const DevInfo &dev, cudaStream_t st) {
     const size_t smem = ExLayout<D>(job.F, job.sa.quads, TC).total;
-    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
     auto kern = k_explain<D, TC>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_shared(kern, smem, dev);
     if (err == cudaSuccess) err = set_carveout(kern, D, TC, smem);
     if (err != cudaSuccess) return err;
     const int64_t blocks = (n + TC - 1) / TC;
@@ -590,9 +590,8 @@ template <int D>
 cudaError_t values_t(const unsigned char *codes, int64_t n, const ExplainJob &job, float *values, const DevInfo &dev,
                      cudaStream_t st) {
     const size_t smem = (size_t)job.sa.quads * 16;
-    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
     auto kern = k_values<D>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = allow_shared(kern, smem, dev);
     if (err != cudaSuccess) return err;
     const dim3 grid((unsigned)((job.T + kValueWarps - 1) / kValueWarps), (unsigned)((n + 31) / 32));
     err = launch_dependent(kern, grid, 32 * kValueWarps, smem, st, codes, job, values);
@@ -604,10 +603,8 @@ template <int D, int TC>
 cudaError_t batch_t(const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items, int *n_items, int F_max,
                     int q_max, int grid, const DevInfo &dev, cudaStream_t st) {
     const size_t smem = ExLayout<D>(F_max, q_max, TC).total;
-    if (smem > dev.smem_optin) return cudaErrorInvalidConfiguration;
     auto kern = k_explain_batch<D, TC>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
+    cudaError_t err = allow_shared(kern, smem, dev, kBatchShared);
     if (err == cudaSuccess) err = set_carveout(kern, D, TC, smem);
     if (err != cudaSuccess) return err;
     if (grid <= 0) grid = dev.sms * explain_blocks_per_sm(D, F_max, q_max, TC, dev);

@@ -522,7 +522,7 @@ static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const Tre
                 count_launches(2);
             }
             auto kern = fb ? k_explain_iv_fold<D, SMEM, true> : k_explain_iv_fold<D, SMEM, false>;
-            err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            err = allow_shared(kern, smem, dev);
             if (err == cudaSuccess)
                 err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIvThreads, smem);
             if (err != cudaSuccess) return err;
@@ -533,7 +533,7 @@ static cudaError_t iv_t(const float *C, int64_t n, int64_t ldc, int F, const Tre
     }
     if (!done) {
         auto kern = k_explain_iv<D, SMEM>;
-        err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        err = allow_shared(kern, smem, dev);
         if (err == cudaSuccess) err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kIvThreads, smem);
         if (err != cudaSuccess) return err;
         const int64_t grid = std::min<int64_t>(cap, (int64_t)dev.sms * std::max(per_sm, 1));

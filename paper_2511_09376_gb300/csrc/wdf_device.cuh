@@ -57,6 +57,16 @@ __device__ __forceinline__ void subtree_entries(const uint32_t (&dw)[Shape<D>::N
     }
 }
 
+// Lets blocks of a kernel take smem bytes of dynamic shared memory beside `fixed` of its own.  The
+// limit belongs to the kernel, not to the launch, so every caller sets the same one, all that
+// a block may have: with each call's own size, host threads in calls on different ensembles
+// lowered it under one another between setting it and launching.
+template <class K>
+inline cudaError_t allow_shared(K kern, size_t smem, const DevInfo &dev, size_t fixed = 0) {
+    if (smem + fixed > dev.smem_optin) return cudaErrorInvalidConfiguration;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(dev.smem_optin - fixed));
+}
+
 // Dependent launches (launch_dependent): early lets the next kernel's blocks start once all blocks
 // of this one are under way; previous_done waits for the kernel before, whose results the
 // next loads may read.
