@@ -165,10 +165,10 @@ wdf_status wdf_set_metric(wdf_ensemble *ens, wdf_metric metric);
  * dimension ldphi >= F): Algorithm 3 step 4 / Eq. "bg_shap_derivation" step (g).
  * C and phi live in the same memory kind.  WDF_EINVAL if no background was set.
  * Device kind: asynchronous; the rows' decision codes (four to twelve bits per code column
- * and row, at most 2^20 rows at a time) and, for calls of few rows, node values (at most
- * 320 MB) or partial sums live in a temporary stream-ordered allocation from the context's
- * pool (which keeps up to 384 MB between calls), so calls on different streams never share
- * scratch memory.  Host kind: copies through the ensemble's device staging buffers, in up
+ * and row, at most 2^20 rows at a time) and, where they make the call faster, node values or
+ * partial sums (at most 320 MB; a call that cannot have them runs without) live in a
+ * temporary stream-ordered allocation from the context's pool (which keeps up to 384 MB
+ * between calls), so calls on different streams never share scratch memory.  Host kind: copies through the ensemble's device staging buffers, in up
  * to eight chunks, and returns once phi is written on the host.  phi of a row does not depend on the other rows of the call (the same
  * floating-point additions in the same order).
  */

@@ -168,10 +168,11 @@ void plan_groups(const wdf_batch *b, const std::vector<int> &tile_rows, std::vec
     }
 }
 
-// Scratch for the planned parts, grown like the code arena.
-wdf_status place_parts(wdf_batch *b, const std::vector<Req> &reqs) {
+// Scratch for the planned parts, grown like the code arena.  Without memory for it the call
+// runs with whole tiles.
+wdf_status place_parts(wdf_batch *b, std::vector<Req> *reqs) {
     size_t total = 0;
-    for (const Req &r : reqs) {
+    for (const Req &r : *reqs) {
         const wdf::Packed &p = b->ens[(size_t)r.e]->pk;
         if (r.groups > 1)
             total = r.parts_off + (size_t)wdf::explain_parts(p.T, p.D) * (size_t)r.n * (size_t)p.F * sizeof(float);
@@ -184,7 +185,14 @@ wdf_status place_parts(wdf_batch *b, const std::vector<Req> &reqs) {
         b->d_parts = nullptr;
         b->parts_cap = 0;
         const size_t cap = std::min(std::max<size_t>(total + total / 2, 1 << 20), kPartsBytes);
-        WDF_CUDA(cudaMalloc((void **)&b->d_parts, cap));
+        const cudaError_t e = cudaMalloc((void **)&b->d_parts, cap);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            b->d_parts = nullptr;
+            for (Req &r : *reqs) r.groups = 1;
+            return WDF_OK;
+        }
+        WDF_CUDA(e);
         b->parts_cap = cap;
     }
     return WDF_OK;
@@ -466,7 +474,7 @@ wdf_status wdf_batch_explain(wdf_batch *b, int32_t n_requests, const int32_t *en
     count_needs(b, reqs, tiles, &need_reqs, &need_items, &need_eitems, &need_tiles);
     s = ensure_blob(b, need_reqs, need_items, need_eitems, need_tiles);
     if (s == WDF_OK) s = place_codes(b, &reqs);
-    if (s == WDF_OK) s = place_parts(b, reqs);
+    if (s == WDF_OK) s = place_parts(b, &reqs);
     if (s == WDF_OK) s = wait_copied(b);
     if (s == WDF_OK) {
         for (size_t c = 0; c < b->cls.size(); ++c) fill_class(b, (int)c, reqs, b->cls[c].tile_rows);
@@ -557,7 +565,7 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
             std::vector<int> tiles;
             for (const Cls &o : b->cls) tiles.push_back(&o == &k ? tc : o.tile_rows);
             plan_groups(b, tiles, &reqs);
-            s = place_parts(b, reqs);
+            s = place_parts(b, &reqs);
             if (s != WDF_OK) break;
             fill_class(b, (int)c, reqs, tc);
             cudaError_t e = cudaMemcpyAsync(b->d_blob, b->h_blob, b->blob_bytes, cudaMemcpyHostToDevice, st);

@@ -5,6 +5,7 @@
 #include <utility>
 #include <vector>
 
+#include "explain_plan.h"
 #include "k_explain.cuh"
 
 namespace wdf {
@@ -178,44 +179,6 @@ static cudaError_t explain_values(const unsigned char *codes, int64_t n, const E
 // Rows per encoded chunk: the decision codes of a chunk live in a stream-ordered
 // scratch allocation (so concurrent calls on other streams never share it).
 constexpr int64_t kExplainChunkRows = 1 << 20;
-// Most scratch of the node values; the context's pool keeps as much between calls.
-constexpr int64_t kValuesBytes = 320ll << 20;
-
-// How a call is spread over the GPU: splits = 0: node values (k_values, k_sum_values), else the
-// tile kernel with its tiles' parts on that many blocks.  The least of estimated microseconds:
-//  - tile kernel: its waves of resident blocks times a tile's walk of its trees, 0.034 us per
-//    tree and leaf position at full occupancy, down to half of it with a block to itself;
-//    split, the parts' sums are written and read once more;
-//  - node values: 1.4 ps (depth 8: 2.2) per row and flush position, 8 ps per row and feature.
-// Measured at 200 trees of depth 6, 127 features (node values / parts on blocks / one block a
-// tile): 1,000 rows 36 / 70 / 205 us, 2,000 rows 56 / 71, 4,000 rows 100 / 86, 8,000 rows 177 /
-// 121; 1000 trees of depth 8, 100 rows 236 / 728; 500 trees of depth 7, 777 rows 130 / 156 /
-// 1380; 50 trees of depth 4, 255 features, 20,000 rows 87 / 49 (all before k_sum_values took its
-// parts side by side, which only moves the line further to where node values already win).
-static int explain_splits(int D, int64_t n, const ExplainJob &job, int tile_rows, const DevInfo &dev) {
-    const int P = explain_parts(job.T, D);
-    const int64_t per_sm = explain_blocks_per_sm(D, job.F, job.sa.quads, tile_rows, dev);
-    const int64_t tiles = (n + tile_rows - 1) / tile_rows, room = (int64_t)dev.sms * per_sm;
-    const double walk = 0.034 * job.T * (1 << D);
-    int best = 1;
-    double least = 0.0;
-    for (int s = 1; s <= P; ++s) {
-        const double full = (double)(tiles * s) / (double)room;
-        const double waves = (double)((tiles * s + room - 1) / room) * ((P + s - 1) / s) / P;
-        const double cost = 15.0 + waves * walk * (full < 1.0 ? 0.5 + 0.5 * full : 1.0) +
-                            (s > 1 ? 4.0 + 2e-6 * (double)P * (double)n * job.F : 0.0);
-        if (s == 1 || cost < least) {
-            best = s;
-            least = cost;
-        }
-    }
-    const int64_t rows = (n + 31) / 32 * 32, positions = (int64_t)job.T * flush_len(D);
-    if (rows * positions <= kValuesBytes / (int64_t)sizeof(float)) {
-        const double cost = 20.0 + (double)rows * ((D == 8 ? 2.2e-6 : 1.4e-6) * (double)positions + 8e-6 * job.F);
-        if (cost < least) best = 0;
-    }
-    return best;
-}
 
 cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const ExplainJob &job, float *phi,
                            int64_t ldp, int tile_rows, const DevInfo &dev, cudaStream_t st) {
@@ -226,16 +189,17 @@ cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const 
     const int64_t chunk = std::min(n, kExplainChunkRows);
     const int64_t pad = 128;  // every tile size divides it
     const size_t code_bytes = (size_t)((chunk + pad - 1) / pad * pad) / 32 * job.sa.quads * 16;
-    const int splits = explain_splits(D, chunk, job, tile_rows, dev);
-    const bool values = splits == 0;  // then one chunk
-    const size_t scratch_floats = values ? (size_t)((n + 31) / 32 * 32) * job.T * flush_len(D)
-                                         : (splits > 1 ? (size_t)explain_parts(job.T, D) * chunk * job.F : 0);
-    const size_t at = (code_bytes + 255) & ~(size_t)255;
+    ExplainPlan plan = explain_plan(D, chunk, job.T, job.F, tile_rows, dev.sms,
+                                    explain_blocks_per_sm(D, job.F, job.sa.quads, tile_rows, dev));
     unsigned char *codes = nullptr;
-    cudaError_t err =
-        cudaMallocFromPoolAsync(reinterpret_cast<void **>(&codes), at + scratch_floats * sizeof(float), dev.pool, st);
+    cudaError_t err = take_scratch(&plan, chunk, code_bytes, cudaErrorMemoryAllocation, [&](size_t bytes) {
+        const cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&codes), bytes, dev.pool, st);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();  // reported by its return value alone
+        return e;
+    });
     if (err != cudaSuccess) return err;
-    float *scratch = scratch_floats ? reinterpret_cast<float *>(codes + at) : nullptr;
+    const int splits = plan.splits;
+    float *scratch = plan.scratch_floats ? reinterpret_cast<float *>(codes + scratch_at(code_bytes)) : nullptr;
     for (int64_t r0 = 0; r0 < n && err == cudaSuccess; r0 += chunk) {
         const int64_t rows = std::min(chunk, n - r0);
         err = launch_encode_slices(C + r0 * ldc, rows, ldc, job.sa, (rows + pad - 1) / pad * pad, codes, dev, st);
@@ -253,21 +217,26 @@ cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const 
                 }
             }
         }
-        switch (D) {
-#define WDF_EXPLAIN_CASE(d)                                                                                       \
-    case d:                                                                                                       \
-        err = values ? explain_values<d>(codes, rows, job, out, ldp, scratch, dev, st)                            \
-                     : explain_depth<d>(codes, rows, job, out, ldp, tile_rows, splits, scratch, dev, st);         \
+        for (int64_t q0 = 0; q0 < rows && err == cudaSuccess; q0 += plan.rows) {
+            const int64_t here = std::min(plan.rows, rows - q0);
+            const unsigned char *block = codes + (size_t)(q0 / 32) * job.sa.quads * 16;
+            float *to = out + q0 * ldp;
+            switch (D) {
+#define WDF_EXPLAIN_CASE(d)                                                                                     \
+    case d:                                                                                                     \
+        err = splits == 0 ? explain_values<d>(block, here, job, to, ldp, scratch, dev, st)                      \
+                          : explain_depth<d>(block, here, job, to, ldp, tile_rows, splits, scratch, dev, st);   \
         break;
-            WDF_EXPLAIN_CASE(2) WDF_EXPLAIN_CASE(3) WDF_EXPLAIN_CASE(4) WDF_EXPLAIN_CASE(5)
-            WDF_EXPLAIN_CASE(6) WDF_EXPLAIN_CASE(7) WDF_EXPLAIN_CASE(8)
+                WDF_EXPLAIN_CASE(2) WDF_EXPLAIN_CASE(3) WDF_EXPLAIN_CASE(4) WDF_EXPLAIN_CASE(5)
+                WDF_EXPLAIN_CASE(6) WDF_EXPLAIN_CASE(7) WDF_EXPLAIN_CASE(8)
 #undef WDF_EXPLAIN_CASE
-        }
-        if (err == cudaSuccess && splits > 1) {
-            k_add_parts<<<(unsigned)((rows * job.F + 255) / 256), 256, 0, st>>>(scratch, explain_parts(job.T, D), rows,
-                                                                               job.F, out, ldp);
-            count_launches(1);
-            err = cudaGetLastError();
+            }
+            if (err == cudaSuccess && splits > 1) {
+                k_add_parts<<<(unsigned)((here * job.F + 255) / 256), 256, 0, st>>>(
+                    scratch, explain_parts(job.T, D), here, job.F, to, ldp);
+                count_launches(1);
+                err = cudaGetLastError();
+            }
         }
         if (ev1) {  // the pair is kept only once both ends are recorded
             std::lock_guard<std::mutex> lk(g_tmu);
