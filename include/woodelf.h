@@ -200,9 +200,10 @@ wdf_status wdf_expected_value(const wdf_ensemble *ens, double *out, void *stream
  * (1/n) sum_c |phi[c,i]| and mean[i] = (1/n) sum_c phi[c,i], accumulated in FP64 in a
  * fixed order (the paper's global attribution combines many local attributions,
  * section "Introduction"), so the result does not depend on scheduling.  With packed
- * rows (ldphi == n_features <= 512, 16-byte aligned phi) short runs of 8 values are
- * first summed as exact-error FP32 pairs (TwoSum; within 2^-42 of the run's exact sum)
- * and each pair is then added in FP64.  mean_abs and mean are device arrays of F
+ * rows (ldphi == n_features <= 512, 16-byte aligned phi) a thread's elements are summed in
+ * FP32 parts that lose nothing an FP64 sum keeps (runs of 16 within 2^-57 of their largest
+ * element, the runs' sums in three FP32) and added in FP64 after that; elements of 2^123 and
+ * more, infinities and NaN in FP64 from the start.  mean_abs and mean are device arrays of F
  * doubles.  Asynchronous.
  */
 wdf_status wdf_global_attribution(wdf_ctx *ctx, const float *phi, int64_t n, int64_t ldphi, int32_t n_features,

@@ -2,7 +2,7 @@
 // accumulated in FP64 (the paper's global attribution combines many local
 // attributions, section "Introduction").  Two passes with a fixed summation order, so
 // the result does not depend on scheduling: row blocks write FP64 partial sums, then
-// one thread per feature adds the partials in block order.
+// 32 threads per feature add them.
 #include <algorithm>
 #include <cstdint>
 
@@ -66,22 +66,26 @@ __global__ void __launch_bounds__(256) k_colsum_partial(const float *__restrict_
 //
 // FP64 adds and conversions run at two a clock and SM on this GPU, so the sums stay in FP32
 // without giving up FP64 results:
-//  - A run of kRun elements of a column is cut at a common power of two: with 2^e the largest
-//    magnitude's binade and M = 1.5 * 2^(e + log2 kRun), q = (x + M) - M is x rounded to a
-//    multiple of 2^(e + log2 kRun - 23), so the run's sum of q (and of |q|) is exact; the rest
-//    r = x - q is exact too and below 2^-20 of the largest, and its plain sum is within about
-//    2^-42 of the run's, relative to the largest element.  r carries x's sign into the sum of
-//    magnitudes.  Seven adds per element and both sums, where an error-free addition per
-//    element takes fourteen.
-//  - The run's two parts go into a thread's sum of three FP32 (h + m + l by error-free
+//  - A run of kRun elements of a column is cut twice at common powers of two.  With 2^e the
+//    largest magnitude's binade and M = 1.5 * 2^(e + 4), q = (x + M) - M is x rounded to a
+//    multiple of 2^(e - 19), so the run's sum of q (and of |q|) is exact.  The rest r = x - q is
+//    exact too and at most 2^(e - 20); cut the same way at multiples of 2^(e - 40) its sum is
+//    exact as well.  What is then left of an element is exact, at most 2^(e - 41), and zero for all
+//    elements of 2^(e - 17) and more; its plain sum is within 2^(e - 57) of the run's (15
+//    additions of partial sums of at most 2^(e - 37), each off by at most 2^-24 of its result).
+//    q and the rests carry x's sign into the sum of magnitudes.
+//  - The run's three parts go into a thread's sum of three FP32 (h + m + l by error-free
 //    TwoSum, the last plain), some 2^-60 of it, and that into FP64 once per thread.
+// So a thread's sum is FP64's but for its last rounding.  (With one cut and a plain sum of r, one
+// large element and fifteen just below 2^-20 of it were 6e-14 of the mean off.)
 // Elements of 2^123 and more, infinities and NaN take plain FP64 sums over the thread's
 // elements instead (nothing above is exact for them).
-// Bound by reading phi: 1,000,000 x 127 (508 MB) in 80 us, 6.3 TB/s; it was 350 us with two
-// FP64 adds per eight elements and sum, and 1.6 waves of blocks.  Two blocks of 254 threads
-// per SM keep 130 KB of loads in flight, so one wave of 304 blocks is enough.
+// Bound by reading phi: 1,000,000 x 127 (508 MB), the whole call: 94 us (5.4 TB/s), 88 with one cut,
+// 380 with two FP64 adds per eight elements and sum and 1.6 waves of blocks.  Two blocks of 254
+// threads per SM keep 130 KB of loads in flight, so one wave of 304 blocks is enough.
 constexpr int kRun = 16;
-constexpr uint32_t kRunShift = 4;  // log2 kRun
+constexpr uint32_t kRunShift = 4;    // log2 kRun
+constexpr uint32_t kRestShift = 17;  // the second cut's M: 1.5 * 2^(e - 17) (below 2^-109 of FP32's range every r is cut to itself)
 
 struct Sum3 {
     float h = 0.0f, m = 0.0f, l = 0.0f;
@@ -91,9 +95,10 @@ struct Sum3 {
         s = t;
         return e;
     }
-    __device__ __forceinline__ void add(float q, float r) {
+    __device__ __forceinline__ void add(float q, float r, float rest) {
         l += two_sum(m, two_sum(h, q));
         l += two_sum(m, r);
+        l += rest;
     }
     __device__ __forceinline__ double value() const { return (double)h + ((double)m + (double)l); }
 };
@@ -129,18 +134,22 @@ __global__ void __launch_bounds__(kVecMaxF, 1) k_colsum_vec(const float *__restr
                 mx = fmaxf(mx, fabsf(x[k]));
             }
             top = fmaxf(top, mx);
-            const float M = __uint_as_float((__float_as_uint(mx) & 0x7F800000u) + (kRunShift << 23) + 0x00400000u);
-            float q1 = 0.0f, qa = 0.0f, rs = 0.0f, ra = 0.0f;
+            const uint32_t e = __float_as_uint(mx) & 0x7F800000u, e2 = max(e, kRestShift << 23) - (kRestShift << 23);
+            const float M = __uint_as_float(e + (kRunShift << 23) + 0x00400000u), M2 = __uint_as_float(e2 + 0x00400000u);
+            float q1 = 0.0f, qa = 0.0f, r1 = 0.0f, ra = 0.0f, d1 = 0.0f, da = 0.0f;
 #pragma unroll
             for (int k = 0; k < kRun; ++k) {
-                const float q = (x[k] + M) - M, r = x[k] - q;
+                const float sign = __uint_as_float((__float_as_uint(x[k]) & 0x80000000u) | 0x3F800000u);
+                const float q = (x[k] + M) - M, rest = x[k] - q, r = (rest + M2) - M2, d = rest - r;
                 q1 += q;
                 qa += fabsf(q);
-                rs += r;
-                ra += __uint_as_float(__float_as_uint(r) ^ (__float_as_uint(x[k]) & 0x80000000u));
+                r1 += r;
+                ra = fmaf(r, sign, ra);
+                d1 += d;
+                da = fmaf(d, sign, da);
             }
-            S[j].add(q1, rs);
-            A[j].add(qa, ra);
+            S[j].add(q1, r1, d1);
+            A[j].add(qa, ra, da);
         }
     }
     double sum[4], mag[4];
