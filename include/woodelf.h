@@ -168,9 +168,12 @@ wdf_status wdf_set_metric(wdf_ensemble *ens, wdf_metric metric);
  * and row, at most 2^20 rows at a time) and, where they make the call faster, node values or
  * partial sums (at most 320 MB; a call that cannot have them runs without) live in a
  * temporary stream-ordered allocation from the context's pool (which keeps up to 384 MB
- * between calls), so calls on different streams never share scratch memory.  Host kind: copies through the ensemble's device staging buffers, in up
- * to eight chunks, and returns once phi is written on the host.  phi of a row does not depend on the other rows of the call (the same
- * floating-point additions in the same order).
+ * between calls), so calls on different streams never share scratch memory.  Host kind:
+ * copies through the ensemble's device staging buffers, in up to eight chunks (of at most
+ * 524,288 rows: more of them above 4,194,304 rows), and returns once phi is written on the
+ * host.  phi of a row does not depend on the other rows of the call (the same floating-point
+ * additions in the same order).  32 rows of phi have to fit a block's shared memory: ensembles of
+ * more than about 1,770 features are refused (WDF_ECUDA), here and in batches and servers.
  */
 wdf_status wdf_explain(wdf_ensemble *ens, const float *C, int64_t n, int64_t ldc, wdf_memkind kind,
                        float *phi, int64_t ldphi, void *stream);

@@ -420,7 +420,8 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
     chk(dalloc(&e->d_t32, (size_t)e->G * K * N, &e->bytes));
     chk(dalloc(&e->d_rec, p.rec.size(), &e->bytes));
     chk(dalloc(&e->d_meta, p.meta.size(), &e->bytes));
-    chk(dalloc(&e->d_image, (size_t)wdf::kImages * p.T * wdf::image_bytes(p.D), &e->bytes));
+    e->wide = !wdf::explain_fits(p.D, p.F, p.quads, 32, false, ctx->dev);
+    chk(dalloc(&e->d_image, (size_t)(e->wide ? 1 : wdf::kImages) * p.T * wdf::image_bytes(p.D), &e->bytes));
     chk(dalloc(&e->d_vlist, std::max<size_t>(p.vlist.size(), 1), &e->bytes));
     chk(dalloc(&e->d_voff, p.voff.size(), &e->bytes));
     int32_t *flfeat = nullptr;  // inputs of the images
@@ -455,7 +456,7 @@ wdf_status wdf_load_ensemble(wdf_ctx *ctx, int32_t n_features, int32_t n_trees, 
                        cudaMemcpyHostToDevice));
         chk(cudaMemcpy(e->d_sthr, p.sthr.data(), p.sthr.size() * 4, cudaMemcpyHostToDevice));
         if (e->n_tiles) chk(cudaMemcpy(e->d_tiles, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice));
-        chk(wdf::launch_images(p.D, p.T, e->d_unit, e->d_meta, flfeat, flrep, e->d_image, 0));
+        chk(wdf::launch_images(p.D, p.T, e->wide, e->d_unit, e->d_meta, flfeat, flrep, e->d_image, 0));
         // step 2 of Algorithm 3 depends only on the path signatures: build the tables now
         chk(wdf::launch_tables(p.D, e->metric, e->d_keys, e->G, e->d_t32, nullptr, 0));
         chk(cudaStreamSynchronize(0));

@@ -43,6 +43,7 @@ wdf_status fail(wdf_status s, const std::string &msg) {
 
 struct Cls {
     int D = 0, room = 0, F_max = 0, q_max = 0, thr_max = 0, tile_rows = 0;
+    bool wide = false;
     std::vector<int> members;  // batch ensemble indices, in job-slot order
     int cap_reqs = 0, cap_items = 0, cap_eitems = 0, cap_tiles = 0;
     size_t off_jobs = 0, off_reqs = 0, off_items = 0, off_count = 0, off_eitems = 0, off_ecount = 0;
@@ -97,6 +98,10 @@ struct Req {
 int class_room(const wdf_ensemble *e, const wdf::DevInfo &dev) {
     const int blocks = wdf::explain_blocks_per_sm(e->pk.D, e->pk.F, e->pk.quads, 32, dev);
     return blocks >= 7 ? 3 : blocks >= 5 ? 2 : blocks >= 3 ? 1 : 0;
+}
+
+bool tile_fits(const Cls &k, int tile_rows, const wdf::DevInfo &dev) {
+    return (!k.wide || tile_rows == 32) && wdf::explain_fits(k.D, k.F_max, k.q_max, tile_rows, k.wide, dev);
 }
 
 void drop_graph(wdf_batch *b) {
@@ -320,7 +325,7 @@ wdf_status capture(wdf_batch *b) {
                 k.D, reinterpret_cast<const wdf::ExplainJob *>(b->d_blob + k.off_jobs),
                 reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),
                 reinterpret_cast<const int4 *>(b->d_blob + k.off_items),
-                reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.q_max, k.tile_rows, 0, b->ctx->dev,
+                reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.q_max, k.tile_rows, k.wide, 0, b->ctx->dev,
                 b->branch[c]);
         if (e == cudaSuccess) e = cudaEventRecord(b->ev_join[c], b->branch[c]);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(b->cap, b->ev_join[c], 0);
@@ -394,13 +399,21 @@ wdf_status wdf_batch_create(wdf_ctx *ctx, int32_t n_ensembles, wdf_ensemble *con
     for (int i = 0; i < n_ensembles; ++i) {
         const int D = b->ens[(size_t)i]->pk.D, room = class_room(b->ens[(size_t)i], ctx->dev);
         int c = -1;
-        for (size_t k = 0; k < b->cls.size(); ++k)
-            if (b->cls[k].D == D && b->cls[k].room == room) c = (int)k;
+        const bool wide = b->ens[(size_t)i]->wide;
+        for (size_t k = 0; k < b->cls.size(); ++k) {
+            const Cls &o = b->cls[k];
+            // its blocks hold the most features and the most codes of any member
+            if (o.D == D && o.room == room && o.wide == wide &&
+                wdf::explain_fits(D, std::max(o.F_max, b->ens[(size_t)i]->pk.F),
+                                  std::max(o.q_max, b->ens[(size_t)i]->pk.quads), 32, wide, ctx->dev))
+                c = (int)k;
+        }
         if (c < 0) {
             b->cls.push_back(Cls());
             c = (int)b->cls.size() - 1;
             b->cls.back().D = D;
             b->cls.back().room = room;
+            b->cls.back().wide = wide;
         }
         Cls &k = b->cls[(size_t)c];
         k.F_max = std::max(k.F_max, b->ens[(size_t)i]->pk.F);
@@ -418,7 +431,7 @@ wdf_status wdf_batch_create(wdf_ctx *ctx, int32_t n_ensembles, wdf_ensemble *con
     for (size_t c = 0; c < b->cls.size() && e == cudaSuccess; ++c) {
         Cls &k = b->cls[c];
         k.tile_rows = wdf::default_tile_rows(k.D, k.F_max, k.q_max, ctx->dev);
-        if (wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, k.tile_rows) > ctx->dev.smem_optin) {
+        if (!tile_fits(k, k.tile_rows, ctx->dev)) {
             e = cudaErrorInvalidConfiguration;
             break;
         }
@@ -536,7 +549,7 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
         int hit = 0;
         for (const auto &row : cached)
             if (row[0] == k.D && row[1] == fkey && row[2] == xkey && (row[3] == 32 || row[3] == 64 || row[3] == 128) &&
-                wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, row[3]) <= b->ctx->dev.smem_optin)
+                tile_fits(k, row[3], b->ctx->dev))
                 hit = row[3];
         if (hit) {
             k.tile_rows = hit;
@@ -561,7 +574,7 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
             }
         }
         for (int tc : cand) {
-            if (wdf::explain_smem_bytes(k.D, k.F_max, k.q_max, tc) > b->ctx->dev.smem_optin) continue;
+            if (!tile_fits(k, tc, b->ctx->dev)) continue;
             std::vector<int> tiles;
             for (const Cls &o : b->cls) tiles.push_back(&o == &k ? tc : o.tile_rows);
             plan_groups(b, tiles, &reqs);
@@ -580,7 +593,7 @@ wdf_status wdf_batch_autotune(wdf_batch *b, int32_t n_requests, const int32_t *e
                                                   reinterpret_cast<const wdf::BatchRequest *>(b->d_blob + k.off_reqs),
                                                   reinterpret_cast<const int4 *>(b->d_blob + k.off_items),
                                                   reinterpret_cast<int *>(b->d_blob + k.off_count), k.F_max, k.q_max, tc,
-                                                  0, b->ctx->dev, st);
+                                                  k.wide, 0, b->ctx->dev, st);
             }
             if (e == cudaSuccess) e = cudaEventRecord(e1, st);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);

@@ -35,7 +35,9 @@ struct ExplainPlan {
 // depth 8 and 134 features: 63.8 ms with the parts of all rows at once (1.26 GB), 64.5 in slices,
 // 67.5 with whole tiles; 100,000 rows, 400 trees of depth 8 and 500 features 22.3 (1.6 GB), 22.8
 // and 27.9 (blocks at work on the same part share its folded vectors in the L2 cache).
-inline ExplainPlan explain_plan(int D, int64_t n, int T, int F, int tile_rows, int sms, int64_t per_sm) {
+// values: a row block's codes fit the shared memory of the node values' kernel.
+inline ExplainPlan explain_plan(int D, int64_t n, int T, int F, int tile_rows, int sms, int64_t per_sm,
+                                bool values = true) {
     const int P = explain_parts(T, D);
     const int64_t room = (int64_t)sms * per_sm;
     const double walk = 0.034 * T * (1 << D);
@@ -63,7 +65,7 @@ inline ExplainPlan explain_plan(int D, int64_t n, int T, int F, int tile_rows, i
         }
     }
     const int64_t rows = (n + 31) / 32 * 32, positions = (int64_t)T * flush_len(D);
-    if (rows <= kScratchBytes / 4 / positions) {
+    if (values && rows <= kScratchBytes / 4 / positions) {
         const double cost = 20.0 + (double)rows * ((D == 8 ? 2.2e-6 : 1.4e-6) * (double)positions + 8e-6 * F);
         if (cost < least) best = ExplainPlan{0, n, (size_t)(rows * positions)};
     }

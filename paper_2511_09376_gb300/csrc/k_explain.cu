@@ -53,25 +53,35 @@ WDF_EXPLAIN_DEPTH(5, extern)
 WDF_EXPLAIN_DEPTH(6, extern)
 WDF_EXPLAIN_DEPTH(7, extern)
 WDF_EXPLAIN_DEPTH(8, extern)
+WDF_EXPLAIN_WIDE(2, extern)
+WDF_EXPLAIN_WIDE(3, extern)
+WDF_EXPLAIN_WIDE(4, extern)
+WDF_EXPLAIN_WIDE(5, extern)
+WDF_EXPLAIN_WIDE(6, extern)
+WDF_EXPLAIN_WIDE(7, extern)
+WDF_EXPLAIN_WIDE(8, extern)
 
 template <int D>
 static cudaError_t explain_depth(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi,
                                  int64_t ldp, int tile_rows, int splits, float *scratch, const DevInfo &dev,
                                  cudaStream_t st) {
+    if (job.wide) return explain_t<D, 32, true>(codes, n, job, phi, ldp, splits, scratch, dev, st);
     switch (tile_rows) {
-        case 32: return explain_t<D, 32>(codes, n, job, phi, ldp, splits, scratch, dev, st);
-        case 128: return explain_t<D, 128>(codes, n, job, phi, ldp, splits, scratch, dev, st);
-        default: return explain_t<D, 64>(codes, n, job, phi, ldp, splits, scratch, dev, st);
+        case 32: return explain_t<D, 32, false>(codes, n, job, phi, ldp, splits, scratch, dev, st);
+        case 128: return explain_t<D, 128, false>(codes, n, job, phi, ldp, splits, scratch, dev, st);
+        default: return explain_t<D, 64, false>(codes, n, job, phi, ldp, splits, scratch, dev, st);
     }
 }
 
 template <int D>
 static cudaError_t batch_depth(const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items, int *n_items,
-                               int F_max, int q_max, int tile_rows, int grid, const DevInfo &dev, cudaStream_t st) {
+                               int F_max, int q_max, int tile_rows, bool wide, int grid, const DevInfo &dev,
+                               cudaStream_t st) {
+    if (wide) return batch_t<D, 32, true>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
     switch (tile_rows) {
-        case 32: return batch_t<D, 32>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
-        case 128: return batch_t<D, 128>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
-        default: return batch_t<D, 64>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
+        case 32: return batch_t<D, 32, false>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
+        case 128: return batch_t<D, 128, false>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
+        default: return batch_t<D, 64, false>(jobs, reqs, items, n_items, F_max, q_max, grid, dev, st);
     }
 }
 
@@ -184,13 +194,16 @@ cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const 
                            int64_t ldp, int tile_rows, const DevInfo &dev, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
     if (D < 2 || D > 8) return cudaErrorInvalidValue;
+    if (job.wide) tile_rows = 32;
     if (tile_rows <= 0) tile_rows = default_tile_rows(D, job.F, job.sa.quads, dev);
-    if (explain_smem_bytes(D, job.F, job.sa.quads, tile_rows) > dev.smem_optin) return cudaErrorInvalidConfiguration;
+    if (explain_smem_bytes(D, job.F, job.sa.quads, tile_rows, job.wide) > dev.smem_optin)
+        return cudaErrorInvalidConfiguration;
     const int64_t chunk = std::min(n, kExplainChunkRows);
     const int64_t pad = 128;  // every tile size divides it
     const size_t code_bytes = (size_t)((chunk + pad - 1) / pad * pad) / 32 * job.sa.quads * 16;
     ExplainPlan plan = explain_plan(D, chunk, job.T, job.F, tile_rows, dev.sms,
-                                    explain_blocks_per_sm(D, job.F, job.sa.quads, tile_rows, dev));
+                                    explain_blocks_per_sm(D, job.F, job.sa.quads, tile_rows, dev),
+                                    (size_t)job.sa.quads * 16 <= dev.smem_optin);
     unsigned char *codes = nullptr;
     cudaError_t err = take_scratch(&plan, chunk, code_bytes, cudaErrorMemoryAllocation, [&](size_t bytes) {
         const cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void **>(&codes), bytes, dev.pool, st);
@@ -249,25 +262,25 @@ cudaError_t launch_explain(int D, const float *C, int64_t n, int64_t ldc, const 
 }
 
 cudaError_t launch_explain_batch(int D, const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items,
-                                 int *n_items, int F_max, int q_max, int tile_rows, int grid, const DevInfo &dev,
-                                 cudaStream_t st) {
+                                 int *n_items, int F_max, int q_max, int tile_rows, bool wide, int grid,
+                                 const DevInfo &dev, cudaStream_t st) {
     switch (D) {
-        case 2: return batch_depth<2>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
-        case 3: return batch_depth<3>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
-        case 4: return batch_depth<4>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
-        case 5: return batch_depth<5>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
-        case 6: return batch_depth<6>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
-        case 7: return batch_depth<7>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
-        case 8: return batch_depth<8>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, grid, dev, st);
+        case 2: return batch_depth<2>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
+        case 3: return batch_depth<3>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
+        case 4: return batch_depth<4>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
+        case 5: return batch_depth<5>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
+        case 6: return batch_depth<6>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
+        case 7: return batch_depth<7>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
+        case 8: return batch_depth<8>(jobs, reqs, items, n_items, F_max, q_max, tile_rows, wide, grid, dev, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
-// One block per (tree, image).
-__global__ void k_images(int D, int T, const UnitNode *__restrict__ unit, const TreeMeta *__restrict__ meta,
+// One block per (tree, image).  wide: the one image of an ensemble of wide tiles.
+__global__ void k_images(int D, int T, bool wide, const UnitNode *__restrict__ unit, const TreeMeta *__restrict__ meta,
                          const int32_t *__restrict__ flfeat, const uint8_t *__restrict__ flrep,
                          unsigned char *__restrict__ image) {
-    const int t = blockIdx.x, i = blockIdx.y, tid = threadIdx.x, nt = blockDim.x, xs = image_rows(i) + 1;
+    const int t = blockIdx.x, i = blockIdx.y, tid = threadIdx.x, nt = blockDim.x, xs = wide ? 32 : image_rows(i) + 1;
     const int UPT = units_per_tree(D), CU = chunk_units(D), GS = gather_group(D), GB = flush_group_len(D) / 8;
     const int CP = chunk_positions(D);
     unsigned char *dst = image + ((size_t)i * T + t) * image_bytes(D);
@@ -299,17 +312,17 @@ __global__ void k_images(int D, int T, const UnitNode *__restrict__ unit, const 
         reinterpret_cast<UnitNode *>(dst)[tid] = src[(tid < UPT ? tid : 0) * 32 + 31];
 }
 
-cudaError_t launch_images(int D, int T, const UnitNode *unit, const TreeMeta *meta, const int32_t *flfeat,
+cudaError_t launch_images(int D, int T, bool wide, const UnitNode *unit, const TreeMeta *meta, const int32_t *flfeat,
                           const uint8_t *flrep, unsigned char *image, cudaStream_t st) {
-    k_images<<<dim3((unsigned)T, kImages), 128, 0, st>>>(D, T, unit, meta, flfeat, flrep, image);
+    k_images<<<dim3((unsigned)T, (unsigned)(wide ? 1 : kImages)), 128, 0, st>>>(D, T, wide, unit, meta, flfeat, flrep, image);
     count_launches(1);
     return cudaGetLastError();
 }
 
-size_t explain_smem_bytes(int D, int F, int quads, int tile_rows) {
+size_t explain_smem_bytes(int D, int F, int quads, int tile_rows, bool wide) {
     switch (D * 1000 + tile_rows) {
 #define WDF_SMEM_CASE(d, tc) \
-    case d * 1000 + tc: return ExLayout<d>(F, quads, tc).total;
+    case d * 1000 + tc: return ExLayout<d>(F, quads, tc, wide && tc == 32).total;
         WDF_SMEM_CASE(2, 32) WDF_SMEM_CASE(2, 64) WDF_SMEM_CASE(2, 128)
         WDF_SMEM_CASE(3, 32) WDF_SMEM_CASE(3, 64) WDF_SMEM_CASE(3, 128)
         WDF_SMEM_CASE(4, 32) WDF_SMEM_CASE(4, 64) WDF_SMEM_CASE(4, 128)

@@ -69,7 +69,7 @@ struct ExplainCfg {
 WDF_HD constexpr int explain_threads(int tc) { return 2 * tc; }
 
 // Shared memory of one block: code tile (TC / 32 blocks of quads) | phi tile ((F + 1) x (TC + 1)
-// floats, feature-major, row F a scratch row) | per warp, a ring of SLOTS chunks and their line
+// floats, feature-major, row F a scratch row; wide: no code tile and rows of TC floats) | per warp, a ring of SLOTS chunks and their line
 // maps, then the nodes above a tree's units.  (Depth 8 a tree at a time, 33.5 KB a block instead
 // of 24.7: 3063 us where the above took 2655, 3371 where 191 features take 3090; depth 7 a unit
 // at a time 3 % slower.)
@@ -80,9 +80,9 @@ struct ExLayout {
     static constexpr int SLOTS = chunk_units(D) > 1 ? 2 : 3;
     static constexpr int LINE = chunk_bytes(D), SLOT = LINE + (chunk_units(D) > 2 ? 8 * chunk_units(D) : 16);
     static constexpr int WARP = SLOTS * SLOT + (unit_top(D) > 1 ? 8 * (int)sizeof(UnitNode) : 0);
-    __host__ __device__ ExLayout(int F, int quads, int TC) {
-        x = (size_t)(TC / 32) * quads * 16;
-        p = ((size_t)(F + 1) * (TC + 1) * 4 + 15) & ~(size_t)15;
+    __host__ __device__ ExLayout(int F, int quads, int TC, bool wide = false) {
+        x = wide ? 0 : (size_t)(TC / 32) * quads * 16;
+        p = ((size_t)(F + 1) * (wide ? TC : TC + 1) * 4 + 15) & ~(size_t)15;
         total = x + p + (size_t)(TC / 16) * WARP;
     }
 };
@@ -254,30 +254,45 @@ __device__ __forceinline__ void unit_sums(const UnitSlots<D> &v, int u, float (&
 // phi, the other makes its next decisions and has its next gathers in flight.  A row's phi
 // fixes how many rows an SM can hold; two warps per 32 rows double the warps that hide the
 // gathers' and the shared memory's latency.  The turns also fix the order of the additions.
-template <int D, int TC>
+//
+// WIDE: the form of ensembles whose tile does not fit a block's shared memory otherwise (from some
+// 1,400 features of 16 to 255 thresholds on, to about 1,770).  The codes are read where they lie, in global memory, and a
+// feature's phi row is 32 floats, rotated by the feature's number (row r of feature f in word (r + f)
+// mod 32) so that its storing reads all banks, as the 33 floats of the other form do.  The same
+// additions in the same order.  48,640 rows, 17 thresholds a feature, the last width of the other form's
+// and the first of this one's at about: depth 6 18.0 / 18.6 ms (380 trees), depth 7 15.9 / 20.1 (185),
+// depth 8 16.9 / 14.8 (94); so the other form stays where it fits.
+template <int D, int TC, bool WIDE>
 __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsigned char *__restrict__ codes,
                                              int64_t n, float *__restrict__ phi, int64_t ldp, int64_t c0, int part0,
                                              int part1, float *__restrict__ scratch, unsigned char *smem_raw) {
     using X = ExplainCfg<D>;
-    constexpr int XS = TC + 1, GS = X::GS, TOP = X::TOP, UPT = X::UPT;
+    static_assert(!WIDE || TC == 32, "wide tiles have 32 rows");
+    constexpr int XS = WIDE ? TC : TC + 1, GS = X::GS, TOP = X::TOP, UPT = X::UPT;
     constexpr int NT = explain_threads(TC), SLOTS = ExLayout<D>::SLOTS, SLOT = ExLayout<D>::SLOT;
     constexpr int FB = flush_group_bottom(D), GL = flush_group_len(D), LW = X::LW;
     constexpr int IMG = image_bytes(D), CHUNK = chunk_bytes(D), LINE = ExLayout<D>::LINE;
     constexpr int CU = chunk_units(D), CPT = tree_chunks(D);
     const int F = job.F, T = job.T, quads = job.sa.quads;
-    const ExLayout<D> L(F, quads, TC);
+    const ExLayout<D> L(F, quads, TC, WIDE);
     uint4 *sx = reinterpret_cast<uint4 *>(smem_raw);
     float *sp = reinterpret_cast<float *>(smem_raw + L.x);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, pair = warp >> 1, half = warp & 1;
     unsigned char *ring = smem_raw + L.x + L.p + (size_t)warp * ExLayout<D>::WARP;  // this warp's
     const uint2 *above = reinterpret_cast<const uint2 *>(ring + SLOTS * SLOT);
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(codes) + (c0 / 32) * quads;
+    const uint4 *src = reinterpret_cast<const uint4 *>(codes) + (c0 / 32) * quads;
+    if (!WIDE)
         for (int i = tid; i < TC / 32 * quads; i += NT) sx[i] = __ldg(src + i);
-    }
     for (int i = tid; i < (F + 1) * XS; i += NT) sp[i] = 0.0f;
-    float *myphi = sp + 32 * pair + lane;
-    const uint4 *block = sx + pair * quads;
+    float *myphi = WIDE ? sp : sp + 32 * pair + lane;
+    const uint4 *block = WIDE ? src : sx + pair * quads;
+    // this lane's phi in the row that starts at o (a multiple of 32 x feature)
+    auto rotate = [&](int (&o)[8]) {
+        if (WIDE) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) o[q] += (lane + (o[q] >> 5)) & 31;
+        }
+    };
     auto turn = [&]() {
         // constant barrier numbers: a block with a variable one reserves all sixteen, and an SM
         // holds four such blocks
@@ -357,12 +372,16 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         const unsigned char *rep = slot + chunk_repeats(D) + i * (GL / 8);
         int o[8];
         load_offsets8(off, o);
+        rotate(o);
         float up[GS > 1 ? GS - 1 : 1];
         unit_sums<D>(v, u, up, top);
 #pragma unroll
         for (int b = 0; b < GL / 8; ++b) {
             int on[8];
-            if (b + 1 < GL / 8) load_offsets8(off + 8 * (b + 1), on);  // off the chain of phi round trips
+            if (b + 1 < GL / 8) {  // off the chain of phi round trips
+                load_offsets8(off + 8 * (b + 1), on);
+                rotate(on);
+            }
             float x[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -379,6 +398,7 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
         }
         if (UPT > 1 && u == UPT - 1 && mine) {
             load_offsets8(off + (CU - i) * GL, o);
+            rotate(o);
             float x[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) x[q] = q < UPT - 1 ? top[q < UPT - 1 ? q : 0] : 0.0f;
@@ -434,9 +454,10 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
             if (row >= n) break;
             float *dst = scratch ? scratch + ((size_t)part * n + row) * F : phi + row * ldp;
             for (int f = lane; f < F; f += 32) {
-                const float x = sp[f * XS + 32 * pair + r];
+                float &y = sp[f * XS + (WIDE ? (r + f) & 31 : 32 * pair + r)];
+                const float x = y;
                 dst[f] = part > part0 && !scratch ? dst[f] + x : x;
-                sp[f * XS + 32 * pair + r] = 0.0f;
+                y = 0.0f;
             }
         }
         turn();
@@ -445,12 +466,12 @@ __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsign
 
 // Block (tile, y): parts [P y / gridDim.y, P (y + 1) / gridDim.y) of the tile's rows (scratch
 // non-null when there is more than one y).
-template <int D, int TC>
-__global__ void __launch_bounds__(explain_threads(TC), kExplainWarps * 16 / TC) k_explain(const unsigned char *__restrict__ codes, int64_t n, ExplainJob job, float *__restrict__ phi, int64_t ldp,
+template <int D, int TC, bool WIDE>
+__global__ void __launch_bounds__(explain_threads(TC), WIDE ? 1 : kExplainWarps * 16 / TC) k_explain(const unsigned char *__restrict__ codes, int64_t n, ExplainJob job, float *__restrict__ phi, int64_t ldp,
               float *__restrict__ scratch) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P = explain_parts(job.T, D), y = blockIdx.y, Y = gridDim.y;
-    explain_tile<D, TC>(job, codes, n, phi, ldp, (int64_t)blockIdx.x * TC, P * y / Y, P * (y + 1) / Y, scratch, smem_raw);
+    explain_tile<D, TC, WIDE>(job, codes, n, phi, ldp, (int64_t)blockIdx.x * TC, P * y / Y, P * (y + 1) / Y, scratch, smem_raw);
 }
 
 // Few rows: the node values of 32 rows and one tree per warp, every tree at once, position i of
@@ -522,9 +543,8 @@ __global__ void __launch_bounds__(32 * kValueWarps) k_values(const unsigned char
 // the tail.  The item count n_items[0] is read from device memory, so one captured graph serves
 // batches of any size up to its capacity.  Which block computes a tile does not change any
 // row's arithmetic, nor do the groups: parts are always added in their order.
-constexpr size_t kBatchShared = 16;  // room for the two words below
-template <int D, int TC>
-__global__ void __launch_bounds__(explain_threads(TC), kExplainWarps * 16 / TC) k_explain_batch(const ExplainJob *__restrict__ jobs,
+template <int D, int TC, bool WIDE>
+__global__ void __launch_bounds__(explain_threads(TC), WIDE ? 1 : kExplainWarps * 16 / TC) k_explain_batch(const ExplainJob *__restrict__ jobs,
                                                          const BatchRequest *__restrict__ reqs,
                                                          const int4 *__restrict__ items, int *n_items) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -540,7 +560,7 @@ __global__ void __launch_bounds__(explain_threads(TC), kExplainWarps * 16 / TC) 
         const BatchRequest rq = reqs[it.y];
         const int group = it.z >> kBatchGroupShift, P = explain_parts(job.T, D), groups = rq.groups;
         const int64_t c0 = ((int64_t)(it.z & ((1 << kBatchGroupShift) - 1)) << 31) | (uint32_t)it.w;
-        explain_tile<D, TC>(job, rq.codes, rq.n, rq.phi, rq.ldp, c0, P * group / groups, P * (group + 1) / groups,
+        explain_tile<D, TC, WIDE>(job, rq.codes, rq.n, rq.phi, rq.ldp, c0, P * group / groups, P * (group + 1) / groups,
                             groups > 1 ? rq.parts : nullptr, smem_raw);
         __syncthreads();
         if (groups > 1) {  // the last of the tile's items adds its parts
@@ -572,11 +592,11 @@ cudaError_t set_carveout(K kern, int D, int tile_rows, size_t smem) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, percent);
 }
 
-template <int D, int TC>
+template <int D, int TC, bool WIDE>
 cudaError_t explain_t(const unsigned char *codes, int64_t n, const ExplainJob &job, float *phi, int64_t ldp,
                       int splits, float *scratch, const DevInfo &dev, cudaStream_t st) {
-    const size_t smem = ExLayout<D>(job.F, job.sa.quads, TC).total;
-    auto kern = k_explain<D, TC>;
+    const size_t smem = ExLayout<D>(job.F, job.sa.quads, TC, WIDE).total;
+    auto kern = k_explain<D, TC, WIDE>;
     cudaError_t err = allow_shared(kern, smem, dev);
     if (err == cudaSuccess) err = set_carveout(kern, D, TC, smem);
     if (err != cudaSuccess) return err;
@@ -599,11 +619,11 @@ cudaError_t values_t(const unsigned char *codes, int64_t n, const ExplainJob &jo
     return err != cudaSuccess ? err : cudaGetLastError();
 }
 
-template <int D, int TC>
+template <int D, int TC, bool WIDE>
 cudaError_t batch_t(const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items, int *n_items, int F_max,
                     int q_max, int grid, const DevInfo &dev, cudaStream_t st) {
-    const size_t smem = ExLayout<D>(F_max, q_max, TC).total;
-    auto kern = k_explain_batch<D, TC>;
+    const size_t smem = ExLayout<D>(F_max, q_max, TC, WIDE).total;
+    auto kern = k_explain_batch<D, TC, WIDE>;
     cudaError_t err = allow_shared(kern, smem, dev, kBatchShared);
     if (err == cudaSuccess) err = set_carveout(kern, D, TC, smem);
     if (err != cudaSuccess) return err;
@@ -615,11 +635,13 @@ cudaError_t batch_t(const ExplainJob *jobs, const BatchRequest *reqs, const int4
 
 // Explicit instantiation of the kernels of one (depth, tile rows) pair; each pair is
 // compiled in one of the k_explain_d*.cu translation units.
-#define WDF_EXPLAIN_TILE(d, tc, spec)                                                                            \
-    spec template cudaError_t explain_t<d, tc>(const unsigned char *, int64_t, const ExplainJob &, float *,       \
-                                               int64_t, int, float *, const DevInfo &, cudaStream_t);            \
-    spec template cudaError_t batch_t<d, tc>(const ExplainJob *, const BatchRequest *, const int4 *, int *, int,  \
-                                             int, int, const DevInfo &, cudaStream_t);
+#define WDF_EXPLAIN_FORM(d, tc, wide, spec)                                                                      \
+    spec template cudaError_t explain_t<d, tc, wide>(const unsigned char *, int64_t, const ExplainJob &, float *, \
+                                                     int64_t, int, float *, const DevInfo &, cudaStream_t);      \
+    spec template cudaError_t batch_t<d, tc, wide>(const ExplainJob *, const BatchRequest *, const int4 *, int *, \
+                                                   int, int, int, const DevInfo &, cudaStream_t);
+#define WDF_EXPLAIN_TILE(d, tc, spec) WDF_EXPLAIN_FORM(d, tc, false, spec)
+#define WDF_EXPLAIN_WIDE(d, spec) WDF_EXPLAIN_FORM(d, 32, true, spec)
 #define WDF_EXPLAIN_VALUES(d, spec)                                                                              \
     spec template cudaError_t values_t<d>(const unsigned char *, int64_t, const ExplainJob &, float *,           \
                                           const DevInfo &, cudaStream_t);

@@ -34,12 +34,13 @@ struct SliceArrays {
 // Everything the consumer kernel needs about one ensemble.
 struct ExplainJob {
     SliceArrays sa;
-    const unsigned char *image;  // [kImages][T][image_bytes(D)] (tree_layout.h)
+    const unsigned char *image;  // [kImages, wide: 1][T][image_bytes(D)] (tree_layout.h)
     const float *sfold;     // folded slot vectors [T][NS][2^(D+1)][slots_per_entry], entry e at line_pos(e), then
                             // (depth 8) the root slots [T][NS][2^(D+1)]
     const int32_t *vlist, *voff;  // nodes of every feature and part in the order of addition (Packed)
     const uint32_t *lines;  // per tree lines_words(D) words: byte s = line map of subtree s
     int T, F;
+    int wide;  // tiles take the wide form
 };
 // Where the consumer gathers land.  A warp's 32-byte gathers of one bottom subtree are
 // served a quarter warp at a time, one L1 wavefront per distinct 128-byte line, and a
@@ -184,8 +185,9 @@ cudaError_t launch_base_value(int D, const uint32_t *hist, const int32_t *group_
                               const double *leaf_w_rows, int n_live, int64_t m, double *out, cudaStream_t st);
 
 // The tree images (tree_layout.h) from the unit nodes, the metadata, the features flfeat
-// [T][flush_len(D)] and repeats flrep [T][flush_batches(D)] of the flush positions.
-cudaError_t launch_images(int D, int T, const UnitNode *unit, const TreeMeta *meta, const int32_t *flfeat,
+// [T][flush_len(D)] and repeats flrep [T][flush_batches(D)] of the flush positions: kImages, or
+// the one of an ensemble of wide tiles.
+cudaError_t launch_images(int D, int T, bool wide, const UnitNode *unit, const TreeMeta *meta, const int32_t *flfeat,
                           const uint8_t *flrep, unsigned char *image, cudaStream_t st);
 
 // Step 4: phi of n consumer rows, tile_rows consumer rows per block (32, 64 or 128;
@@ -201,7 +203,13 @@ void explain_timing(bool on);
 cudaError_t explain_timing_read(double *ms, int64_t *launches);
 // quads: 16-byte quads of a 32-row code block.
 int default_tile_rows(int D, int F, int quads, const DevInfo &dev);
-size_t explain_smem_bytes(int D, int F, int quads, int tile_rows);
+// Shared memory of a block; wide: of the form for ensembles whose 32 rows do not fit otherwise
+// (k_explain.cuh).
+size_t explain_smem_bytes(int D, int F, int quads, int tile_rows, bool wide = false);
+constexpr size_t kBatchShared = 16;  // what a block of the batch kernel has beside that
+inline bool explain_fits(int D, int F, int quads, int tile_rows, bool wide, const DevInfo &dev) {
+    return explain_smem_bytes(D, F, quads, tile_rows, wide) + kBatchShared <= dev.smem_optin;
+}
 int explain_blocks_per_sm(int D, int F, int quads, int tile_rows, const DevInfo &dev);
 
 // Decision codes of a ragged batch's rows: items (request, group of packs, first 32-row block,
@@ -214,10 +222,10 @@ cudaError_t launch_encode_batch(const ExplainJob *jobs, const BatchRequest *reqs
 // Step 4 for a ragged batch of one depth: a persistent grid (grid <= 0: one wave at full
 // occupancy) walks the work items (job, request, first row split as hi/lo words);
 // *n_items is read on the device; the rows' codes come from launch_encode_batch.  F_max and q_max bound the
-// feature count and the quads of a code block of every job.
+// feature count and the quads of a code block of every job.  wide: the jobs are (tile_rows 32).
 cudaError_t launch_explain_batch(int D, const ExplainJob *jobs, const BatchRequest *reqs, const int4 *items,
-                                 int *n_items, int F_max, int q_max, int tile_rows, int grid, const DevInfo &dev,
-                                 cudaStream_t st);
+                                 int *n_items, int F_max, int q_max, int tile_rows, bool wide, int grid,
+                                 const DevInfo &dev, cudaStream_t st);
 
 // Interaction values (k_interactions.cu).  Pair tables t2 [G][2^D][P * 2^D] (P =
 // D(D-1)/2 position pairs) for metric 0 (Shapley) or 1 (Banzhaf); the contraction is

@@ -161,7 +161,8 @@ static_assert(flush_batches(8) <= 64, "batch flags are one 64-bit word per tree"
 // batches and the last batch in bits 8-15 and 16-23; per batch the positions whose feature an
 // earlier position of the batch has (0xFF when they repeat among themselves).  After the
 // chunks, with several levels above the units, the nodes of those.  The offsets depend on the
-// tile's rows, so an ensemble has an image of its trees for every tile size.
+// tile's rows, so an ensemble has an image of its trees for every tile size (one of wide tiles,
+// k_explain.cuh, only theirs).
 WDF_HD constexpr int chunk_units(int D) { return D == 8 ? 1 : units_per_tree(D); }
 WDF_HD constexpr int tree_chunks(int D) { return units_per_tree(D) / chunk_units(D); }
 WDF_HD constexpr int chunk_positions(int D) {

@@ -48,6 +48,7 @@ struct wdf_ensemble {
     float *d_t32 = nullptr;
     wdf::NodeRec *d_rec = nullptr;
     wdf::TreeMeta *d_meta = nullptr;
+    bool wide = false;  // explain calls take wide tiles (k_explain.cuh)
     unsigned char *d_image = nullptr;  // the trees as the consumer kernel stages them (tree_layout.h)
     // tensor-core contraction: split operand stages (A for any mode, B for bpk_mode),
     // 128-row tiles, wait-expiry flag
@@ -71,7 +72,7 @@ struct wdf_ensemble {
                                 (int)pk.scol.size(), pk.spack[0].levels, {pk.qbase[0], pk.qbase[1], pk.qbase[2]}, pk.quads};
     }
     wdf::TreeArrays arrays() const { return wdf::TreeArrays{d_nodes, d_rec, d_meta}; }
-    wdf::ExplainJob job() const { return wdf::ExplainJob{slices(), d_image, d_sfold, d_vlist, d_voff, d_lines, pk.T, pk.F}; }
+    wdf::ExplainJob job() const { return wdf::ExplainJob{slices(), d_image, d_sfold, d_vlist, d_voff, d_lines, pk.T, pk.F, wide}; }
     // background state (set_background)
     int has_bg = 0;
     int64_t m = 0;
