@@ -683,8 +683,8 @@ def ragged_compare(args) -> dict:
         "batched": {"rows_per_s": rows / (batch_ms * 1e-3), "ms_per_step": batch_ms, "contraction": SPLIT_BF16,
                     "graph_launches_per_step": 1, "kernels_per_step": (l2 - l1) // args.ragged_steps,
                     "tile_rows": tiles,
-                    "how": "one wdf_batch_explain: a CUDA graph with one persistent kernel per depth class, "
-                           "autotuned consumer tiles"},
+                    "how": "one wdf_batch_explain: a CUDA graph with one persistent kernel per class (of one depth), "
+                           "autotuned consumer tiles (tile_rows: the smallest of a depth)"},
         "batched_vs_plain": plain_ms / batch_ms,
         "max_abs_diff_batched_vs_plain": diff,
         "accuracy": "both arms within |phi - oracle| <= 1e-6 + 1e-5 |oracle| of the FP64 oracle "

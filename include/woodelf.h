@@ -229,12 +229,14 @@ wdf_status wdf_global_attribution(wdf_ctx *ctx, const float *phi, int64_t n, int
  * ldc[i]) against ensembles[ensemble_index[i]] into phi[i] (device, stride ldphi[i]).
  * Stream-ordered and asynchronous; the caller may reuse its request arrays on return.
  * WDF_EINVAL for an index out of range, a missing background or bad sizes.
- * wdf_batch_autotune: runs each depth class's kernel on the given requests with every
+ * wdf_batch_autotune: runs each class's kernel on the given requests with every
  * consumer-tile size that fits (32, 64, 128 rows), reps timed runs each, and keeps the
  * fastest per class (phi is written with valid results).  cache_path (nullable): a text
  * file of "depth features code_bytes tile_rows ms" lines (features and decision-code
- * bytes per row of the class, rounded up to 32) read first and appended to.  Synchronous.  wdf_batch_tile_rows reports the tile size of a depth class (-1 if
- * the batch has none).
+ * bytes per row of the class, rounded up to 32) read first and appended to.  Synchronous.
+ * wdf_batch_tile_rows reports the tile size of a depth's ensembles, the smallest where they
+ * are in several classes (its multiples are then tile borders of every one of them), -1 if
+ * the batch has none of that depth.
  */
 typedef struct wdf_batch wdf_batch;
 wdf_status wdf_batch_create(wdf_ctx *ctx, int32_t n_ensembles, wdf_ensemble *const *ensembles, wdf_batch **out);

@@ -623,7 +623,7 @@ wdf_status wdf_batch_tile_rows(const wdf_batch *b, int32_t depth, int32_t *tile_
     if (!b || !tile_rows) return fail(WDF_EINVAL, "null argument");
     *tile_rows = -1;
     for (const Cls &k : b->cls)
-        if (k.D == depth) *tile_rows = k.tile_rows;
+        if (k.D == depth && (*tile_rows < 0 || k.tile_rows < *tile_rows)) *tile_rows = k.tile_rows;
     return WDF_OK;
 }
 
