@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(32 * kCountWarps, 1) k_bg_count(const unsigned
     using S = Shape<D>;
     using N = Unit<D>;
     static_assert(N::TOP <= 1, "one m16 of ancestor patterns");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, W = blockDim.x >> 5;
     const int chunk = blockIdx.x % chunks, slice = blockIdx.x / chunks, nslices = gridDim.x / chunks;
     const int unit = min(chunk * W + warp, units - 1);  // a spare warp repeats the last unit and adds nothing
@@ -310,8 +310,8 @@ __global__ void __launch_bounds__(512, 1) k_bg_add(const unsigned char *__restri
     using S = Shape<D>;
     using N = Unit<D>;
     constexpr int GS = N::NSU, TOP = N::TOP, CELLS = GS * S::E;
-    static_assert(N::H == 5, "units of 31 nodes");
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    static_assert(N::H == 5 && CELLS % 8 == 0, "units of 31 nodes, counters in whole 32 bytes");
+    extern __shared__ __align__(32) unsigned char smem_raw[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 6, half = (tid >> 5) & 1, W = blockDim.x >> 6;
     const int chunk = blockIdx.x % chunks, slice = blockIdx.x / chunks, nslices = gridDim.x / chunks;
     const bool spare = chunk * W + warp >= units;
@@ -376,7 +376,9 @@ __global__ void __launch_bounds__(512, 1) k_bg_add(const unsigned char *__restri
 #pragma unroll
             for (int k = 1; k < TOP; ++k) path = 2u * path + ((__shfl_sync(0xFFFFFFFFu, tw, 2 * (k - 1) + b) >> lane) & 1u);
             // byte offsets, entry e of subtree j at 4 (j E + e): R of the children of the unit's
-            // nodes above its subtrees, 32 bytes (eight entries) apart
+            // nodes above its subtrees, 32 bytes (eight entries) apart; the entry's own bits are ORed
+            // in below, so the counters lie on a 32-byte boundary (the array does, and so many tiles
+            // and units into it)
             uint32_t R[GS - 1];
             R[0] = 64u * path | ((w[b] << 5) & 32u);
 #pragma unroll
