@@ -248,9 +248,9 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
     constexpr int P = D * (D - 1) / 2, PP = (P + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ncol = sa.n_cols;
-    int *scode = reinterpret_cast<int *>(smem_raw);
-    uint32_t *sdw = reinterpret_cast<uint32_t *>(smem_raw + iv_up16((size_t)ncol * 4));
-    float *acc = reinterpret_cast<float *>(smem_raw + iv_up16((size_t)ncol * 4) + iv_up16((size_t)T * NW * 4));
+    uint16_t *scode = reinterpret_cast<uint16_t *>(smem_raw);  // codes of at most kSliceBits bits
+    uint32_t *sdw = reinterpret_cast<uint32_t *>(smem_raw + iv_up16((size_t)ncol * 2));
+    float *acc = reinterpret_cast<float *>(smem_raw + iv_up16((size_t)ncol * 2) + iv_up16((size_t)T * NW * 4));
     const int tid = threadIdx.x;
     const int64_t ntri = (int64_t)F * (F - 1) / 2;
     for (int64_t row = blockIdx.x; row < n; row += gridDim.x) {
@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv(const float *__restri
         }
         const float *x = C + row * ldc;
         for (int c = tid; c < ncol; c += kIvThreads)
-            scode[c] = decision_code(__ldg(x + __ldg(&sa.col[c].feature)), sa, c);
+            scode[c] = (uint16_t)decision_code(__ldg(x + __ldg(&sa.col[c].feature)), sa, c);
         __syncthreads();
         // decision words of every tree (bit v of word v / 32: left at inner node v)
         for (int t = tid; t < T; t += kIvThreads) {
@@ -353,9 +353,9 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__r
     constexpr int UP = (D - 4) * (1 << (D - 2)) + 2 > 1 ? (D - 4) * (1 << (D - 2)) + 2 : 1;  // sum of depths, nodes 0..NS-2
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int ncol = sa.n_cols;
-    int *scode = reinterpret_cast<int *>(smem_raw);
-    uint32_t *sdw = reinterpret_cast<uint32_t *>(smem_raw + iv_up16((size_t)ncol * 4));
-    float *acc = reinterpret_cast<float *>(smem_raw + iv_up16((size_t)ncol * 4) + iv_up16((size_t)T * NW * 4));
+    uint16_t *scode = reinterpret_cast<uint16_t *>(smem_raw);  // codes of at most kSliceBits bits
+    uint32_t *sdw = reinterpret_cast<uint32_t *>(smem_raw + iv_up16((size_t)ncol * 2));
+    float *acc = reinterpret_cast<float *>(smem_raw + iv_up16((size_t)ncol * 2) + iv_up16((size_t)T * NW * 4));
     const int tid = threadIdx.x;
     const int64_t ntri = (int64_t)F * (F - 1) / 2;
     for (int64_t row = blockIdx.x; row < n; row += gridDim.x) {
@@ -367,7 +367,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__r
         }
         const float *x = C + row * ldc;
         for (int c = tid; c < ncol; c += kIvThreads)
-            scode[c] = decision_code(__ldg(x + __ldg(&sa.col[c].feature)), sa, c);
+            scode[c] = (uint16_t)decision_code(__ldg(x + __ldg(&sa.col[c].feature)), sa, c);
         __syncthreads();
         for (int t = tid; t < T; t += kIvThreads) {
             if constexpr (FB) {
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kIvThreads) k_explain_iv_fold(const float *__r
 
 size_t iv_smem_bytes(int D, int F, int T, int n_cols, bool smem_acc) {
     const int NW = ((1 << D) - 1 + 31) / 32;
-    return iv_up16((size_t)n_cols * 4) + iv_up16((size_t)T * NW * 4) +
+    return iv_up16((size_t)n_cols * 2) + iv_up16((size_t)T * NW * 4) +
            (smem_acc ? iv_up16((size_t)F * (F - 1) / 2 * 4) : 0);
 }
 
