@@ -60,6 +60,13 @@ cudaError_t dalloc(T **p, size_t count, int64_t *bytes) {
     return e;
 }
 
+// Allocates *p unless an earlier call did (one of several buffers that failed half-way leaves the
+// others null: each is checked by itself).
+template <typename T>
+cudaError_t need(T **p, size_t count, int64_t *bytes) {
+    return *p ? cudaSuccess : dalloc(p, count, bytes);
+}
+
 template <typename T>
 void dfree(T *&p) {
     if (p) cudaFree(p);
@@ -204,13 +211,13 @@ wdf_status count_device_rows(wdf_ensemble *ens, const float *B, int64_t m, int64
 // mode) once, the B stages (the tables split for this mode) whenever the mode changes.
 wdf_status ensure_tensor_core_state(wdf_ensemble *e, int mode) {
     const wdf::Packed &p = e->pk;
-    if (!e->d_tiles128) {
+    if (!e->d_apk) {
         std::vector<int4> tiles;
         for (int gi = 0; gi < e->G; ++gi)
             for (int r0 = p.group_off[(size_t)gi]; r0 < p.group_off[(size_t)gi + 1]; r0 += 128)
                 tiles.push_back(make_int4(gi, r0, std::min(r0 + 128, p.group_off[(size_t)gi + 1]), 0));
-        WDF_CUDA(dalloc(&e->d_tiles128, std::max<size_t>(tiles.size(), 1), &e->bytes));
-        WDF_CUDA(dalloc(&e->d_err, 1, &e->bytes));
+        WDF_CUDA(need(&e->d_tiles128, std::max<size_t>(tiles.size(), 1), &e->bytes));
+        WDF_CUDA(need(&e->d_err, 1, &e->bytes));
         WDF_CUDA(cudaMemset(e->d_err, 0, sizeof(int)));
         if (!tiles.empty())
             WDF_CUDA(cudaMemcpy(e->d_tiles128, tiles.data(), tiles.size() * sizeof(int4), cudaMemcpyHostToDevice));
@@ -253,16 +260,14 @@ wdf_status ensure_frequency_state(wdf_ensemble *ens, wdf_precision precision, bo
     const wdf::Packed &p = ens->pk;
     const int K = 1 << p.D, N = p.D << p.D;
     const size_t hist_n = (size_t)p.T * p.NS * (2 * K);
-    if (!ens->d_hist) {
-        WDF_CUDA(dalloc(&ens->d_hist, hist_n, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_scale, (size_t)ens->n_live, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_sfold, hist_n * (wdf::slots_per_entry(p.D) + wdf::extra_slots(p.D)), &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_lines, (size_t)p.T * wdf::lines_words(p.D), &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_base, wdf::kBaseBlocks + 1, &ens->bytes));
-    }
-    if ((path_dependent || precision != WDF_FP32) && !ens->d_S) {
-        if (!ens->d_A) WDF_CUDA(dalloc(&ens->d_A, (size_t)ens->n_live * K, &ens->bytes));
-        WDF_CUDA(dalloc(&ens->d_S, (size_t)ens->n_live * N, &ens->bytes));
+    WDF_CUDA(need(&ens->d_hist, hist_n, &ens->bytes));
+    WDF_CUDA(need(&ens->d_scale, (size_t)ens->n_live, &ens->bytes));
+    WDF_CUDA(need(&ens->d_sfold, hist_n * (wdf::slots_per_entry(p.D) + wdf::extra_slots(p.D)), &ens->bytes));
+    WDF_CUDA(need(&ens->d_lines, (size_t)p.T * wdf::lines_words(p.D), &ens->bytes));
+    WDF_CUDA(need(&ens->d_base, wdf::kBaseBlocks + 1, &ens->bytes));
+    if (path_dependent || precision != WDF_FP32) {
+        WDF_CUDA(need(&ens->d_A, (size_t)ens->n_live * K, &ens->bytes));
+        WDF_CUDA(need(&ens->d_S, (size_t)ens->n_live * N, &ens->bytes));
     }
     ens->has_bg = 0;
     if (precision != WDF_FP32) return ensure_tensor_core_state(ens, tc_mode(precision));
