@@ -25,11 +25,11 @@ struct ExplainPlan {
 //    tree and leaf position at full occupancy, down to half of it with a block to itself;
 //    split, the parts' sums are written and read once more;
 //  - node values: 1.4 ps (depth 8: 2.2) per row and flush position, 8 ps per row and feature.
-// Measured at 200 trees of depth 6, 127 features (node values / parts on blocks / one block a
-// tile): 1,000 rows 36 / 70 / 205 us, 2,000 rows 56 / 71, 4,000 rows 100 / 86, 8,000 rows 177 /
-// 121; 1000 trees of depth 8, 100 rows 236 / 728; 500 trees of depth 7, 777 rows 130 / 156 /
-// 1380; 50 trees of depth 4, 255 features, 20,000 rows 87 / 49 (all before k_sum_values took its
-// parts side by side, which only moves the line further to where node values already win).
+// Measured (node values / parts on blocks / one block a tile): 200 trees of depth 6, 127 features,
+// 1,000 rows 29 / 68 / 211 us, 2,000 rows 47 / 68, 4,000 rows 88 / 82, 8,000 rows - / 118 / 224; 1000
+// trees of depth 8, 100 rows 99 / 706; 500 trees of depth 7, 777 rows 88 / 156 / 1149; 50 trees of
+// depth 4, 255 features, 20,000 rows 82 / 51.  The line is drawn a little early for calls of about
+// 4,000 rows of shallow trees (500 of depth 4: 60 / 79) and 1,000 of 100 trees of depth 8 (74 / 92).
 // Neither form takes more than kScratchBytes: node values are not chosen beyond, and split tiles
 // run one slice of the rows after another (a multiple of 128 rows).  293,300 rows, 1000 trees of
 // depth 8 and 134 features: 63.8 ms with the parts of all rows at once (1.26 GB), 64.5 in slices,
