@@ -104,8 +104,9 @@ wdf_status wdf_ensemble_info(const wdf_ensemble *ens, wdf_info *out);
 
 /*
  * Set the background B (m x F, leading dimension ldb) and run the consumer-independent
- * half of Algorithm 3: background pattern counts (step 1), pattern-pair tables (step
- * 2) and their contraction (step 3), in the given precision.  B is not retained; its
+ * half of Algorithm 3: background pattern counts (step 1), then the values of every leaf's
+ * patterns (steps 2 and 3), in the given precision: in WDF_FP32 straight from the counts by
+ * subset sums, else by contracting the pattern-pair tables.  B is not retained; its
  * decision codes pass through a buffer the ensemble keeps (up to 2^20 rows of codes).
  * Calls on one ensemble must not overlap on the GPU.
  * WDF_EUNSUPPORTED: m == 0 (an empty background is the path-dependent variant), or more
@@ -185,10 +186,11 @@ wdf_status wdf_explain(wdf_ensemble *ens, const float *C, int64_t n, int64_t ldc
  * "banzhaf_simplified_formula_interactions") when it is WDF_BANZHAF.
  * C: n x F consumer rows (DEVICE memory, row stride ldc >= F).  out: DEVICE memory, row
  * r of the result at out + r * ldo (ldo >= F * F), F x F row-major per row: symmetric,
- * out[i][j] = out[j][i] = the value of the pair (i, j), diagonal 0.  FP32 results from
- * an FP32 contraction of FP64-built tables; the additions into one element come from
- * many threads, so the last bits may change between runs.  Stream-ordered; takes a
- * temporary stream-ordered allocation (pair tables and per-leaf pair vectors).
+ * out[i][j] = out[j][i] = the value of the pair (i, j), diagonal 0.  FP32 results, from
+ * background counts by subset sums, from path-dependent frequencies by an FP32
+ * contraction of FP64-built tables; the additions into one element come from many
+ * threads, so the last bits may change between runs.  Stream-ordered; takes a temporary
+ * stream-ordered allocation (pair vectors; path-dependent: and pair tables).
  * WDF_EINVAL without a background (or path-dependent frequencies), for null pointers
  * or short strides. */
 wdf_status wdf_explain_interactions(wdf_ensemble *ens, const float *C, int64_t n, int64_t ldc, float *out,
@@ -256,7 +258,9 @@ wdf_status wdf_batch_tile_rows(const wdf_batch *batch, int32_t depth, int32_t *t
  * queued request in turn (round robin, so a large request does not hold back the ones
  * behind it) until the wave has max_wave_requests parts, about 16M rows x trees of
  * work, or the next part's device buffers (2 * rows * F * 4 bytes) would exceed
- * device_budget_bytes; it runs the wave as copies in, ONE batch launch
+ * device_budget_bytes (which counts these buffers only: beside them each slot's batch
+ * keeps its codes and up to 128 MB of partial sums, and the context's pool up to 384 MB
+ * between waves); it runs the wave as copies in, ONE batch launch
  * (wdf_batch_explain) and copies out on the slot's stream.  Waves of different slots
  * overlap on the GPU.  With four or more slots, slot 0 is an express slot: it takes only
  * requests of at most 2^20 rows x trees of remaining work, in waves of at most 2^22

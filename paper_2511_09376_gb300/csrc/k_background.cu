@@ -9,7 +9,6 @@
 // item 3, applied two levels up).
 #include <algorithm>
 #include <cmath>
-#include <cstdlib>
 
 #include "launch.h"
 #include "wdf_device.cuh"

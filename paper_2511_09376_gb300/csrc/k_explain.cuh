@@ -1,7 +1,7 @@
 // Consumer side of Algorithm 3, step 4 (Eq. "bg_shap_derivation" step (g)):
 // phi[c, i] = sum over trees and leaves of s_{l,i}[P[l][c]].
 //
-// A block takes a tile of consumer rows, one thread per row.  It stages its rows' sliced
+// A block takes a tile of consumer rows, two warps per 32 rows, a lane per row.  It stages its rows' sliced
 // decision codes (tree_layout.h) in shared memory together with a per-row phi accumulator
 // (feature-major) and walks the trees.  Per unit of a tree (31 nodes, eight bottom subtrees)
 // each warp
@@ -14,7 +14,8 @@
 //   - sums the slots of the nodes above the bottom subtrees in registers and adds every
 //     node's value into phi[feature of the node] in the fixed flush order of tree_layout.h, a
 //     batch at a time: a batch that repeats no feature reads its phi values before writing
-//     any, so the shared-memory round trips overlap; any other batch adds one by one.
+//     any, so the shared-memory round trips overlap; another batch adds its features' first
+//     positions so and the repeats after them (one by one where they repeat among themselves).
 //     Pass-through nodes add into a scratch row, a batch of pass-through nodes only is
 //     skipped.
 // The trees come in parts (explain_parts): a part's sums start from zero and are added to
@@ -34,7 +35,6 @@
 // translation unit so that they compile in parallel.
 #pragma once
 #include <algorithm>
-#include <cstdlib>
 
 #include "tree_layout.h"
 #include "launch.h"
