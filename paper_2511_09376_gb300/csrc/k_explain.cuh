@@ -259,9 +259,9 @@ __device__ __forceinline__ void unit_sums(const UnitSlots<D> &v, int u, float (&
 // 1,400 features of 16 to 255 thresholds on, to about 1,770).  The codes are read where they lie, in global memory, and a
 // feature's phi row is 32 floats, rotated by the feature's number (row r of feature f in word (r + f)
 // mod 32) so that its storing reads all banks, as the 33 floats of the other form do.  The same
-// additions in the same order.  48,640 rows, 17 thresholds a feature, the last width of the other form's
-// and the first of this one's at about: depth 6 18.0 / 18.6 ms (380 trees), depth 7 15.9 / 20.1 (185),
-// depth 8 16.9 / 14.8 (94); so the other form stays where it fits.
+// additions in the same order.  48,640 rows, 17 thresholds a feature, on both sides of the border (the
+// other form / this one): depth 6 18.0 / 18.6 ms (380 trees, 1,390 / 1,405 features), depth 7 15.9 / 20.1
+// (185, 1,375 / 1,402), depth 8 16.9 / 14.8 (94, 1,375 / 1,400); so the other form stays where it fits.
 template <int D, int TC, bool WIDE>
 __device__ __forceinline__ void explain_tile(const ExplainJob &job, const unsigned char *__restrict__ codes,
                                              int64_t n, float *__restrict__ phi, int64_t ldp, int64_t c0, int part0,
